@@ -11,7 +11,6 @@
 
 namespace keepkv {
 
-constexpr int kTile = 64;          // entries per K/V tile of the decode kernel
 constexpr int kDecMaxCtas = 512;    // upper bound on the persistent decode grid (sizes the partial pool)
 
 constexpr int kMaxUnits = 4096;    // B * H_kv that keepkv_compress accepts (per-unit tables live in shared memory)

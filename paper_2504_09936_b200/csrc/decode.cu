@@ -1,36 +1,41 @@
 // keepkv_decode_attention: Electoral-Votes attention (Eq. 6) over the cache, with the per-entry
 // score estimate of Eq. 8 advanced in the same pass.
 //
-// Work is the list of all 64-entry tiles of all (sequence, kv-head) units, in unit order.  A
-// persistent grid (two CTAs per SM) cuts the list into equal contiguous ranges, so ragged batches
-// and any number of units load every SM alike; a unit whose tiles fall into several ranges is
-// finished by the last of those CTAs to arrive (one ticket per unit), in a fixed order, so results
-// are bit-reproducible.
+// Work.  Every unit's entries are cut into groups of 32; a CTA owns a contiguous range of groups and walks it in tiles
+// of up to 128 entries, a segment being the part of its range that lies in one unit.  Up to two units per SM, the grid is
+// one cluster of 8, 4, 2 or 1 CTAs per unit; if the units are about equally long -- every steady-state step -- the CTAs
+// of a cluster split their unit evenly and send their partial results to each other's shared memory: one cluster
+// barrier, then each folds its share of the outputs in rank order.  (Through global memory -- fence, ticket, the last to
+// arrive reads the others' partials -- the same meeting took 1.5 to 4 us behind the next launch's loads.)  Otherwise the
+// list of all groups is cut into equal ranges, and a unit that lies in several of them is finished through global memory
+// by the last of their CTAs to arrive (one ticket per unit), in a fixed order, so results are bit-reproducible.
 //
-// With a moderate number of units (two dozen to one per SM) the grid is launched as clusters of S <= 8 CTAs, one
-// cluster per unit, S * units <= two CTAs per SM.  If the units are about equally long -- every steady-state
-// step -- a cluster splits its unit's tiles evenly, and the S partial results meet in distributed shared
-// memory instead of global memory: each CTA leaves its partial in its own shared memory, a cluster barrier,
-// each CTA folds 1/S of the outputs from its peers' memories (in rank order), a second barrier.  Ragged
-// batches fall back to the equal ranges over the whole list, whatever the launch shape.
-//
-// One CTA = 4 warps.  Thread 0 also walks the range as producer: per tile it issues TMA loads of the
-// K and V tiles (128-byte swizzled boxes), bulk copies of the tile's votes and lscore, and a small
-// descriptor, into a ring of shared-memory stages guarded by full/empty mbarriers, two tiles ahead
-// of the arithmetic.  The two warp pairs take alternate tiles; a warp owns 32 entries of its tile:
-// the G query heads of the unit are the
-// rows of an m16n8k16 bf16 MMA (rows >= G are zero), so K is read once for all heads; logits come
-// out in fp32; the vote weight enters as + log2 p_i before the online softmax
-// (p_i e^{l_i} = 2^{l_i log2 e + log2 p_i}), and the probabilities go back into the tensor core
-// split into a bf16 head (A rows 0-7) and a bf16 remainder (A rows 8-15), so that P.V keeps
-// fp32-level accuracy in one MMA.  The Eq. 8 update is done one entry per lane, from the logits the
-// warp exchanges through shared memory.
+// Bound: the K / V stream; for a few units also the chain of one tile -- load, first product, softmax, second product,
+// 0.5 + 0.4 + 0.5 us after the load.  The arithmetic is arranged so that it costs few instructions and registers
+// (112-128 registers at 224 threads, two CTAs per SM; the mma.sync form of this kernel needed 255 at 128 threads and took
+// 16.2 us where this takes 14.3 us: 64 units of 1702 entries, G = 4, d = 128; 27.7 -> 23.0 us: 512 units of 442, G = 1).
+// Roles of the seven warps:
+//   warps 0-3  one entry per thread: logits of the G heads from tensor memory, Eq. 8, softmax weights; then one
+//              channel per thread: the tile's weighted value sum from tensor memory is added to the segment's;
+//   warps 4-5  tensor cores: S[entry, head] = K Q^T (M = 128 entries, the key tile as it lies in the ring) and
+//              O[channel, head] = V^T P (M = 128 channels, the value tile read as an MN-major operand), one elected
+//              thread each, fp32 accumulators in tensor memory; they also stage the unit's queries, patch the
+//              appended row, publish the new lengths and write the results of sequences without entries;
+//   warp 6     one thread: TMA copies of key and value tiles, alternating, into a ring of three 128-entry slots.
+// The weights p_i e^{l_i} = 2^{l_i log2 e + log2 p_i} enter the second product split into a bf16 head (columns 0-7) and
+// a bf16 remainder (columns 8-15), so that it keeps fp32-level accuracy; its accumulator is fresh for every tile, so a
+// growing maximum rescales G registers per thread and nothing in tensor memory.
+// At d = 64 a value tile has 64 channels: the two halves of a tile's entries take the upper and lower 64 rows of the
+// product (columns 0-15 for the first half, 16-31 for the second) and are added when the segment ends.
 //
 // keepkv_decode_step runs the same kernel with the step's new token (Eq. 2) folded in: lengths count the fresh
-// entry from the start; the warp that owns its row patches it into the tile it has just received (and stores
-// it to the cache), so that the attention sees it.  The new lengths are published when nobody reads the old
-// ones any more: every CTA copies the lengths into shared memory first and then signs off on a counter, and
-// the last one to sign off writes them (batches beyond kSeqCache sequences: the last CTA to finish does).
+// entry from the start; warps 4 and 5 patch its row into the tiles they have just received (and stores it to the cache). The new
+// lengths are published when nobody reads the old ones any more: every CTA copies the lengths into shared memory first
+// and then signs off on a counter, and the last one to sign off writes them (batches beyond kSeqCache sequences: the
+// last CTA to finish does).
+//
+// Every wait is bounded.  One that runs out marks the CTA (s_abort): its warps go on through their barriers without
+// waiting and without arithmetic, copies and products in flight get a bounded time to end, KEEPKV_DEV_TIMEOUT is raised.
 #include <mutex>
 
 #include "common.cuh"
@@ -38,50 +43,29 @@
 
 namespace keepkv {
 
-constexpr int kDecConsumers = 4;                  // warps per CTA
-constexpr int kDecThreads = 32 * kDecConsumers;   // 128 threads leave each of them up to 255 registers at two CTAs per SM
-constexpr int kSeqCache = 256;                    // sequence lengths a CTA keeps in shared memory
+constexpr int kDecThreads = 224;   // four softmax warps, two tensor-core warps, copy warp
+constexpr int kDecTile = 128;      // entries of a tile: lanes of tensor memory
+constexpr int kGroup = 32;         // entries of a work group: granularity of the split and of a partial tile's copies
+constexpr int kSeqCache = 256;     // sequence lengths a CTA keeps in shared memory
+constexpr int kDecTmemCols = 128;  // S: 2 x 16 columns, O: 2 x 16 (d = 64: 2 x 32)
+constexpr int kMinGroups = 2;      // groups a range of the equal split holds at least
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 
-// Descriptor the producer leaves with every tile.
-struct TileDesc {
-  int u;          // unit
-  int tile;       // tile index inside the unit
-  int len;        // valid entries of the unit
-  int flags;      // bit 0: first tile of this CTA's segment of the unit, bit 1: last tile of the segment
-  int c_first;    // first CTA that holds a segment of the unit
-  int nparts;     // CTAs that hold a segment of the unit
-  int u_next;     // unit of the next tile of this CTA's range when this tile ends its unit, else -1
-  int fresh;      // row inside the tile of the entry this call appends, -1 if the tile does not hold it
-};
-
 template <int D>
 struct DecSmem {
-  static constexpr int kSub = D / 64;
-  static constexpr int kSubBytes = kTile * 128;
-  static constexpr int kK = 0;
-  static constexpr int kV = kSub * kSubBytes;
-  static constexpr int kVotes = 2 * kSub * kSubBytes;
-  static constexpr int kLscore = kVotes + kTile * 4;
-  static constexpr int kTxBytes = kLscore + kTile * 4;                 // what the async copies deliver
-  static constexpr int kDesc = kTxBytes;
-  static constexpr int kStride = (kDesc + 32 + 1023) / 1024 * 1024;    // sub-tiles need 1024-byte alignment
-  static constexpr int kStages = D == 128 ? 3 : 6;
-  // Per consumer warp one region that serves two purposes at different times: while the warp works on
-  // a tile, the logits it exchanges (f32 [8 heads][32 entries]) and the log2 votes (f32 [32]); while a
-  // segment is combined, the warp's numerators (f32 [4 heads][D]).  A warp writes its numerators only
-  // after its own tile work, and the others read them only between the barriers of the combine.
-  static constexpr int kWarpRegion = (4 * D * 4 > 8 * 32 * 4 + 32 * 4) ? 4 * D * 4 : 8 * 32 * 4 + 32 * 4;
-  static constexpr int kComb = kStages * kStride;
-  static constexpr int kML = kComb + kDecConsumers * kWarpRegion;      // f32 [4 warps][8][2]
-  static constexpr int kBytes = kML + kDecConsumers * 8 * 2 * 4;
+  static constexpr int kSub = D / 64;                        // 64-channel (128-byte) sub-tiles of a row
+  static constexpr int kSubBytes = kDecTile * 128;
+  static constexpr int kSlotBytes = kSub * kSubBytes;        // a key or a value tile
+  static constexpr int kSlots = D == 128 ? 3 : 6;            // two CTAs per SM
+  static constexpr int kQ = kSlots * kSlotBytes;             // bf16 [2][kSub][8 heads][64], swizzled
+  static constexpr int kQBytes = kSub * 1024;
+  static constexpr int kP = kQ + 2 * kQBytes;                // bf16 [2 halves of the tile][16][64], swizzled
+  // what the CTAs of a cluster send one another when their unit ends: f32 [rank][16 maxima and sums], then numerators
+  static constexpr int kInbox = kP + 4096;
+  template <int G> static constexpr int bytes() { return kInbox + (8 * 16 + G * D) * 4; }
+  // (the query operand's columns 8-15, which nobody reads, are whatever follows a sub-tile of kQ: always inside)
 };
-
-// Byte offset of 16-byte chunk `chunk` (0..D/8-1) of tile row `row` inside a swizzled K or V tile.
-__device__ __forceinline__ uint32_t swz(int row, int chunk) {
-  return (uint32_t)((chunk >> 3) * (kTile * 128) + row * 128 + (((chunk & 7) ^ (row & 7)) << 4));
-}
 
 __device__ __forceinline__ float ex2f(float x) {
   float y;
@@ -108,56 +92,68 @@ struct PartRec {
   float acc[G * D];
 };
 
-// kEarly: the variant for KEEPKV_FLAG_CACHE_IDLE (a compile-time choice: as a run-time branch the same code lost the
-// gain and 0.4 us more, measured).
+// Position of a role in its CTA's range.
+struct DecWalk {
+  int b, h;        // sequence, kv head
+  int len, gb;     // entries of the unit, its groups
+  int g, left;     // first group of the current tile inside the unit; groups left in the range, this tile included
+  int start;       // list position of the unit's first group (equal ranges only)
+  int fresh;       // row of the entry this call appends to the unit, -1 if none
+  bool first;      // the tile opens a segment
+  __device__ __forceinline__ int groups() const { return min(kDecTile / kGroup, min(gb - g, left)); }
+  __device__ __forceinline__ bool last(int n) const { return n == left || g + n == gb; }
+};
+
+// kEarly: the variant for KEEPKV_FLAG_CACHE_IDLE (lengths, votes, scores and tiles are requested before the wait for the
+// preceding kernel).
 template <int D, int G, bool kEarly>
 __global__ void __launch_bounds__(kDecThreads, 2)
-decode_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapV, keepkv_params p,
+decode_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapV,
+              keepkv_params p,
               keepkv_cache c, const __nv_bfloat16 *__restrict__ q, __nv_bfloat16 *__restrict__ out,
               float *__restrict__ lse, int update_scores, int *counters, PartRec<D, G> *pool, int32_t *status_dev,
               const uint4 *__restrict__ k_new, const uint4 *__restrict__ v_new, int spin_limit, int withhold) {
   using SL = DecSmem<D>;
-  constexpr int S = SL::kStages;
-  constexpr int KS = D / 16;   // k-steps of the QK^T product
-  constexpr int NT = D / 8;    // 8-channel n-tiles of the PV product
+  constexpr int S = SL::kSlots;
+  constexpr int NO = D == 128 ? 16 : 32;   // columns of the second product
+  constexpr uint32_t IDESC_S = umma_idesc_bf16(128, 16), IDESC_O = umma_idesc_bf16(128, NO) | kUmmaTransposeA;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t full_bar[S], empty_bar[S];
-  __shared__ int s_scan[8], s_tbmax[4];
-  __shared__ int s_start[4];   // b, h, tile of the first tile of this CTA's range
+  __shared__ __align__(8) uint64_t bars[2 * S + 8];   // full[S], empty[S], s_full[2], o_full[2], p_full[2], drain[2]
+  __shared__ __align__(16) float s_wmax[2][8][4];     // per-warp maxima of a tile
+  __shared__ float s_wsum[4][8];                      // per-warp sums of a segment
+  __shared__ int s_scan[8], s_tbmax[8];
+  __shared__ int s_start[5];        // b, h, group, unit's list position, groups of this CTA's range
+  __shared__ uint32_t s_tmem;
   __shared__ volatile int s_abort;
-  __shared__ volatile int s_issued, s_stop;   // tiles the producer has handed over; first tile that never will be
   __shared__ int s_last, s_finisher;
-  __shared__ int s_seq[kSeqCache];   // the lengths as they were when the kernel started
+  __shared__ int s_seq[kSeqCache];  // the lengths as they were when the kernel started
 
-  // dynamic shared memory is only guaranteed 16-byte aligned: round up to the swizzle atom
-  // (the offset is added to the array itself, so that the compiler still knows every derived pointer as shared memory)
   uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-  const uint32_t smem_base = smem_u32(smem);
+  const uint32_t sbase = smem_u32(smem);
+  const uint32_t bar_full = smem_u32(&bars[0]), bar_empty = smem_u32(&bars[S]), bar_s = smem_u32(&bars[2 * S]);
+  const uint32_t bar_o = smem_u32(&bars[2 * S + 2]), bar_p = smem_u32(&bars[2 * S + 4]), bar_drain = smem_u32(&bars[2 * S + 6]);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int cta = blockIdx.x, grid = gridDim.x;
   const int U = p.B * p.H_kv;
 
   if (tid == 0) {
-    for (int i = 0; i < S; ++i) { mbar_init(smem_u32(&full_bar[i]), 1); mbar_init(smem_u32(&empty_bar[i]), kDecConsumers); }
+    for (int i = 0; i < S; ++i) { mbar_init(bar_full + 8 * i, 1); mbar_init(bar_empty + 8 * i, 1); }
+    for (int i = 0; i < 2; ++i) { mbar_init(bar_s + 8 * i, 1); mbar_init(bar_o + 8 * i, 1); }
+    for (int i = 0; i < 2; ++i) { mbar_init(bar_p + 8 * i, 4); mbar_init(bar_drain + 8 * i, 1); }
     s_abort = 0;
-    s_issued = 0;
-    s_stop = 0x7fffffff;
     s_start[0] = p.B;
+    s_start[4] = 0;
     mbar_fence_init();
-    fence_proxy_async_smem();
-    prefetch_tensormap(&mapK);
-    prefetch_tensormap(&mapV);
   }
-  // With KEEPKV_FLAG_CACHE_IDLE the preceding kernel of the stream does not write this cache: the lengths and the
-  // first tiles are then requested before the wait for that kernel, behind whose tail they arrive.  Everything else
-  // (queries, the token to append, the workspace, every write) stays behind the wait.
-  constexpr bool early = kEarly;
-  if (!early) {
+  if (tid == 32) { prefetch_tensormap(&mapK); prefetch_tensormap(&mapV); }
+  const int csize = (int)cluster_nctarank(), crank = (int)cluster_ctarank(), cshift = 31 - __clz(csize);   // (1, 2, 4 or 8)
+  if (csize > 1) cluster_arrive();   // waited for below: nobody writes to a CTA that has not started
+  if (!kEarly) {
     pdl_wait();      // everything above ran while the previous kernel of the stream was finishing
     pdl_trigger();
   }
 
-  // ---- the tile list: every thread sums a block of consecutive sequences, a block scan gives the offsets
+  // ---- the list of groups: every thread sums a block of consecutive sequences, a block scan gives the offsets
   // entries of sequence b this call attends to: with a token to append, the fresh entry counts
   const bool cached = p.B <= kSeqCache;   // then every thread copies the lengths of its block of sequences below
   auto old_len = [&](int b) { return cached ? s_seq[b] : c.seq_len[b]; };
@@ -166,633 +162,554 @@ decode_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ 
     if (k_new && n >= 0 && n < p.N_cap) ++n;
     return max(0, min(n, p.N_cap));
   };
-  auto tiles_of = [&](int b) { return (len_of(b) + kTile - 1) / kTile; };
+  auto fresh_of = [&](int b) { const int n = old_len(b); return k_new && n >= 0 && n < p.N_cap ? n : -1; };
+  auto groups_of = [&](int b) { return (len_of(b) + kGroup - 1) / kGroup; };
   const int per = (p.B + kDecThreads - 1) / kDecThreads;
   const int b_lo = min(p.B, tid * per), b_hi = min(p.B, b_lo + per);
-  int mine = 0, tb_max = 0;
+  int mine = 0, gb_max = 0;
   for (int b = b_lo; b < b_hi; ++b) {
     if (cached) s_seq[b] = c.seq_len[b];   // read back by this thread here, by the others after the barrier below
-    const int tb = tiles_of(b);
-    mine += tb;
-    tb_max = max(tb_max, tb);
+    const int n = groups_of(b);
+    mine += n;
+    gb_max = max(gb_max, n);
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) tb_max = max(tb_max, __shfl_xor_sync(0xffffffffu, tb_max, o));
+  gb_max = __reduce_max_sync(0xffffffffu, gb_max);
   int incl = mine;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const int y = __shfl_up_sync(0xffffffffu, incl, o);
     if (lane >= o) incl += y;
   }
-  if (lane == 31) { s_scan[warp] = incl; s_tbmax[warp] = tb_max; }
+  if (lane == 31) { s_scan[warp] = incl; s_tbmax[warp] = gb_max; }
   __syncthreads();
   int before = incl - mine, total_b = 0;
-  for (int w = 0; w < kDecConsumers; ++w) {
+#pragma unroll
+  for (int w = 0; w < kDecThreads / 32; ++w) {
     if (w < warp) before += s_scan[w];
     total_b += s_scan[w];
+    gb_max = max(gb_max, s_tbmax[w]);
   }
-  const long long T = (long long)total_b * p.H_kv;
-  // Equal ranges of `chunk` tiles per CTA.  When every unit has the same number of tiles and a range holds more than
-  // one unit, the range is rounded up to whole units (if that costs at most an eighth more tiles per CTA): no unit is
-  // then cut between two CTAs, and none of them needs the partial results and the ticket.
-  int chunk = (int)((T + grid - 1) / grid);
+  const int T = total_b * p.H_kv;   // (below 2^26: the rows of a cache are indexed by 32-bit TMA coordinates)
   // one cluster per unit, if the launch has them and no sequence is much longer than the average
-  const int csize = (int)cluster_nctarank(), crank = (int)cluster_ctarank();
-  tb_max = max(max(s_tbmax[0], s_tbmax[1]), max(s_tbmax[2], s_tbmax[3]));
-  if (tb_max > 0 && (long long)tb_max * p.B == total_b && chunk > tb_max) {
-    const int up = (chunk + tb_max - 1) / tb_max * tb_max;
+  const bool split = grid == U << cshift && (long long)gb_max * p.B * 4 <= 5LL * total_b;
+  int chunk = max((T + grid - 1) / grid, kMinGroups);
+  // Equal ranges: when every unit has the same number of groups and a range holds more than one unit, the range is
+  // rounded up to whole units (if that costs at most an eighth more): no unit is then cut between two CTAs.
+  if (gb_max > 0 && gb_max * p.B == total_b && chunk > gb_max) {
+    const int up = (chunk + gb_max - 1) / gb_max * gb_max;
     if (up * 8 <= chunk * 9) chunk = up;
   }
-  const bool aligned = csize > 1 && grid == U * csize && total_b > 0 && (long long)tb_max * p.B * 4 <= 5LL * total_b;
-  long long g0 = min(T, (long long)cta * chunk), g1 = min(T, g0 + chunk);
-  int tb_unit = 0;   // aligned: tiles of this cluster's unit
-  if (aligned) {
-    const int ub = (cta / csize) / p.H_kv;
-    tb_unit = tiles_of(ub);
-    const int t_lo = (int)((long long)crank * tb_unit / csize), t_hi = (int)((long long)(crank + 1) * tb_unit / csize);
-    g0 = t_lo;   // only the tile count matters below
-    g1 = t_hi;
-    if (tid == 0 && t_hi > t_lo) { s_start[0] = ub; s_start[1] = (cta / csize) % p.H_kv; s_start[2] = t_lo; }
-  }
-  const int ntiles = (int)(g1 - g0);
-  if (!aligned && ntiles > 0 && (long long)before * p.H_kv <= g0 && g0 < (long long)(before + mine) * p.H_kv) {
-    long long at = (long long)before * p.H_kv;
-    for (int b = b_lo; b < b_hi; ++b) {
-      const int tb = tiles_of(b);
-      const long long span = (long long)tb * p.H_kv;
-      if (g0 < at + span) {
-        const int r = (int)(g0 - at);
-        s_start[0] = b; s_start[1] = r / tb; s_start[2] = r % tb;
-        break;
+  if (split) {
+    if (tid == 0) {
+      const int u = cta >> cshift, b = u / p.H_kv, gb = groups_of(b);
+      const int lo = (crank * gb) >> cshift, hi = ((crank + 1) * gb) >> cshift;
+      s_start[0] = b; s_start[1] = u % p.H_kv; s_start[2] = lo; s_start[3] = 0; s_start[4] = hi - lo;
+    }
+  } else {
+    const int g0 = (int)min((long long)T, (long long)cta * chunk), g1 = min(T, g0 + chunk);
+    if (g1 > g0 && before * p.H_kv <= g0 && g0 < (before + mine) * p.H_kv) {
+      int at = before * p.H_kv;
+      for (int b = b_lo; b < b_hi; ++b) {
+        const int gb = groups_of(b), span = gb * p.H_kv;
+        if (g0 < at + span) {
+          const int r = g0 - at;
+          s_start[0] = b; s_start[1] = r / gb; s_start[2] = r % gb; s_start[3] = g0 - r % gb; s_start[4] = g1 - g0;
+          break;
+        }
+        at += span;
       }
-      at += span;
     }
   }
   __syncthreads();
-  // ------------------------------------------------------------ producer state (thread 0)
-  int pb = 0, ph = 0, ptile = 0, plen = 0, ptb = 1, pit = 0;
-  if (tid == 0 && ntiles > 0) {
-    pb = s_start[0]; ph = s_start[1]; ptile = s_start[2];
-    plen = len_of(pb);
-    ptb = (plen + kTile - 1) / kTile;
-  }
-  // Issues the copies of tile `pit` of the range (thread 0 only); false if the stage never came free.
-  auto issue_tile = [&]() -> bool {
-    const int it = pit, stage = it % S;
-    if (!mbar_wait_n(smem_u32(&empty_bar[stage]), ((it / S) & 1) ^ 1, spin_limit)) return false;
-    const long long cur = g0 + it;
-    const int u = pb * p.H_kv + ph;
-    const long long us = cur - ptile, ue = us + ptb;
-    TileDesc d;
-    d.u = u; d.tile = ptile; d.len = plen;
-    d.flags = ((it == 0 || ptile == 0) ? 1 : 0) | ((it == ntiles - 1 || ptile == ptb - 1) ? 2 : 0);
-    if (aligned) {   // every CTA of the cluster holds a partial (possibly empty) unless the unit is a single tile
-      d.c_first = 0;
-      d.nparts = ptb == 1 ? 1 : csize;
-    } else if (T < 0x7fffffffLL) {   // (64-bit divisions cost this one thread hundreds of cycles per tile)
-      d.c_first = (int)us / chunk;
-      d.nparts = ((int)ue - 1) / chunk - d.c_first + 1;
-    } else {
-      d.c_first = (int)(us / chunk);
-      d.nparts = (int)((ue - 1) / chunk) - d.c_first + 1;
-    }
-    d.u_next = -1;
-    d.fresh = -1;
-    if (k_new) {
-      const int old = old_len(pb);   // the fresh entry goes to row `old` of the unit
-      if (old >= 0 && old < p.N_cap && old / kTile == ptile) d.fresh = old % kTile;
-    }
-    const size_t ubase = (size_t)u * p.N_cap;
-    const int row = (int)ubase + ptile * kTile;
-    const int this_tile = ptile;
-    // next tile of the list (units without entries have no tiles)
-    if (++ptile == ptb && it + 1 < ntiles) {
-      ptile = 0;
-      if (++ph == p.H_kv) {
-        ph = 0;
+  DecWalk w;
+  w.b = s_start[0]; w.h = s_start[1]; w.g = s_start[2]; w.start = s_start[3]; w.left = s_start[4];
+  w.first = true;
+  w.len = w.left > 0 ? len_of(w.b) : 0;
+  w.gb = (w.len + kGroup - 1) / kGroup;
+  w.fresh = w.left > 0 ? fresh_of(w.b) : -1;
+  // to the next tile: n groups of this one are done
+  auto advance = [&](DecWalk &w, int n) {
+    w.g += n;
+    w.left -= n;
+    w.first = false;
+    if (w.g == w.gb && w.left > 0) {
+      w.g = 0;
+      w.first = true;
+      w.start += w.gb;
+      if (++w.h == p.H_kv) {
+        w.h = 0;
         do {
-          ++pb;
-          plen = len_of(pb);
-          ptb = (plen + kTile - 1) / kTile;
-        } while (ptb == 0);
+          ++w.b;
+          w.len = len_of(w.b);
+          w.gb = (w.len + kGroup - 1) / kGroup;
+        } while (w.gb == 0);   // (sequences without entries have no groups)
+        w.fresh = fresh_of(w.b);
       }
-      d.u_next = pb * p.H_kv + ph;
     }
-    uint8_t *st = smem + stage * SL::kStride;
-    *reinterpret_cast<TileDesc *>(st + SL::kDesc) = d;
-    const uint32_t bar = smem_u32(&full_bar[stage]);
-    const uint32_t dst = smem_base + stage * SL::kStride;
-    if (it == withhold) {   // test hook: the tile is announced, its copies are never issued
-      ++pit;
-      __threadfence_block();
-      s_issued = pit;
-      return true;
-    }
-    mbar_expect_tx(bar, SL::kTxBytes);
-    tma_load_3d(dst + SL::kK, &mapK, 0, row, 0, bar);   // both 64-channel halves of the tile in one copy
-    tma_load_3d(dst + SL::kV, &mapV, 0, row, 0, bar);
-    bulk_load_1d(dst + SL::kVotes, c.votes + ubase + (size_t)this_tile * kTile, kTile * 4, bar);
-    bulk_load_1d(dst + SL::kLscore, c.lscore + ubase + (size_t)this_tile * kTile, kTile * 4, bar);
-    ++pit;
-    __threadfence_block();
-    s_issued = pit;   // the descriptor of every tile below pit is in place
-    return true;
   };
-  // One cluster per unit: tile `it` of this CTA is tile a_tlo + it of the cluster's unit, so its descriptor needs
-  // none of the walk over sequences and heads above (about 400 cycles per tile of this one thread).
-  const int a_u = aligned ? cta / csize : 0;
-  const int a_len = aligned ? len_of(a_u / p.H_kv) : 0;
-  const int a_tlo = aligned ? (int)g0 : 0;
-  int a_fresh_tile = -1, a_fresh_row = -1;
-  if (aligned && k_new) {
-    const int old = old_len(a_u / p.H_kv);
-    if (old >= 0 && old < p.N_cap) { a_fresh_tile = old / kTile; a_fresh_row = old % kTile; }
-  }
-  auto issue_aligned = [&]() -> bool {
-    const int it = pit, stage = it % S;
-    if (!mbar_wait_n(smem_u32(&empty_bar[stage]), ((it / S) & 1) ^ 1, spin_limit)) return false;
-    const int tile = a_tlo + it;
-    TileDesc d;
-    d.u = a_u; d.tile = tile; d.len = a_len;
-    d.flags = (it == 0 ? 1 : 0) | (it == ntiles - 1 ? 2 : 0);
-    d.c_first = 0;
-    d.nparts = tb_unit == 1 ? 1 : csize;
-    d.u_next = -1;
-    d.fresh = tile == a_fresh_tile ? a_fresh_row : -1;
-    *reinterpret_cast<TileDesc *>(smem + stage * SL::kStride + SL::kDesc) = d;
-    if (it != withhold) {   // (test hook: the tile is announced, its copies are never issued)
-      const uint32_t bar = smem_u32(&full_bar[stage]);
-      const uint32_t dst = smem_base + stage * SL::kStride;
-      const size_t ubase = (size_t)a_u * p.N_cap;
-      const int row = (int)ubase + tile * kTile;
-      mbar_expect_tx(bar, SL::kTxBytes);
-      tma_load_3d(dst + SL::kK, &mapK, 0, row, 0, bar);
-      tma_load_3d(dst + SL::kV, &mapV, 0, row, 0, bar);
-      bulk_load_1d(dst + SL::kVotes, c.votes + ubase + (size_t)tile * kTile, kTile * 4, bar);
-      bulk_load_1d(dst + SL::kLscore, c.lscore + ubase + (size_t)tile * kTile, kTile * 4, bar);
-    }
-    ++pit;
-    __threadfence_block();
-    s_issued = pit;
-    return true;
+  // row inside the current tile of the entry this call appends, -1 if the tile does not hold it
+  auto fresh_row = [&](const DecWalk &w) {
+    const int r = w.fresh - w.g * kGroup;
+    return w.fresh >= 0 && r >= 0 && r < w.groups() * kGroup ? r : -1;
   };
-  auto issue_next = [&]() -> bool { return aligned ? issue_aligned() : issue_tile(); };
-  if (tid == 0) {
-    const int first = early ? S : S - 1;   // nothing else to do before the wait: fill the whole ring
-    while (pit < ntiles && pit < first)
-      if (!issue_next()) { s_stop = pit; s_abort = 1; break; }
-  }
-  if (early) {
-    pdl_wait();
-    pdl_trigger();   // only now: the next launch may run ahead of this one, never of this one's predecessor
-  }
-  if (k_new && cached && tid == kDecThreads - 1) {
-    // every CTA signs off once it holds its copy of the lengths; the last one publishes the new ones (this thread
-    // is not the producer: its wait for the counter hides behind the first tile's flight)
-    if (atomicAdd(&counters[U], 1) == grid - 1) {
-      counters[U] = 0;   // ready for the next call
-      for (int b = 0; b < p.B; ++b) {
-        const int n = s_seq[b];
-        if (n >= 0 && n < p.N_cap) c.seq_len[b] = n + 1;
-        else atomicOr(status_dev, KEEPKV_DEV_APPEND_FULL);
-      }
+  if (csize > 1) cluster_wait();
+  const uint32_t inbox = sbase + SL::kInbox;
+  // Bounded wait that also ends when another warp of the CTA has given up.
+  auto wait_bar = [&](uint32_t bar, uint32_t parity) {
+    for (int k = 0; k < spin_limit; ++k) {
+      if (mbar_try_wait(bar, parity)) return true;
+      if (s_abort) return false;
     }
-  }
+    return false;
+  };
 
-
-  {
-    // ------------------------------------------------------------ the arithmetic
-    const int g = lane >> 2, qd = lane & 3;   // MMA row (query head) and position inside the quad
-    const int pair = warp >> 1;               // the two warp pairs take alternate tiles
-    const int r0 = (warp & 1) * 32;           // this warp's 32 rows inside a tile
-    const int ctid = tid;                     // 0..127
-    constexpr int WR = SL::kWarpRegion / 4;   // floats per warp region
-    float *comb = reinterpret_cast<float *>(smem + SL::kComb);
-    float *cml = reinterpret_cast<float *>(smem + SL::kML);
-    float *sc_w = comb + warp * WR;
-    float *lp_w = sc_w + 8 * 32;
-
-    // sequences without entries: output 0, lse = -inf
-    for (int u = cta; u < U; u += grid) {
-      const int b = u / p.H_kv, h = u % p.H_kv;
-      if (len_of(b) <= 0) {
-        for (int idx = ctid; idx < G * D; idx += 32 * kDecConsumers)
-          out[((size_t)b * p.H_q + h * G) * D + idx] = __float2bfloat16_rn(0.f);
-        if (lse && ctid < G) lse[(size_t)b * p.H_q + h * G + ctid] = -CUDART_INF_F;
+  if (warp == 6) {
+    // ------------------------------------------------------------ copies
+    if (elect_one()) {
+      // order: K0 K1 V0 K2 V1 ... -- a value tile is asked for when the key tile after it has been, so that it arrives
+      // about when its weights are ready and does not sit in the ring before
+      DecWalk ak = w, av = w;
+      int i = 0, tk = 0, tv = 0;
+      uint32_t held = 0;   // slots whose copies the test hook has withheld
+      bool go = true;
+      while (go && av.left > 0) {
+        const bool is_v = ak.left == 0 || tk > tv + 1;
+        DecWalk &a = is_v ? av : ak;
+        const int n = a.groups(), row = (a.b * p.H_kv + a.h) * p.N_cap + a.g * kGroup, slot = i % S;
+        if (i >= S) {
+          // (the ring drains only when the other warps have passed their wait: not a time to poll for)
+          if (kEarly && i == S) pdl_wait();
+          if (!wait_bar(bar_empty + 8 * slot, ((i / S) & 1) ^ 1)) { s_abort = 1; go = false; break; }
+        }
+        if ((is_v ? tv : tk) != withhold) {   // (test hook: these copies are never issued)
+          const uint32_t bar = bar_full + 8 * slot, dst = sbase + slot * SL::kSlotBytes;
+          mbar_expect_tx(bar, (uint32_t)(n * kGroup * 128 * SL::kSub));
+#pragma unroll
+          for (int k = 0; k < kDecTile / kGroup; ++k)
+            if (k < n)
+#pragma unroll
+              for (int sub = 0; sub < SL::kSub; ++sub)
+                tma_load_2d(dst + sub * SL::kSubBytes + k * (kGroup * 128), is_v ? &mapV : &mapK, sub * 64, row + k * kGroup, bar);
+        } else {
+          held |= 1u << slot;
+        }
+        if (is_v) { advance(av, n); ++tv; } else { advance(ak, n); ++tk; }
+        ++i;
       }
+      // nobody leaves before the last copies have landed (bounded; only a CTA that gave up has not waited for them)
+      for (int k = max(0, i - S); k < i; ++k)
+        if (!(held >> (k % S) & 1)) mbar_wait_n(bar_full + 8 * (k % S), (k / S) & 1, spin_limit);
     }
-
+    __syncwarp();
+  } else if (warp == 4 || warp == 5) {
+    // ------------------------------------------------------------ tensor cores
+    // The first product of a tile is issued by warp 4, the second by warp 5: a step of either costs about half a
+    // microsecond of its warp (barrier, patch, eight products, two commits), and one warp doing both was what a CTA's
+    // tiles waited for (1.05 us a tile with every tile at hand).
+    constexpr int CH = D / 8, NQ = (G * CH + 31) / 32;
+    const bool vals = warp == 5;
+    // the unit's row of the token to append: key in warp 4, value in warp 5, with the next unit's in flight
+    uint4 row_now = make_uint4(0, 0, 0, 0), row_next = row_now, qv[NQ];
+    const uint4 *new_rows = vals ? v_new : k_new;
+    auto fetch_unit = [&](const DecWalk &x) {
+      if (!vals) {
+        const uint4 *qu = reinterpret_cast<const uint4 *>(q) + ((size_t)x.b * p.H_q + x.h * G) * CH;
+#pragma unroll
+        for (int k = 0; k < NQ; ++k)
+          qv[k] = lane + 32 * k < G * CH ? qu[lane + 32 * k] : make_uint4(0, 0, 0, 0);
+      }
+      if (k_new && lane < CH) row_next = new_rows[(size_t)(x.b * p.H_kv + x.h) * CH + lane];
+    };
+    if (kEarly) {   // the call's inputs on their way to L2, should they not be there, while the predecessor ends
+      if (w.left > 0) {
+        if (!vals)
+          for (int k = lane; k < G * CH; k += 32) prefetch_l2(reinterpret_cast<const uint4 *>(q) + ((size_t)w.b * p.H_q + w.h * G) * CH + k);
+        if (k_new && lane < CH) prefetch_l2(new_rows + (size_t)(w.b * p.H_kv + w.h) * CH + lane);
+      }
+      pdl_wait();
+    }
+    if (w.left > 0) fetch_unit(w);
+    if (!vals) {
+      // (not before the wait: a predecessor's CTA may still be waiting for tensor memory of its own)
+      tmem_alloc(smem_u32(&s_tmem), kDecTmemCols);
+      tmem_relinquish();
+      tc_fence_before();
+    }
+    asm volatile("bar.sync 2, 192;" ::: "memory");
+    tc_fence_after();
+    const uint32_t tmem = s_tmem;
+    if (vals) {
+      if (k_new && cached && lane == 0) {
+        // every CTA signs off once it holds its copy of the lengths; the last one publishes the new ones
+        if (atomicAdd(&counters[U], 1) == grid - 1) {
+          counters[U] = 0;   // ready for the next call
+          for (int b = 0; b < p.B; ++b) {
+            const int n = s_seq[b];
+            if (n >= 0 && n < p.N_cap) c.seq_len[b] = n + 1;
+            else atomicOr(status_dev, KEEPKV_DEV_APPEND_FULL);
+          }
+        }
+      }
+      // sequences without entries: output 0, lse = -inf
+      for (int u = cta; u < U; u += grid) {
+        const int b = u / p.H_kv, h = u % p.H_kv;
+        if (len_of(b) <= 0) {
+          for (int idx = lane; idx < G * D; idx += 32) out[((size_t)b * p.H_q + h * G) * D + idx] = __float2bfloat16_rn(0.f);
+          if (lse && lane < G) lse[(size_t)b * p.H_q + h * G + lane] = -CUDART_INF_F;
+        }
+      }
+      __syncwarp();
+    }
+    auto swz = [](int row, int chunk) { return (chunk >> 3) * SL::kSubBytes + row * 128 + (((chunk & 7) ^ (row & 7)) << 4); };
+    bool ok = true;
+    for (int t = 0, seg = -1; w.left > 0; ++t) {
+      const int n = w.groups();
+      const int i = !vals ? (t == 0 ? 0 : 2 * t - 1) : (w.left > n ? 2 * t + 2 : 2 * t + 1), slot = i % S;
+      // Weights of tile t for its second product; of tile t - 2 for the first product of tile t, which overwrites that
+      // tile's logits and, entering a unit, the queries used before.
+      const int tp = vals ? t : t - 2;
+      ok = (tp < 0 || wait_bar(bar_p + 8 * (tp & 1), (tp >> 1) & 1)) && wait_bar(bar_full + 8 * slot, (i / S) & 1);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      uint8_t *tile = smem + slot * SL::kSlotBytes;
+      bool wrote = false;
+      if (w.first) {   // a new unit: its row becomes the current one, the next unit's is requested
+        ++seg;
+        if (!vals) {
+#pragma unroll
+          for (int k = 0; k < NQ; ++k) {
+            const int idx = lane + 32 * k, g = idx / CH, ch = idx % CH;
+            if (idx < G * CH)
+              *reinterpret_cast<uint4 *>(smem + SL::kQ + (seg & 1) * SL::kQBytes + (ch >> 3) * 1024 + g * 128 + (((ch & 7) ^ g) << 4)) = qv[k];
+          }
+          wrote = true;
+        }
+        row_now = row_next;
+        if (w.left > w.gb - w.g) {
+          DecWalk nx = w;
+          advance(nx, w.gb - w.g);
+          fetch_unit(nx);
+        }
+      }
+      const int rows = min(n * kGroup, w.len - w.g * kGroup);
+      if (vals && rows < kDecTile) {
+        // missing rows hold unspecified bits: zero those the product reads (their weights are 0, and 0 * NaN is not)
+        const int zend = D == 128 || rows <= 64 ? (rows + 15) & ~15 : kDecTile;
+        wrote |= rows < zend;
+        for (int idx = rows * CH + lane; idx < zend * CH; idx += 32)
+          *reinterpret_cast<uint4 *>(tile + swz(idx / CH, idx % CH)) = make_uint4(0, 0, 0, 0);
+      }
+      if (w.fresh >= 0 && w.g + n == w.gb) {   // the unit's last row, the appended one: into the tile and into the cache
+        if (lane < CH) {
+          *reinterpret_cast<uint4 *>(tile + swz(rows - 1, lane)) = row_now;
+          reinterpret_cast<uint4 *>(vals ? c.V : c.K)[((size_t)(w.b * p.H_kv + w.h) * p.N_cap + w.fresh) * CH + lane] = row_now;
+        }
+        wrote = true;
+      }
+      if (wrote) { fence_proxy_async_smem(); __syncwarp(); }
+      tc_fence_after();
+      if (elect_one()) {
+        const uint32_t at = sbase + slot * SL::kSlotBytes;
+        if (!vals) {
+          const uint64_t kd = umma_desc_sw128(at), qd = umma_desc_sw128(sbase + SL::kQ + (seg & 1) * SL::kQBytes);
+#pragma unroll
+          for (int k = 0; k < D / 16; ++k)   // (descriptor addresses count 16-byte units)
+            umma_bf16(tmem + (t & 1) * 16, kd + (k >> 2) * (SL::kSubBytes / 16) + (k & 3) * 2,
+                      qd + (k >> 2) * 64 + (k & 3) * 2, IDESC_S, k > 0 ? 1u : 0u);
+          umma_commit(bar_s + 8 * (t & 1));
+        } else {
+          const uint64_t vd = umma_desc_sw128_mn(at, D == 128 ? SL::kSubBytes : SL::kSubBytes / 2);
+          const uint64_t pd = umma_desc_sw128(sbase + SL::kP);
+          const int steps = D == 128 || rows <= 64 ? (rows + 15) / 16 : 4;
+#pragma unroll
+          for (int k = 0; k < (D == 128 ? 8 : 4); ++k)
+            if (k < steps)
+              umma_bf16(tmem + 32 + (t & 1) * NO, vd + k * 128, pd + (k >> 2) * 128 + (k & 3) * 2, IDESC_O, k > 0 ? 1u : 0u);
+          umma_commit(bar_o + 8 * (t & 1));
+        }
+        umma_commit(bar_empty + 8 * slot);
+      }
+      __syncwarp();
+      advance(w, n);
+    }
+    if (!ok) {   // products in flight retire (bounded) before tensor memory is given back
+      s_abort = 1;
+      if (elect_one()) umma_commit(bar_drain + 8 * (warp & 1));
+      mbar_wait_n(bar_drain + 8 * (warp & 1), 0, spin_limit);
+    }
+    __syncwarp();
+  } else {
+    // ------------------------------------------------------------ softmax and sums
     const float ln_alpha = p.ema_alpha > 0.f ? __logf(p.ema_alpha) : -CUDART_INF_F;
     const float ln_1ma = log1pf(-p.ema_alpha);
     const float ln_G = __logf((float)G);
-
-    // Q fragments (A operand of QK^T): row g = query head, rows >= G and rows 8-15 are zero.  They are
-    // fetched ahead of the segment that uses them: before the first tile arrives, and while the
-    // previous segment is being combined.
-    uint32_t qa[KS][2];
-    auto load_q = [&](int u) {
-      const int b = u / p.H_kv, h = u % p.H_kv;
-      const __nv_bfloat16 *qrow = q + ((size_t)b * p.H_q + h * G + (g < G ? g : 0)) * D;
-#pragma unroll
-      for (int ks = 0; ks < KS; ++ks) {
-        qa[ks][0] = g < G ? *reinterpret_cast<const uint32_t *>(qrow + ks * 16 + qd * 2) : 0u;
-        qa[ks][1] = g < G ? *reinterpret_cast<const uint32_t *>(qrow + ks * 16 + 8 + qd * 2) : 0u;
+    // vote and score estimate of this thread's entry of a tile, one tile ahead of their use
+    float pv_next = 1.f, ls_next = 0.f;
+    auto fetch_entry = [&](const DecWalk &x) {
+      const int e = x.g * kGroup + tid;
+      if (tid < x.groups() * kGroup && e < x.len) {
+        const size_t at = (size_t)(x.b * p.H_kv + x.h) * p.N_cap + e;
+        pv_next = c.votes[at];
+        if (update_scores) ls_next = c.lscore[at];
       }
     };
-    if (ntiles > 0) load_q(s_start[0] * p.H_kv + s_start[1]);
-    float o[NT][4];
+    if (w.left > 0) fetch_entry(w);
+    if (kEarly) {
+      pdl_wait();
+      pdl_trigger();   // only now: the next launch may run ahead of this one, never of this one's predecessor
+    }
+    asm volatile("bar.sync 2, 192;" ::: "memory");
+    tc_fence_after();
+    const uint32_t lanes = s_tmem + ((uint32_t)(warp * 32) << 16);
+    float *xch = reinterpret_cast<float *>(smem + SL::kP);   // d = 64: the second half's sums at the end of a segment
+    const int half = D == 128 ? 0 : tid >> 6;
+    float m[G], l[G], o[G];
 #pragma unroll
-    for (int nt = 0; nt < NT; ++nt) o[nt][0] = o[nt][1] = o[nt][2] = o[nt][3] = 0.f;
-    float m_run = -CUDART_INF_F, l_run = 0.f;   // running max (base-2 exponent) and per-thread partial sum of head g
-    bool dead = false;                          // a bounded wait ran out: no more waiting, no more arithmetic
-
-    for (int it = 0; it < ntiles; ++it) {
-      const int stage = it % S;
-      // keep the ring S-1 tiles ahead: the stage of tile it-1 is free once all four warps have left it
-      if (tid == 0 && pit < ntiles && pit <= it + S - 1 && s_stop > pit)
-        if (!issue_next()) { s_stop = pit; s_abort = 1; }
-      __syncwarp();
+    for (int g = 0; g < G; ++g) { m[g] = -CUDART_INF_F; l[g] = o[g] = 0.f; }
+    int prev_rows = 0;
+    bool dead = false;
+    // adds the value sums of tile `t` (rows_t of its rows exist) to o
+    auto add_sums = [&](int t, int rows_t) {
+      uint32_t r[16];
+      tc_fence_after();
+      tmem_ld_32x16(lanes + 32 + (t & 1) * NO + half * 16, r);
+      tmem_ld_wait();
+      if (D == 128 || half == 0 || rows_t > 64) {
+#pragma unroll
+        for (int g = 0; g < G; ++g) o[g] += __uint_as_float(r[g]) + __uint_as_float(r[8 + g]);
+      }
+    };
+    for (int t = 0; w.left > 0; ++t) {
+      const int n = w.groups(), i0 = w.g * kGroup, rows = min(n * kGroup, w.len - i0), fresh = fresh_row(w);
+      const bool last = w.last(n), valid = tid < rows;
+      const size_t entry = (size_t)(w.b * p.H_kv + w.h) * p.N_cap + i0 + tid;
+      float pv = pv_next, ls = ls_next;
+      if (tid == fresh) {   // Eq. 2 inside this call: one vote, no score history
+        pv = 1.0f;
+        ls = -CUDART_INF_F;
+      }
+      DecWalk nx = w;
+      advance(nx, n);
+      if (nx.left > 0) fetch_entry(nx);
+      if (!dead) dead = !__all_sync(0xffffffffu, wait_bar(bar_s + 8 * (t & 1), (t >> 1) & 1));
+      float x[G], y[G];
       if (!dead) {
-        int ok = 0;
-        if (lane == 0) ok = !s_abort && mbar_wait_n(smem_u32(&full_bar[stage]), (it / S) & 1, spin_limit);
-        if (!__shfl_sync(0xffffffffu, ok, 0)) { s_abort = 1; dead = true; }
-      }
-      if (dead) {
-        // A wait ran out (here or in another warp): the kernel's result is lost, but its barriers are not.  The warp
-        // walks the rest of its range without waiting for data and without arithmetic, so that it still meets the
-        // others at every barrier of the combines; it only makes sure that the descriptor it acts on exists, and
-        // all four warps stop at the same tile if the producer gave up.
-        int go = 1;
-        if (lane == 0) {
-          int polls = 0;
-          while (s_issued <= it && s_stop > it && polls < spin_limit) { ++polls; __nanosleep(64); }
-          go = s_issued > it;
+        uint32_t s[8];
+        tc_fence_after();
+        tmem_ld_32x8(lanes + (t & 1) * 16, s);
+        tmem_ld_wait();
+        const float lp = lg2f(pv);
+#pragma unroll
+        for (int g = 0; g < G; ++g) {   // (the logits of entries that do not exist may be anything)
+          x[g] = __uint_as_float(s[g]) * p.sm_scale;
+          y[g] = valid ? fmaf(x[g], kLog2e, lp) : -CUDART_INF_F;
+          const float mx = warp_max_redux(y[g]);
+          if (lane == 0) s_wmax[t & 1][g][warp] = mx;
         }
-        if (!__shfl_sync(0xffffffffu, go, 0)) break;
       }
-      const uint32_t st = smem_base + stage * SL::kStride;
-      const uint8_t *stp = smem + stage * SL::kStride;
-      const TileDesc d = *reinterpret_cast<const TileDesc *>(stp + SL::kDesc);
-      const int b = d.u / p.H_kv, h = d.u % p.H_kv;
-
-      const int i_base = d.tile * kTile + r0;     // first entry of this warp's slice
-      const int n_valid = d.len - i_base;         // entries of the slice that exist (may be <= 0 or >= 32)
-      const bool mine = (it & 1) == pair && !dead;
-      const bool patch = mine && d.fresh >= r0 && d.fresh < r0 + 32;
-      if (patch) {
-        // Eq. 2 inside this call: the row of the fresh entry arrived with whatever the cache held; this warp,
-        // the only one to read it, overwrites it in the tile and in the cache (one vote, no score history)
-        constexpr int CH = D / 8;
-        const size_t e = (size_t)d.u * p.N_cap + d.tile * kTile + d.fresh;
-        const int half = lane >> 4, ch = lane & 15;
-        if (ch < CH) {
-          const uint4 val = (half ? v_new : k_new)[(size_t)d.u * CH + ch];
-          *reinterpret_cast<uint4 *>(smem + stage * SL::kStride + (half ? SL::kV : SL::kK) + swz(d.fresh, ch)) = val;
-          reinterpret_cast<uint4 *>(half ? c.V : c.K)[e * CH + ch] = val;
+      asm volatile("bar.sync 1, 128;" ::: "memory");
+      float fac[G];
+      if (!dead) {
+        float pr[G];
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+          const float4 wm = *reinterpret_cast<const float4 *>(s_wmax[t & 1][g]);
+          const float mx = fmaxf(fmaxf(wm.x, wm.y), fmaxf(wm.z, wm.w));
+          const float mn = fmaxf(m[g], mx);
+          const bool any = mn > -CUDART_INF_F;
+          fac[g] = any ? ex2f(m[g] - mn) : 1.f;   // m = -inf gives 0; o and l are 0 then anyway
+          pr[g] = any ? ex2f(y[g] - mn) : 0.f;
+          l[g] = fmaf(l[g], fac[g], pr[g]);
+          m[g] = mn;
         }
-        if (lane == 0) {
-          reinterpret_cast<float *>(smem + stage * SL::kStride + SL::kVotes)[d.fresh] = 1.0f;
-          reinterpret_cast<float *>(smem + stage * SL::kStride + SL::kLscore)[d.fresh] = -CUDART_INF_F;
-          c.votes[e] = 1.0f;
-          if (!update_scores) c.lscore[e] = -CUDART_INF_F;   // otherwise Eq. 8 below writes the first observation
-        }
-        __syncwarp();
-      }
-      if (mine && n_valid > 0) {
-        const bool ragged = n_valid < 32;
-        if (ragged) {
-          // rows past the sequence hold unspecified bits; zero their V so that 0 * garbage cannot turn
-          // into NaN inside the tensor core
-          for (int idx = lane; idx < 32 * (D / 8); idx += 32) {
-            const int r = idx / (D / 8), ch = idx % (D / 8);
-            if (r >= n_valid)
-              *reinterpret_cast<uint4 *>(smem + stage * SL::kStride + SL::kV + swz(r0 + r, ch)) = make_uint4(0, 0, 0, 0);
+        // the weights buffer is free once the previous tile's second product has completed
+        if (t > 0) dead = !__all_sync(0xffffffffu, wait_bar(bar_o + 8 * ((t - 1) & 1), ((t - 1) >> 1) & 1));
+        if (!dead) {
+          uint8_t *pb = smem + SL::kP + (tid >> 6) * 2048 + (tid & 7) * 2;
+          const int ch = (tid & 63) >> 3;
+#pragma unroll
+          for (int g = 0; g < G; ++g) {
+            const __nv_bfloat16 hi = __float2bfloat16_rn(pr[g]);
+            *reinterpret_cast<__nv_bfloat16 *>(pb + g * 128 + ((ch ^ g) << 4)) = hi;
+            *reinterpret_cast<__nv_bfloat16 *>(pb + 1024 + g * 128 + ((ch ^ g) << 4)) = __float2bfloat16_rn(pr[g] - __bfloat162float(hi));
           }
+          fence_proxy_async_smem();
+          tc_fence_before();
           __syncwarp();
+          if (lane == 0) mbar_arrive(bar_p + 8 * (t & 1));
+          if (!w.first) add_sums(t - 1, prev_rows);
+#pragma unroll
+          for (int g = 0; g < G; ++g) o[g] *= fac[g];
         }
-
-        // ---- logits: S[head][entry] for the 32 entries, four independent n-tiles of 8
-        float sc[4][4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) sc[j][0] = sc[j][1] = sc[j][2] = sc[j][3] = 0.f;
-#pragma unroll
-        for (int kk = 0; kk < KS / 2; ++kk) {
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const int row = r0 + j * 8 + (lane & 7);
-            uint32_t b0, b1, b2, b3;
-            ldsm_x4(st + SL::kK + swz(row, kk * 4 + (lane >> 3)), b0, b1, b2, b3);
-            mma_bf16(sc[j], qa[2 * kk][0], 0u, qa[2 * kk][1], 0u, b0, b1);
-            mma_bf16(sc[j], qa[2 * kk + 1][0], 0u, qa[2 * kk + 1][1], 0u, b2, b3);
-          }
-        }
-        // this thread holds head g, entries e(j,t) = 8 j + 2 qd + t of the slice, in natural-log units
-        float x[4][2];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          x[j][0] = sc[j][0] * p.sm_scale;
-          x[j][1] = sc[j][1] * p.sm_scale;
-          if (g < G) *reinterpret_cast<float2 *>(sc_w + g * 32 + j * 8 + qd * 2) = make_float2(x[j][0], x[j][1]);
-        }
-        __syncwarp();
-
-        // ---- one lane per entry: log2 of the vote; Eq. 8 with the kv head's score = mean over its G heads of e^{l}
-        {
-          const int e = lane;
-          const float pv = reinterpret_cast<const float *>(stp + SL::kVotes)[r0 + e];
-          if (update_scores) {
-            float mx = sc_w[e];
-#pragma unroll
-            for (int gg = 1; gg < G; ++gg) mx = fmaxf(mx, sc_w[gg * 32 + e]);
-            float sigma = mx;
-            if (G > 1) {
-              float se = 0.f;
-#pragma unroll
-              for (int gg = 0; gg < G; ++gg) se += ex2f((sc_w[gg * 32 + e] - mx) * kLog2e);
-              sigma = mx + lg2f(se) * kLn2 - ln_G;
-            }
-            const float old = reinterpret_cast<const float *>(stp + SL::kLscore)[r0 + e];
-            float r = sigma;
-            if (old > -CUDART_INF_F && p.ema_alpha > 0.f) {
-              const float a = ln_alpha + old, bb = ln_1ma + sigma;
-              const float hi = fmaxf(a, bb), lo = fminf(a, bb);
-              r = hi + lg2f(1.f + ex2f((lo - hi) * kLog2e)) * kLn2;
-            }
-            if (e < n_valid) c.lscore[(size_t)d.u * p.N_cap + i_base + e] = r;
-          }
-          lp_w[e] = e < n_valid ? lg2f(pv) : -CUDART_INF_F;
-        }
-        __syncwarp();
-
-        // ---- Eq. 6: weights p_i e^{l_i} = 2^{x log2e + log2 p} through an online softmax
-        float mloc = -CUDART_INF_F;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float2 lp = *reinterpret_cast<const float2 *>(lp_w + j * 8 + qd * 2);
-          x[j][0] = fmaf(x[j][0], kLog2e, lp.x);   // -inf for entries past the sequence
-          x[j][1] = fmaf(x[j][1], kLog2e, lp.y);
-          if (ragged) {   // garbage logits of missing entries may be NaN or +inf
-            if (j * 8 + qd * 2 >= n_valid) x[j][0] = -CUDART_INF_F;
-            if (j * 8 + qd * 2 + 1 >= n_valid) x[j][1] = -CUDART_INF_F;
-          }
-          mloc = fmaxf(mloc, fmaxf(x[j][0], x[j][1]));
-        }
-        mloc = fmaxf(mloc, __shfl_xor_sync(0xffffffffu, mloc, 1));
-        mloc = fmaxf(mloc, __shfl_xor_sync(0xffffffffu, mloc, 2));
-        const float m_new = fmaxf(m_run, mloc);
-        const bool grow = m_new > m_run;
-        if (__any_sync(0xffffffffu, grow)) {
-          const float scale = grow ? ex2f(m_run - m_new) : 1.f;   // m_run = -inf gives 0; o and l are 0 then anyway
-          l_run *= scale;
-#pragma unroll
-          for (int nt = 0; nt < NT; ++nt) {
-            o[nt][0] *= scale; o[nt][1] *= scale; o[nt][2] *= scale; o[nt][3] *= scale;
-          }
-          m_run = m_new;
-        }
-        // A fragments of P for the two 16-entry k-steps: a0/a2 = bf16 head (rows 0-7), a1/a3 = bf16
-        // remainder (rows 8-15)
-        uint32_t pa[2][4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float p0 = m_run > -CUDART_INF_F ? ex2f(x[j][0] - m_run) : 0.f;
-          const float p1 = m_run > -CUDART_INF_F ? ex2f(x[j][1] - m_run) : 0.f;
-          l_run += p0 + p1;
-          const uint32_t hi2 = pack_bf16(p0, p1);
-          pa[j >> 1][2 * (j & 1)] = hi2;
-          pa[j >> 1][2 * (j & 1) + 1] = pack_bf16(p0 - bf16_lo(hi2), p1 - bf16_hi(hi2));
-        }
-        // ---- O += P V   (rows 0-7 collect the head part, rows 8-15 the remainder part)
-#pragma unroll
-        for (int ks = 0; ks < 2; ++ks) {
-          const int vrow = r0 + ks * 16 + (lane & 7) + ((lane >> 3) & 1) * 8;
-#pragma unroll
-          for (int np = 0; np < NT / 2; ++np) {
-            uint32_t b0, b1, b2, b3;
-            ldsm_x4_t(st + SL::kV + swz(vrow, np * 2 + (lane >> 4)), b0, b1, b2, b3);
-            mma_bf16(o[2 * np], pa[ks][0], pa[ks][1], pa[ks][2], pa[ks][3], b0, b1);
-            mma_bf16(o[2 * np + 1], pa[ks][0], pa[ks][1], pa[ks][2], pa[ks][3], b2, b3);
-          }
-        }
-        if (ragged || patch) fence_proxy_async_smem();   // the rows written here precede the next TMA write
       }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&empty_bar[stage]));   // this warp is done with the stage
+      prev_rows = rows;
+      // ---- Eq. 8 with the kv head's score = mean over its G heads of e^{l}
+      if (!dead && valid) {
+        if (update_scores) {
+          float mx = x[0];
+#pragma unroll
+          for (int g = 1; g < G; ++g) mx = fmaxf(mx, x[g]);
+          float sigma = mx;
+          if (G > 1) {
+            float se = 0.f;
+#pragma unroll
+            for (int g = 0; g < G; ++g) se += ex2f((x[g] - mx) * kLog2e);
+            sigma = mx + lg2f(se) * kLn2 - ln_G;
+          }
+          float r = sigma;
+          if (ls > -CUDART_INF_F && p.ema_alpha > 0.f) {
+            const float a = ln_alpha + ls, bb = ln_1ma + sigma;
+            const float hi = fmaxf(a, bb), lo = fminf(a, bb);
+            r = hi + lg2f(1.f + ex2f((lo - hi) * kLog2e)) * kLn2;
+          }
+          c.lscore[entry] = r;
+        } else if (tid == fresh) {
+          c.lscore[entry] = -CUDART_INF_F;
+        }
+        if (tid == fresh) c.votes[entry] = 1.0f;
+      }
 
-      if (d.flags & 2) {
-        // ---- end of this CTA's segment of the unit: combine the four warps
-        l_run += __shfl_xor_sync(0xffffffffu, l_run, 1);
-        l_run += __shfl_xor_sync(0xffffffffu, l_run, 2);
-        if (g < G && qd == 0) { cml[(warp * 8 + g) * 2] = m_run; cml[(warp * 8 + g) * 2 + 1] = l_run; }
-        const bool whole = d.nparts == 1;
-        PartRec<D, G> *rec = pool + (size_t)cta * 2 + (d.c_first == cta ? 1 : 0);
-        float osum[NT][2];
+      if (last) {
+        // ---- end of this CTA's segment of the unit
 #pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {
-          osum[nt][0] = o[nt][0] + o[nt][2]; osum[nt][1] = o[nt][1] + o[nt][3];
-          o[nt][0] = o[nt][1] = o[nt][2] = o[nt][3] = 0.f;
+        for (int g = 0; g < G; ++g) {
+          const float sum = warp_sum(l[g]);
+          if (lane == 0) s_wsum[warp][g] = sum;
         }
-        if (d.u_next >= 0) load_q(d.u_next);   // in flight while this segment is combined
-        m_run = -CUDART_INF_F;
-        l_run = 0.f;
-        constexpr int ROUNDS = (G + 3) / 4, RG = G < 4 ? G : 4;
+        if (!dead) dead = !__all_sync(0xffffffffu, wait_bar(bar_o + 8 * (t & 1), (t >> 1) & 1));
+        if (!dead) {
+          add_sums(t, rows);
+          if (D == 64 && half == 1) {
 #pragma unroll
-        for (int rd = 0; rd < ROUNDS; ++rd) {
-          if (g < G && (g >> 2) == rd) {
-#pragma unroll
-            for (int nt = 0; nt < NT; ++nt)
-              *reinterpret_cast<float2 *>(&comb[(size_t)warp * WR + (g & 3) * D + nt * 8 + qd * 2]) =
-                  make_float2(osum[nt][0], osum[nt][1]);
+            for (int g = 0; g < G; ++g) xch[g * 64 + (tid & 63)] = o[g];
           }
-          asm volatile("bar.sync 1, 128;" ::: "memory");
-          for (int idx = ctid; idx < RG * D; idx += 32 * kDecConsumers) {
-            const int gl = idx / D, j = idx % D, gg = rd * 4 + gl;
-            float M = cml[gg * 2];
+        }
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+        int c_first = 0, nparts = csize;
+        if (!split) {
+          c_first = w.start / chunk;
+          nparts = (w.start + w.gb - 1) / chunk - c_first + 1;
+        }
+        const size_t head0 = (size_t)w.b * p.H_q + w.h * G;
+        if (!dead && tid < D) {
+          PartRec<D, G> *rec = pool + (size_t)cta * 2 + (c_first == cta ? 1 : 0);
 #pragma unroll
-            for (int w = 1; w < kDecConsumers; ++w) M = fmaxf(M, cml[(w * 8 + gg) * 2]);
-            float Ls = 0.f, a = 0.f;
-            if (M > -CUDART_INF_F) {
-#pragma unroll
-              for (int w = 0; w < kDecConsumers; ++w) {
-                const float f = ex2f(cml[(w * 8 + gg) * 2] - M);
-                Ls += f * cml[(w * 8 + gg) * 2 + 1];
-                a += f * comb[(size_t)w * WR + gl * D + j];
+          for (int g = 0; g < G; ++g) {
+            const float Ls = (s_wsum[0][g] + s_wsum[1][g]) + (s_wsum[2][g] + s_wsum[3][g]);
+            if (D == 64) o[g] += xch[g * 64 + tid];
+            if (nparts == 1) {
+              out[(head0 + g) * D + tid] = __float2bfloat16_rn(Ls > 0.f ? o[g] / Ls : 0.f);
+              if (lse && tid == 0) lse[head0 + g] = Ls > 0.f ? (m[g] + lg2f(Ls)) * kLn2 : -CUDART_INF_F;
+            } else if (split) {   // to the CTA of the cluster that folds this output
+              // (slices of G * D / csize outputs, powers of two)
+              const int sshift = 31 - __clz(G * D) - cshift, idx = g * D + tid, to = idx >> sshift;
+              st_shared_cluster_f32(mapa_shared(inbox + (128 + ((crank - to) << sshift) + idx) * 4, to), o[g]);
+              if (tid < csize) {
+                st_shared_cluster_f32(mapa_shared(inbox + (crank * 16 + g) * 4, tid), m[g]);
+                st_shared_cluster_f32(mapa_shared(inbox + (crank * 16 + 8 + g) * 4, tid), Ls);
               }
-            }
-            if (whole) {
-              const size_t qo = (size_t)b * p.H_q + h * G + gg;
-              out[qo * D + j] = __float2bfloat16_rn(Ls > 0.f ? a / Ls : 0.f);
-              if (lse && j == 0) lse[qo] = Ls > 0.f ? (M + lg2f(Ls)) * kLn2 : -CUDART_INF_F;
-            } else if (aligned) {   // this CTA's partial stays in its shared memory (the ring is idle by now)
-              float *xr = reinterpret_cast<float *>(smem);
-              xr[16 + gg * D + j] = a;
-              if (j == 0) { xr[gg] = M; xr[8 + gg] = Ls; }
             } else {
-              rec->acc[gg * D + j] = a;
-              if (j == 0) { rec->m[gg] = M; rec->l[gg] = Ls; }
+              rec->acc[g * D + tid] = o[g];
+              if (tid == 0) { rec->m[g] = m[g]; rec->l[g] = Ls; }
             }
           }
-          asm volatile("bar.sync 1, 128;" ::: "memory");
         }
-        if (!whole && !aligned) {
+        if (nparts > 1 && !split) {
           // ---- the last CTA of the unit to arrive merges the partials, in CTA order
           __threadfence();
           asm volatile("bar.sync 1, 128;" ::: "memory");
-          if (ctid == 0) {
-            const int ticket = atomicAdd(&counters[d.u], 1);
-            s_last = (ticket == d.nparts - 1);
-            if (s_last) counters[d.u] = 0;   // ready for the next call
+          if (tid == 0) {
+            const int u = w.b * p.H_kv + w.h;
+            s_last = atomicAdd(&counters[u], 1) == nparts - 1;
+            if (s_last) counters[u] = 0;   // ready for the next call
           }
           asm volatile("bar.sync 1, 128;" ::: "memory");
           if (s_last) {
             __threadfence();
-            // comb[part][head] = (m_k, scale factor 2^{m_k - M}); cml[head] = M
-            constexpr int kMaxParts = kDecConsumers * WR / (2 * G);
-            const int np_ = d.nparts;
-            auto part = [&](int k) { return pool + (size_t)(d.c_first + k) * 2 + (k == 0 ? 1 : 0); };
-            constexpr int NI = (G * D + 32 * kDecConsumers - 1) / (32 * kDecConsumers);   // outputs per thread
-            constexpr int KF = NI <= 4 ? 8 : 4;   // parts the register path holds
-            if (np_ <= KF) {
-              // few parts (the usual case): everything in registers, one round trip to L2
-              float pm[KF][NI], pl[KF][NI], pa_[KF][NI];
+            constexpr int KB = 8;   // parts in flight at a time
+            for (int q4 = tid; q4 < G * D / 4; q4 += 128) {   // four consecutive channels of one head
+              const int g = q4 * 4 / D;
+              float M = -CUDART_INF_F, Ls = 0.f;
+              float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+              for (int k0 = 0; k0 < nparts; k0 += KB) {
+                float pm[KB], pl[KB];
+                float4 pa[KB];
 #pragma unroll
-              for (int k = 0; k < KF; ++k) {
-                const PartRec<D, G> *r = part(k < np_ ? k : 0);
-#pragma unroll
-                for (int i = 0; i < NI; ++i) {
-                  const int idx = min(ctid + i * 32 * kDecConsumers, G * D - 1);
-                  pm[k][i] = k < np_ ? __ldcg(&r->m[idx / D]) : -CUDART_INF_F;
-                  pl[k][i] = __ldcg(&r->l[idx / D]);
-                  pa_[k][i] = __ldcg(&r->acc[idx]);
+                for (int k = 0; k < KB; ++k) {
+                  const int kk = min(k0 + k, nparts - 1);
+                  const PartRec<D, G> *r = pool + (size_t)(c_first + kk) * 2 + (kk == 0 ? 1 : 0);
+                  pm[k] = k0 + k < nparts ? __ldcg(&r->m[g]) : -CUDART_INF_F;
+                  pl[k] = __ldcg(&r->l[g]);
+                  pa[k] = __ldcg(reinterpret_cast<const float4 *>(r->acc) + q4);
                 }
-              }
+                float Mn = M;
 #pragma unroll
-              for (int i = 0; i < NI; ++i) {
-                const int idx = ctid + i * 32 * kDecConsumers;
-                float M = pm[0][i];
+                for (int k = 0; k < KB; ++k) Mn = fmaxf(Mn, pm[k]);
+                if (Mn > -CUDART_INF_F) {
+                  const float f0 = ex2f(M - Mn);
+                  Ls *= f0; acc.x *= f0; acc.y *= f0; acc.z *= f0; acc.w *= f0;
 #pragma unroll
-                for (int k = 1; k < KF; ++k) M = fmaxf(M, pm[k][i]);
-                float Ls = 0.f, a = 0.f;
-#pragma unroll
-                for (int k = 0; k < KF; ++k) {
-                  const float f = pm[k][i] > -CUDART_INF_F ? ex2f(pm[k][i] - M) : 0.f;
-                  Ls = fmaf(f, pl[k][i], Ls);
-                  a = fmaf(f, pa_[k][i], a);
-                }
-                if (idx < G * D) {
-                  const int gg = idx / D, j = idx % D;
-                  const size_t qo = (size_t)b * p.H_q + h * G + gg;
-                  out[qo * D + j] = __float2bfloat16_rn(Ls > 0.f ? a / Ls : 0.f);
-                  if (lse && j == 0) lse[qo] = Ls > 0.f ? (M + lg2f(Ls)) * kLn2 : -CUDART_INF_F;
-                }
-              }
-            } else if (np_ <= kMaxParts) {
-              for (int idx = ctid; idx < np_ * G; idx += 32 * kDecConsumers)
-                comb[idx * 2] = __ldcg(&part(idx / G)->m[idx % G]);
-              asm volatile("bar.sync 1, 128;" ::: "memory");
-              for (int idx = ctid; idx < np_ * G; idx += 32 * kDecConsumers) {
-                const int gg = idx % G;
-                float M = -CUDART_INF_F;
-                for (int k = 0; k < np_; ++k) M = fmaxf(M, comb[(k * G + gg) * 2]);
-                comb[idx * 2 + 1] = M > -CUDART_INF_F ? ex2f(comb[idx * 2] - M) : 0.f;
-                if (idx < G) cml[gg] = M;
-              }
-              asm volatile("bar.sync 1, 128;" ::: "memory");
-              // every thread owns NI outputs; the parts are the outer loop so that all loads of a part
-              // are in flight together
-              float Ls[NI], a[NI];
-#pragma unroll
-              for (int i = 0; i < NI; ++i) Ls[i] = a[i] = 0.f;
-#pragma unroll 2
-              for (int k = 0; k < np_; ++k) {
-                const PartRec<D, G> *r = part(k);
-#pragma unroll
-                for (int i = 0; i < NI; ++i) {
-                  const int idx = ctid + i * 32 * kDecConsumers;
-                  if (idx < G * D) {
-                    const int gg = idx / D;
-                    const float f = comb[(k * G + gg) * 2 + 1];
-                    Ls[i] = fmaf(f, __ldcg(&r->l[gg]), Ls[i]);
-                    a[i] = fmaf(f, __ldcg(&r->acc[idx]), a[i]);
+                  for (int k = 0; k < KB; ++k) {
+                    const float f = ex2f(pm[k] - Mn);
+                    Ls = fmaf(f, pl[k], Ls);
+                    acc.x = fmaf(f, pa[k].x, acc.x); acc.y = fmaf(f, pa[k].y, acc.y);
+                    acc.z = fmaf(f, pa[k].z, acc.z); acc.w = fmaf(f, pa[k].w, acc.w);
                   }
+                  M = Mn;
                 }
               }
-#pragma unroll
-              for (int i = 0; i < NI; ++i) {
-                const int idx = ctid + i * 32 * kDecConsumers;
-                if (idx < G * D) {
-                  const int gg = idx / D, j = idx % D;
-                  const size_t qo = (size_t)b * p.H_q + h * G + gg;
-                  out[qo * D + j] = __float2bfloat16_rn(Ls[i] > 0.f ? a[i] / Ls[i] : 0.f);
-                  if (lse && j == 0) lse[qo] = Ls[i] > 0.f ? (cml[gg] + lg2f(Ls[i])) * kLn2 : -CUDART_INF_F;
-                }
-              }
-            } else {
-              for (int idx = ctid; idx < G * D; idx += 32 * kDecConsumers) {
-                const int gg = idx / D, j = idx % D;
-                float M = -CUDART_INF_F;
-                for (int k = 0; k < np_; ++k) M = fmaxf(M, __ldcg(&part(k)->m[gg]));
-                float Ls = 0.f, a = 0.f;
-                if (M > -CUDART_INF_F) {
-                  for (int k = 0; k < np_; ++k) {
-                    const float f = ex2f(__ldcg(&part(k)->m[gg]) - M);
-                    Ls = fmaf(f, __ldcg(&part(k)->l[gg]), Ls);
-                    a = fmaf(f, __ldcg(&part(k)->acc[gg * D + j]), a);
-                  }
-                }
-                const size_t qo = (size_t)b * p.H_q + h * G + gg;
-                out[qo * D + j] = __float2bfloat16_rn(Ls > 0.f ? a / Ls : 0.f);
-                if (lse && j == 0) lse[qo] = Ls > 0.f ? (M + lg2f(Ls)) * kLn2 : -CUDART_INF_F;
-              }
+              const float inv = Ls > 0.f ? 1.f / Ls : 0.f;
+              *reinterpret_cast<uint2 *>(out + head0 * D + q4 * 4) =
+                  make_uint2(pack_bf16(acc.x * inv, acc.y * inv), pack_bf16(acc.z * inv, acc.w * inv));
+              if (lse && q4 * 4 % D == 0) lse[head0 + g] = Ls > 0.f ? (M + lg2f(Ls)) * kLn2 : -CUDART_INF_F;
             }
           }
-          asm volatile("bar.sync 1, 128;" ::: "memory");   // s_last is reused by the next segment
         }
+#pragma unroll
+        for (int g = 0; g < G; ++g) { m[g] = -CUDART_INF_F; l[g] = o[g] = 0.f; }
       }
+      w = nx;
+    }
+    if (dead) s_abort = 1;
+    if (split && csize > 1 && (s_start[4] == 0 || dead) && tid < csize) {   // no entries here: an empty partial
+#pragma unroll
+      for (int g = 0; g < G; ++g) st_shared_cluster_f32(mapa_shared(inbox + (crank * 16 + g) * 4, tid), -CUDART_INF_F);
     }
   }
 
-  __syncthreads();
-  if (aligned && tb_unit > 1) {
-    // ---- the cluster folds its unit's partials through distributed shared memory: [m[8], l[8], acc[G*D]] per CTA
-    float *xr = reinterpret_cast<float *>(smem);
-    if (ntiles == 0 && tid < 8) { xr[tid] = -CUDART_INF_F; xr[8 + tid] = 0.f; }   // no tiles here: an empty partial
-    cluster_sync_all();
-    const int u = cta / csize, b = u / p.H_kv, h = u % p.H_kv;
-    const int per_cta = G * D / csize;   // outputs this CTA folds
-    const uint32_t xr_addr = smem_u32(xr);
-    for (int k = tid; k < per_cta; k += kDecThreads) {
-      const int idx = crank * per_cta + k, gg = idx / D, j = idx % D;
-      float pm[8], pl[8], pa_[8];
+  __syncwarp();
+  tc_fence_before();
+  if (csize > 1) cluster_sync_all();
+  else __syncthreads();
+  if (split && csize > 1 && warp < 4 && total_b > 0) {
+    // ---- every CTA of the cluster folds its slice of the unit's outputs, in rank order
+    const float *in = reinterpret_cast<const float *>(smem + SL::kInbox);
+    const int slice = (G * D) >> cshift, u = cta >> cshift, b = u / p.H_kv, h = u % p.H_kv;
+    if (len_of(b) > 0) {
+      for (int j = tid; j < slice; j += 128) {
+        const int idx = crank * slice + j, g = idx / D;
+        float M = -CUDART_INF_F, Ls = 0.f, acc = 0.f;
 #pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        pm[r] = -CUDART_INF_F; pl[r] = 0.f; pa_[r] = 0.f;
-        if (r < csize) {
-          const uint32_t ra = mapa_shared(xr_addr, (uint32_t)r);
-          pm[r] = ld_shared_cluster_f32(ra + gg * 4);
-          pl[r] = ld_shared_cluster_f32(ra + (8 + gg) * 4);
-          pa_[r] = ld_shared_cluster_f32(ra + (16 + idx) * 4);
+        for (int r = 0; r < 8; ++r)
+          if (r < csize) M = fmaxf(M, in[r * 16 + g]);
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+          // (an empty partial has no numerators: what its place holds is not even multiplied by zero)
+          if (r < csize && in[r * 16 + g] > -CUDART_INF_F) {
+            const float f = ex2f(in[r * 16 + g] - M);
+            Ls = fmaf(f, in[r * 16 + 8 + g], Ls);
+            acc = fmaf(f, in[128 + r * slice + j], acc);
+          }
         }
+        const size_t head = (size_t)b * p.H_q + h * G + g;
+        out[head * D + idx % D] = __float2bfloat16_rn(Ls > 0.f ? acc / Ls : 0.f);
+        if (lse && idx % D == 0) lse[head] = Ls > 0.f ? (M + lg2f(Ls)) * kLn2 : -CUDART_INF_F;
       }
-      float M = pm[0];
-#pragma unroll
-      for (int r = 1; r < 8; ++r) M = fmaxf(M, pm[r]);
-      float Ls = 0.f, a = 0.f;
-#pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        // a CTA without tiles published m = -inf and nothing else: its numerators are whatever its shared
-        // memory held (0 * NaN would poison the sum), so an empty partial is skipped, not weighted by zero
-        if (pm[r] > -CUDART_INF_F) {
-          const float f = ex2f(pm[r] - M);
-          Ls = fmaf(f, pl[r], Ls);
-          a = fmaf(f, pa_[r], a);
-        }
-      }
-      const size_t qo = (size_t)b * p.H_q + h * G + gg;
-      out[qo * D + j] = __float2bfloat16_rn(Ls > 0.f ? a / Ls : 0.f);
-      if (lse && j == 0) lse[qo] = Ls > 0.f ? (M + lg2f(Ls)) * kLn2 : -CUDART_INF_F;
     }
-    cluster_sync_all();   // nobody leaves while a peer still reads its shared memory
+  }
+  if (warp == 4) {
+    tc_fence_after();
+    tmem_dealloc(s_tmem, kDecTmemCols);
   }
   if (k_new && !cached) {
     // the new lengths are published by the last CTA to get here: every CTA has read the old ones for the last time
@@ -810,20 +727,13 @@ decode_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ 
       }
     }
   }
-  if (s_abort) {
-    // give copies still in flight a bounded chance to land before the CTA's shared memory goes away
-    if (tid == 0) {
-      atomicOr(status_dev, KEEPKV_DEV_TIMEOUT);
-      for (int i = 0; i < S; ++i) { mbar_wait_n(smem_u32(&full_bar[i]), 0, spin_limit); mbar_wait_n(smem_u32(&full_bar[i]), 1, spin_limit); }
-    }
-    __syncthreads();
-  }
+  if (s_abort && tid == 0) atomicOr(status_dev, KEEPKV_DEV_TIMEOUT);
 }
 
 // ---------------------------------------------------------------- host side
 // What a test may change: the number of polls of a bounded wait, and one position of every CTA's tile range
-// that the producer announces without issuing its copies, so that the consumers' wait for it runs out with
-// nothing in flight (keepkv_debug_decode in the header).
+// whose copies are never issued, so that the wait for it runs out with nothing in flight (keepkv_debug_decode in the
+// header).
 static int g_dbg_spin = kSpinLimit;
 static int g_dbg_withhold = -1;
 void decode_debug(int spin_limit, int withhold) {
@@ -831,22 +741,26 @@ void decode_debug(int spin_limit, int withhold) {
   g_dbg_withhold = withhold;
 }
 
-// Tensor maps are a function of (base pointer, rows, D): a serving loop calls with the same few caches over and
-// over, so the encoded maps are kept in a small table instead of being rebuilt by the driver on every launch.
-struct MapKey { const void *base; uint64_t rows; int D; };
-static bool cached_rows_map(CUtensorMap *out, void *base, uint64_t rows, int D) {
-  constexpr int N = 64;
-  static MapKey keys[N];
-  static CUtensorMap maps[N];
-  static int used = 0, next = 0;
+// Tensor maps are a function of (base pointer, rows, D): a serving loop calls with the same caches, two arrays per layer,
+// over and over, so the encoded maps are kept in a bounded table, four places to a bucket, instead of being rebuilt by
+// the driver on every launch (about a microsecond each).
+static bool cached_maps(CUtensorMap *out, void *base, uint64_t rows, int D) {
+  struct Place { const void *base; uint64_t rows; int D; };
+  constexpr int kBuckets = 256, kWays = 4;   // 128 KB: the keys and values of 512 layer caches
+  static Place places[kBuckets][kWays];
+  static CUtensorMap maps[kBuckets][kWays];
+  static uint8_t victim[kBuckets];
   static std::mutex mu;
+  const int at = (int)((((uint64_t)(uintptr_t)base >> 8) * 0x9E3779B97F4A7C15ull) >> 56);
   std::lock_guard<std::mutex> lock(mu);
-  for (int i = 0; i < used; ++i)
-    if (keys[i].base == base && keys[i].rows == rows && keys[i].D == D) { *out = maps[i]; return true; }
-  if (!make_bf16_halves_map(out, base, rows, D, kTile)) return false;
-  const int slot = used < N ? used++ : (next++ % N);
-  keys[slot] = MapKey{base, rows, D};
-  maps[slot] = *out;
+  for (int i = 0; i < kWays; ++i) {
+    const Place &k = places[at][i];
+    if (k.base == base && k.rows == rows && k.D == D) { *out = maps[at][i]; return true; }
+  }
+  if (!make_bf16_rows_map(out, base, rows, D, kGroup)) return false;
+  const int i = victim[at]++ % kWays;
+  places[at][i] = Place{base, rows, D};
+  maps[at][i] = *out;
   return true;
 }
 template <int D, int G, bool E>
@@ -854,7 +768,7 @@ static void launch_t(const keepkv_params &p, const keepkv_cache &c, const void *
                      int update_scores, char *ws, const WsLayout &L, int32_t *status_dev, const void *k_new,
                      const void *v_new, LaunchCtx &ctx) {
   using SL = DecSmem<D>;
-  constexpr size_t smem_bytes = (size_t)SL::kBytes + 1024;
+  constexpr size_t smem_bytes = (size_t)SL::template bytes<G>() + 1024;
   static_assert(sizeof(PartRec<D, G>) == (16 + G * D) * 4, "partial record layout");
   static bool attr_done_dev[64] = {};
   int dev = 0;
@@ -865,56 +779,30 @@ static void launch_t(const keepkv_params &p, const keepkv_cache &c, const void *
   }
   CUtensorMap mapK, mapV;
   const uint64_t rows = (uint64_t)p.B * p.H_kv * p.N_cap;
-  if (!cached_rows_map(&mapK, c.K, rows, D) || !cached_rows_map(&mapV, c.V, rows, D)) {
+  if (!cached_maps(&mapK, c.K, rows, D) || !cached_maps(&mapV, c.V, rows, D)) {
     if (ctx.err == cudaSuccess) ctx.err = cudaErrorInvalidValue;
     return;
   }
-  // two CTAs per SM, never more than tiles could exist or than the partial pool holds
-  const long long max_tiles = (long long)p.B * p.H_kv * (p.N_cap / kTile);   // N_cap % 64 == 0: at least one
-  long long grid = 2LL * sm_count();
-  if (grid > kDecMaxCtas) grid = kDecMaxCtas;
-  // Two dozen units to one per SM: one cluster per unit, with as many CTAs per cluster (8, 4 or 2) as two per SM
-  // allow -- provided all clusters are resident at once and at least 0.6 of the CTA slots are used (16 units
-  // x 8 = 128 CTAs ran 17.3 us where the equal ranges over the whole list took 15.9 us).  The idle-cache variant
-  // takes clusters from 0.2 of the slots on: the slots a small launch leaves free are where the next launch's CTAs
-  // start reading (16 units x 8: 13.3 us against 15.4 us; 8 short units x 8: 8.1 against 11.8 us).
-  const int U = p.B * p.H_kv;
-  int cs = 1;
-  if (2 * U <= grid && p.N_cap / kTile >= 2) {
-    static int max_clusters_dev[64][4] = {};   // per device and log2(cluster size); 0 = not asked yet, -1 = none
-    for (int c = 8; c > 1 && cs == 1; c >>= 1) {
-      if ((long long)U * c > grid || (E ? 5LL * U * c < 1 * grid : 5LL * U * c < 3 * grid)) continue;
-      if (c == 8 && 4LL * U * c > 3 * grid) continue;   // 32 clusters of 8 are all resident, yet ran 16.7 us against 14.2 us
-      const int li = c == 8 ? 3 : (c == 4 ? 2 : 1);
-      int &mc = max_clusters_dev[dev & 63][li];
-      if (mc == 0) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)(U * c));
-        cfg.blockDim = dim3(kDecThreads);
-        cfg.dynamicSmemBytes = smem_bytes;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = (unsigned)c;
-        at[0].val.clusterDim.y = 1;
-        at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, decode_kernel<D, G, E>, &cfg) != cudaSuccess) { n = 0; cudaGetLastError(); }
-        mc = n > 0 ? n : -1;
-      }
-      if (U <= mc) cs = c;
-    }
-  }
+  // Two CTAs per SM.  One per SM, with the next launch's CTAs resident beside this one's, measured 10-15 % slower: three
+  // slots of 32 KB on an SM do not cover the latency of a loaded memory system, six do.
+  const int U = p.B * p.H_kv, slots = 2 * sm_count() < kDecMaxCtas ? 2 * sm_count() : kDecMaxCtas;
+  // One cluster of 8, 4, 2 or 1 CTAs per unit, the most that are resident at once and still get a tile each (8 units of
+  // 1656 entries: 6.3 us with 8 CTAs, 7.8 us with 4, 9.6 us with 18 that meet in global memory).
+  int cs = U <= slots ? 1 : 0;
+  for (int k = 8; k > 1 && cs == 1; k >>= 1)
+    if (U * k <= slots && p.N_cap / k >= kDecTile) cs = k;
+  // Few long units: clusters would leave most of the chip idle, so the list of groups is cut into equal ranges (16 units
+  // of 32768: 51 us against 54 us; the gap widens with fewer units).
+  if (5 * U * cs < 2 * slots && p.N_cap > 1024 * cs) cs = 0;
   if (cs > 1) {
     launch_pdl_cluster(decode_kernel<D, G, E>, dim3((unsigned)(U * cs)), dim3(kDecThreads), smem_bytes, ctx.stream, cs,
-        mapK, mapV, p, c, reinterpret_cast<const __nv_bfloat16 *>(q), reinterpret_cast<__nv_bfloat16 *>(out), lse,
-        update_scores, reinterpret_cast<int *>(ws + L.counters), reinterpret_cast<PartRec<D, G> *>(ws + L.part_pool),
-        status_dev, reinterpret_cast<const uint4 *>(k_new), reinterpret_cast<const uint4 *>(v_new), g_dbg_spin, g_dbg_withhold);
+      mapK, mapV, p, c, reinterpret_cast<const __nv_bfloat16 *>(q), reinterpret_cast<__nv_bfloat16 *>(out), lse,
+      update_scores, reinterpret_cast<int *>(ws + L.counters), reinterpret_cast<PartRec<D, G> *>(ws + L.part_pool),
+      status_dev, reinterpret_cast<const uint4 *>(k_new), reinterpret_cast<const uint4 *>(v_new), g_dbg_spin, g_dbg_withhold);
     KEEPKV_CHECK_LAUNCH(ctx);
     return;
   }
-  if (grid > max_tiles) grid = max_tiles;
+  const int grid = cs ? U : slots;
   launch_pdl(decode_kernel<D, G, E>, dim3((unsigned)grid), dim3(kDecThreads), smem_bytes, ctx.stream,
       mapK, mapV, p, c, reinterpret_cast<const __nv_bfloat16 *>(q), reinterpret_cast<__nv_bfloat16 *>(out), lse,
       update_scores, reinterpret_cast<int *>(ws + L.counters), reinterpret_cast<PartRec<D, G> *>(ws + L.part_pool),

@@ -77,6 +77,39 @@ def test_decode_one_cluster_per_unit(B, H_kv, G, d, lens):
     assert torch.equal(out.view(torch.int16), out2.view(torch.int16)) and torch.equal(lse.view(torch.int32), lse2.view(torch.int32))
 
 
+@pytest.mark.parametrize("G,d", [(1, 64), (8, 64), (2, 128), (8, 128)])
+@pytest.mark.parametrize("lens", [
+    [1, 31, 32, 33, 127, 128, 129, 160, 255, 257, 384, 515],    # unequal: equal ranges over the list of 32-entry groups
+    [509, 510, 511, 512, 513, 514],                             # similar: one cluster per unit
+    [2900],                                                     # two long units: ranges of a unit that meet in memory
+])
+def test_decode_group_and_tile_edges(G, d, lens):
+    """Lengths around the 32-entry groups and 128-entry tiles of the decode kernel, the step's token appended (it opens a
+    group for some sequences), with NaN in every row past a sequence: the oracle's rules of check_decode_unit."""
+    H_kv, B = 2, len(lens)
+    p = kb.make_params(B=B, H_q=H_kv * G, H_kv=H_kv, d=d, N_cap=-(-(max(lens) + 1) // 64) * 64, ema_alpha=0.9)
+    cache = random_cache(p, lens, seed=G + d + len(lens), vote_max=4, scored_frac=0.7)
+    for b, n in enumerate(lens):
+        cache.K[b, :, n:] = float("nan")
+        cache.V[b, :, n:] = float("nan")
+    rng = np.random.default_rng(21)
+    mk = lambda *s: f32_to_dev_bf16(rng.standard_normal(s).astype(np.float32))
+    q, kn, vn = _q(p, 5), mk(B, H_kv, d), mk(B, H_kv, d)
+    twin = kb.Cache(cache.K.clone(), cache.V.clone(), cache.votes.clone(), cache.lscore.clone(), cache.seq_len.clone())
+    ws, st = kb.new_workspace(p), kb.new_status()
+    kb.keepkv_append(p, twin, kn, vn, st)
+    hc = HostCache(twin)
+    out, lse = torch.empty_like(q), torch.empty(B, p.H_q, dtype=torch.float32, device="cuda")
+    kb.keepkv_decode_step(p, cache, q, kn, vn, out, lse, True, ws, st)
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0 and torch.equal(cache.seq_len, twin.seq_len)
+    assert torch.equal(cache.K.view(torch.int16), twin.K.view(torch.int16)) and torch.equal(cache.V.view(torch.int16), twin.V.view(torch.int16))
+    assert torch.equal(cache.votes, twin.votes)
+    ls_after = to_f64(cache.lscore).reshape(B * H_kv, -1)
+    for u in range(B * H_kv):
+        check_decode_unit(p, u, hc, to_f64(q), to_f64(out), to_f64(lse), ls_after, what=f"edges G={G} d={d}")
+
+
 def test_decode_without_score_update_leaves_lscore():
     p = kb.make_params(B=2, H_q=8, H_kv=2, d=128, N_cap=256)
     cache = random_cache(p, [256, 100], seed=3)

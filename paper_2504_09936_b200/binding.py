@@ -43,6 +43,7 @@ STATS_FIELDS = ("n_retained", "n_evicted", "n_merged", "n_below_T", "n_guard_gro
                 "reserved")
 
 _lib = None
+_raw_stream, _current_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
 
 
 def lib() -> C.CDLL:
@@ -102,6 +103,7 @@ class Cache:
     lscore: torch.Tensor   # f32  [B, H_kv, N_cap]
     seq_len: torch.Tensor  # i32  [B]
     _c: keepkv_cache = field(default=None, repr=False)
+    _ref: object = field(default=None, repr=False)
 
     @staticmethod
     def empty(p: keepkv_params, device="cuda") -> "Cache":
@@ -120,9 +122,16 @@ class Cache:
                                    self.lscore.data_ptr(), self.seq_len.data_ptr())
         return self._c
 
+    def ref(self):
+        """The same, as the pointer argument of a call."""
+        if self._ref is None:
+            self._ref = C.byref(self.c())
+        return self._ref
+
 
 def _stream(stream=None) -> int:
-    return (stream if stream is not None else torch.cuda.current_stream()).cuda_stream
+    # (the handle alone: building torch.cuda.current_stream()'s object takes 3 us, most of what the binding adds to a call)
+    return stream.cuda_stream if stream is not None else _raw_stream(_current_device())
 
 
 def _ptr(t):
@@ -147,19 +156,19 @@ def new_status(device="cuda") -> torch.Tensor:
 
 
 def keepkv_append(p, cache: Cache, k_new, v_new, status, stream=None):
-    _check(lib().keepkv_append(C.byref(p), C.byref(cache.c()), k_new.data_ptr(), v_new.data_ptr(), status.data_ptr(),
+    _check(lib().keepkv_append(C.byref(p), cache.ref(), k_new.data_ptr(), v_new.data_ptr(), status.data_ptr(),
                                _stream(stream)), "keepkv_append")
 
 
 def keepkv_decode_attention(p, cache: Cache, q, out, lse, update_scores: bool, ws, status, stream=None):
-    _check(lib().keepkv_decode_attention(C.byref(p), C.byref(cache.c()), q.data_ptr(), out.data_ptr(), _ptr(lse),
+    _check(lib().keepkv_decode_attention(C.byref(p), cache.ref(), q.data_ptr(), out.data_ptr(), _ptr(lse),
                                          int(update_scores), ws.data_ptr(), ws.numel(), status.data_ptr(),
                                          _stream(stream)), "keepkv_decode_attention")
 
 
 def keepkv_decode_step(p, cache: Cache, q, k_new, v_new, out, lse, update_scores: bool, ws, status, stream=None):
     """keepkv_append followed by keepkv_decode_attention in one launch."""
-    _check(lib().keepkv_decode_step(C.byref(p), C.byref(cache.c()), q.data_ptr(), k_new.data_ptr(), v_new.data_ptr(),
+    _check(lib().keepkv_decode_step(C.byref(p), cache.ref(), q.data_ptr(), k_new.data_ptr(), v_new.data_ptr(),
                                     out.data_ptr(), _ptr(lse), int(update_scores), ws.data_ptr(), ws.numel(),
                                     status.data_ptr(), _stream(stream)), "keepkv_decode_step")
 
@@ -168,7 +177,7 @@ def keepkv_decode_attention_static(p, cache: Cache, q, out, lse, update_scores: 
     """keepkv_decode_attention without a caller workspace, for code that cannot allocate device memory:
     the scratch is a fixed array inside the library (shared by all calls on the GPU, so keep them
     on one stream; make the first call on a device outside stream capture)."""
-    _check(lib().keepkv_decode_attention_static(C.byref(p), C.byref(cache.c()), q.data_ptr(), out.data_ptr(),
+    _check(lib().keepkv_decode_attention_static(C.byref(p), cache.ref(), q.data_ptr(), out.data_ptr(),
                                                 _ptr(lse), int(update_scores), status.data_ptr(), _stream(stream)),
            "keepkv_decode_attention_static")
 
@@ -176,7 +185,7 @@ def keepkv_decode_attention_static(p, cache: Cache, q, out, lse, update_scores: 
 def keepkv_prefill_scores(p, cache: Cache, q_window, status, stream=None):
     """q_window: bf16 CUDA tensor [B, H_q, W, d], the last W prompt queries, oldest first (Eq. 8, first case)."""
     assert q_window.is_contiguous() and q_window.dim() == 4
-    _check(lib().keepkv_prefill_scores(C.byref(p), C.byref(cache.c()), q_window.data_ptr(), int(q_window.shape[2]),
+    _check(lib().keepkv_prefill_scores(C.byref(p), cache.ref(), q_window.data_ptr(), int(q_window.shape[2]),
                                        status.data_ptr(), _stream(stream)), "keepkv_prefill_scores")
 
 
@@ -184,7 +193,7 @@ def keepkv_compress(p, src: Cache, dst: Cache, budget, ws, status, n_recent_dev=
                     target=None, stats=None, stream=None):
     """budget: int (same for every sequence) or an int32 CUDA tensor [B]."""
     bdev, bsc = (budget.data_ptr(), 0) if isinstance(budget, torch.Tensor) else (None, int(budget))
-    _check(lib().keepkv_compress(C.byref(p), C.byref(src.c()), C.byref(dst.c()), bdev, bsc, _ptr(n_recent_dev),
+    _check(lib().keepkv_compress(C.byref(p), src.ref(), dst.ref(), bdev, bsc, _ptr(n_recent_dev),
                                  _ptr(retained_idx), _ptr(target), _ptr(stats), ws.data_ptr(), ws.numel(),
                                  status.data_ptr(), _stream(stream)), "keepkv_compress")
 
@@ -194,7 +203,7 @@ def keepkv_compress_scored(p, src: Cache, dst: Cache, select_score, budget, ws, 
     """keepkv_compress with the caller's importance scores (fp32 CUDA tensor [B, H_kv, N_cap]) driving the selection."""
     assert select_score.dtype == torch.float32 and select_score.is_contiguous()
     bdev, bsc = (budget.data_ptr(), 0) if isinstance(budget, torch.Tensor) else (None, int(budget))
-    _check(lib().keepkv_compress_scored(C.byref(p), C.byref(src.c()), C.byref(dst.c()), select_score.data_ptr(), bdev,
+    _check(lib().keepkv_compress_scored(C.byref(p), src.ref(), dst.ref(), select_score.data_ptr(), bdev,
                                         bsc, _ptr(n_recent_dev), _ptr(retained_idx), _ptr(target), _ptr(stats),
                                         ws.data_ptr(), ws.numel(), status.data_ptr(), _stream(stream)),
            "keepkv_compress_scored")
@@ -213,7 +222,7 @@ def keepkv_complete_load_host(p, K_host, V_host, seq_len_host, dev: Cache, strea
     for t in (K_host, V_host, seq_len_host):
         assert not t.is_cuda and t.is_contiguous()
     _check(lib().keepkv_complete_load_host(C.byref(p), K_host.data_ptr(), V_host.data_ptr(), seq_len_host.data_ptr(),
-                                           C.byref(dev.c()), _stream(stream)), "keepkv_complete_load_host")
+                                           dev.ref(), _stream(stream)), "keepkv_complete_load_host")
 
 
 def keepkv_compress_inplace(p, cache: Cache, pos, pos_len, n_seen, budget, ws, status, n_recent_dev=None, moved_from=None,
@@ -222,7 +231,7 @@ def keepkv_compress_inplace(p, cache: Cache, pos, pos_len, n_seen, budget, ws, s
     for t in (pos, pos_len, n_seen):
         assert t.dtype == torch.int32 and t.is_cuda and t.is_contiguous()
     bdev, bsc = (budget.data_ptr(), 0) if isinstance(budget, torch.Tensor) else (None, int(budget))
-    _check(lib().keepkv_compress_inplace(C.byref(p), C.byref(cache.c()), pos.data_ptr(), pos_len.data_ptr(), n_seen.data_ptr(),
+    _check(lib().keepkv_compress_inplace(C.byref(p), cache.ref(), pos.data_ptr(), pos_len.data_ptr(), n_seen.data_ptr(),
                                          bdev, bsc, _ptr(n_recent_dev), _ptr(moved_from), _ptr(target), _ptr(stats),
                                          ws.data_ptr(), ws.numel(), status.data_ptr(), _stream(stream)),
            "keepkv_compress_inplace")
@@ -233,7 +242,7 @@ def keepkv_compress_merge_first(p, cache: Cache, scratch: Cache, budget, ws, sta
     """Prefill compression, merge-first policy (Section 3.4): similar entries of the prompt are merged with each
     other, then the selection cuts the result to the budget.  In place on `cache`; `scratch` is destroyed."""
     bdev, bsc = (budget.data_ptr(), 0) if isinstance(budget, torch.Tensor) else (None, int(budget))
-    _check(lib().keepkv_compress_merge_first(C.byref(p), C.byref(cache.c()), C.byref(scratch.c()), bdev, bsc,
+    _check(lib().keepkv_compress_merge_first(C.byref(p), cache.ref(), scratch.ref(), bdev, bsc,
                                              _ptr(n_recent_dev), _ptr(retained_idx), _ptr(stats), ws.data_ptr(),
                                              ws.numel(), status.data_ptr(), _stream(stream)),
            "keepkv_compress_merge_first")
@@ -241,7 +250,7 @@ def keepkv_compress_merge_first(p, cache: Cache, scratch: Cache, budget, ws, sta
 
 def keepkv_decode_step_host(p, cache: Cache, q_host, k_new_host, v_new_host, out_host, q_dev, k_new_dev, v_new_dev,
                             out_dev, update_scores: bool, ws, status, stream=None):
-    _check(lib().keepkv_decode_step_host(C.byref(p), C.byref(cache.c()), q_host.data_ptr(), k_new_host.data_ptr(),
+    _check(lib().keepkv_decode_step_host(C.byref(p), cache.ref(), q_host.data_ptr(), k_new_host.data_ptr(),
                                          v_new_host.data_ptr(), out_host.data_ptr(), q_dev.data_ptr(),
                                          k_new_dev.data_ptr(), v_new_dev.data_ptr(), out_dev.data_ptr(),
                                          int(update_scores), ws.data_ptr(), ws.numel(), status.data_ptr(),

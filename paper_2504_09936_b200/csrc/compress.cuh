@@ -228,7 +228,7 @@ __device__ __forceinline__ void offer4(Top2 &ta, Top2 &tb, float a0, float a1, f
     if (!__any_sync(0xffffffffu, (int)s >= 0)) return;   // no lane has a value that is not below its cut
   }
   ta.insert(a0 * w.x, idx); tb.insert(a1 * w.y, idx + 1); ta.insert(a2 * w.z, idx + 2); tb.insert(a3 * w.w, idx + 3);
-  if (TEST) ta.cut = fmaxf(ta.best, tb.best) - ta.thr;
+  if (TEST) ta.cut = fmaxf(ta.cut, fmaxf(ta.best, tb.best) - ta.thr);   // (a cut only rises: it may have started above the best)
 }
 
 // ------------------------------------------------------------------ the interface's cosine

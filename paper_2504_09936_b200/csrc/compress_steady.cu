@@ -327,14 +327,12 @@ steady_compress_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, cons
       tc_fence_before();
       __syncthreads();             // everyone's; and everyone has finished the previous iteration
       tc_fence_after();
-      if (tid == 0 && !s_abort) {
-        const uint32_t a_base = sbase + SL::kA, b_base = sbase + SL::kRing + (i % S) * SL::kStageBytes;
+      if (warp == 0 && !__any_sync(0xffffffffu, s_abort) && elect_one()) {
+        const uint64_t ad = umma_desc_sw128(sbase + SL::kA), bd = umma_desc_sw128(sbase + SL::kRing + (i % S) * SL::kStageBytes);
 #pragma unroll
-        for (int k = 0; k < KSTEPS; ++k) {
-          const uint64_t ad = umma_desc_sw128(a_base + (k >> 2) * (kStEv * 128) + (k & 3) * 32);
-          const uint64_t bd = umma_desc_sw128(b_base + (k >> 2) * (kStN * 128) + (k & 3) * 32);
-          umma_bf16(tmem + (i & 1) * kStN, ad, bd, IDESC, k > 0 ? 1u : 0u);
-        }
+        for (int k = 0; k < KSTEPS; ++k)   // (descriptor addresses count 16-byte units)
+          umma_bf16(tmem + (i & 1) * kStN, ad + (k >> 2) * (kStEv * 8) + (k & 3) * 2, bd + (k >> 2) * (kStN * 8) + (k & 3) * 2,
+                    IDESC, k > 0 ? 1u : 0u);
         umma_commit(bar_t_full + 8 * (i & 1));
       }
       // the previous product has completed: its stage can be refilled and its accumulator drained

@@ -186,7 +186,7 @@ prefill_scores_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
-    if (lane == 0) {
+    if (elect_one()) {
       int n_units = 0;
       for (int it = 0; it < ntiles && !s_abort; ++it) {
         const int u = wk.b * p.H_kv + wk.h;
@@ -213,7 +213,7 @@ prefill_scores_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    if (elect_one()) {
       int n_units = 0;
       for (int it = 0; it < ntiles && !s_abort; ++it) {
         if (it == 0 || wk.tile == 0) {
@@ -224,15 +224,13 @@ prefill_scores_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_con
         if (!mbar_wait(bar_a_full + 8 * s, (it / kPfStages) & 1) ||
             !mbar_wait(bar_t_empty + 8 * a, ((it >> 1) & 1) ^ 1)) { s_abort = 1; break; }
         tc_fence_after();
-        const uint32_t a_base = sbase + SL::kA + s * SL::kABytes, b_base = sbase + SL::kB;
+        const uint64_t ad = umma_desc_sw128(sbase + SL::kA + s * SL::kABytes), bd = umma_desc_sw128(sbase + SL::kB);
 #pragma unroll
         for (int hf = 0; hf < TP; ++hf) {   // the 128-entry tiles of the hand-over, each into its own columns
 #pragma unroll
-          for (int k = 0; k < KSTEPS; ++k) {
-            const uint64_t ad = umma_desc_sw128(a_base + (k >> 2) * (ROWS * 128) + hf * (kPfM * 128) + (k & 3) * 32);
-            const uint64_t bd = umma_desc_sw128(b_base + (k >> 2) * (NB * 128) + (k & 3) * 32);
-            umma_bf16(tmem + (a * TP + hf) * NB, ad, bd, IDESC, k > 0 ? 1u : 0u);
-          }
+          for (int k = 0; k < KSTEPS; ++k)   // (descriptor addresses count 16-byte units)
+            umma_bf16(tmem + (a * TP + hf) * NB, ad + (k >> 2) * (ROWS * 8) + hf * (kPfM * 8) + (k & 3) * 2,
+                      bd + (k >> 2) * (NB * 8) + (k & 3) * 2, IDESC, k > 0 ? 1u : 0u);
         }
         umma_commit(bar_a_empty + 8 * s);
         umma_commit(bar_t_full + 8 * a);

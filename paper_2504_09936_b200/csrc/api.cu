@@ -32,7 +32,9 @@ WsLayout ws_layout(const keepkv_params &p) {
   L.ret_idx = take(U * N * 4);
   L.target = take(U * N * 4);
   L.ev_idx = take(U * N * 4);
+  // (the search reads whole 256-entry tiles of these two)
   L.inv_norm = take(U * N * 4);
+  L.norm_ext = take(U * N * 16 + 4096);
   L.nom_v = take(U * N * C * 16);
   L.nom_si = take(U * N * C * 4);
   L.grp_key = take(U * Np2 * 4);

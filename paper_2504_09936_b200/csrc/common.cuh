@@ -29,6 +29,7 @@ struct WsLayout {
   size_t target;      // i32 [U,N]          per source entry: slot, -1 dropped, -2 retained
   size_t ev_idx;      // i32 [U,N]          source indices of evicted entries, ascending
   size_t inv_norm;    // f32 [U,N]          1/|k| of each retained key (tree-summed; only ranks candidates)
+  size_t norm_ext;    // bf16 [U,N,8]       |k| of the same in three terms, as more channels of the search's columns
   size_t nom_v;       // float4 [U,N,C]     per evicted row and column chunk: best, second cosine, unused, best slot
   size_t nom_si;      // i32 [U,N,C]        slot of the second-best cosine
   size_t grp_key;     // u32 [U,Npow2]      (slot << 16 | evicted position) of merged entries, sorted
@@ -70,7 +71,7 @@ void launch_compress(const keepkv_params &p, const keepkv_cache &src, const keep
                      LaunchCtx &ctx, const float *select_key = nullptr);
 // tcgen05 similarity search: for every evicted key the two largest cosines over the retained keys
 void launch_nominate(const keepkv_params &p, const keepkv_cache &src, const keepkv_cache &dst, const int32_t *ev_idx,
-                     const UnitInfo *unit_info, const float *inv_norm, int32_t *sched, float4 *nom_v, int32_t *nom_si,
+                     const UnitInfo *unit_info, const float *inv_norm, const uint4 *norm_ext, int32_t *sched, float4 *nom_v, int32_t *nom_si,
                      int nom_chunks, int32_t *status_dev, LaunchCtx &ctx, int self_mask = 0);
 // Algorithm 1 in place on a cache with a position array (compress.cu)
 void launch_compress_inplace(const keepkv_params &p, const keepkv_cache &c, int32_t *pos, int32_t *pos_len, int32_t *n_seen,

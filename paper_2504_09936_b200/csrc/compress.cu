@@ -219,12 +219,12 @@ select_kernel(keepkv_params p, keepkv_cache src, int32_t *dst_seq_len, const int
 
 // ------------------------------------------------------------------ compact
 // grid (up to 32, U), 256 threads, 64 slots per CTA and sweep.  Sixteen lanes move one retained row (a 16-byte piece of
-// K and of V each); a warp has eight rows in flight.  The same lanes tree-sum the squared key for
-// the inverse norm the similarity search ranks with.
+// K and of V each); a warp has eight rows in flight.  The same lanes tree-sum the squared key
+// and, where a similarity search follows (norm_ext given), write what it needs of the key's norm.
 template <int D>
 __global__ void __launch_bounds__(256)
 compact_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, const int32_t *__restrict__ ret_idx,
-               const UnitInfo *__restrict__ unit_info, float *__restrict__ inv_norm) {
+               const UnitInfo *__restrict__ unit_info, float *__restrict__ inv_norm, uint4 *__restrict__ norm_ext) {
   constexpr int CH = D / 8;       // 16-byte chunks per row
   pdl_wait();
   pdl_trigger();
@@ -265,7 +265,10 @@ compact_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, const int32_
     ss += __shfl_xor_sync(0xffffffffu, ss, 4);
     ss += __shfl_xor_sync(0xffffffffu, ss, 8);
     if (si[r] >= 0 && ch == 0) {
-      inv_norm[base + slot[r]] = rsqrtf(ss);
+      if (norm_ext) {
+        norm_ext[base + slot[r]] = ext_col(sqrtf(ss));
+        inv_norm[base + slot[r]] = rsqrtf(ss);
+      }
       dst.votes[base + slot[r]] = src.votes[base + si[r]];
       dst.lscore[base + slot[r]] = src.lscore[base + si[r]];
     }
@@ -518,6 +521,7 @@ static void launch_compress_t(const keepkv_params &p, const keepkv_cache &src, c
   int32_t *sched = reinterpret_cast<int32_t *>(ws + L.sched);
   int32_t *ev_idx = reinterpret_cast<int32_t *>(ws + L.ev_idx);
   float *inv_norm = reinterpret_cast<float *>(ws + L.inv_norm);
+  uint4 *norm_ext = reinterpret_cast<uint4 *>(ws + L.norm_ext);
   float4 *nom_v = reinterpret_cast<float4 *>(ws + L.nom_v);
   int32_t *nom_si = reinterpret_cast<int32_t *>(ws + L.nom_si);
   uint32_t *grp_key = reinterpret_cast<uint32_t *>(ws + L.grp_key);
@@ -546,12 +550,13 @@ static void launch_compress_t(const keepkv_params &p, const keepkv_cache &src, c
   KEEPKV_CHECK_LAUNCH(ctx);
   if (ret_bound <= 0) return;   // nothing is kept: every entry is dropped, which select has recorded
   const int cgx = (ret_bound + 63) / 64 < 32 ? (ret_bound + 63) / 64 : 32;   // the retained count is only known on the device
-  launch_pdl(compact_kernel<D>, dim3(cgx, U), dim3(256), 0, ctx.stream, p, src, dst, ret_idx, ui,
-             inv_norm);
-  KEEPKV_CHECK_LAUNCH(ctx);
   // T = +inf: no cosine can exceed it, nothing merges -- the eviction strategy alone (what follows a merge-first pass)
-  if (isinf(p.merge_threshold) && p.merge_threshold > 0.f) return;
-  launch_nominate(p, src, dst, ev_idx, ui, inv_norm, sched, nom_v, nom_si, L.nom_chunks, status_dev, ctx);
+  const bool merges = !(isinf(p.merge_threshold) && p.merge_threshold > 0.f);
+  launch_pdl(compact_kernel<D>, dim3(cgx, U), dim3(256), 0, ctx.stream, p, src, dst, ret_idx, ui, inv_norm,
+             merges ? norm_ext : nullptr);
+  KEEPKV_CHECK_LAUNCH(ctx);
+  if (!merges) return;
+  launch_nominate(p, src, dst, ev_idx, ui, inv_norm, norm_ext, sched, nom_v, nom_si, L.nom_chunks, status_dev, ctx);
   launch_pdl(resolve_kernel<D>, dim3(L.nom_chunks, U), dim3(kResolveThreads), (size_t)smem_keys * 4, ctx.stream,
       p, src, dst, ev_idx, ui, nom_v, nom_si, sched, L.nom_chunks, ret_idx, target, grp_key, L.key_stride, grp_head,
       stats, smem_keys, 0);
@@ -580,7 +585,8 @@ static void launch_compress_t(const keepkv_params &p, const keepkv_cache &src, c
 //   merge       -> Eq. A.3 for units with many groups
 template <int D>
 __global__ void __launch_bounds__(256)
-mf_prepare_kernel(keepkv_params p, keepkv_cache src, int32_t *ev_idx, UnitInfo *unit_info, float *__restrict__ inv_norm) {
+mf_prepare_kernel(keepkv_params p, keepkv_cache src, int32_t *ev_idx, UnitInfo *unit_info, float *__restrict__ inv_norm,
+                  uint4 *__restrict__ norm_ext) {
   constexpr int CH = D / 8;
   pdl_wait();
   pdl_trigger();
@@ -605,7 +611,7 @@ mf_prepare_kernel(keepkv_params p, keepkv_cache src, int32_t *ev_idx, UnitInfo *
     ss += __shfl_xor_sync(0xffffffffu, ss, 2);
     ss += __shfl_xor_sync(0xffffffffu, ss, 4);
     ss += __shfl_xor_sync(0xffffffffu, ss, 8);
-    if (i < len && ch == 0) { inv_norm[base + i] = rsqrtf(ss); ev_idx[base + i] = i; }
+    if (i < len && ch == 0) { inv_norm[base + i] = rsqrtf(ss); norm_ext[base + i] = ext_col(sqrtf(ss)); ev_idx[base + i] = i; }
   }
 }
 
@@ -747,6 +753,7 @@ static void launch_compress_merge_first_t(const keepkv_params &p, const keepkv_c
   int32_t *target = reinterpret_cast<int32_t *>(ws + L.target);
   int32_t *ev_idx = reinterpret_cast<int32_t *>(ws + L.ev_idx);
   float *inv_norm = reinterpret_cast<float *>(ws + L.inv_norm);
+  uint4 *norm_ext = reinterpret_cast<uint4 *>(ws + L.norm_ext);
   float4 *nom_v = reinterpret_cast<float4 *>(ws + L.nom_v);
   int32_t *nom_si = reinterpret_cast<int32_t *>(ws + L.nom_si);
   uint32_t *grp_key = reinterpret_cast<uint32_t *>(ws + L.grp_key);
@@ -768,10 +775,10 @@ static void launch_compress_merge_first_t(const keepkv_params &p, const keepkv_c
   // ---- pass 1: similar entries merged with each other, cache -> scratch (every head keeps its own length for now)
   int gx = 2 * sm_count() / U;
   gx = gx < 1 ? 1 : (gx > 32 ? 32 : gx);
-  launch_pdl(mf_prepare_kernel<D>, dim3(gx, U), dim3(256), 0, ctx.stream, p, cache, ev_idx, ui, inv_norm);
+  launch_pdl(mf_prepare_kernel<D>, dim3(gx, U), dim3(256), 0, ctx.stream, p, cache, ev_idx, ui, inv_norm, norm_ext);
   KEEPKV_CHECK_LAUNCH(ctx);
   // rows and columns are the same keys: the "retained" operand of the search is the prompt itself
-  launch_nominate(p, cache, cache, ev_idx, ui, inv_norm, sched, nom_v, nom_si, L.nom_chunks, status_dev, ctx, 1);
+  launch_nominate(p, cache, cache, ev_idx, ui, inv_norm, norm_ext, sched, nom_v, nom_si, L.nom_chunks, status_dev, ctx, 1);
   launch_pdl(resolve_kernel<D>, dim3(L.nom_chunks, U), dim3(kResolveThreads), (size_t)smem_keys * 4, ctx.stream,
       p, cache, cache, ev_idx, ui, nom_v, nom_si, sched, L.nom_chunks, ret1, target, grp_key, L.key_stride, grp_head,
       st1, smem_keys, 1);
@@ -780,7 +787,7 @@ static void launch_compress_merge_first_t(const keepkv_params &p, const keepkv_c
              L.key_stride, ui, st1);
   KEEPKV_CHECK_LAUNCH(ctx);
   const int cgx = (p.N_cap + 63) / 64 < 32 ? (p.N_cap + 63) / 64 : 32;
-  launch_pdl(compact_kernel<D>, dim3(cgx, U), dim3(256), 0, ctx.stream, p, cache, scratch, ret1, ui, inv_norm);
+  launch_pdl(compact_kernel<D>, dim3(cgx, U), dim3(256), 0, ctx.stream, p, cache, scratch, ret1, ui, inv_norm, (uint4 *)nullptr);
   KEEPKV_CHECK_LAUNCH(ctx);
   launch_pdl(group_kernel<D>, dim3(U), dim3(kResolveThreads), (size_t)smem_keys * 4, ctx.stream, p, cache, scratch, ret1,
              ev_idx, target, ui, grp_key, L.key_stride, grp_head, st1, smem_keys);
@@ -799,7 +806,7 @@ static void launch_compress_merge_first_t(const keepkv_params &p, const keepkv_c
              (const int32_t *)eff_budget, 0, n_recent_dev, ret2, target, ev_idx, ui, st2, (const float *)nullptr,
              (const int32_t *)unit_len, (int32_t *)nullptr, (const int32_t *)nullptr, (const int32_t *)nullptr, status_dev);
   KEEPKV_CHECK_LAUNCH(ctx);
-  launch_pdl(compact_kernel<D>, dim3(cgx, U), dim3(256), 0, ctx.stream, p, scratch, cache, ret2, ui, inv_norm);
+  launch_pdl(compact_kernel<D>, dim3(cgx, U), dim3(256), 0, ctx.stream, p, scratch, cache, ret2, ui, inv_norm, (uint4 *)nullptr);
   KEEPKV_CHECK_LAUNCH(ctx);
   if (ret_idx_out || stats_out) {
     launch_pdl(mf_compose_kernel, dim3(4, U), dim3(256), 0, ctx.stream, p, cache.seq_len, ret1, ret2, ret_idx_out, st1, ui,
@@ -833,7 +840,7 @@ void launch_compress_merge_first(const keepkv_params &p, const keepkv_cache &cac
 template <int D>
 __global__ void __launch_bounds__(256)
 ip_prepare_kernel(keepkv_params p, keepkv_cache c, const int32_t *__restrict__ target, int32_t *ident, UnitInfo *unit_info,
-                  float *__restrict__ inv_norm) {
+                  float *__restrict__ inv_norm, uint4 *__restrict__ norm_ext) {
   constexpr int CH = D / 8;
   pdl_wait();
   pdl_trigger();
@@ -856,6 +863,7 @@ ip_prepare_kernel(keepkv_params p, keepkv_cache c, const int32_t *__restrict__ t
     ss += __shfl_xor_sync(0xffffffffu, ss, 4);
     ss += __shfl_xor_sync(0xffffffffu, ss, 8);
     if (i < len && ch == 0) {
+      norm_ext[base + i] = ext_col(kept ? sqrtf(ss) : kExtNever);
       inv_norm[base + i] = kept ? rsqrtf(ss) : __int_as_float(0x7fffffff);   // a row that is not retained is no column
       ident[base + i] = i;   // the slot of a target is its row
     }
@@ -931,6 +939,7 @@ static void launch_compress_inplace_t(const keepkv_params &p, const keepkv_cache
   int32_t *kept = reinterpret_cast<int32_t *>(ws + L.kept);        // retained rows, ascending
   int32_t *ev_idx = reinterpret_cast<int32_t *>(ws + L.ev_idx);
   float *inv_norm = reinterpret_cast<float *>(ws + L.inv_norm);
+  uint4 *norm_ext = reinterpret_cast<uint4 *>(ws + L.norm_ext);
   float4 *nom_v = reinterpret_cast<float4 *>(ws + L.nom_v);
   int32_t *nom_si = reinterpret_cast<int32_t *>(ws + L.nom_si);
   uint32_t *grp_key = reinterpret_cast<uint32_t *>(ws + L.grp_key);
@@ -950,13 +959,13 @@ static void launch_compress_inplace_t(const keepkv_params &p, const keepkv_cache
   KEEPKV_CHECK_LAUNCH(ctx);
   int gx = 2 * sm_count() / U;
   gx = gx < 1 ? 1 : (gx > 32 ? 32 : gx);
-  launch_pdl(ip_prepare_kernel<D>, dim3(gx, U), dim3(256), 0, ctx.stream, p, c, (const int32_t *)target, ident, ui, inv_norm);
+  launch_pdl(ip_prepare_kernel<D>, dim3(gx, U), dim3(256), 0, ctx.stream, p, c, (const int32_t *)target, ident, ui, inv_norm, norm_ext);
   KEEPKV_CHECK_LAUNCH(ctx);
   const bool merges = !(isinf(p.merge_threshold) && p.merge_threshold > 0.f);
   if (merges) {
     launch_pdl(ip_columns_kernel, dim3((U + 127) / 128), dim3(128), 0, ctx.stream, ui, U, 1);
     KEEPKV_CHECK_LAUNCH(ctx);
-    launch_nominate(p, c, c, ev_idx, ui, inv_norm, sched, nom_v, nom_si, L.nom_chunks, status_dev, ctx);
+    launch_nominate(p, c, c, ev_idx, ui, inv_norm, norm_ext, sched, nom_v, nom_si, L.nom_chunks, status_dev, ctx);
     launch_pdl(resolve_kernel<D>, dim3(L.nom_chunks, U), dim3(kResolveThreads), (size_t)smem_keys * 4, ctx.stream,
         p, c, c, ev_idx, ui, nom_v, nom_si, sched, L.nom_chunks, ident, target, grp_key, L.key_stride, grp_head,
         stats, smem_keys, 0);

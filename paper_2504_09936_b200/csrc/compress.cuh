@@ -231,6 +231,26 @@ __device__ __forceinline__ void offer4(Top2 &ta, Top2 &tb, float a0, float a1, f
   if (TEST) ta.cut = fmaxf(ta.cut, fmaxf(ta.best, tb.best) - ta.thr);   // (a cut only rises: it may have started above the best)
 }
 
+// ------------------------------------------------------------------ the cut inside the product
+// c |k_c| as six products of bf16 terms (c = c1 + c2 + c3 and likewise the norm; what is left out is below 2^-23 of it):
+// eight more channels of a row and of a column, whose product subtracts it from the accumulator.
+constexpr float kExtNever = 1.2676506e30f;   // 2^100: a row no column reaches, a column that reaches no row
+__device__ __forceinline__ void bf16_terms(float x, float &t1, float &t2, float &t3) {
+  t1 = __bfloat162float(__float2bfloat16_rn(x));
+  t2 = __bfloat162float(__float2bfloat16_rn(x - t1));
+  t3 = x - t1 - t2;
+}
+__device__ __forceinline__ uint4 ext_row(float c) {
+  float a, b, d;
+  bf16_terms(c, a, b, d);
+  return make_uint4(pack_bf16(-a, -a), pack_bf16(-b, -a), pack_bf16(-b, -d), 0u);
+}
+__device__ __forceinline__ uint4 ext_col(float n) {
+  float a, b, d;
+  bf16_terms(n, a, b, d);
+  return make_uint4(pack_bf16(a, b), pack_bf16(a, d), pack_bf16(b, a), 0u);
+}
+
 // ------------------------------------------------------------------ the interface's cosine
 // One warp evaluates cos(k_e, k_a) and cos(k_e, k_b) in the fixed fp32 arithmetic of the interface:
 // dot and squared norms by fused multiply-add from 0 over channels 0..D-1, then dot/(sqrtf(n_e)*sqrtf(n_c)).

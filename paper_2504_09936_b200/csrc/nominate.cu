@@ -5,104 +5,131 @@
 // ranking is closer than the accumulation error allows, the caller re-evaluates the candidates in
 // the fixed fp32 arithmetic the interface defines (see resolve_kernel in compress.cu).
 //
+// Only columns whose cosine exceeds the merge threshold matter: an entry whose best cosine does not exceed it is dropped
+// whatever its best column was.  So the product itself subtracts the threshold: eight more channels -- the row's cut
+// (threshold less a margin, times the row's norm) and the column's norm, both as three bf16 terms, six cross products --
+// make the accumulator  k_e . k_c - cut_e |k_c|,  and 32 columns are screened by 20 maxima and one vote.  What passes (a
+// fifth of the 32 x 32 blocks at a threshold of 0.8 on keys with outlier channels) is looked at four columns at a time.
+// For a threshold below kNomStatic, where nearly every block would pass, those channels are zero and the screen is the
+// running cut itself: one packed multiply-add per two columns.
+//
 // Work item = (unit, 128 evicted rows, one chunk of 256-column tiles of the unit's retained keys).
 // A persistent grid of one CTA per SM walks the items.  Inside a CTA:
-//   warp 0      TMA producer: retained-key tiles (256 rows x D, 128-byte swizzle) from the compacted
-//               dst cache into a 2-stage ring;
-//   warp 1      one thread issues tcgen05.mma (M=128, N=256, K=16, bf16 -> fp32) into one of two
-//               256-column accumulators in tensor memory and commits to the ring / accumulator barriers;
-//   warps 2-3   gather the 128 evicted rows of the next item from the src cache into the other swizzled A tile;
-//   warps 4-19  drain the accumulators with tcgen05.ld: four warps per 32-lane quarter, each 64 of a tile's 256
-//               columns, scaling by the retained keys' inverse norms and tracking the row's top two.
-// Bound: the drain's instructions.  It looks only at columns that can matter: those above the running cut of their row,
-// which starts just below the merge threshold (an entry whose best cosine does not exceed it is dropped whatever its
-// best column was) and follows the row's best.  32 columns are screened by 16 packed multiply-adds (value * inverse norm
-// - cut, two columns each), 16 three-input maxima and one vote: 1.4 instructions per (row, column) pair where testing
-// groups of four against a cut that starts at minus infinity took 14.6.
-// Every wait is bounded; a wait that runs out raises KEEPKV_DEV_TIMEOUT, the CTA stops issuing work,
-// drains what is in flight, frees its tensor memory and returns.
-#include <type_traits>
-
+//   warp 0      copies: column tiles (256 rows x D, 128-byte swizzle, and their norms), 64 channels at a time into a
+//               4-stage ring, so that three quarters of it are in flight while one is multiplied;
+//   warp 1      tensor cores: M = 128, N = 256, bf16 -> fp32, into one of two accumulators in tensor memory;
+//   warps 2-3   gather the evicted rows of the next item from the src cache into the other A tile;
+//   warps 4-19  drain: four warps per 32 rows, 64 of a tile's 256 columns each.
+// Bound: the tensor pipe at the rate it sustains (with its extra sixteenth of the channels) and, beside it, the hand-overs.
+// Measured, 64 units of 6554 x 1638 keys of 128 channels, 176 GFLOP: 525 us when every accumulator was scaled by its
+// column's norm and tested against a cut that starts at minus infinity (1.46 instructions per row and column of a warp),
+// 378 us with the scaled values screened 32 at a time against a cut that starts at the threshold (0.85), 205 us in this
+// form; without the drain it is 177 us.  256 rows an item, as two products of N = 128 a column tile, measured equal.
+// Every wait is bounded; a wait that runs out raises KEEPKV_DEV_TIMEOUT, every warp of the CTA leaves its loop, what is
+// in flight gets a bounded time to end, tensor memory is freed.
 #include "compress.cuh"
 #include "ptx.cuh"
 
 namespace keepkv {
 
-constexpr int kNomM = 128;        // evicted rows per item (tensor-memory lanes)
-constexpr int kNomN = 256;        // retained columns per tile
-constexpr int kNomStages = 2;     // B ring
-constexpr int kNomDrainWarps = 16; // four per 32-lane quarter of tensor memory, each a quarter of a tile's columns
-constexpr int kNomGatherWarps = 2;   // (20 warps: 96 registers each)
+constexpr int kNomM = 128;         // evicted rows per item (tensor-memory lanes)
+constexpr int kNomN = 256;         // retained columns per tile
+constexpr int kNomStages = 4;      // column ring: 64 channels of a tile each
+constexpr int kNomDrainWarps = 16;
+constexpr int kNomGatherWarps = 2; // (20 warps in all: 96 registers a thread)
 constexpr int kNomThreads = 32 * (2 + kNomGatherWarps + kNomDrainWarps);
+constexpr float kNomStatic = 0.5f; // thresholds from here on are subtracted by the product
 
 template <int D>
 struct NomSmem {
   static constexpr int kSub = D / 64;                     // 64-channel (128-byte) K atoms per row
   static constexpr int kABytes = kSub * kNomM * 128;
-  static constexpr int kBBytes = kSub * kNomN * 128;
-  static constexpr int kA = 0;
-  static constexpr int kB = 2 * kABytes;                  // two A tiles: the next item is gathered while this one is drained
-  static constexpr int kInv = kB + kNomStages * kBBytes;  // f32 [16 warps][64]   inverse norms of the warp's columns
-  static constexpr int kRowInv = kInv + 16 * 64 * 4;      // f32 [2][128]         inverse norms of the staged rows
-  static constexpr int kXchg = kRowInv + 2 * 128 * 4;     // u32 [3][128][3][3]   exchange between the column quarters
-  static constexpr int kCoarse = kXchg + 3 * 128 * 9 * 4; // i32 [kMaxUnits / 32] row tiles before each 32 units
-  static constexpr int kFine = kCoarse + kMaxUnits / 32 * 4;   // u16 [kMaxUnits] and before each unit among its 32
-  static constexpr int kBytes = kFine + kMaxUnits * 2;
+  static constexpr int kBBytes = kNomN * 128;
+  static constexpr int kTiles = kNomStages / kSub;        // column tiles the ring holds
+  static constexpr int kA = 0;                            // [2]: the next item is gathered while this one runs
+  static constexpr int kB = 2 * kABytes;
+  static constexpr int kAX = kB + kNomStages * kBBytes;   // [2][128] x 16 B  eight more channels of the rows
+  static constexpr int kBX = kAX + 2 * kNomM * 16;        // [kTiles][256] x 16 B  and of the columns
+  static constexpr int kZero = kBX + kTiles * kNomN * 16; // [256] x 16 B  and eight more that are zero, for all of them
+  // Inverse norms of the columns outlive their tile's stages: when tile t + 2 has been multiplied, tile t has been drained.
+  static constexpr int kInvTiles = kTiles + 2 <= 4 ? 4 : 8;
+  static constexpr int kInv = kZero + kNomN * 16;              // f32 [kInvTiles][256]
+  static constexpr int kRowInv = kInv + kInvTiles * kNomN * 4; // f32 [2][128]        inverse norms of the staged rows
+  static constexpr int kXchg = kRowInv + 2 * kNomM * 4;        // u32 [2][128][3][3]  results of the later column quarters
+  static constexpr int kCoarse = kXchg + 2 * kNomM * 36;       // i32 [kMaxUnits / 32]  row tiles before each 32 units
+  static constexpr int kBytes = kCoarse + kMaxUnits / 32 * 4;
 };
 
-struct NomItem { int u, m_tile, chunk, t0, t1, n_ev, n_ret; };
+// Four columns idx..idx+3: accumulators a_i, inverse norms w_i.  Skipped by the whole warp unless a row has one at its cut.
+// (What is left of a missing column's inverse norm may have any sign: -inf stays -inf.)
+__device__ __forceinline__ void offer4_above(Top2 &ta, Top2 &tb, float a0, float a1, float a2, float a3, const float4 w,
+                                             int idx) {
+  const float v0 = a0 * fabsf(w.x), v1 = a1 * fabsf(w.y), v2 = a2 * fabsf(w.z), v3 = a3 * fabsf(w.w);
+  if (!__any_sync(0xffffffffu, max3(fmaxf(v0, v1), v2, v3) >= ta.cut)) return;
+  ta.insert(v0, idx); tb.insert(v1, idx + 1); ta.insert(v2, idx + 2); tb.insert(v3, idx + 3);
+  ta.cut = fmaxf(ta.cut, fmaxf(ta.best, tb.best) - ta.thr);   // (it only rises: it may have started above the best)
+}
 
-// Row tiles before each unit, in two levels (a unit has at most 384 of them, 32 units fewer than 2^16).
-struct NomPrefix {
-  const int *coarse;
-  const uint16_t *fine;
-  __device__ __forceinline__ int operator[](int u) const { return coarse[u >> 5] + fine[u]; }
-};
+struct __align__(16) NomItem { int u, m0, chunk, t0, t1, n_ev, n_ret, pad; };
 
-__device__ __forceinline__ NomItem nom_item(int item, int C, const NomPrefix prefix, int U, const UnitInfo *unit_info) {
+// The whole warp looks an item up: among the units' row tiles first by groups of 32 units, then inside the group.
+__device__ __forceinline__ NomItem nom_item(int item, int C, const int *coarse, int U, const UnitInfo *unit_info) {
+  const int lane = threadIdx.x & 31, groups = (U + 31) >> 5;
   NomItem it;
   const int mg = item / C;
   it.chunk = item % C;
-  int lo = 0, hi = U;   // largest u with prefix[u] <= mg
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (prefix[mid] <= mg) lo = mid; else hi = mid;
+  int g = -1;   // last group that starts at or before mg
+  for (int k = 0; k < groups; k += 32) {
+    const bool le = k + lane < groups && coarse[k + lane] <= mg;
+    g += __popc(__ballot_sync(0xffffffffu, le));
   }
-  it.u = lo;
-  it.m_tile = mg - prefix[lo];
-  const UnitInfo ui = unit_info[lo];
-  it.n_ev = ui.n_ev;
-  it.n_ret = ui.n_ret;
-  const int T = (ui.n_ret + kNomN - 1) / kNomN;
-  it.t0 = (int)((long long)it.chunk * T / C);
-  it.t1 = (int)((long long)(it.chunk + 1) * T / C);
+  const int u = g * 32 + lane;
+  int n_ev = 0, n_ret = 0;
+  if (u < U) { const UnitInfo ui = unit_info[u]; n_ev = ui.n_ev; n_ret = ui.n_ret; }
+  const int tiles = (n_ev + kNomM - 1) / kNomM;
+  int x = tiles;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  const int r = mg - coarse[g];
+  const int at = __ffs(__ballot_sync(0xffffffffu, x > r)) - 1;   // (mg lies in this group, so one lane's sum exceeds r)
+  it.u = g * 32 + at;
+  it.m0 = (r - __shfl_sync(0xffffffffu, x - tiles, at)) * kNomM;
+  it.n_ev = __shfl_sync(0xffffffffu, n_ev, at);
+  it.n_ret = __shfl_sync(0xffffffffu, n_ret, at);
+  const int T = (it.n_ret + kNomN - 1) / kNomN;
+  it.t0 = it.chunk * T / C;
+  it.t1 = (it.chunk + 1) * T / C;
+  it.pad = 0;
   return it;
 }
 
-template <int D>
+// kCut: the product subtracts the rows' cuts (a compile-time choice: both screens in one kernel spill registers).
+template <int D, bool kCut>
 __global__ void __launch_bounds__(kNomThreads, 1)
 nominate_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, const __nv_bfloat16 *__restrict__ srcK,
                 const int32_t *__restrict__ ev_idx, const UnitInfo *__restrict__ unit_info,
-                const float *__restrict__ inv_norm, int32_t *sched, float4 *__restrict__ nom_v,
-                int32_t *__restrict__ nom_si, int C_max, int32_t *status_dev, int self_mask) {
+                const float *__restrict__ inv_norm, const uint4 *__restrict__ norm_ext, int32_t *sched,
+                float4 *__restrict__ nom_v, int32_t *__restrict__ nom_si, int C_max, int32_t *status_dev, int self_mask) {
   using SL = NomSmem<D>;
-  constexpr int KSTEPS = D / 16;
   constexpr uint32_t IDESC = umma_idesc_bf16(kNomM, kNomN);
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t bars[13];   // a_ready[2], b_full[2], b_empty[2], t_full[2], t_empty[2], drain, a_empty[2]
+  // a_ready[2], a_empty[2], b_full[4], b_empty[4], t_full[2], t_empty[2], drain, x_full[4][2]
+  __shared__ __align__(8) uint64_t bars[4 + 2 * kNomStages + 4 + 1 + 8];
   __shared__ uint32_t s_tmem;
-  __shared__ int s_wtot[kNomThreads / 32];
+  __shared__ __align__(16) NomItem s_item[2];   // what the staged rows belong to; n_ev < 0: the CTA's items are done
+  __shared__ int s_wtot[kNomThreads / 32], s_wmax[kNomThreads / 32];
   __shared__ volatile int s_abort;
 
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const uint32_t sbase = smem_u32(smem);
-  const uint32_t bar_a_ready = smem_u32(&bars[0]);
-  const uint32_t bar_b_full = smem_u32(&bars[2]), bar_b_empty = smem_u32(&bars[4]);
-  const uint32_t bar_t_full = smem_u32(&bars[6]), bar_t_empty = smem_u32(&bars[8]);
-  const uint32_t bar_drain = smem_u32(&bars[10]), bar_a_empty = smem_u32(&bars[11]);
+  const uint32_t bar_a_ready = smem_u32(&bars[0]), bar_a_empty = smem_u32(&bars[2]);
+  const uint32_t bar_b_full = smem_u32(&bars[4]), bar_b_empty = smem_u32(&bars[8]);
+  const uint32_t bar_t_full = smem_u32(&bars[12]), bar_t_empty = smem_u32(&bars[14]);
+  const uint32_t bar_drain = smem_u32(&bars[16]), bar_x = smem_u32(&bars[17]);
   int *coarse = reinterpret_cast<int *>(smem + SL::kCoarse);
-  uint16_t *fine = reinterpret_cast<uint16_t *>(smem + SL::kFine);
-  const NomPrefix prefix{coarse, fine};
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int U = p.B * p.H_kv;
@@ -111,11 +138,11 @@ nominate_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, const
     for (int i = 0; i < 2; ++i) {
       mbar_init(bar_a_ready + 8 * i, kNomGatherWarps);
       mbar_init(bar_a_empty + 8 * i, 1 + kNomDrainWarps);
-      mbar_init(bar_b_full + 8 * i, 1);
-      mbar_init(bar_b_empty + 8 * i, 1);
       mbar_init(bar_t_full + 8 * i, 1);
       mbar_init(bar_t_empty + 8 * i, kNomDrainWarps);
     }
+    for (int i = 0; i < kNomStages; ++i) { mbar_init(bar_b_full + 8 * i, 1); mbar_init(bar_b_empty + 8 * i, 1); }
+    for (int i = 0; i < 8; ++i) mbar_init(bar_x + 8 * i, 3);
     mbar_init(bar_drain, 1);
     s_abort = 0;
     mbar_fence_init();
@@ -126,21 +153,20 @@ nominate_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, const
     tmem_alloc(smem_u32(&s_tmem), 512);
     tmem_relinquish();
   }
+  if (tid >= 64 && tid < 64 + kNomN) {
+    reinterpret_cast<uint4 *>(smem + SL::kZero)[tid - 64] = make_uint4(0, 0, 0, 0);
+    fence_proxy_async_smem();
+  }
   pdl_wait();      // barrier set-up and tensor-memory allocation overlap the previous kernel's tail
   pdl_trigger();
-  int total_m = 0;
-  {   // exclusive prefix of 128-row tiles over the units: one unit per thread and pass
-    int run = 0;
+  int total_m = 0, t_max = 0;
+  {   // exclusive prefix of 128-row tiles over the units, kept for every 32nd: one unit per thread and pass
     for (int u0 = 0; u0 < U; u0 += kNomThreads) {
       const int u = u0 + tid;
-      const int t = u < U ? (unit_info[u].n_ev + kNomM - 1) / kNomM : 0;
-      int x = t;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-      }
-      if (lane == 31) s_wtot[warp] = x;
+      int t = 0, cols = 0;
+      if (u < U) { const UnitInfo ui = unit_info[u]; t = (ui.n_ev + kNomM - 1) / kNomM; cols = ui.n_ret; }
+      const int sum = __reduce_add_sync(0xffffffffu, t), mx = __reduce_max_sync(0xffffffffu, cols);
+      if (lane == 0) { s_wtot[warp] = sum; s_wmax[warp] = mx; }
       __syncthreads();
       int off = 0, tot = 0;
 #pragma unroll
@@ -148,116 +174,171 @@ nominate_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, const
         const int v = s_wtot[w];
         off += w < warp ? v : 0;
         tot += v;
+        t_max = max(t_max, s_wmax[w]);
       }
-      if (u < U) fine[u] = (uint16_t)(x - t);
-      if (lane == 0 && u < U) coarse[u >> 5] = run + off;
-      run += tot;
+      if (lane == 0 && u < U) coarse[u >> 5] = total_m + off;
+      total_m += tot;
       __syncthreads();
     }
-    total_m = run;
+    t_max = (t_max + kNomN - 1) / kNomN;
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
 
   const uint32_t tmem = s_tmem;
-  // few row tiles: split every row's columns into chunks so that all SMs get one item (a second wave
-  // of items would cost more in fixed latency than the shorter items save)
-  int C = total_m > 0 ? (int)gridDim.x / total_m : 1;
-  C = max(1, min(C, C_max));
+  // Column chunks per row tile: what makes the longest CTA shortest, an item costing about a tile and a half beside its
+  // tiles (first columns, publishing).  Without chunks 192 items on 148 CTAs take as long as 296.
+  int C = 1;
+  {
+    int cost = 0x7fffffff;
+    for (int c = 1; c <= C_max; ++c) {
+      const int rounds = (total_m * c + (int)gridDim.x - 1) / (int)gridDim.x, k = rounds * (2 * ((t_max + c - 1) / c) + 3);
+      if (k < cost) { cost = k; C = c; }
+    }
+  }
   const int n_items = total_m * C;
   if (blockIdx.x == 0 && tid == 0) sched[0] = C;
 
   if (warp == 0) {
-    // ------------------------------------------------------------ TMA producer
-    if (elect_one()) {
-      int ring = 0;
-      for (int item = blockIdx.x; item < n_items && !s_abort; item += gridDim.x) {
-        const NomItem it = nom_item(item, C, prefix, U, unit_info);
-        for (int t = it.t0; t < it.t1; ++t, ++ring) {
-          const int s = ring & 1;
-          if (!mbar_wait(bar_b_empty + 8 * s, ((ring >> 1) & 1) ^ 1)) { s_abort = 1; break; }
-          mbar_expect_tx(bar_b_full + 8 * s, SL::kBBytes);
-          const uint32_t dst = sbase + SL::kB + s * SL::kBBytes;
-          const int row = it.u * p.N_cap + t * kNomN;
+    // ------------------------------------------------------------ column tiles
+    int ring = 0, n_tiles = 0;
+    bool ok = true;
+    for (int n_done = 0; ok; ++n_done) {   // (watches the rows' barrier only: an item's last product waits for its columns)
+      if (!__all_sync(0xffffffffu, !s_abort && mbar_wait(bar_a_ready + 8 * (n_done & 1), (n_done >> 1) & 1))) { s_abort = 1; break; }
+      const NomItem it = s_item[n_done & 1];
+      if (it.n_ev < 0) break;
+      for (int t = it.t0; ok && t < it.t1; ++t, ++n_tiles) {
+        const int row = it.u * p.N_cap + t * kNomN;
 #pragma unroll
-          for (int sub = 0; sub < SL::kSub; ++sub)
-            tma_load_2d(dst + sub * (kNomN * 128), &mapB, sub * 64, row, bar_b_full + 8 * s);
+        for (int sub = 0; sub < SL::kSub; ++sub, ++ring) {
+          const int s = ring % kNomStages;
+          ok = __all_sync(0xffffffffu, !s_abort && mbar_wait(bar_b_empty + 8 * s, ((ring / kNomStages) & 1) ^ 1));
+          if (!ok) { s_abort = 1; break; }
+          if (elect_one()) {
+            const uint32_t full = bar_b_full + 8 * s;
+            const bool last = sub == SL::kSub - 1;
+            mbar_expect_tx(full, SL::kBBytes + (last ? kNomN * 20 : 0));
+            tma_load_2d(sbase + SL::kB + s * SL::kBBytes, &mapB, sub * 64, row, full);
+            if (last) {
+              bulk_load_1d(sbase + SL::kBX + n_tiles % SL::kTiles * (kNomN * 16), norm_ext + row, kNomN * 16, full);
+              bulk_load_1d(sbase + SL::kInv + n_tiles % SL::kInvTiles * (kNomN * 4), inv_norm + row, kNomN * 4, full);
+            }
+          }
+          __syncwarp();
         }
       }
     }
   } else if (warp == 1) {
-    // ------------------------------------------------------------ MMA issuer
-    if (elect_one()) {
-      int ring = 0, acc = 0, n_done = 0;
-      for (int item = blockIdx.x; item < n_items && !s_abort; item += gridDim.x) {
-        const NomItem it = nom_item(item, C, prefix, U, unit_info);
-        if (it.t0 == it.t1) continue;
-        const int abuf = n_done & 1;
-        if (!mbar_wait(bar_a_ready + 8 * abuf, (n_done >> 1) & 1)) { s_abort = 1; break; }
-        ++n_done;
-        tc_fence_after();
-        for (int t = it.t0; t < it.t1; ++t, ++ring, ++acc) {
-          const int s = ring & 1, a = acc & 1;
-          if (!mbar_wait(bar_b_full + 8 * s, (ring >> 1) & 1) ||
-              !mbar_wait(bar_t_empty + 8 * a, ((acc >> 1) & 1) ^ 1)) { s_abort = 1; break; }
-          tc_fence_after();
-          const uint64_t ad = umma_desc_sw128(sbase + SL::kA + abuf * SL::kABytes), bd = umma_desc_sw128(sbase + SL::kB + s * SL::kBBytes);
+    // ------------------------------------------------------------ products
+    int ring = 0, acc = 0;
+    bool ok = true;
+    for (int n_done = 0; ok; ++n_done) {
+      const int buf = n_done & 1;
+      ok = __all_sync(0xffffffffu, !s_abort && mbar_wait(bar_a_ready + 8 * buf, (n_done >> 1) & 1));
+      if (!ok) break;
+      const NomItem it = s_item[buf];
+      if (it.n_ev < 0) break;
+      for (int t = it.t0; ok && t < it.t1; ++t, ++acc) {
+        const int a = acc & 1;
+        ok = __all_sync(0xffffffffu, !s_abort && mbar_wait(bar_t_empty + 8 * a, ((acc >> 1) & 1) ^ 1));
 #pragma unroll
-          for (int k = 0; k < KSTEPS; ++k)   // (descriptor addresses count 16-byte units)
-            umma_bf16(tmem + a * kNomN, ad + (k >> 2) * (kNomM * 8) + (k & 3) * 2, bd + (k >> 2) * (kNomN * 8) + (k & 3) * 2,
-                      IDESC, k > 0 ? 1u : 0u);
-          umma_commit(bar_b_empty + 8 * s);   // the stage may be refilled once these MMAs have read it
-          umma_commit(bar_t_full + 8 * a);    // the accumulator is complete
+        for (int sub = 0; sub < SL::kSub; ++sub, ++ring) {
+          const int s = ring % kNomStages;
+          ok = ok && __all_sync(0xffffffffu, !s_abort && mbar_wait(bar_b_full + 8 * s, (ring / kNomStages) & 1));
+          if (!ok) break;
+          tc_fence_after();
+          if (elect_one()) {
+            const uint64_t ad = umma_desc_sw128(sbase + SL::kA + buf * SL::kABytes + sub * (kNomM * 128));
+            const uint64_t bd = umma_desc_sw128(sbase + SL::kB + s * SL::kBBytes);
+            const uint32_t dt = tmem + a * kNomN;
+#pragma unroll
+            for (int k = 0; k < 4; ++k)   // (descriptor addresses count 16-byte units)
+              umma_bf16(dt, ad + k * 2, bd + k * 2, IDESC, sub + k > 0 ? 1u : 0u);
+            if (sub == SL::kSub - 1) {
+              const uint32_t zero = sbase + SL::kZero;
+              if (kCut)
+                umma_bf16(dt, umma_desc_plain(sbase + SL::kAX + buf * (kNomM * 16), zero),
+                          umma_desc_plain(sbase + SL::kBX + acc % SL::kTiles * (kNomN * 16), zero), IDESC, 1u);
+              umma_commit(bar_t_full + 8 * a);
+            }
+            umma_commit(bar_b_empty + 8 * s);   // the stage may be refilled once these have read it
+          }
+          __syncwarp();
         }
-        umma_commit(bar_a_empty + 8 * abuf);  // the rows have been read
       }
-      umma_commit(bar_drain);
-      mbar_wait(bar_drain, 0);   // every MMA issued above has retired (bounded)
+      if (elect_one()) umma_commit(bar_a_empty + 8 * buf);          // the rows have been read
+      __syncwarp();
     }
+    if (!ok) s_abort = 1;
+    if (elect_one()) umma_commit(bar_drain);
+    mbar_wait(bar_drain, 0);   // every product issued above has retired (bounded)
   } else if (warp < 2 + kNomGatherWarps) {
-    // ------------------------------------------------------------ rows of the next item: 64 per warp, sixteen lanes each
+    // ------------------------------------------------------------ rows of the next item, kNomM / kNomGatherWarps a warp
+    // Asynchronous copies straight into the swizzled tile, all in flight together; then a row per lane for the norms.
     float *rowinv = reinterpret_cast<float *>(smem + SL::kRowInv);
-    const int r0 = (warp - 2) * 64, ch = lane & 15, sub = lane >> 4;
+    constexpr int RW = kNomM / kNomGatherWarps, CH = D / 8, RI = 32 / CH;   // rows a warp, 16-byte chunks a row, rows a copy
+    const int r0 = (warp - 2) * RW;
     int n_done = 0;
-    for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
-      const NomItem it = nom_item(item, C, prefix, U, unit_info);
-      if (it.t0 == it.t1) continue;
+    for (int item = blockIdx.x;; item += gridDim.x) {
+      NomItem it = {0, 0, 0, 0, 0, -1, 0, 0};
+      if (item < n_items) it = nom_item(item, C, coarse, U, unit_info);
       const int buf = n_done & 1;
       const size_t ubase = (size_t)it.u * p.N_cap;
-      const int m0 = it.m_tile * kNomM + r0;
-      const int mine0 = m0 + lane < it.n_ev ? ev_idx[ubase + m0 + lane] : -1;
-      const int mine1 = m0 + 32 + lane < it.n_ev ? ev_idx[ubase + m0 + 32 + lane] : -1;
+      if (it.n_ev >= 0 && it.t0 == it.t1) {   // a chunk without tiles (fewer tiles than chunks): an empty result
+        for (int i = it.m0 + r0 + lane; i < min(it.m0 + r0 + RW, it.n_ev); i += 32) {
+          const size_t o = (ubase + i) * C_max + it.chunk;
+          nom_v[o] = make_float4(-CUDART_INF_F, -CUDART_INF_F, 0.f, __int_as_float(-1));
+          nom_si[o] = -1;
+        }
+        continue;
+      }
+      const int m0 = it.m0 + r0;
+      int mine[RW / 32];
+#pragma unroll
+      for (int k = 0; k < RW / 32; ++k) mine[k] = it.n_ev >= 0 && m0 + 32 * k + lane < it.n_ev ? ev_idx[ubase + m0 + 32 * k + lane] : -1;
       if (n_done >= 2 && !__all_sync(0xffffffffu, !s_abort && mbar_wait(bar_a_empty + 8 * buf, ((n_done >> 1) - 1) & 1))) {
         s_abort = 1;
         break;
       }
       ++n_done;
+      if (warp == 2 && lane == 0) s_item[buf] = it;
+      if (it.n_ev < 0) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_a_ready + 8 * buf);
+        break;
+      }
+      const uint32_t At = SL::kA + buf * SL::kABytes;
+      const int ch = lane % CH, sub = lane / CH;
+#pragma unroll
+      for (int k = 0; k < RW / 32; ++k) {
+#pragma unroll
+        for (int i = 0; i < 32; i += RI) {
+          const int e = __shfl_sync(0xffffffffu, mine[k], i + sub), r = r0 + 32 * k + i + sub;
+          cp_async_16(sbase + At + (ch >> 3) * (kNomM * 128) + r * 128 + (((ch & 7) ^ (r & 7)) << 4),
+                      srcK + (ubase + (e >= 0 ? e : 0)) * D + ch * 8, e >= 0);
+        }
+      }
+      cp_async_commit();
+      cp_async_wait<0>();
+      __syncwarp();
 #pragma unroll 1
-      for (int half = 0; half < 4; ++half) {
-        uint4 val[8];
+      for (int k = 0; k < RW / 32; ++k) {
+        const int r = r0 + 32 * k + lane;
+        float s0 = 0.f, s1 = 0.f;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const int e = __shfl_sync(0xffffffffu, half < 2 ? mine0 : mine1, (half & 1) * 16 + 2 * k + sub);
-          val[k] = make_uint4(0, 0, 0, 0);
-          if (e >= 0 && ch < D / 8) val[k] = *reinterpret_cast<const uint4 *>(srcK + (ubase + e) * D + ch * 8);
+        for (int c = 0; c < CH; ++c) {
+          const uint4 v = *reinterpret_cast<const uint4 *>(smem + At + (c >> 3) * (kNomM * 128) + r * 128 + (((c & 7) ^ (r & 7)) << 4));
+          const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+          for (int q = 0; q < 4; ++q) { s0 = fmaf(bf16_lo(w[q]), bf16_lo(w[q]), s0); s1 = fmaf(bf16_hi(w[q]), bf16_hi(w[q]), s1); }
         }
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const int r = r0 + half * 16 + 2 * k + sub;
-          float ss = 0.f;
-          const uint32_t w[4] = {val[k].x, val[k].y, val[k].z, val[k].w};
-#pragma unroll
-          for (int q = 0; q < 4; ++q) { const float a = bf16_lo(w[q]), b = bf16_hi(w[q]); ss = fmaf(a, a, ss); ss = fmaf(b, b, ss); }
-          ss += __shfl_xor_sync(0xffffffffu, ss, 1);
-          ss += __shfl_xor_sync(0xffffffffu, ss, 2);
-          ss += __shfl_xor_sync(0xffffffffu, ss, 4);
-          ss += __shfl_xor_sync(0xffffffffu, ss, 8);
-          if (ch < D / 8)
-            *reinterpret_cast<uint4 *>(smem + SL::kA + buf * SL::kABytes + (ch >> 3) * (kNomM * 128) + r * 128 +
-                                       (((ch & 7) ^ (r & 7)) << 4)) = val[k];
-          if (ch == 0) rowinv[buf * 128 + r] = rsqrtf(ss);
-        }
+        // (a row that does not exist, or of norm zero: a cut no column reaches)
+        const float ri = rsqrtf(s0 + s1);
+        if (kCut)
+          *reinterpret_cast<uint4 *>(smem + SL::kAX + buf * (kNomM * 16) + r * 16) =
+              ext_row(ri < CUDART_INF_F ? (p.merge_threshold - 2.f * kRankEps) / ri : kExtNever);
+        rowinv[buf * kNomM + r] = ri;
       }
       fence_proxy_async_smem();
       __syncwarp();
@@ -265,154 +346,125 @@ nominate_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, const
     }
   } else {
     // ------------------------------------------------------------ accumulator drain
-    const int ew = warp - 2 - kNomGatherWarps, quarter = warp & 3, cq = ew >> 2;   // cq: which 64 columns of a tile
-    const int row = quarter * 32 + lane;                        // tensor-memory lane = row of the item
-    float *inv_w = reinterpret_cast<float *>(smem + SL::kInv) + ew * 64;
+    const int ew = warp - 2 - kNomGatherWarps, quarter = warp & 3;   // (a warp reads the lanes 32 (warp mod 4) ..)
+    const int cq = ew >> 2;                                          // which 64 of a tile's columns
+    const int row = quarter * 32 + lane;                             // row of the item
+    const uint32_t xbar = bar_x + 16 * quarter;
     const float *rowinv = reinterpret_cast<const float *>(smem + SL::kRowInv);
     uint32_t *xchg = reinterpret_cast<uint32_t *>(smem + SL::kXchg);
-    const size_t n_total = (size_t)U * p.N_cap;
-    int acc = 0, n_done = 0, x3 = 0;
-    bool dead = false;
-    for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
-      const NomItem it = nom_item(item, C, prefix, U, unit_info);
-      const size_t ubase = (size_t)it.u * p.N_cap;
-      const int m0 = it.m_tile * kNomM;
+    int acc = 0, x_phase = 0;   // x_phase: a bit per set of A tiles
+    for (int n_done = 0;; ++n_done) {
       const int buf = n_done & 1;
-      if (it.t0 == it.t1) {   // a chunk without tiles (fewer tiles than chunks): publish an empty result
-        if (cq == 0 && m0 + row < it.n_ev) {
-          const size_t o = (ubase + m0 + row) * C_max + it.chunk;
-          nom_v[o] = make_float4(-CUDART_INF_F, -CUDART_INF_F, 0.f, __int_as_float(-1));
-          nom_si[o] = -1;
-        }
-        continue;
-      }
-      // inverse norms of this warp's columns, two per lane, one tile ahead of their use
-      auto fetch_inv = [&](int t) {
-        const size_t g = ubase + t * kNomN + cq * 64 + 2 * lane;
-        return g + 1 < n_total ? *reinterpret_cast<const float2 *>(inv_norm + g) : make_float2(0.f, 0.f);
-      };
-      float2 inv_next = fetch_inv(it.t0);
-      if (!dead) {
-        const bool ok = !s_abort && mbar_wait(bar_a_ready + 8 * buf, (n_done >> 1) & 1);
-        if (!__all_sync(0xffffffffu, ok)) { dead = true; s_abort = 1; }
-      }
-      const float rinv = rowinv[buf * 128 + row];
-      __syncwarp();
-      if (lane == 0 && !dead) mbar_arrive(bar_a_empty + 8 * buf);
-      ++n_done;
-      // Values are compared before the division by |k_e|: the closeness margin and the threshold scale with it.  A row
-      // that does not exist, or whose norm is zero, takes no column.
-      Top2 top, topb;   // two trackers over alternate groups of four columns: two independent dependency chains
+      if (!__all_sync(0xffffffffu, !s_abort && mbar_wait(bar_a_ready + 8 * buf, (n_done >> 1) & 1))) { s_abort = 1; break; }
+      const NomItem it = s_item[buf];
+      if (it.n_ev < 0) break;
+      const size_t ubase = (size_t)it.u * p.N_cap;
+      const bool row_ok = it.m0 + row < it.n_ev;
+      // Values are compared before the division by |k_e|: the closeness margin and the threshold scale with it.
+      const float rinv = rowinv[buf * kNomM + row];
+      const bool live = it.m0 + quarter * 32 < it.n_ev;   // some of this warp's rows exist
+      Top2 top, topb;   // two lists over alternate columns: two independent dependency chains
       top.init(2.f * kRankEps / rinv);
       topb.init(top.thr);
-      top.cut = m0 + row < it.n_ev && rinv < CUDART_INF_F ? (p.merge_threshold - 2.f * kRankEps) / rinv : CUDART_INF_F;
-      const bool open = p.merge_threshold == -CUDART_INF_F;   // no threshold: the first tile's lists start cold
-
+      const float cut0 = (p.merge_threshold - 2.f * kRankEps) / rinv;
+      top.cut = row_ok && rinv < CUDART_INF_F ? cut0 : CUDART_INF_F;
+      bool ok = true;
       for (int t = it.t0; t < it.t1; ++t, ++acc) {
         const int a = acc & 1;
-        const int c0 = t * kNomN + cq * 64;
-        __syncwarp();
-        *reinterpret_cast<float2 *>(inv_w + 2 * lane) = inv_next;
-        __syncwarp();
-        if (t + 1 < it.t1) inv_next = fetch_inv(t + 1);
-        if (!dead && !__all_sync(0xffffffffu, mbar_wait(bar_t_full + 8 * a, (acc >> 1) & 1))) { dead = true; s_abort = 1; }
-        if (dead) continue;
-        // nothing to track if this warp's 32 rows lie past the evicted entries or its columns past the
-        // retained ones: release the accumulator without reading it
-        const bool live = m0 + quarter * 32 < it.n_ev && c0 < it.n_ret;
-        if (!live) {
-          tc_fence_before();
-          if (lane == 0) mbar_arrive(bar_t_empty + 8 * a);
-          continue;
-        }
+        ok = __all_sync(0xffffffffu, !s_abort && mbar_wait(bar_t_full + 8 * a, (acc >> 1) & 1));
+        if (!ok) break;
         tc_fence_after();
+        const int c0 = t * kNomN + cq * 64, n_valid = it.n_ret - c0;   // this warp's columns that exist, if positive
         const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + a * kNomN + cq * 64;
-        const int n_valid = it.n_ret - c0;   // columns of this quarter that exist
         // rows and columns are the same entries (self_mask): the column of the row's own key does not count
-        const int diag = self_mask ? m0 + row - c0 : -1;
-        const bool crosses = self_mask && m0 + quarter * 32 < c0 + 64 && c0 <= m0 + quarter * 32 + 31;
+        const int diag = self_mask ? it.m0 + row - c0 : -1;
+        const int diag0 = it.m0 + quarter * 32 - c0;
 #pragma unroll 1
-        for (int jg = 0; jg < 2; ++jg) {   // 32 columns at a time: the register budget of 20 warps
+        for (int off = 0; live && off < 64 && off < n_valid; off += 32) {   // 32 columns at a time: the register budget of 20 warps
           uint32_t r[32];
-          tmem_ld_32x32(taddr + jg * 32, r);
+          tmem_ld_32x32(taddr + off, r);
           tmem_ld_wait();
-          if (jg == 1) {   // everything this warp needs from the accumulator is in registers
-            tc_fence_before();
-            if (lane == 0) mbar_arrive(bar_t_empty + 8 * a);
-          }
-          const int off = jg * 32;
-          const bool ragged = n_valid < off + 32 || crosses;   // columns past n_ret hold other rows' data
-          // `masked` is a compile-time flag: only the last tile of a row of tiles has columns to mask, and a
-          // run-time test inside the unrolled loop would be turned into selects that every group pays for
-          auto drain32 = [&](auto test, auto masked) {
+          // the last columns may hold other rows' data, and the row's own key does not count
+          const bool masked = n_valid < off + 32 || (self_mask && diag0 < off + 32 && off < diag0 + 32);
+          if (masked) {
 #pragma unroll
-            for (int i = 0; i < 32; i += 4) {
-              float4 iv = *reinterpret_cast<const float4 *>(inv_w + off + i);
-              float a0 = __uint_as_float(r[i]), a1 = __uint_as_float(r[i + 1]);
-              float a2 = __uint_as_float(r[i + 2]), a3 = __uint_as_float(r[i + 3]);
-              if (decltype(masked)::value) {   // a masked column contributes -inf
-                if (off + i >= n_valid || off + i == diag) { a0 = -CUDART_INF_F; iv.x = 1.f; }
-                if (off + i + 1 >= n_valid || off + i + 1 == diag) { a1 = -CUDART_INF_F; iv.y = 1.f; }
-                if (off + i + 2 >= n_valid || off + i + 2 == diag) { a2 = -CUDART_INF_F; iv.z = 1.f; }
-                if (off + i + 3 >= n_valid || off + i + 3 == diag) { a3 = -CUDART_INF_F; iv.w = 1.f; }
+            for (int i = 0; i < 32; ++i)
+              if (off + i >= n_valid || off + i == diag) r[i] = 0xff800000u;   // -inf
+          }
+          const float4 *wv = reinterpret_cast<const float4 *>(smem + SL::kInv + acc % SL::kInvTiles * (kNomN * 4)) + (cq * 64 + off) / 4;
+          if constexpr (kCut) {
+            // groups of four columns; what lies above the row's cut is positive (NaNs never show)
+            float gm[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+              gm[i] = max3(fmaxf(__uint_as_float(r[4 * i]), __uint_as_float(r[4 * i + 1])), __uint_as_float(r[4 * i + 2]), __uint_as_float(r[4 * i + 3]));
+            const float all = max3(max3(gm[0], gm[1], gm[2]), max3(gm[3], gm[4], gm[5]), fmaxf(gm[6], gm[7]));
+            if (__any_sync(0xffffffffu, all > 0.f)) {
+#pragma unroll
+              for (int i = 0; i < 8; ++i) {
+                if (!__any_sync(0xffffffffu, gm[i] > 0.f)) continue;
+                const float4 w = wv[i];
+                const int c = c0 + off + 4 * i;
+                top.insert(fmaf(__uint_as_float(r[4 * i]), fabsf(w.x), cut0), c);
+                topb.insert(fmaf(__uint_as_float(r[4 * i + 1]), fabsf(w.y), cut0), c + 1);
+                top.insert(fmaf(__uint_as_float(r[4 * i + 2]), fabsf(w.z), cut0), c + 2);
+                topb.insert(fmaf(__uint_as_float(r[4 * i + 3]), fabsf(w.w), cut0), c + 3);
               }
-              offer4<decltype(test)::value>(top, topb, a0, a1, a2, a3, iv, c0 + off + i);
             }
-          };
-          if (open && t == it.t0) {
-            if (ragged) drain32(std::false_type{}, std::true_type{});
-            else drain32(std::false_type{}, std::false_type{});
-            if (jg == 1) top.cut = m0 + row < it.n_ev ? fmaxf(top.best, topb.best) - top.thr : CUDART_INF_F;
-          } else if (ragged) {
-            drain32(std::true_type{}, std::true_type{});
           } else {
             const uint64_t ncut = pack_f32x2(-top.cut, -top.cut);
-            float m0_ = -1.f, m1_ = -1.f;   // largest value - cut, if any reaches it (NaNs, zero-norm keys, never do)
+            float m_a = -1.f, m_b = -1.f;   // largest value - cut, if any reaches it
 #pragma unroll
             for (int i = 0; i < 32; i += 4) {
-              const float4 iv = *reinterpret_cast<const float4 *>(inv_w + off + i);
+              const float4 w = wv[i / 4];
               float d0, d1, d2, d3;
-              unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(r[i]), __uint_as_float(r[i + 1])), pack_f32x2(iv.x, iv.y), ncut), d0, d1);
-              unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(r[i + 2]), __uint_as_float(r[i + 3])), pack_f32x2(iv.z, iv.w), ncut), d2, d3);
-              m0_ = max3(m0_, d0, d1);
-              m1_ = max3(m1_, d2, d3);
+              unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(r[i]), __uint_as_float(r[i + 1])), pack_f32x2(w.x, w.y), ncut), d0, d1);
+              unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(r[i + 2]), __uint_as_float(r[i + 3])), pack_f32x2(w.z, w.w), ncut), d2, d3);
+              m_a = max3(m_a, d0, d1);
+              m_b = max3(m_b, d2, d3);
             }
-            if (__any_sync(0xffffffffu, fmaxf(m0_, m1_) >= 0.f)) drain32(std::true_type{}, std::false_type{});
+            if (__any_sync(0xffffffffu, fmaxf(m_a, m_b) >= 0.f || top.cut == -CUDART_INF_F)) {
+#pragma unroll
+              for (int i = 0; i < 32; i += 4)   // groups of four columns that hold a candidate of some row
+                offer4_above(top, topb, __uint_as_float(r[i]), __uint_as_float(r[i + 1]), __uint_as_float(r[i + 2]),
+                             __uint_as_float(r[i + 3]), wv[i / 4], c0 + off + i);
+            }
           }
         }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_t_empty + 8 * a);
       }
+      if (!ok) { s_abort = 1; break; }
       top.insert_any(topb.best, topb.bi);
       top.insert_any(topb.second, topb.si);
-      // ---- Combine the four column quarters of each row and publish the chunk's result.  The warps of the later quarters
-      // leave theirs and go on; only the first quarter's warp waits for them.  They can be two items ahead of it at most
-      // (it releases an accumulator before it folds), so the exchange area and the barrier rotate over three.
-      uint32_t *x = xchg + (size_t)(x3 * 128 + row) * 9;
-      if (cq > 0) {   // slots are below 65535 (N_cap <= 49152); -1 = none
+      // ---- Fold the four warps' results of each row and publish the chunk's.  Those of the later columns leave theirs and
+      // go on.  They can be one item ahead at most: the item after that is not gathered before this one is folded.
+      uint32_t *x = xchg + (size_t)(buf * kNomM + row) * 9;
+      if (cq) {   // slots are below 65535 (N_cap <= 49152); -1 = none
         uint32_t *xw = x + (cq - 1) * 3;
         xw[0] = __float_as_uint(top.best);
         xw[1] = __float_as_uint(top.second);
         xw[2] = (uint32_t)(top.bi + 1) | ((uint32_t)(top.si + 1) << 16);
-        __threadfence_block();
-        if (dead)   // no longer paced by the accumulators: stay in step
-          asm volatile("bar.sync %0, 128;" ::"r"(1 + quarter + 4 * x3) : "memory");
-        else
-          asm volatile("bar.arrive %0, 128;" ::"r"(1 + quarter + 4 * x3) : "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(xbar + 8 * buf);
       } else {
-        asm volatile("bar.sync %0, 128;" ::"r"(1 + quarter + 4 * x3) : "memory");
+        if (!__all_sync(0xffffffffu, !s_abort && mbar_wait(xbar + 8 * buf, (x_phase >> buf) & 1))) { s_abort = 1; break; }
 #pragma unroll
-        for (int w = 0; w < 3; ++w) {   // ascending columns: a later quarter holds higher slots, ties keep the earlier one
-          const uint32_t *xw = x + w * 3;
-          const uint32_t sl = xw[2];
-          top.insert_any(__uint_as_float(xw[0]), (int)(sl & 0xffffu) - 1);
-          top.insert_any(__uint_as_float(xw[1]), (int)(sl >> 16) - 1);
+        for (int w = 0; w < 3; ++w) {
+          const uint32_t sl = x[3 * w + 2];
+          top.insert_any(__uint_as_float(x[3 * w]), (int)(sl & 0xffffu) - 1);
+          top.insert_any(__uint_as_float(x[3 * w + 1]), (int)(sl >> 16) - 1);
         }
-        if (m0 + row < it.n_ev) {
-          const size_t o = (ubase + m0 + row) * C_max + it.chunk;
+        if (row_ok) {
+          const size_t o = (ubase + it.m0 + row) * C_max + it.chunk;
           nom_v[o] = make_float4(top.best * rinv, top.second * rinv, 0.f, __int_as_float(top.bi));
           nom_si[o] = top.si;
         }
       }
-      x3 = x3 == 2 ? 0 : x3 + 1;
+      x_phase ^= 1 << buf;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar_a_empty + 8 * buf);
     }
   }
 
@@ -423,7 +475,7 @@ nominate_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, const
     if (tid == 0) {
       atomicOr(status_dev, KEEPKV_DEV_TIMEOUT);
       // copies still in flight get a bounded chance to land before the shared memory goes away
-      for (int i = 0; i < 2; ++i) { mbar_wait(bar_b_full + 8 * i, 0); mbar_wait(bar_b_full + 8 * i, 1); }
+      for (int i = 0; i < kNomStages; ++i) { mbar_wait(bar_b_full + 8 * i, 0); mbar_wait(bar_b_full + 8 * i, 1); }
     }
     __syncthreads();
   }
@@ -434,10 +486,10 @@ nominate_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, const
   }
 }
 
-template <int D>
+template <int D, bool kCut>
 static void launch_nominate_t(const keepkv_params &p, const keepkv_cache &src, const keepkv_cache &dst,
-                              const int32_t *ev_idx, const UnitInfo *unit_info, const float *inv_norm, int32_t *sched,
-                              float4 *nom_v, int32_t *nom_si, int nom_chunks, int32_t *status_dev, LaunchCtx &ctx,
+                              const int32_t *ev_idx, const UnitInfo *unit_info, const float *inv_norm,
+                              const uint4 *norm_ext, int32_t *sched, float4 *nom_v, int32_t *nom_si, int nom_chunks, int32_t *status_dev, LaunchCtx &ctx,
                               int self_mask) {
   using SL = NomSmem<D>;
   constexpr size_t smem_bytes = (size_t)SL::kBytes + 1024;
@@ -445,7 +497,7 @@ static void launch_nominate_t(const keepkv_params &p, const keepkv_cache &src, c
   int dev = 0;
   cudaGetDevice(&dev);
   if (!attr_done_dev[dev & 63]) {
-    cudaFuncSetAttribute(nominate_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+    cudaFuncSetAttribute(nominate_kernel<D, kCut>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
     attr_done_dev[dev & 63] = true;
   }
   CUtensorMap mapB;
@@ -453,19 +505,19 @@ static void launch_nominate_t(const keepkv_params &p, const keepkv_cache &src, c
     if (ctx.err == cudaSuccess) ctx.err = cudaErrorInvalidValue;
     return;
   }
-  launch_pdl(nominate_kernel<D>, dim3(sm_count()), dim3(kNomThreads), smem_bytes, ctx.stream,
-      mapB, p, reinterpret_cast<const __nv_bfloat16 *>(src.K), ev_idx, unit_info, inv_norm, sched, nom_v, nom_si,
+  launch_pdl(nominate_kernel<D, kCut>, dim3(sm_count()), dim3(kNomThreads), smem_bytes, ctx.stream,
+      mapB, p, reinterpret_cast<const __nv_bfloat16 *>(src.K), ev_idx, unit_info, inv_norm, norm_ext, sched, nom_v, nom_si,
       nom_chunks, status_dev, self_mask);
   KEEPKV_CHECK_LAUNCH(ctx);
 }
 
 void launch_nominate(const keepkv_params &p, const keepkv_cache &src, const keepkv_cache &dst, const int32_t *ev_idx,
-                     const UnitInfo *unit_info, const float *inv_norm, int32_t *sched, float4 *nom_v, int32_t *nom_si,
+                     const UnitInfo *unit_info, const float *inv_norm, const uint4 *norm_ext, int32_t *sched, float4 *nom_v, int32_t *nom_si,
                      int nom_chunks, int32_t *status_dev, LaunchCtx &ctx, int self_mask) {
-  if (p.d == 128)
-    launch_nominate_t<128>(p, src, dst, ev_idx, unit_info, inv_norm, sched, nom_v, nom_si, nom_chunks, status_dev, ctx, self_mask);
-  else
-    launch_nominate_t<64>(p, src, dst, ev_idx, unit_info, inv_norm, sched, nom_v, nom_si, nom_chunks, status_dev, ctx, self_mask);
+  const bool cut = p.merge_threshold >= kNomStatic;
+  auto launch = p.d == 128 ? (cut ? launch_nominate_t<128, true> : launch_nominate_t<128, false>)
+                           : (cut ? launch_nominate_t<64, true> : launch_nominate_t<64, false>);
+  launch(p, src, dst, ev_idx, unit_info, inv_norm, norm_ext, sched, nom_v, nom_si, nom_chunks, status_dev, ctx, self_mask);
 }
 
 }  // namespace keepkv

@@ -52,6 +52,11 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
       "l"(map), "r"(x), "r"(y), "r"(bar)
       : "memory");
 }
+__device__ __forceinline__ void bulk_load_1d(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(bar)
+               : "memory");
+}
 __device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p) : "memory"); }
 __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap *map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
@@ -128,6 +133,11 @@ __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.
 __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t smem_addr) {
   return (uint64_t)((smem_addr & 0x3FFFFu) >> 4) | (1ull << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) |
          (2ull << 61);
+}
+// The descriptor of 16 channels of a K-major operand without swizzle: rows of 16 bytes, the first eight channels at `lo`,
+// the others at `hi` (above it).
+__device__ __forceinline__ uint64_t umma_desc_plain(uint32_t lo, uint32_t hi) {
+  return (uint64_t)((lo & 0x3FFFFu) >> 4) | ((uint64_t)((hi - lo) >> 4) << 16) | ((uint64_t)(128 >> 4) << 32) | (1ull << 46);
 }
 // The same rows read as an MN-major operand (the 128-byte rows run along M, the 8-row groups along K): `mn_stride` bytes
 // between two 64-element atoms of M, 8-row groups of K 1024 bytes apart.

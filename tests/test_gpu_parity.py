@@ -215,6 +215,36 @@ def test_compress_staged_parity(d, G, T, guard):
     assert n_excused <= 1
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("T", [0.9, 0.5, 0.4999])
+def test_compress_search_at_tile_edges(d, T):
+    """Row counts around 128 and column counts around 256 (the tiles of the similarity search), thresholds on both sides
+    of where the search subtracts them in the product, clustered keys (members on either side of every threshold), a key
+    of norm zero and exact duplicates: targets, votes and lengths are the oracle's."""
+    B, H_kv, G = 5, 2, 2
+    n_ret, n_ev = [256, 257, 511, 40, 512], [127, 128, 129, 1, 257]
+    lens = [a + b for a, b in zip(n_ret, n_ev)]
+    p = kb.make_params(B=B, H_q=H_kv * G, H_kv=H_kv, d=d, N_cap=832, period=0, n_sink=4, n_recent=20, merge_threshold=T)
+    src = random_cache(p, lens, seed=d, vote_max=3, scored_frac=1.0)
+    rng = np.random.default_rng(int(T * 100) + d)
+    U = B * H_kv
+    K = np.empty((U, p.N_cap, d), dtype=np.float32)
+    for u in range(U):
+        centers = 3.0 * rng.standard_normal((50, d)).astype(np.float32)
+        K[u] = centers[rng.integers(0, 50, p.N_cap)] + rng.uniform(0.2, 4.0, (p.N_cap, 1)) * rng.standard_normal((p.N_cap, d))
+    K[:, 30] = 0.0
+    K[:, 25] = K[:, 12]; K[:, 26] = K[:, 12]
+    src.K.copy_(f32_to_dev_bf16(K).view(B, H_kv, p.N_cap, d))
+    src.lscore.mul_(0.25).add_(1.5)                # positive log-scores keep the rescale factors inside the guard
+    budgets = torch.tensor(n_ret, dtype=torch.int32, device="cuda")
+    dst, ret, tgt, stats = _run_compress(p, src, budgets)
+    hs, hd = HostCache(src), HostCache(dst)
+    assert list(hd.seq_len) == n_ret
+    for u in range(U):
+        check_compress_unit(p, u, n_ret[u // H_kv], p.n_recent, hs, hd, ret, tgt, stats, what=f"search edges T={T}", max_tolerated=4)
+    assert stats[:, 2].sum() > 0 and stats[:, 3].sum() > 0      # some merged, some below the threshold
+
+
 def test_compress_ragged_budgets_and_copy_through():
     """Per-sequence budgets and recent windows; a sequence within its budget is copied in order."""
     B, H_kv, G, d = 3, 2, 2, 128

@@ -11,21 +11,23 @@
 
 namespace keepkv {
 
-constexpr int kWarpSelectMax = 2048;   // candidate sets up to this size are searched by one warp, without block barriers
-
 // ------------------------------------------------------------------ select
-// One CTA per unit.  The keys of the whole unit live in shared memory; the heavy-hitter threshold
-// is found by a 4-pass radix select over the candidates [lo, hi), and one ordered pass writes the
-// retained list, the evicted list and the per-entry marks.
+// One CTA per unit.  The keys of the whole unit live in shared memory.  The heavy-hitter threshold is found by
+// histograms of kSelBins bins over the range the candidates' keys really span: the bin that holds the n-th largest becomes
+// the next range, so three passes settle any 32-bit key (the leading byte of most keys coincides, so a histogram of fixed
+// digits has its counts in a few bins: four passes with one atomic per distinct digit of a warp took 49 us for 64 units
+// of 8192 where this kernel takes 22 us, 95 us for 128 of up to 16384 where it takes 32 us).  Then every warp counts what it keeps of a contiguous run of entries, one
+// block scan gives the places, and the retained list, the evicted list and the per-entry marks are written in order.
+constexpr int kSelBins = 2048;
 __global__ void __launch_bounds__(1024)
 select_kernel(keepkv_params p, keepkv_cache src, int32_t *dst_seq_len, const int32_t *budget_dev, int budget_scalar,
               const int32_t *n_recent_dev, int32_t *ret_idx, int32_t *target, int32_t *ev_idx, UnitInfo *unit_info,
               keepkv_stats *stats, const float *__restrict__ select_key, const int32_t *__restrict__ unit_len,
               int32_t *pos, const int32_t *pos_len, const int32_t *n_seen, int32_t *status_dev) {
   extern __shared__ uint32_t keys[];
-  __shared__ int hist[256];
-  __shared__ int warp_tot[32];
-  __shared__ uint32_t s_prefix;
+  __shared__ int hist[kSelBins];
+  __shared__ int warp_tot[32], warp_tie[32];
+  __shared__ uint32_t warp_min[32], warp_max[32], s_key;
   __shared__ int s_kr, s_cnt;
   const int u = blockIdx.x, b = u / p.H_kv, h = u % p.H_kv, tid = threadIdx.x;
   pdl_wait();
@@ -48,8 +50,9 @@ select_kernel(keepkv_params p, keepkv_cache src, int32_t *dst_seq_len, const int
   }
   const size_t base = (size_t)u * p.N_cap;
   // Short units need few threads, and every barrier below costs by the warp: the surplus warps leave.
-  const int nthr = min((int)blockDim.x, max(128, ((len + 3) / 4 + 31) & ~31)), nw = nthr >> 5;
+  const int nthr = min((int)blockDim.x, len > 4096 ? 1024 : (len > 1024 ? 512 : 128)), nw = nthr >> 5;
   if (tid >= nthr) return;
+  const int lane = tid & 31, warp = tid >> 5;
   if (pos) {
     // A cache that is not in token order (in-place compression): sinks and recent window are told by the token
     // position of a row, not by the row.  Rows from pos_len[b] on are the tokens appended since the last call, in
@@ -74,136 +77,108 @@ select_kernel(keepkv_params p, keepkv_cache src, int32_t *dst_seq_len, const int
     lo = 0;
     hi = len;
   } else {
+#pragma unroll 4
     for (int i = tid; i < len; i += nthr) {
       // the caller's scores where given, else kappa = ln p + lscore
       keys[i] = select_key ? ordered_key(select_key[base + i]) : kappa_key(src.votes[base + i], src.lscore[base + i]);
     }
   }
+  // the range of the candidates' keys (a thread reads back what it wrote)
+  uint32_t k_lo = 0xffffffffu, k_hi = 0u;
+  for (int i = tid; i < len; i += nthr)
+    if (i >= lo && i < hi) { k_lo = min(k_lo, keys[i]); k_hi = max(k_hi, keys[i]); }
+  k_lo = __reduce_min_sync(0xffffffffu, k_lo);
+  k_hi = __reduce_max_sync(0xffffffffu, k_hi);
+  if (lane == 0) { warp_min[warp] = k_lo; warp_max[warp] = k_hi; }
   __syncthreads();
+  for (int w = 0; w < nw; ++w) { k_lo = min(k_lo, warp_min[w]); k_hi = max(k_hi, warp_max[w]); }
 
-  uint32_t kth = 0;
-  int n_tie = 0, tot_ties = 0;
-  const int m_cand = hi - lo;
-  if (n_heavy > 0 && m_cand <= kWarpSelectMax) {
-    // few candidates (every steady-state compression): warp 0 alone finds the threshold, so the four
-    // digit passes cost no block barrier
-    if (tid < 32) {
-      uint32_t k_ = 0;
-      int nt_ = 0, tt_ = 0;
-      warp_radix_select(keys, lo, hi, n_heavy, hist, k_, nt_, tt_);
-      if (tid == 0) { s_prefix = k_; s_kr = nt_; s_cnt = tt_; }
-    }
-    __syncthreads();
-    kth = s_prefix;
-    n_tie = s_kr;
-    tot_ties = s_cnt;
-  } else if (n_heavy > 0) {
-    uint32_t prefix = 0, mask = 0;
+  uint32_t kth = 0;    // the n_heavy-th largest key
+  int n_tie = 0;       // how many entries equal to it are taken, lowest index first
+  int tot_ties = 0;    // how many entries equal to it exist
+  if (n_heavy > 0) {
     int kr = n_heavy;
-    const int lane = tid & 31;
-    for (int pass = 3; pass >= 0; --pass) {
-      for (int i = tid; i < 256; i += nthr) hist[i] = 0;
+    for (;;) {
+      const int shift = max(0, 21 - __clz(k_hi - k_lo));   // (bits of the span less the 11 of a bin number)
+      const int bpt = kSelBins / nthr;                     // bins a thread
+      for (int i = tid; i < kSelBins; i += nthr) hist[i] = 0;
       __syncthreads();
-      for (int start = lo; start < hi; start += nthr) {
-        const int i = start + tid;
-        const uint32_t k = i < hi ? keys[i] : 0u;
-        const bool in = i < hi && (k & mask) == prefix;
-        // one shared-memory atomic per distinct bin of the warp (the leading bytes of most keys coincide)
-        const int bin = in ? (int)((k >> (8 * pass)) & 255u) : -1 - lane;
-        const unsigned peers = __match_any_sync(0xffffffffu, bin);
-        if (in && lane == __ffs(peers) - 1) atomicAdd(&hist[bin], __popc(peers));
+      for (int i = lo + tid; i < hi; i += nthr) {
+        const uint32_t k = keys[i];
+        if (k >= k_lo && k <= k_hi) atomicAdd(&hist[(k - k_lo) >> shift], 1);
       }
       __syncthreads();
-      if (tid < 32) {
-        // bins are scanned from the top: lane l owns bins 8l..8l+7
-        int c[8], sum = 0;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) { c[j] = hist[8 * lane + j]; sum += c[j]; }
-        int x = sum;   // becomes the count in bins of lanes >= lane
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int y = __shfl_down_sync(0xffffffffu, x, o);
-          if (lane + o < 32) x += y;
-        }
-        const int above = x - sum;
-        if (above < kr && x >= kr) {
-          int cum = above, bin = 0, cnt = 0;
-          bool found = false;
-#pragma unroll
-          for (int j = 7; j >= 0; --j) {
-            if (!found) {
-              if (cum + c[j] >= kr) { bin = j; cnt = c[j]; found = true; }
-              else cum += c[j];
-            }
-          }
-          s_prefix = prefix | ((uint32_t)(8 * lane + bin) << (8 * pass));
-          s_kr = kr - cum;
-          s_cnt = cnt;
-        }
+      // bins from the top: thread t owns bins kSelBins - 1 - t * bpt downwards
+      int sum = 0;
+      for (int j = 0; j < bpt; ++j) sum += hist[kSelBins - 1 - tid * bpt - j];
+      int tot;
+      int above = block_excl_sum(sum, warp_tot, tot, nw);
+      if (above < kr && above + sum >= kr) {
+        int bin = kSelBins - 1 - tid * bpt;
+        while (above + hist[bin] < kr) above += hist[bin--];
+        s_key = (uint32_t)bin;
+        s_kr = kr - above;
+        s_cnt = hist[bin];
       }
-      __syncthreads();   // s_prefix is not written again before the second barrier of the next pass
-      prefix = s_prefix;
+      __syncthreads();   // (not written again before the barriers of the next pass)
+      k_lo += s_key << shift;
+      k_hi = min(k_hi, k_lo + ((1u << shift) - 1u));
       kr = s_kr;
-      mask |= 0xFFu << (8 * pass);
+      if (shift == 0) break;
     }
-    kth = prefix;        // the n_heavy-th largest key
-    n_tie = kr;          // how many entries equal to it are taken, lowest index first
-    tot_ties = s_cnt;    // how many entries equal to it exist (the last pass counted full keys)
+    kth = k_lo;
+    n_tie = kr;
+    tot_ties = s_cnt;
   }
 
-  // One ordered pass writes both lists: every thread owns a run of consecutive entries, so one block
-  // scan per sweep gives the slots.  The rank among keys equal to the threshold is needed only if
-  // some of them lose.
+  // A warp owns a run of consecutive entries.  Pass 1 counts the entries above the threshold and equal to it, a scan over
+  // the warps gives the places, pass 2 writes.  Ties are ranked only if some of them lose.
   const bool rank_ties = n_heavy > 0 && n_tie < tot_ties;
-  auto valid_key = [&](int i) { return i < len ? keys[i] : 0u; };
-  constexpr int RUN = 4;
-  int base_tie = 0, base_keep = 0;
-  for (int start = 0; start < len; start += nthr * RUN) {
-    const int i0 = start + tid * RUN;
-    bool keepf[RUN], tief[RUN];
-    int n_t = 0;
-#pragma unroll
-    for (int r = 0; r < RUN; ++r) {
-      const int i = i0 + r;
-      const uint32_t k = valid_key(i);
-      const bool valid = i < len, in_mid = valid && i >= lo && i < hi && !(pos && k == 0u);
-      tief[r] = false;
-      if (!in_mid) {
-        keepf[r] = valid;
-      } else {
-        tief[r] = n_heavy > 0 && k == kth;
-        keepf[r] = n_heavy > 0 && k > kth;   // ties are added below
-        n_t += tief[r] ? 1 : 0;
-      }
+  const int run = ((len + nw - 1) / nw + 31) & ~31, e0 = min(len, warp * run), e1 = min(len, e0 + run);
+  auto classify = [&](int i, bool &keep, bool &tie) {
+    const bool valid = i < e1;
+    const uint32_t k = valid ? keys[i] : 0u;
+    const bool mid = valid && i >= lo && i < hi && !(pos && k == 0u);
+    tie = mid && n_heavy > 0 && k == kth;
+    keep = valid && (!mid || (n_heavy > 0 && k > kth) || (tie && !rank_ties));
+  };
+  int n_k = 0, n_t = 0;
+  for (int i0 = e0; i0 < e1; i0 += 32) {
+    bool keep, tie;
+    classify(i0 + lane, keep, tie);
+    n_k += __popc(__ballot_sync(0xffffffffu, keep));
+    n_t += __popc(__ballot_sync(0xffffffffu, tie));
+  }
+  if (lane == 0) { warp_tot[warp] = n_k; warp_tie[warp] = n_t; }
+  __syncthreads();
+  int slot = 0, tie_rank = 0, base_keep = 0;
+  {
+    int ties = 0;
+    for (int w = 0; w < nw; ++w) {
+      if (w == warp) { slot = base_keep; tie_rank = ties; }
+      base_keep += warp_tot[w];
+      if (rank_ties) base_keep += max(0, min(n_tie - ties, warp_tie[w]));
+      ties += warp_tie[w];
     }
-    if (n_heavy > 0) {
-      int tie_rank = base_tie, tot_tie = 0;
-      if (rank_ties) tie_rank += block_excl_sum(n_t, warp_tot, tot_tie, nw);
-#pragma unroll
-      for (int r = 0; r < RUN; ++r)
-        if (tief[r]) { keepf[r] = !rank_ties || tie_rank < n_tie; ++tie_rank; }
-      base_tie += tot_tie;
+  }
+  for (int i0 = e0; i0 < e1; i0 += 32) {
+    const int i = i0 + lane;
+    bool keep, tie;
+    classify(i, keep, tie);
+    const unsigned below = (1u << lane) - 1u;
+    if (rank_ties) {
+      const unsigned tb = __ballot_sync(0xffffffffu, tie);
+      keep = keep || (tie && tie_rank + __popc(tb & below) < n_tie);
+      tie_rank += __popc(tb);
     }
-    int n_k = 0;
-#pragma unroll
-    for (int r = 0; r < RUN; ++r) n_k += keepf[r] ? 1 : 0;
-    int tot_keep;
-    int slot = base_keep + block_excl_sum(n_k, warp_tot, tot_keep, nw);
-#pragma unroll
-    for (int r = 0; r < RUN; ++r) {
-      const int i = i0 + r;
-      if (i < len) {
-        if (keepf[r]) {
-          ret_idx[base + slot] = i;
-          target[base + i] = -2;
-          ++slot;
-        } else {
-          ev_idx[base + (i - slot)] = i;
-          target[base + i] = -1;
-        }
-      }
+    const unsigned kb = __ballot_sync(0xffffffffu, keep);
+    const int at = slot + __popc(kb & below);
+    if (i < e1) {
+      if (keep) ret_idx[base + at] = i;
+      else ev_idx[base + (i - at)] = i;
+      target[base + i] = keep ? -2 : -1;
     }
-    base_keep += tot_keep;
+    slot += __popc(kb);
   }
   if (tid == 0) {
     UnitInfo ui{len, base_keep, len - base_keep, 0, 0, 0, base_keep, 0};   // (pad0: the retained count once more, for the in-place path)
@@ -544,7 +519,7 @@ static void launch_compress_t(const keepkv_params &p, const keepkv_cache &src, c
                            select_key, ctx);
     return;
   }
-  launch_pdl(select_kernel, dim3(U), dim3(512), sel_smem, ctx.stream, p, src, dst.seq_len, budget_dev, budget_scalar,
+  launch_pdl(select_kernel, dim3(U), dim3(1024), sel_smem, ctx.stream, p, src, dst.seq_len, budget_dev, budget_scalar,
              n_recent_dev, ret_idx, target, ev_idx, ui, stats, select_key, (const int32_t *)nullptr, (int32_t *)nullptr,
              (const int32_t *)nullptr, (const int32_t *)nullptr, status_dev);
   KEEPKV_CHECK_LAUNCH(ctx);
@@ -802,7 +777,7 @@ static void launch_compress_merge_first_t(const keepkv_params &p, const keepkv_c
              eff_budget);
   KEEPKV_CHECK_LAUNCH(ctx);
   int32_t *ret2 = grp_head;   // (free again: the groups are merged)
-  launch_pdl(select_kernel, dim3(U), dim3(512), (size_t)p.N_cap * sizeof(uint32_t), ctx.stream, p, scratch, cache.seq_len,
+  launch_pdl(select_kernel, dim3(U), dim3(1024), (size_t)p.N_cap * sizeof(uint32_t), ctx.stream, p, scratch, cache.seq_len,
              (const int32_t *)eff_budget, 0, n_recent_dev, ret2, target, ev_idx, ui, st2, (const float *)nullptr,
              (const int32_t *)unit_len, (int32_t *)nullptr, (const int32_t *)nullptr, (const int32_t *)nullptr, status_dev);
   KEEPKV_CHECK_LAUNCH(ctx);
@@ -953,7 +928,7 @@ static void launch_compress_inplace_t(const keepkv_params &p, const keepkv_cache
     cudaFuncSetAttribute(resolve_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, 32768 * 4);
     attr_done_dev[dev & 63] = true;
   }
-  launch_pdl(select_kernel, dim3(U), dim3(512), (size_t)p.N_cap * sizeof(uint32_t), ctx.stream, p, c, (int32_t *)nullptr,
+  launch_pdl(select_kernel, dim3(U), dim3(1024), (size_t)p.N_cap * sizeof(uint32_t), ctx.stream, p, c, (int32_t *)nullptr,
              budget_dev, budget_scalar, n_recent_dev, kept, target, ev_idx, ui, stats, (const float *)nullptr,
              (const int32_t *)nullptr, pos, (const int32_t *)pos_len, (const int32_t *)n_seen, status_dev);
   KEEPKV_CHECK_LAUNCH(ctx);

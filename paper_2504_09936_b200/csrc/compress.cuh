@@ -65,56 +65,9 @@ __device__ __forceinline__ uint32_t kappa_key(float pv, float ls) {
   return ordered_key(kappa);
 }
 
-// One warp finds the kr-th largest of keys[lo..hi) by four 8-bit digit passes (hist: 256 ints of shared
-// memory owned by the warp).  Returns, in every lane: kth = that key, n_tie = how many entries equal to it
-// belong to the kr largest (lowest index first), tot_ties = how many entries equal to it exist.
-__device__ __forceinline__ void warp_radix_select(const uint32_t *keys, int lo, int hi, int kr, int *hist, uint32_t &kth,
-                                                  int &n_tie, int &tot_ties) {
-  const int lane = threadIdx.x & 31;
-  uint32_t prefix = 0, mask = 0;
-  int cnt_last = 0;
-  for (int pass = 3; pass >= 0; --pass) {
-#pragma unroll
-    for (int j = 0; j < 8; ++j) hist[8 * lane + j] = 0;
-    __syncwarp();
-    for (int i = lo + lane; i < hi; i += 32) {
-      const uint32_t k = keys[i];
-      if ((k & mask) == prefix) atomicAdd(&hist[(k >> (8 * pass)) & 255u], 1);
-    }
-    __syncwarp();
-    int c[8], sum = 0;   // bins are scanned from the top: lane l owns bins 8l..8l+7
-#pragma unroll
-    for (int j = 0; j < 8; ++j) { c[j] = hist[8 * lane + j]; sum += c[j]; }
-    int x = sum;   // becomes the count in bins of lanes >= lane
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_down_sync(0xffffffffu, x, o);
-      if (lane + o < 32) x += y;
-    }
-    const int above = x - sum;
-    const bool here = above < kr && x >= kr;
-    int cum = above, bin = 0, cnt = 0;
-    bool found = false;
-#pragma unroll
-    for (int j = 7; j >= 0; --j) {
-      if (!found) {
-        if (cum + c[j] >= kr) { bin = j; cnt = c[j]; found = true; }
-        else cum += c[j];
-      }
-    }
-    const int src_lane = __ffs(__ballot_sync(0xffffffffu, here)) - 1;
-    prefix |= (uint32_t)__shfl_sync(0xffffffffu, 8 * lane + bin, src_lane) << (8 * pass);
-    kr = __shfl_sync(0xffffffffu, kr - cum, src_lane);
-    cnt_last = __shfl_sync(0xffffffffu, cnt, src_lane);
-    mask |= 0xFFu << (8 * pass);
-    __syncwarp();
-  }
-  kth = prefix;
-  n_tie = kr;
-  tot_ties = cnt_last;
-}
-
-// The same search by a whole block of 256 threads (one histogram bin per thread); three barriers per digit.
+// A block of 256 threads finds the kr-th largest of keys[0..n) by four 8-bit digit passes, one histogram bin per thread and
+// three barriers per digit: kth = that key, n_tie = how many entries equal to it belong to the kr largest (lowest index
+// first), tot_ties = how many entries equal to it exist.
 // sh: three words of shared memory.  Results in every thread.
 __device__ __forceinline__ void block_radix_select(const uint32_t *keys, int n, int kr, int *hist, uint32_t *sh,
                                                    uint32_t &kth, int &n_tie, int &tot_ties) {

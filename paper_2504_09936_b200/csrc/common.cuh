@@ -16,7 +16,7 @@ constexpr int kDecMaxCtas = 512;    // upper bound on the persistent decode grid
 constexpr int kMaxUnits = 4096;    // B * H_kv that keepkv_compress accepts (per-unit tables live in shared memory)
 constexpr int kNomChunksMax = 8;   // upper bound on the column chunks a row's similarity search is split into
 
-// n_keys / ticket: entries to merge appended so far and resolve CTAs finished (select_kernel zeroes them)
+// n_keys: entries to merge appended so far; ticket: they are sorted already (select_kernel zeroes both)
 struct UnitInfo { int len, n_ret, n_ev, n_groups, n_keys, ticket, pad0, pad1; };
 
 // Byte offsets of the arrays kept in the caller's workspace.  U = B*H_kv, N = N_cap.

@@ -262,16 +262,21 @@ compact_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, const int32_
 // settle, would need a coincidence of order 1e-8 per row; exact duplicates are handled, because equal
 // keys give equal values and the lower slot stays in front.)
 // Rows that need the exact chain are queued and shared out over the warps of the CTA (coalesced row
-// loads into shared memory, the sequential chains on three lanes).  The last CTA of a unit to finish
-// sorts the entries to merge by (slot, position), which makes every group contiguous and ascending.
-constexpr int kMergeInline = 32;   // units with at most this many groups are merged by resolve_kernel itself
+// loads into shared memory, the sequential chains on three lanes).  A unit of at most kResolveThreads evicted
+// entries (every steady-state compression) is one CTA's: it sorts the entries to merge by (slot, position), which makes
+// every group contiguous and ascending, and merges them if the groups are few.  The entries to merge of larger units go to
+// a list that group_kernel sorts.
+constexpr int kMergeInline = 32;   // units with at most this many groups are merged where they are sorted
 constexpr int kResolveThreads = 512;
 constexpr int kResolveWarps = kResolveThreads / 32;
+constexpr int kGroupThreads = 1024;
+constexpr int kGroupSmem = 212992; // bytes of counters and keys group_kernel may hold
+constexpr int kGroupRank = 128;    // members of one group up to which a key finds its place among its neighbours
 
 // Sorts the M entries to merge of unit u by (slot, position) -- which makes every group contiguous and ascending --,
 // publishes the sorted members and the start of every group, and merges the groups itself when there are few.
-// Called by a whole CTA of kResolveThreads threads.  keys: where the M keys are now (key_smem when `single`, else gk).
-template <int D>
+// Called by a whole CTA of NT threads.  keys: where the M keys are now (key_smem when `single`, else gk).
+template <int D, int NT>
 __device__ __forceinline__ void group_and_merge(const keepkv_params &p, const keepkv_cache &src, const keepkv_cache &dst,
                                                 int u, size_t base, int n_ev, int M, bool single, uint32_t *key_smem,
                                                 int smem_keys, uint32_t *gk, const int32_t *__restrict__ ret_idx,
@@ -282,10 +287,10 @@ __device__ __forceinline__ void group_and_merge(const keepkv_params &p, const ke
   while (Mp < M) Mp <<= 1;
   uint32_t *keys = (single || Mp <= smem_keys) ? key_smem : gk;
   if (keys != gk && !single)
-    for (int i = tid; i < M; i += kResolveThreads) keys[i] = __ldcg(&gk[i]);
-  for (int i = M + tid; i < Mp; i += kResolveThreads) keys[i] = 0xFFFFFFFFu;
+    for (int i = tid; i < M; i += NT) keys[i] = __ldcg(&gk[i]);
+  for (int i = M + tid; i < Mp; i += NT) keys[i] = 0xFFFFFFFFu;
   __syncthreads();
-  if (Mp <= kResolveThreads && keys == key_smem) {
+  if (Mp <= NT && keys == key_smem) {
     // few keys (all distinct): every thread finds the rank of its key by counting, one barrier
     uint32_t mine = 0xFFFFFFFFu;
     int rank = 0;
@@ -300,7 +305,7 @@ __device__ __forceinline__ void group_and_merge(const keepkv_params &p, const ke
     // bitonic sort, ascending
     for (int k = 2; k <= Mp; k <<= 1) {
       for (int jj = k >> 1; jj > 0; jj >>= 1) {
-        for (int i = tid; i < Mp; i += kResolveThreads) {
+        for (int i = tid; i < Mp; i += NT) {
           const int ixj = i ^ jj;
           if (ixj > i) {
             const uint32_t a = keys[i], b = keys[ixj];
@@ -313,7 +318,7 @@ __device__ __forceinline__ void group_and_merge(const keepkv_params &p, const ke
   }
   // publish the sorted members and the start of every group
   int n_groups = 0;
-  for (int i0 = 0; i0 < M; i0 += kResolveThreads) {
+  for (int i0 = 0; i0 < M; i0 += NT) {
     const int i = i0 + tid;
     const bool head = i < M && (i == 0 || (keys[i] >> 16) != (keys[i - 1] >> 16));
     int tot;
@@ -330,7 +335,7 @@ __device__ __forceinline__ void group_and_merge(const keepkv_params &p, const ke
   if (n_groups <= kMergeInline) {
     // few groups (every steady-state compression): merge them here, one warp per group
     __syncthreads();   // the keys and group starts written above are visible to the whole CTA
-    for (int g = warp; g < n_groups; g += kResolveWarps) {
+    for (int g = warp; g < n_groups; g += NT / 32) {
       const int beg = grp_head[base + g], n = grp_head[base + g + 1] - beg;
       const int c = (int)(gk[beg] >> 16);
       merge_group<D>(p, src, dst, c, ret_idx[base + c], [&](int t) { return ev_idx[base + (gk[beg + t] & 0xFFFFu)]; }, n,
@@ -345,12 +350,12 @@ __global__ void __launch_bounds__(kResolveThreads)
 resolve_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, const int32_t *__restrict__ ev_idx,
                UnitInfo *unit_info, const float4 *__restrict__ nom_v, const int32_t *__restrict__ nom_si,
                const int32_t *__restrict__ sched, int C_max, const int32_t *__restrict__ ret_idx, int32_t *target,
-               uint32_t *grp_key, int key_stride, int32_t *grp_head, keepkv_stats *stats, int smem_keys, int decide_only) {
-  extern __shared__ uint32_t key_smem[];
+               uint32_t *grp_key, int key_stride, int32_t *grp_head, keepkv_stats *stats, int decide_only) {
+  __shared__ uint32_t key_smem[kResolveThreads];
   __shared__ float ke_s[kResolveWarps][D];
   __shared__ float kc_s[kResolveWarps][2][D];
   __shared__ int warp_tot[32];
-  __shared__ int s_nq[2], s_base, s_last;
+  __shared__ int s_nq[2], s_base;
   __shared__ int q_tid[kResolveThreads], q_e[kResolveThreads], q_kind[kResolveThreads], q_a[kResolveThreads],
       q_b[kResolveThreads];
   __shared__ int res_slot[kResolveThreads], res_merge[kResolveThreads];
@@ -364,10 +369,7 @@ resolve_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, const int32_
   uint32_t *gk = grp_key + (size_t)u * key_stride;
   const int C = sched[0];
   const float T = p.merge_threshold;
-  // CTAs of the unit that have rows; the others leave at once.  A unit whose rows fit one pass of one CTA
-  // (every steady-state compression) needs no exchange through global memory.
-  const int n_cta = min((int)gridDim.x, (ui.n_ev + kResolveThreads - 1) / kResolveThreads);
-  if ((int)blockIdx.x >= n_cta) return;
+  if ((int)blockIdx.x * kResolveThreads >= ui.n_ev) return;
   const bool single = ui.n_ev <= kResolveThreads && !decide_only;
   if (tid == 0) { s_nq[0] = s_nq[1] = 0; s_base = 0; }
   __syncthreads();
@@ -444,27 +446,104 @@ resolve_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, const int32_
       if (merge) gk[s_base + off] = ((uint32_t)slot << 16) | (uint32_t)j;
     }
   }
-  if (decide_only) return;
-  int M;
-  if (single) {
-    M = s_base;
-  } else {
-    // ---- the last CTA of the unit to arrive groups the entries
-    __threadfence();
+  if (!single) return;
+  if (tid == 0) unit_info[u].ticket = 1;   // this unit's entries are sorted
+  group_and_merge<D, kResolveThreads>(p, src, dst, u, base, ui.n_ev, s_base, true, key_smem, kResolveThreads, gk, ret_idx, ev_idx,
+                                      target, grp_head, unit_info, stats, warp_tot);
+}
+
+// One CTA per unit: the unit's key list (in global memory, any order) sorted into groups by counting -- a histogram of the
+// slots in shared memory, a scan, every key to its group, its rank there from its neighbours: nine barriers, where a
+// bitonic sort of 4096 keys has 78.  Lists that do not fit, or hold a group of more than kGroupRank members, are sorted
+// bitonically after all.  (With the sort at the end of resolve_kernel by a unit's last CTA, at a few CTAs a unit, the two
+// steps took 45 us for 64 units of 6554 entries and 113 us for 128 units of up to 14746.)
+template <int D>
+__global__ void __launch_bounds__(kGroupThreads)
+group_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, const int32_t *__restrict__ ret_idx,
+             const int32_t *__restrict__ ev_idx, int32_t *target, UnitInfo *unit_info, uint32_t *grp_key, int key_stride,
+             int32_t *grp_head, keepkv_stats *stats, int smem_words) {
+  extern __shared__ uint32_t key_smem[];
+  __shared__ int warp_tot[32];
+  __shared__ int s_max;
+  constexpr int NT = kGroupThreads;
+  const int tid = threadIdx.x, u = blockIdx.x;
+  pdl_wait();
+  pdl_trigger();
+  const UnitInfo ui = unit_info[u];
+  if (ui.ticket) return;   // resolve_kernel has sorted this unit's
+  const size_t base = (size_t)u * p.N_cap;
+  uint32_t *gk = grp_key + (size_t)u * key_stride;
+  const int M = ui.n_keys, n_slots = ui.n_ret;
+  if (n_slots + M <= smem_words) {
+    int *cnt = reinterpret_cast<int *>(key_smem);
+    uint32_t *out = key_smem + n_slots;
+    for (int i = tid; i < n_slots; i += NT) cnt[i] = 0;
+    if (tid == 0) s_max = 0;
     __syncthreads();
-    if (tid == 0) s_last = atomicAdd(&unit_info[u].ticket, 1) == n_cta - 1;
+    int most = 0;
+#pragma unroll 4
+    for (int i = tid; i < M; i += NT) most = max(most, atomicAdd(&cnt[gk[i] >> 16], 1) + 1);
+    most = __reduce_max_sync(0xffffffffu, most);
+    if ((tid & 31) == 0) atomicMax(&s_max, most);
     __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    M = *reinterpret_cast<volatile int *>(&unit_info[u].n_keys);
+    if (s_max <= kGroupRank) {
+      // a thread owns a run of slots: keys and groups before it, in one packed scan
+      const int per = (n_slots + NT - 1) / NT, lo = min(n_slots, tid * per), hi = min(n_slots, lo + per);
+      int mine = 0;
+      for (int s = lo; s < hi; ++s) mine += cnt[s] + (cnt[s] > 0 ? 1 << 16 : 0);
+      int tot;
+      unsigned at = (unsigned)block_excl_sum(mine, warp_tot, tot, NT / 32);
+      for (int s = lo; s < hi; ++s) {
+        const int n = cnt[s];
+        cnt[s] = (int)(at & 0xffffu);
+        if (n > 0) {
+          grp_head[base + (at >> 16)] = (int)(at & 0xffffu);
+          at += (1u << 16) + (unsigned)n;
+        }
+      }
+      const int n_groups = (int)((unsigned)tot >> 16);
+      __syncthreads();
+#pragma unroll 4
+      for (int i = tid; i < M; i += NT) {
+        const uint32_t k = gk[i];
+        out[atomicAdd(&cnt[k >> 16], 1)] = k;
+      }
+      __syncthreads();
+      for (int i = tid; i < M; i += NT) {
+        const uint32_t k = out[i], slot = k >> 16;
+        int j = i - 1, less = 0;
+        for (; j >= 0 && (out[j] >> 16) == slot; --j) less += out[j] < k ? 1 : 0;
+        const int beg = j + 1;
+        for (j = i + 1; j < M && (out[j] >> 16) == slot; ++j) less += out[j] < k ? 1 : 0;
+        gk[beg + less] = k;
+      }
+      if (tid == 0) {
+        grp_head[base + n_groups] = M;
+        unit_info[u].n_groups = n_groups;
+        stats[u].n_below_T = ui.n_ev - M;
+      }
+      return;
+    }
+    __syncthreads();   // the counters make room for keys
   }
-  group_and_merge<D>(p, src, dst, u, base, ui.n_ev, M, single, key_smem, smem_keys, gk, ret_idx, ev_idx, target, grp_head,
-                     unit_info, stats, warp_tot);
+  group_and_merge<D, NT>(p, src, dst, u, base, ui.n_ev, M, false, key_smem, smem_words, gk, ret_idx, ev_idx, target, grp_head,
+                         unit_info, stats, warp_tot);
+}
+
+// What the two kernels are launched with.
+static int resolve_grid(const keepkv_params &p) { return (p.N_cap + kResolveThreads - 1) / kResolveThreads; }   // a pass each
+static int group_words(const keepkv_params &p, const WsLayout &L) {
+  const int words = p.N_cap + L.key_stride;
+  return words < kGroupSmem / 4 ? words : kGroupSmem / 4;
+}
+// No unit can evict more than the entries one CTA of resolve_kernel sorts.
+static bool all_small(const keepkv_params &p, const int32_t *budget_dev, int32_t budget_scalar) {
+  return !budget_dev && p.N_cap - budget_scalar <= kResolveThreads;
 }
 
 // ------------------------------------------------------------------ merge
 // Units with many groups (the first compression of a long prompt): warps of several CTAs share them.
-// Units with few groups were already merged by resolve_kernel, which left n_groups = 0 here.
+// Units whose few groups were merged where they were sorted have n_groups = 0 here.
 template <int D>
 __global__ void __launch_bounds__(256)
 merge_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, const int32_t *__restrict__ ret_idx,
@@ -504,14 +583,13 @@ static void launch_compress_t(const keepkv_params &p, const keepkv_cache &src, c
   const int ret_bound = budget_dev ? p.N_cap : (budget_scalar < p.N_cap ? budget_scalar : p.N_cap);
 
   const size_t sel_smem = (size_t)p.N_cap * sizeof(uint32_t);
-  const int smem_keys = L.key_stride < 32768 ? L.key_stride : 32768;
   static bool attr_done_dev[64] = {};   // opt-in to large dynamic shared memory once per device
   int dev = 0;
   cudaGetDevice(&dev);
   bool &attr_done = attr_done_dev[dev & 63];
   if (!attr_done) {
     cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 49152 * 4);
-    cudaFuncSetAttribute(resolve_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, 32768 * 4);
+    cudaFuncSetAttribute(group_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGroupSmem);
     attr_done = true;
   }
   if (p.flags & KEEPKV_FLAG_COMPRESS_STEADY) {   // the caller vouches for every unit: one kernel does it all
@@ -532,10 +610,15 @@ static void launch_compress_t(const keepkv_params &p, const keepkv_cache &src, c
   KEEPKV_CHECK_LAUNCH(ctx);
   if (!merges) return;
   launch_nominate(p, src, dst, ev_idx, ui, inv_norm, norm_ext, sched, nom_v, nom_si, L.nom_chunks, status_dev, ctx);
-  launch_pdl(resolve_kernel<D>, dim3(L.nom_chunks, U), dim3(kResolveThreads), (size_t)smem_keys * 4, ctx.stream,
+  launch_pdl(resolve_kernel<D>, dim3(resolve_grid(p), U), dim3(kResolveThreads), 0, ctx.stream,
       p, src, dst, ev_idx, ui, nom_v, nom_si, sched, L.nom_chunks, ret_idx, target, grp_key, L.key_stride, grp_head,
-      stats, smem_keys, 0);
+      stats, 0);
   KEEPKV_CHECK_LAUNCH(ctx);
+  if (!all_small(p, budget_dev, budget_scalar)) {
+    launch_pdl(group_kernel<D>, dim3(U), dim3(kGroupThreads), (size_t)group_words(p, L) * 4, ctx.stream, p, src, dst, ret_idx,
+               ev_idx, target, ui, grp_key, L.key_stride, grp_head, stats, group_words(p, L));
+    KEEPKV_CHECK_LAUNCH(ctx);
+  }
   int gx = 4096 / U;
   gx = gx < 1 ? 1 : (gx > 32 ? 32 : gx);
   launch_pdl(merge_kernel<D>, dim3(gx, U), dim3(256), 0, ctx.stream, p, src, dst, ret_idx, ev_idx, target, ui, grp_key,
@@ -664,23 +747,6 @@ mf_mark_kernel(keepkv_params p, int32_t *unit_len, int32_t *ret_idx, int32_t *ta
   }
 }
 
-// One CTA per unit: the unit's key list (in global memory) sorted into groups; few groups are merged here.
-template <int D>
-__global__ void __launch_bounds__(kResolveThreads)
-group_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, const int32_t *__restrict__ ret_idx,
-             const int32_t *__restrict__ ev_idx, int32_t *target, UnitInfo *unit_info, uint32_t *grp_key, int key_stride,
-             int32_t *grp_head, keepkv_stats *stats, int smem_keys) {
-  extern __shared__ uint32_t key_smem[];
-  __shared__ int warp_tot[32];
-  pdl_wait();
-  pdl_trigger();
-  const int u = blockIdx.x;
-  const UnitInfo ui = unit_info[u];
-  const size_t base = (size_t)u * p.N_cap;
-  group_and_merge<D>(p, src, dst, u, base, ui.n_ev, ui.n_keys, false, key_smem, smem_keys, grp_key + (size_t)u * key_stride,
-                     ret_idx, ev_idx, target, grp_head, unit_info, stats, warp_tot);
-}
-
 // Budget of each sequence for the eviction pass: the caller's, capped by the sequence's shortest merged head (the
 // heads of a sequence share one seq_len, so they must all end at the same length).
 __global__ void mf_budget_kernel(keepkv_params p, const int32_t *budget_dev, int budget_scalar, const int32_t *unit_len,
@@ -737,14 +803,12 @@ static void launch_compress_merge_first_t(const keepkv_params &p, const keepkv_c
   keepkv_stats *st2 = reinterpret_cast<keepkv_stats *>(ws + L.stats);
   int32_t *unit_len = reinterpret_cast<int32_t *>(ws + L.unit_len);
   int32_t *eff_budget = reinterpret_cast<int32_t *>(ws + L.eff_budget);
-  const int smem_keys = L.key_stride < 32768 ? L.key_stride : 32768;
   static bool attr_done_dev[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
   if (!attr_done_dev[dev & 63]) {
     cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 49152 * 4);
-    cudaFuncSetAttribute(resolve_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, 32768 * 4);
-    cudaFuncSetAttribute(group_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, 32768 * 4);
+    cudaFuncSetAttribute(group_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGroupSmem);
     attr_done_dev[dev & 63] = true;
   }
   // ---- pass 1: similar entries merged with each other, cache -> scratch (every head keeps its own length for now)
@@ -754,9 +818,9 @@ static void launch_compress_merge_first_t(const keepkv_params &p, const keepkv_c
   KEEPKV_CHECK_LAUNCH(ctx);
   // rows and columns are the same keys: the "retained" operand of the search is the prompt itself
   launch_nominate(p, cache, cache, ev_idx, ui, inv_norm, norm_ext, sched, nom_v, nom_si, L.nom_chunks, status_dev, ctx, 1);
-  launch_pdl(resolve_kernel<D>, dim3(L.nom_chunks, U), dim3(kResolveThreads), (size_t)smem_keys * 4, ctx.stream,
+  launch_pdl(resolve_kernel<D>, dim3(resolve_grid(p), U), dim3(kResolveThreads), 0, ctx.stream,
       p, cache, cache, ev_idx, ui, nom_v, nom_si, sched, L.nom_chunks, ret1, target, grp_key, L.key_stride, grp_head,
-      st1, smem_keys, 1);
+      st1, 1);
   KEEPKV_CHECK_LAUNCH(ctx);
   launch_pdl(mf_mark_kernel, dim3(U), dim3(1024), 0, ctx.stream, p, unit_len, ret1, target, ev_idx, grp_head, grp_key,
              L.key_stride, ui, st1);
@@ -764,8 +828,8 @@ static void launch_compress_merge_first_t(const keepkv_params &p, const keepkv_c
   const int cgx = (p.N_cap + 63) / 64 < 32 ? (p.N_cap + 63) / 64 : 32;
   launch_pdl(compact_kernel<D>, dim3(cgx, U), dim3(256), 0, ctx.stream, p, cache, scratch, ret1, ui, inv_norm, (uint4 *)nullptr);
   KEEPKV_CHECK_LAUNCH(ctx);
-  launch_pdl(group_kernel<D>, dim3(U), dim3(kResolveThreads), (size_t)smem_keys * 4, ctx.stream, p, cache, scratch, ret1,
-             ev_idx, target, ui, grp_key, L.key_stride, grp_head, st1, smem_keys);
+  launch_pdl(group_kernel<D>, dim3(U), dim3(kGroupThreads), (size_t)group_words(p, L) * 4, ctx.stream, p, cache, scratch, ret1,
+             ev_idx, target, ui, grp_key, L.key_stride, grp_head, st1, group_words(p, L));
   KEEPKV_CHECK_LAUNCH(ctx);
   int mgx = 4096 / U;
   mgx = mgx < 1 ? 1 : (mgx > 32 ? 32 : mgx);
@@ -919,13 +983,12 @@ static void launch_compress_inplace_t(const keepkv_params &p, const keepkv_cache
   int32_t *nom_si = reinterpret_cast<int32_t *>(ws + L.nom_si);
   uint32_t *grp_key = reinterpret_cast<uint32_t *>(ws + L.grp_key);
   int32_t *grp_head = reinterpret_cast<int32_t *>(ws + L.grp_head);
-  const int smem_keys = L.key_stride < 32768 ? L.key_stride : 32768;
   static bool attr_done_dev[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
   if (!attr_done_dev[dev & 63]) {
     cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 49152 * 4);
-    cudaFuncSetAttribute(resolve_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, 32768 * 4);
+    cudaFuncSetAttribute(group_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGroupSmem);
     attr_done_dev[dev & 63] = true;
   }
   launch_pdl(select_kernel, dim3(U), dim3(1024), (size_t)p.N_cap * sizeof(uint32_t), ctx.stream, p, c, (int32_t *)nullptr,
@@ -941,10 +1004,15 @@ static void launch_compress_inplace_t(const keepkv_params &p, const keepkv_cache
     launch_pdl(ip_columns_kernel, dim3((U + 127) / 128), dim3(128), 0, ctx.stream, ui, U, 1);
     KEEPKV_CHECK_LAUNCH(ctx);
     launch_nominate(p, c, c, ev_idx, ui, inv_norm, norm_ext, sched, nom_v, nom_si, L.nom_chunks, status_dev, ctx);
-    launch_pdl(resolve_kernel<D>, dim3(L.nom_chunks, U), dim3(kResolveThreads), (size_t)smem_keys * 4, ctx.stream,
+    launch_pdl(resolve_kernel<D>, dim3(resolve_grid(p), U), dim3(kResolveThreads), 0, ctx.stream,
         p, c, c, ev_idx, ui, nom_v, nom_si, sched, L.nom_chunks, ident, target, grp_key, L.key_stride, grp_head,
-        stats, smem_keys, 0);
+        stats, 0);
     KEEPKV_CHECK_LAUNCH(ctx);
+    if (!all_small(p, budget_dev, budget_scalar)) {
+      launch_pdl(group_kernel<D>, dim3(U), dim3(kGroupThreads), (size_t)group_words(p, L) * 4, ctx.stream, p, c, c, ident, ev_idx,
+                 target, ui, grp_key, L.key_stride, grp_head, stats, group_words(p, L));
+      KEEPKV_CHECK_LAUNCH(ctx);
+    }
     int mgx = 4096 / U;
     mgx = mgx < 1 ? 1 : (mgx > 32 ? 32 : mgx);
     launch_pdl(merge_kernel<D>, dim3(mgx, U), dim3(256), 0, ctx.stream, p, c, c, ident, ev_idx, target, ui, grp_key,

@@ -32,7 +32,7 @@ struct WsLayout {
   size_t norm_ext;    // bf16 [U,N,8]       |k| of the same in three terms, as more channels of the search's columns
   size_t nom_v;       // float4 [U,N,C]     per evicted row and column chunk: best, second cosine, unused, best slot
   size_t nom_si;      // i32 [U,N,C]        slot of the second-best cosine
-  size_t grp_key;     // u32 [U,Npow2]      (slot << 16 | evicted position) of merged entries, sorted
+  size_t grp_key;     // u32 [U,Npow2]      (slot << 16 | source index) of merged entries, sorted
   size_t grp_head;    // i32 [U,N]          position in grp_key where each group starts
   size_t stats;       // keepkv_stats [U]   used when the caller passes no stats array
   size_t stats2;      // keepkv_stats [U]   merge-first: statistics of the merge pass

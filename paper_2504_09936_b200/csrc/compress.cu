@@ -279,9 +279,7 @@ constexpr int kGroupRank = 128;    // members of one group up to which a key fin
 template <int D, int NT>
 __device__ __forceinline__ void group_and_merge(const keepkv_params &p, const keepkv_cache &src, const keepkv_cache &dst,
                                                 int u, size_t base, int n_ev, int M, bool single, uint32_t *key_smem,
-                                                int smem_keys, uint32_t *gk, const int32_t *__restrict__ ret_idx,
-                                                const int32_t *__restrict__ ev_idx, int32_t *target, int32_t *grp_head,
-                                                UnitInfo *unit_info, keepkv_stats *stats, int *warp_tot) {
+                                                int smem_keys, uint32_t *gk, int32_t *target, int32_t *grp_head, UnitInfo *unit_info, keepkv_stats *stats, int *warp_tot) {
   const int tid = threadIdx.x, warp = tid >> 5;
   int Mp = 1;
   while (Mp < M) Mp <<= 1;
@@ -335,12 +333,14 @@ __device__ __forceinline__ void group_and_merge(const keepkv_params &p, const ke
   if (n_groups <= kMergeInline) {
     // few groups (every steady-state compression): merge them here, one warp per group
     __syncthreads();   // the keys and group starts written above are visible to the whole CTA
+    MergeCount count;
     for (int g = warp; g < n_groups; g += NT / 32) {
       const int beg = grp_head[base + g], n = grp_head[base + g + 1] - beg;
       const int c = (int)(gk[beg] >> 16);
-      merge_group<D>(p, src, dst, c, ret_idx[base + c], [&](int t) { return ev_idx[base + (gk[beg + t] & 0xFFFFu)]; }, n,
-                     target + base, base, stats + u);
+      merge_group<D>(p, src, dst, c, dst, base + c, [&](int t) { return (int)(gk[beg + t] & 0xFFFFu); }, n,
+                     target + base, base, count);
     }
+    count.flush(stats + u);
   }
 }
 
@@ -349,8 +349,7 @@ template <int D>
 __global__ void __launch_bounds__(kResolveThreads)
 resolve_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, const int32_t *__restrict__ ev_idx,
                UnitInfo *unit_info, const float4 *__restrict__ nom_v, const int32_t *__restrict__ nom_si,
-               const int32_t *__restrict__ sched, int C_max, const int32_t *__restrict__ ret_idx, int32_t *target,
-               uint32_t *grp_key, int key_stride, int32_t *grp_head, keepkv_stats *stats, int decide_only) {
+               const int32_t *__restrict__ sched, int C_max, int32_t *target, uint32_t *grp_key, int key_stride, int32_t *grp_head, keepkv_stats *stats, int decide_only) {
   __shared__ uint32_t key_smem[kResolveThreads];
   __shared__ float ke_s[kResolveWarps][D];
   __shared__ float kc_s[kResolveWarps][2][D];
@@ -433,7 +432,7 @@ resolve_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, const int32_
     if (single) {   // this CTA holds all rows of the unit: its keys never leave shared memory
       if (valid) {
         target[base + e] = merge ? slot : -1;
-        if (merge) key_smem[off] = ((uint32_t)slot << 16) | (uint32_t)j;
+        if (merge) key_smem[off] = ((uint32_t)slot << 16) | (uint32_t)e;
       }
       if (tid == 0) s_base = tot;
       __syncthreads();
@@ -443,13 +442,12 @@ resolve_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, const int32_
     __syncthreads();
     if (valid) {
       target[base + e] = merge ? slot : -1;
-      if (merge) gk[s_base + off] = ((uint32_t)slot << 16) | (uint32_t)j;
+      if (merge) gk[s_base + off] = ((uint32_t)slot << 16) | (uint32_t)e;
     }
   }
   if (!single) return;
   if (tid == 0) unit_info[u].ticket = 1;   // this unit's entries are sorted
-  group_and_merge<D, kResolveThreads>(p, src, dst, u, base, ui.n_ev, s_base, true, key_smem, kResolveThreads, gk, ret_idx, ev_idx,
-                                      target, grp_head, unit_info, stats, warp_tot);
+  group_and_merge<D, kResolveThreads>(p, src, dst, u, base, ui.n_ev, s_base, true, key_smem, kResolveThreads, gk, target, grp_head, unit_info, stats, warp_tot);
 }
 
 // One CTA per unit: the unit's key list (in global memory, any order) sorted into groups by counting -- a histogram of the
@@ -459,8 +457,7 @@ resolve_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, const int32_
 // steps took 45 us for 64 units of 6554 entries and 113 us for 128 units of up to 14746.)
 template <int D>
 __global__ void __launch_bounds__(kGroupThreads)
-group_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, const int32_t *__restrict__ ret_idx,
-             const int32_t *__restrict__ ev_idx, int32_t *target, UnitInfo *unit_info, uint32_t *grp_key, int key_stride,
+group_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, int32_t *target, UnitInfo *unit_info, uint32_t *grp_key, int key_stride,
              int32_t *grp_head, keepkv_stats *stats, int smem_words) {
   extern __shared__ uint32_t key_smem[];
   __shared__ int warp_tot[32];
@@ -526,12 +523,15 @@ group_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, const int32_t 
     }
     __syncthreads();   // the counters make room for keys
   }
-  group_and_merge<D, NT>(p, src, dst, u, base, ui.n_ev, M, false, key_smem, smem_words, gk, ret_idx, ev_idx, target, grp_head,
-                         unit_info, stats, warp_tot);
+  group_and_merge<D, NT>(p, src, dst, u, base, ui.n_ev, M, false, key_smem, smem_words, gk, target, grp_head, unit_info, stats, warp_tot);
 }
 
 // What the two kernels are launched with.
 static int resolve_grid(const keepkv_params &p) { return (p.N_cap + kResolveThreads - 1) / kResolveThreads; }   // a pass each
+static int merge_grid(const keepkv_params &p) {
+  const int n = 4096 / (p.B * p.H_kv);
+  return n < 1 ? 1 : (n > 128 ? 128 : n);
+}
 static int group_words(const keepkv_params &p, const WsLayout &L) {
   const int words = p.N_cap + L.key_stride;
   return words < kGroupSmem / 4 ? words : kGroupSmem / 4;
@@ -546,22 +546,30 @@ static bool all_small(const keepkv_params &p, const int32_t *budget_dev, int32_t
 // Units whose few groups were merged where they were sorted have n_groups = 0 here.
 template <int D>
 __global__ void __launch_bounds__(256)
-merge_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, const int32_t *__restrict__ ret_idx,
-             const int32_t *__restrict__ ev_idx, int32_t *target, const UnitInfo *__restrict__ unit_info,
+merge_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, int32_t *target, const UnitInfo *__restrict__ unit_info,
              const uint32_t *__restrict__ grp_key, int key_stride, const int32_t *__restrict__ grp_head,
              keepkv_stats *stats) {
   const int u = blockIdx.y;
   pdl_wait();
   pdl_trigger();
-  const UnitInfo ui = unit_info[u];
+  const int n_groups = unit_info[u].n_groups, step = gridDim.x * 8;
   const size_t base = (size_t)u * p.N_cap;
   const uint32_t *gk = grp_key + (size_t)u * key_stride;
-  for (int g = blockIdx.x * 8 + (threadIdx.x >> 5); g < ui.n_groups; g += gridDim.x * 8) {
-    const int beg = grp_head[base + g], n = grp_head[base + g + 1] - beg;
+  const int32_t *head = grp_head + base;
+  int g = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (g >= n_groups) return;
+  int beg = head[g], end = head[g + 1];
+  MergeCount count;
+  while (g < n_groups) {
+    const int nx = min(g + step, n_groups - 1), nbeg = head[nx], nend = head[nx + 1];   // the next group's, in flight meanwhile
     const int c = (int)(gk[beg] >> 16);
-    merge_group<D>(p, src, dst, c, ret_idx[base + c], [&](int t) { return ev_idx[base + (gk[beg + t] & 0xFFFFu)]; }, n,
-                   target + base, base, stats + u);
+    merge_group<D>(p, src, dst, c, dst, base + c, [&](int t) { return (int)(gk[beg + t] & 0xFFFFu); }, end - beg, target + base,
+                   base, count);
+    g += step;
+    beg = nbeg;
+    end = nend;
   }
+  count.flush(stats + u);
 }
 
 // ------------------------------------------------------------------ host side
@@ -611,17 +619,15 @@ static void launch_compress_t(const keepkv_params &p, const keepkv_cache &src, c
   if (!merges) return;
   launch_nominate(p, src, dst, ev_idx, ui, inv_norm, norm_ext, sched, nom_v, nom_si, L.nom_chunks, status_dev, ctx);
   launch_pdl(resolve_kernel<D>, dim3(resolve_grid(p), U), dim3(kResolveThreads), 0, ctx.stream,
-      p, src, dst, ev_idx, ui, nom_v, nom_si, sched, L.nom_chunks, ret_idx, target, grp_key, L.key_stride, grp_head,
+      p, src, dst, ev_idx, ui, nom_v, nom_si, sched, L.nom_chunks, target, grp_key, L.key_stride, grp_head,
       stats, 0);
   KEEPKV_CHECK_LAUNCH(ctx);
   if (!all_small(p, budget_dev, budget_scalar)) {
-    launch_pdl(group_kernel<D>, dim3(U), dim3(kGroupThreads), (size_t)group_words(p, L) * 4, ctx.stream, p, src, dst, ret_idx,
-               ev_idx, target, ui, grp_key, L.key_stride, grp_head, stats, group_words(p, L));
+    launch_pdl(group_kernel<D>, dim3(U), dim3(kGroupThreads), (size_t)group_words(p, L) * 4, ctx.stream, p, src, dst,
+               target, ui, grp_key, L.key_stride, grp_head, stats, group_words(p, L));
     KEEPKV_CHECK_LAUNCH(ctx);
   }
-  int gx = 4096 / U;
-  gx = gx < 1 ? 1 : (gx > 32 ? 32 : gx);
-  launch_pdl(merge_kernel<D>, dim3(gx, U), dim3(256), 0, ctx.stream, p, src, dst, ret_idx, ev_idx, target, ui, grp_key,
+  launch_pdl(merge_kernel<D>, dim3(merge_grid(p), U), dim3(256), 0, ctx.stream, p, src, dst, target, ui, grp_key,
              L.key_stride, grp_head, stats);
   KEEPKV_CHECK_LAUNCH(ctx);
 }
@@ -675,7 +681,7 @@ mf_prepare_kernel(keepkv_params p, keepkv_cache src, int32_t *ev_idx, UnitInfo *
 
 // One CTA per unit.  partner[e] (in `target`): the entry e would merge into, or -1.  Writes the kept list (ret_idx),
 // the member list (ev_idx), target[e] = slot of the partner for a member / -2 for a kept entry, the group keys
-// (slot << 16 | position among the members), sizes and the initial statistics.  slot_of: scratch [N] per unit.
+// (slot << 16 | entry), sizes and the initial statistics.  slot_of: scratch [N] per unit.
 __global__ void __launch_bounds__(1024)
 mf_mark_kernel(keepkv_params p, int32_t *unit_len, int32_t *ret_idx, int32_t *target, int32_t *ev_idx, int32_t *slot_of,
                uint32_t *grp_key, int key_stride, UnitInfo *unit_info, keepkv_stats *stats) {
@@ -726,7 +732,7 @@ mf_mark_kernel(keepkv_params p, int32_t *unit_len, int32_t *ret_idx, int32_t *ta
     const int so = slot_of[base + e];
     if (so < 0) {
       const int pos = -1 - so, slot = slot_of[base + tg[e]];
-      gk[pos] = ((uint32_t)slot << 16) | (uint32_t)pos;
+      gk[pos] = ((uint32_t)slot << 16) | (uint32_t)e;
       slot_of[base + e] = -0x40000000 + slot;   // remembered for the rewrite below
     }
   }
@@ -819,7 +825,7 @@ static void launch_compress_merge_first_t(const keepkv_params &p, const keepkv_c
   // rows and columns are the same keys: the "retained" operand of the search is the prompt itself
   launch_nominate(p, cache, cache, ev_idx, ui, inv_norm, norm_ext, sched, nom_v, nom_si, L.nom_chunks, status_dev, ctx, 1);
   launch_pdl(resolve_kernel<D>, dim3(resolve_grid(p), U), dim3(kResolveThreads), 0, ctx.stream,
-      p, cache, cache, ev_idx, ui, nom_v, nom_si, sched, L.nom_chunks, ret1, target, grp_key, L.key_stride, grp_head,
+      p, cache, cache, ev_idx, ui, nom_v, nom_si, sched, L.nom_chunks, target, grp_key, L.key_stride, grp_head,
       st1, 1);
   KEEPKV_CHECK_LAUNCH(ctx);
   launch_pdl(mf_mark_kernel, dim3(U), dim3(1024), 0, ctx.stream, p, unit_len, ret1, target, ev_idx, grp_head, grp_key,
@@ -828,12 +834,10 @@ static void launch_compress_merge_first_t(const keepkv_params &p, const keepkv_c
   const int cgx = (p.N_cap + 63) / 64 < 32 ? (p.N_cap + 63) / 64 : 32;
   launch_pdl(compact_kernel<D>, dim3(cgx, U), dim3(256), 0, ctx.stream, p, cache, scratch, ret1, ui, inv_norm, (uint4 *)nullptr);
   KEEPKV_CHECK_LAUNCH(ctx);
-  launch_pdl(group_kernel<D>, dim3(U), dim3(kGroupThreads), (size_t)group_words(p, L) * 4, ctx.stream, p, cache, scratch, ret1,
-             ev_idx, target, ui, grp_key, L.key_stride, grp_head, st1, group_words(p, L));
+  launch_pdl(group_kernel<D>, dim3(U), dim3(kGroupThreads), (size_t)group_words(p, L) * 4, ctx.stream, p, cache, scratch,
+             target, ui, grp_key, L.key_stride, grp_head, st1, group_words(p, L));
   KEEPKV_CHECK_LAUNCH(ctx);
-  int mgx = 4096 / U;
-  mgx = mgx < 1 ? 1 : (mgx > 32 ? 32 : mgx);
-  launch_pdl(merge_kernel<D>, dim3(mgx, U), dim3(256), 0, ctx.stream, p, cache, scratch, ret1, ev_idx, target, ui, grp_key,
+  launch_pdl(merge_kernel<D>, dim3(merge_grid(p), U), dim3(256), 0, ctx.stream, p, cache, scratch, target, ui, grp_key,
              L.key_stride, grp_head, st1);
   KEEPKV_CHECK_LAUNCH(ctx);
   // ---- pass 2: the eviction strategy alone, scratch -> cache
@@ -1005,17 +1009,15 @@ static void launch_compress_inplace_t(const keepkv_params &p, const keepkv_cache
     KEEPKV_CHECK_LAUNCH(ctx);
     launch_nominate(p, c, c, ev_idx, ui, inv_norm, norm_ext, sched, nom_v, nom_si, L.nom_chunks, status_dev, ctx);
     launch_pdl(resolve_kernel<D>, dim3(resolve_grid(p), U), dim3(kResolveThreads), 0, ctx.stream,
-        p, c, c, ev_idx, ui, nom_v, nom_si, sched, L.nom_chunks, ident, target, grp_key, L.key_stride, grp_head,
+        p, c, c, ev_idx, ui, nom_v, nom_si, sched, L.nom_chunks, target, grp_key, L.key_stride, grp_head,
         stats, 0);
     KEEPKV_CHECK_LAUNCH(ctx);
     if (!all_small(p, budget_dev, budget_scalar)) {
-      launch_pdl(group_kernel<D>, dim3(U), dim3(kGroupThreads), (size_t)group_words(p, L) * 4, ctx.stream, p, c, c, ident, ev_idx,
+      launch_pdl(group_kernel<D>, dim3(U), dim3(kGroupThreads), (size_t)group_words(p, L) * 4, ctx.stream, p, c, c,
                  target, ui, grp_key, L.key_stride, grp_head, stats, group_words(p, L));
       KEEPKV_CHECK_LAUNCH(ctx);
     }
-    int mgx = 4096 / U;
-    mgx = mgx < 1 ? 1 : (mgx > 32 ? 32 : mgx);
-    launch_pdl(merge_kernel<D>, dim3(mgx, U), dim3(256), 0, ctx.stream, p, c, c, ident, ev_idx, target, ui, grp_key,
+    launch_pdl(merge_kernel<D>, dim3(merge_grid(p), U), dim3(256), 0, ctx.stream, p, c, c, target, ui, grp_key,
                L.key_stride, grp_head, stats);
     KEEPKV_CHECK_LAUNCH(ctx);
   }

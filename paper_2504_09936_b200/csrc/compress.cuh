@@ -1,6 +1,8 @@
 // Device helpers shared by the kernels of keepkv_compress (compress.cu: the general pipeline;
 // compress_steady.cu: the single-kernel path of a steady-state compression).
 #pragma once
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace keepkv {
@@ -234,12 +236,29 @@ __device__ __forceinline__ void exact_cosines(const __nv_bfloat16 *ke, const __n
 // One warp per group.  With a_i = ln p_i + lscore_i over the group K'_e (target first, then members
 // ascending):  omega = softmax(a),  v_r = sum omega_i v_i,  k_r = gamma * sum omega_i k_i,
 // gamma = L / lambda_bar,  L = LSE(a) - ln(sum p),  lambda_bar = sum omega_i lscore_i,  p_r = sum p,
-// lscore_r = L   (Eq. A.3 in logarithms).  c: the target's slot in dst, ci: its source index,
-// member(t): source index of the t-th member (ascending), target_u: the unit's per-entry targets.
+// lscore_r = L   (Eq. A.3 in logarithms).  c: the target's slot in dst, (tc, ti): a cache and row that hold the target as
+// it was, member(t): source index of the t-th member (ascending), target_u: the unit's per-entry targets.
+// Bound: the chain of dependent loads of the warp with the largest group.  So the target is read where it was copied to (its
+// source index would be one load more), members are known by source index, the first kMergePre rows are requested with the
+// votes, before the weights are known, the others eight at a time, and beyond 31 members every lane weighs its own (one
+// after the other in all lanes, a group of 45 was what 35 us of a launch over 15000 groups waited for).
+constexpr int kMergePre = 4;
+
+// What a warp has merged: added to the unit's statistics once, when it has done all its groups.
+struct MergeCount {
+  int merged = 0, groups = 0, guarded = 0, most = 0;
+  __device__ __forceinline__ void flush(keepkv_stats *st) const {
+    if ((threadIdx.x & 31) || !groups) return;
+    if (merged) { atomicAdd(&st->n_merged, merged); atomicMax(&st->max_group, most); }
+    if (guarded) atomicAdd(&st->n_guard_groups, guarded);
+    atomicAdd(&st->n_groups, groups);
+  }
+};
 template <int D, typename MemberFn>
 __device__ __forceinline__ void merge_group(const keepkv_params &p, const keepkv_cache &src, const keepkv_cache &dst,
-                                            int c, int ci, MemberFn member, int n, int32_t *target_u, size_t base,
-                                            keepkv_stats *st) {
+                                            int c, const keepkv_cache &tc, size_t ti, MemberFn member, int n, int32_t *target_u,
+                                            size_t base,
+                                            MergeCount &count) {
   constexpr int EPL = D / 32;
   const int lane = threadIdx.x & 31;
   const float *votes = src.votes + base, *ls = src.lscore + base;
@@ -254,21 +273,22 @@ __device__ __forceinline__ void merge_group(const keepkv_params &p, const keepkv
   double lbar = 0.0, L, Ps;
 #pragma unroll
   for (int e = 0; e < EPL; ++e) { ka[e] = 0.f; va[e] = 0.f; }
-  auto accumulate = [&](int i, float om) {
+  using Row = typename std::conditional<EPL == 4, uint2, uint32_t>::type;   // a lane's part of a row
+  const Row *rK = reinterpret_cast<const Row *>(sK) + lane, *rV = reinterpret_cast<const Row *>(sV) + lane;
+  const Row *qK = reinterpret_cast<const Row *>(reinterpret_cast<const __nv_bfloat16 *>(tc.K) + ti * D) + lane;
+  const Row *qV = reinterpret_cast<const Row *>(reinterpret_cast<const __nv_bfloat16 *>(tc.V) + ti * D) + lane;
+  auto add_row = [&](const Row kk, const Row vv, float om) {
     if constexpr (EPL == 4) {
-      const uint2 kk = *reinterpret_cast<const uint2 *>(sK + (size_t)i * D + lane * 4);
-      const uint2 vv = *reinterpret_cast<const uint2 *>(sV + (size_t)i * D + lane * 4);
       ka[0] = fmaf(om, bf16_lo(kk.x), ka[0]); ka[1] = fmaf(om, bf16_hi(kk.x), ka[1]);
       ka[2] = fmaf(om, bf16_lo(kk.y), ka[2]); ka[3] = fmaf(om, bf16_hi(kk.y), ka[3]);
       va[0] = fmaf(om, bf16_lo(vv.x), va[0]); va[1] = fmaf(om, bf16_hi(vv.x), va[1]);
       va[2] = fmaf(om, bf16_lo(vv.y), va[2]); va[3] = fmaf(om, bf16_hi(vv.y), va[3]);
     } else {
-      const uint32_t kk = *reinterpret_cast<const uint32_t *>(sK + (size_t)i * D + lane * 2);
-      const uint32_t vv = *reinterpret_cast<const uint32_t *>(sV + (size_t)i * D + lane * 2);
       ka[0] = fmaf(om, bf16_lo(kk), ka[0]); ka[1] = fmaf(om, bf16_hi(kk), ka[1]);
       va[0] = fmaf(om, bf16_lo(vv), va[0]); va[1] = fmaf(om, bf16_hi(vv), va[1]);
     }
   };
+  auto accumulate = [&](int i, float om) { add_row(rK[(size_t)i * 32], rV[(size_t)i * 32], om); };
   auto wsum_d = [](double v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -283,8 +303,17 @@ __device__ __forceinline__ void merge_group(const keepkv_params &p, const keepkv
   if (n < 32) {
     // the usual case: lane 0 holds the target, lane t the t-th member, so that their votes and scores are
     // fetched together and the row loads of the accumulation do not wait on one another
-    const int idx = lane == 0 ? ci : (lane <= n ? member(lane - 1) : -1);
-    const float pv = idx >= 0 ? votes[idx] : 0.f, lsv = idx >= 0 ? ls[idx] : 0.f;
+    const int idx = lane == 0 ? 0 : (lane <= n ? member(lane - 1) : -1);
+    Row kp[kMergePre], vp[kMergePre];
+#pragma unroll
+    for (int t = 0; t < kMergePre; ++t) {
+      const int i = __shfl_sync(0xffffffffu, idx, t);
+      if (t == 0) { kp[t] = __ldcg(qK); vp[t] = __ldcg(qV); }
+      else if (t <= n) { kp[t] = rK[(size_t)i * 32]; vp[t] = rV[(size_t)i * 32]; }
+    }
+    float pv = 0.f, lsv = 0.f;
+    if (lane == 0) { pv = __ldcg(tc.votes + ti); lsv = __ldcg(tc.lscore + ti); }
+    else if (idx >= 0) { pv = votes[idx]; lsv = ls[idx]; }
     // fp32 first: with |L| and |lambda_bar| away from zero its error (about 1e-6 absolute) is far below bf16
     // resolution in gamma; only a group near the cancellation is evaluated again in fp64 (a warp-uniform choice)
     float om;
@@ -310,16 +339,23 @@ __device__ __forceinline__ void merge_group(const keepkv_params &p, const keepkv
       lbar = wsum_d(omd * (double)lsv);
       om = (float)omd;
     }
-#pragma unroll 4
-    for (int t = 0; t <= n; ++t) accumulate(__shfl_sync(0xffffffffu, idx, t), __shfl_sync(0xffffffffu, om, t));
+#pragma unroll
+    for (int t = 0; t < kMergePre; ++t) {
+      const float w = __shfl_sync(0xffffffffu, om, t);
+      if (t <= n) add_row(kp[t], vp[t], w);
+    }
+#pragma unroll 8
+    for (int t = kMergePre; t <= n; ++t) accumulate(__shfl_sync(0xffffffffu, idx, t), __shfl_sync(0xffffffffu, om, t));
   } else {
-    const double a_c = log((double)votes[ci]) + (double)ls[ci];
+    // Larger groups: 32 members at a time, one a lane, three times over (maximum, sums, weights with the rows); fp64.
+    const float pc = __ldcg(tc.votes + ti), lc = __ldcg(tc.lscore + ti);
+    const double a_c = log((double)pc) + (double)lc;
     double M = a_c;
     for (int t = lane; t < n; t += 32) { const int e = member(t); M = fmax(M, log((double)votes[e]) + (double)ls[e]); }
     M = wmax_d(M);
     double Z = 0.0;
     Ps = 0.0;
-    if (lane == 0) { Z = exp(a_c - M); Ps = (double)votes[ci]; }
+    if (lane == 0) { Z = exp(a_c - M); Ps = (double)pc; }
     for (int t = lane; t < n; t += 32) {
       const int e = member(t);
       Z += exp(log((double)votes[e]) + (double)ls[e] - M);
@@ -329,14 +365,23 @@ __device__ __forceinline__ void merge_group(const keepkv_params &p, const keepkv
     Ps = wsum_d(Ps);
     const double Lam = M + log(Z);
     L = Lam - log(Ps);
-    // every lane walks all members (the rows are spread over the lanes by channel), so lambda_bar is summed per lane
-    for (int t = -1; t < n; ++t) {
-      const int i = t < 0 ? ci : member(t);
-      const double lsi = (double)ls[i];
-      const double omd = exp(log((double)votes[i]) + lsi - Lam);
-      lbar += omd * lsi;
-      accumulate(i, (float)omd);
+    const double om_c = exp(a_c - Lam);
+    lbar = lane == 0 ? om_c * (double)lc : 0.0;
+    add_row(__ldcg(qK), __ldcg(qV), (float)om_c);
+    for (int t0 = 0; t0 < n; t0 += 32) {
+      const int e = t0 + lane < n ? member(t0 + lane) : 0;
+      double omd = 0.0;
+      if (t0 + lane < n) {
+        const double lsi = (double)ls[e];
+        omd = exp(log((double)votes[e]) + lsi - Lam);
+        lbar += omd * lsi;
+      }
+      const float om = (float)omd;
+      const int m = min(32, n - t0);
+#pragma unroll 8
+      for (int t = 0; t < m; ++t) accumulate(__shfl_sync(0xffffffffu, e, t), __shfl_sync(0xffffffffu, om, t));
     }
+    lbar = wsum_d(lbar);
   }
   const double gamma_d = L / lbar;
   const float gamma = (float)gamma_d;
@@ -344,7 +389,8 @@ __device__ __forceinline__ void merge_group(const keepkv_params &p, const keepkv
   if (!ok) {
     // guard: the members are dropped after all and the target keeps the row copied by compaction
     for (int t = lane; t < n; t += 32) target_u[member(t)] = -1;
-    if (lane == 0) { atomicAdd(&st->n_guard_groups, 1); atomicAdd(&st->n_groups, 1); }
+    ++count.guarded;
+    ++count.groups;
     return;
   }
   __nv_bfloat16 *dK = reinterpret_cast<__nv_bfloat16 *>(dst.K) + (base + c) * D;
@@ -362,10 +408,10 @@ __device__ __forceinline__ void merge_group(const keepkv_params &p, const keepkv
   if (lane == 0) {
     dst.votes[base + c] = (float)Ps;
     dst.lscore[base + c] = (float)L;
-    atomicAdd(&st->n_merged, n);
-    atomicAdd(&st->n_groups, 1);
-    atomicMax(&st->max_group, n);
   }
+  count.merged += n;
+  ++count.groups;
+  count.most = max(count.most, n);
 }
 
 // the single-kernel path of a steady-state compression (compress_steady.cu)

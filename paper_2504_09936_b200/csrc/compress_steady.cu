@@ -472,12 +472,14 @@ steady_compress_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, cons
   }
   __syncthreads();
   // ---- Algorithm 1, merge step: one warp per group
+  MergeCount count;
   for (int gi = warp; gi < n_groups; gi += kStWarps) {
     const int beg = ghead[gi], n = ghead[gi + 1] - beg;
     const int c = (int)(skey[beg] >> 16);
-    merge_group<D>(p, src, dst, c, ret(c), [&](int t) { return ev[skey[beg + t] & 0xFFFFu]; }, n, target + base, base,
-                   stats + u);
+    merge_group<D>(p, src, dst, c, src, base + ret(c), [&](int t) { return ev[skey[beg + t] & 0xFFFFu]; }, n, target + base, base,
+                   count);
   }
+  count.flush(stats + u);
 }
 
 template <int D>

@@ -245,6 +245,29 @@ def test_compress_search_at_tile_edges(d, T):
     assert stats[:, 2].sum() > 0 and stats[:, 3].sum() > 0      # some merged, some below the threshold
 
 
+@pytest.mark.parametrize("size", [127, 128, 129, 200])
+@pytest.mark.parametrize("n", [900, 1700])
+def test_compress_group_of_given_size(size, n):
+    """One target with `size` members on either side of where grouping by counting gives way to the sort, in units of up to
+    and of more than one CTA of the decision (512 evicted entries), beside ordinary groups: the oracle's targets and rows."""
+    B, H_kv, G, d, budget = 1, 2, 2, 128, 500
+    p = kb.make_params(B=B, H_q=H_kv * G, H_kv=H_kv, d=d, N_cap=1728, period=0, n_sink=4, n_recent=300, merge_threshold=0.8)
+    src = random_cache(p, [n], seed=size + n, vote_max=3, scored_frac=1.0)
+    rng = np.random.default_rng(size)
+    K = rng.standard_normal((H_kv, p.N_cap, d)).astype(np.float32)
+    K[:, 260:360] = K[:, 660:760] + 0.3 * rng.standard_normal((H_kv, 100, d))     # pairs, some retained, some not
+    rows = 40 + rng.permutation(210)[:size]                                       # evicted: their scores are the lowest
+    K[:, rows] = K[:, 2:3] + 0.3 * rng.standard_normal((H_kv, size, d))           # close to a sink
+    src.K.copy_(f32_to_dev_bf16(K).view(B, H_kv, p.N_cap, d))
+    src.lscore.mul_(0.25).add_(1.5)
+    src.lscore[:, :, 40:250] = 0.5
+    dst, ret, tgt, stats = _run_compress(p, src, budget)
+    hs, hd = HostCache(src), HostCache(dst)
+    for u in range(H_kv):
+        check_compress_unit(p, u, budget, p.n_recent, hs, hd, ret, tgt, stats, what=f"group of {size}", max_tolerated=4)
+        assert np.sum(tgt[u] == 2) >= size
+
+
 def test_compress_ragged_budgets_and_copy_through():
     """Per-sequence budgets and recent windows; a sequence within its budget is copied in order."""
     B, H_kv, G, d = 3, 2, 2, 128

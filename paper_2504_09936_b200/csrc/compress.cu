@@ -12,13 +12,11 @@
 namespace keepkv {
 
 // ------------------------------------------------------------------ select
-// One CTA per unit.  The keys of the whole unit live in shared memory.  The heavy-hitter threshold is found by
-// histograms of kSelBins bins over the range the candidates' keys really span: the bin that holds the n-th largest becomes
-// the next range, so three passes settle any 32-bit key (the leading byte of most keys coincides, so a histogram of fixed
-// digits has its counts in a few bins: four passes with one atomic per distinct digit of a warp took 49 us for 64 units
-// of 8192 where this kernel takes 22 us, 95 us for 128 of up to 16384 where it takes 32 us).  Then every warp counts what it keeps of a contiguous run of entries, one
-// block scan gives the places, and the retained list, the evicted list and the per-entry marks are written in order.
-constexpr int kSelBins = 2048;
+// One CTA per unit.  The keys of the whole unit live in shared memory; the heavy-hitter threshold is found by range_select.
+// Then every warp counts what it keeps of a contiguous run of entries, one block scan gives the places, and the retained
+// list, the evicted list and the per-entry marks are written 32 consecutive entries at a time.  49 -> 22 us for 64 units of
+// 8192, 95 -> 32 us for 128 of up to 16384, against four passes over 8-bit digits and an ordered pass with three block
+// barriers every 2048 entries.
 __global__ void __launch_bounds__(1024)
 select_kernel(keepkv_params p, keepkv_cache src, int32_t *dst_seq_len, const int32_t *budget_dev, int budget_scalar,
               const int32_t *n_recent_dev, int32_t *ret_idx, int32_t *target, int32_t *ev_idx, UnitInfo *unit_info,
@@ -27,8 +25,8 @@ select_kernel(keepkv_params p, keepkv_cache src, int32_t *dst_seq_len, const int
   extern __shared__ uint32_t keys[];
   __shared__ int hist[kSelBins];
   __shared__ int warp_tot[32], warp_tie[32];
-  __shared__ uint32_t warp_min[32], warp_max[32], s_key;
-  __shared__ int s_kr, s_cnt;
+  __shared__ uint32_t warp_min[32], warp_max[32];
+  __shared__ int s_sel[3];
   const int u = blockIdx.x, b = u / p.H_kv, h = u % p.H_kv, tid = threadIdx.x;
   pdl_wait();
   pdl_trigger();
@@ -96,40 +94,7 @@ select_kernel(keepkv_params p, keepkv_cache src, int32_t *dst_seq_len, const int
   uint32_t kth = 0;    // the n_heavy-th largest key
   int n_tie = 0;       // how many entries equal to it are taken, lowest index first
   int tot_ties = 0;    // how many entries equal to it exist
-  if (n_heavy > 0) {
-    int kr = n_heavy;
-    for (;;) {
-      const int shift = max(0, 21 - __clz(k_hi - k_lo));   // (bits of the span less the 11 of a bin number)
-      const int bpt = kSelBins / nthr;                     // bins a thread
-      for (int i = tid; i < kSelBins; i += nthr) hist[i] = 0;
-      __syncthreads();
-      for (int i = lo + tid; i < hi; i += nthr) {
-        const uint32_t k = keys[i];
-        if (k >= k_lo && k <= k_hi) atomicAdd(&hist[(k - k_lo) >> shift], 1);
-      }
-      __syncthreads();
-      // bins from the top: thread t owns bins kSelBins - 1 - t * bpt downwards
-      int sum = 0;
-      for (int j = 0; j < bpt; ++j) sum += hist[kSelBins - 1 - tid * bpt - j];
-      int tot;
-      int above = block_excl_sum(sum, warp_tot, tot, nw);
-      if (above < kr && above + sum >= kr) {
-        int bin = kSelBins - 1 - tid * bpt;
-        while (above + hist[bin] < kr) above += hist[bin--];
-        s_key = (uint32_t)bin;
-        s_kr = kr - above;
-        s_cnt = hist[bin];
-      }
-      __syncthreads();   // (not written again before the barriers of the next pass)
-      k_lo += s_key << shift;
-      k_hi = min(k_hi, k_lo + ((1u << shift) - 1u));
-      kr = s_kr;
-      if (shift == 0) break;
-    }
-    kth = k_lo;
-    n_tie = kr;
-    tot_ties = s_cnt;
-  }
+  if (n_heavy > 0) range_select(keys, lo, hi, k_lo, k_hi, n_heavy, nthr, hist, s_sel, warp_tot, kth, n_tie, tot_ties);
 
   // A warp owns a run of consecutive entries.  Pass 1 counts the entries above the threshold and equal to it, a scan over
   // the warps gives the places, pass 2 writes.  Ties are ranked only if some of them lose.

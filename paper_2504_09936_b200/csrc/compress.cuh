@@ -10,15 +10,18 @@ namespace keepkv {
 constexpr float kRankEps = 1e-4f;   // tensor-core cosines closer than this are re-evaluated in the interface's fp32 chain
 
 // ------------------------------------------------------------------ block scans
+// The barrier of the threads that take part (the block, unless the kernel has warps with other work).
+struct BlockSync { __device__ __forceinline__ void operator()() const { __syncthreads(); } };
 // Exclusive prefix count of `flag` over the first nw warps of the block in thread order (the other
 // warps have left the kernel); total returned through `total`.
-__device__ __forceinline__ int block_excl_count(bool flag, int *warp_tot, int &total, int nw) {
+template <typename Sync = BlockSync>
+__device__ __forceinline__ int block_excl_count(bool flag, int *warp_tot, int &total, int nw, Sync sync = Sync()) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned bal = __ballot_sync(0xffffffffu, flag);
   const int in_warp = __popc(bal & ((1u << lane) - 1u));
-  __syncthreads();  // warp_tot may still be read from the previous call
+  sync();  // warp_tot may still be read from the previous call
   if (lane == 0) warp_tot[warp] = __popc(bal);
-  __syncthreads();
+  sync();
   int off = 0, tot = 0;
   for (int w = 0; w < nw; ++w) {
     const int t = warp_tot[w];
@@ -33,7 +36,8 @@ __device__ __forceinline__ int block_excl_count(bool flag, int *warp_tot, int &t
 }
 
 // Exclusive prefix sum of small non-negative ints over the block (thread order).
-__device__ __forceinline__ int block_excl_sum(int v, int *warp_tot, int &total, int nw) {
+template <typename Sync = BlockSync>
+__device__ __forceinline__ int block_excl_sum(int v, int *warp_tot, int &total, int nw, Sync sync = Sync()) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int x = v;
 #pragma unroll
@@ -41,9 +45,9 @@ __device__ __forceinline__ int block_excl_sum(int v, int *warp_tot, int &total, 
     const int y = __shfl_up_sync(0xffffffffu, x, o);
     if (lane >= o) x += y;
   }
-  __syncthreads();
+  sync();
   if (lane == 31) warp_tot[warp] = x;
-  __syncthreads();
+  sync();
   int off = 0, tot = 0;
   for (int w = 0; w < nw; ++w) {
     const int t = warp_tot[w];
@@ -67,65 +71,48 @@ __device__ __forceinline__ uint32_t kappa_key(float pv, float ls) {
   return ordered_key(kappa);
 }
 
-// A block of 256 threads finds the kr-th largest of keys[0..n) by four 8-bit digit passes, one histogram bin per thread and
-// three barriers per digit: kth = that key, n_tie = how many entries equal to it belong to the kr largest (lowest index
-// first), tot_ties = how many entries equal to it exist.
-// sh: three words of shared memory.  Results in every thread.
-__device__ __forceinline__ void block_radix_select(const uint32_t *keys, int n, int kr, int *hist, uint32_t *sh,
-                                                   uint32_t &kth, int &n_tie, int &tot_ties) {
-  const int tid = threadIdx.x, lane = tid & 31;
-  uint32_t prefix = 0, mask = 0;
-  for (int pass = 3; pass >= 0; --pass) {
-    hist[tid] = 0;
-    __syncthreads();
-    for (int start = 0; start < n; start += 256) {
-      const int i = start + tid;
-      const uint32_t k = i < n ? keys[i] : 0u;
-      const bool in = i < n && (k & mask) == prefix;
-      // one shared-memory atomic per distinct bin among the warp's keys that are still in the race (the leading
-      // bytes of most keys coincide; in the later passes few keys are left)
-      const unsigned racing = __ballot_sync(0xffffffffu, in);
-      if (in) {
-        const int bin = (int)((k >> (8 * pass)) & 255u);
-        const unsigned peers = __match_any_sync(racing, bin);
-        if (lane == __ffs(peers) - 1) atomicAdd(&hist[bin], __popc(peers));
-      }
+// nthr threads (a power of two, 64 to 1024; thread tid) find the kr-th largest of keys[lo..hi), all of which lie in
+// [k_lo, k_hi], by histograms of kSelBins bins over that range: the bin that holds it becomes the next range, so three
+// passes settle any 32-bit key.  (The leading byte of most keys coincides: fixed 8-bit digits put the counts into a few
+// bins, which took a pass more and one atomic per distinct digit of a warp.)  kth = that key, n_tie = how many entries
+// equal to it belong to the kr largest (lowest index first), tot_ties = how many entries equal to it exist.
+// hist: kSelBins words, sh: three, warp_tot: one per warp of shared memory.
+constexpr int kSelBins = 2048;
+template <typename Sync = BlockSync>
+__device__ __forceinline__ void range_select(const uint32_t *keys, int lo, int hi, uint32_t k_lo, uint32_t k_hi, int kr, int nthr,
+                                             int *hist, int *sh, int *warp_tot, uint32_t &kth, int &n_tie, int &tot_ties,
+                                             Sync sync = Sync()) {
+  const int tid = threadIdx.x, bpt = kSelBins / nthr;
+  for (;;) {
+    const int shift = max(0, 21 - __clz(k_hi - k_lo));   // (bits of the span less the 11 of a bin number)
+    for (int i = tid; i < kSelBins; i += nthr) hist[i] = 0;
+    sync();
+    for (int i = lo + tid; i < hi; i += nthr) {
+      const uint32_t k = keys[i];
+      if (k >= k_lo && k <= k_hi) atomicAdd(&hist[(k - k_lo) >> shift], 1);
     }
-    __syncthreads();
-    if (tid < 32) {
-      int c[8], sum = 0;   // bins are scanned from the top: lane l owns bins 8l..8l+7
-#pragma unroll
-      for (int j = 0; j < 8; ++j) { c[j] = hist[8 * lane + j]; sum += c[j]; }
-      int x = sum;   // becomes the count in bins of lanes >= lane
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_down_sync(0xffffffffu, x, o);
-        if (lane + o < 32) x += y;
-      }
-      const int above = x - sum;
-      if (above < kr && x >= kr) {
-        int cum = above, bin = 0, cnt = 0;
-        bool found = false;
-#pragma unroll
-        for (int j = 7; j >= 0; --j) {
-          if (!found) {
-            if (cum + c[j] >= kr) { bin = j; cnt = c[j]; found = true; }
-            else cum += c[j];
-          }
-        }
-        sh[0] = prefix | ((uint32_t)(8 * lane + bin) << (8 * pass));
-        sh[1] = (uint32_t)(kr - cum);
-        sh[2] = (uint32_t)cnt;
-      }
+    sync();
+    // bins from the top: thread t owns bins kSelBins - 1 - t * bpt downwards
+    int sum = 0;
+    for (int j = 0; j < bpt; ++j) sum += hist[kSelBins - 1 - tid * bpt - j];
+    int tot;
+    int above = block_excl_sum(sum, warp_tot, tot, nthr >> 5, sync);
+    if (above < kr && above + sum >= kr) {
+      int bin = kSelBins - 1 - tid * bpt;
+      while (above + hist[bin] < kr) above += hist[bin--];
+      sh[0] = bin;
+      sh[1] = kr - above;
+      sh[2] = hist[bin];
     }
-    __syncthreads();   // sh is not written again before the second barrier of the next pass
-    prefix = sh[0];
-    kr = (int)sh[1];
-    mask |= 0xFFu << (8 * pass);
+    sync();   // (not written again before the barriers of the next pass)
+    k_lo += (uint32_t)sh[0] << shift;
+    k_hi = min(k_hi, k_lo + ((1u << shift) - 1u));
+    kr = sh[1];
+    if (shift == 0) break;
   }
-  kth = prefix;
+  kth = k_lo;
   n_tie = kr;
-  tot_ties = (int)sh[2];
+  tot_ties = sh[2];
 }
 
 // ------------------------------------------------------------------ tensor-core ranking: top two of a row
@@ -170,20 +157,14 @@ struct Top2 {
 // values within thr of its best.  (A cut from the smaller best lets through everything between the two bests,
 // and with 32 rows per warp the warp-wide skip then hardly ever fires.)
 // a_i: accumulators, w_i: inverse norms of the four columns idx..idx+3.
-// TEST = false (the first tile of an item, where nearly every group holds a new candidate for some row):
-// all four columns are inserted without the skip test, so nothing but the select chains is on the
-// critical path.
-template <bool TEST>
 __device__ __forceinline__ void offer4(Top2 &ta, Top2 &tb, float a0, float a1, float a2, float a3, const float4 w,
                                        int idx) {
-  if (TEST) {
-    const float ncut = -ta.cut;
-    const uint32_t s = __float_as_uint(fmaf(a0, w.x, ncut)) & __float_as_uint(fmaf(a1, w.y, ncut)) &
-                       __float_as_uint(fmaf(a2, w.z, ncut)) & __float_as_uint(fmaf(a3, w.w, ncut));
-    if (!__any_sync(0xffffffffu, (int)s >= 0)) return;   // no lane has a value that is not below its cut
-  }
+  const float ncut = -ta.cut;
+  const uint32_t s = __float_as_uint(fmaf(a0, w.x, ncut)) & __float_as_uint(fmaf(a1, w.y, ncut)) &
+                     __float_as_uint(fmaf(a2, w.z, ncut)) & __float_as_uint(fmaf(a3, w.w, ncut));
+  if (!__any_sync(0xffffffffu, (int)s >= 0)) return;   // no lane has a value that is not below its cut
   ta.insert(a0 * w.x, idx); tb.insert(a1 * w.y, idx + 1); ta.insert(a2 * w.z, idx + 2); tb.insert(a3 * w.w, idx + 3);
-  if (TEST) ta.cut = fmaxf(ta.cut, fmaxf(ta.best, tb.best) - ta.thr);   // (a cut only rises: it may have started above the best)
+  ta.cut = fmaxf(ta.cut, fmaxf(ta.best, tb.best) - ta.thr);   // (a cut only rises: it may have started above the best)
 }
 
 // ------------------------------------------------------------------ the cut inside the product

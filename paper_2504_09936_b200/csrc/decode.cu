@@ -36,6 +36,7 @@
 //
 // Every wait is bounded.  One that runs out marks the CTA (s_abort): its warps go on through their barriers without
 // waiting and without arithmetic, copies and products in flight get a bounded time to end, KEEPKV_DEV_TIMEOUT is raised.
+#include <atomic>
 #include <mutex>
 
 #include "common.cuh"
@@ -48,7 +49,9 @@ constexpr int kDecTile = 128;      // entries of a tile: lanes of tensor memory
 constexpr int kGroup = 32;         // entries of a work group: granularity of the split and of a partial tile's copies
 constexpr int kSeqCache = 256;     // sequence lengths a CTA keeps in shared memory
 constexpr int kDecTmemCols = 128;  // S: 2 x 16 columns, O: 2 x 16 (d = 64: 2 x 32)
+constexpr int kSlack = 32;         // groups that cost a CTA about as much as the cuts of the equal split
 constexpr int kMinGroups = 2;      // groups a range of the equal split holds at least
+constexpr int kOneCtaSmem = 120 * 1024;   // more than half of an SM's shared memory
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 
@@ -63,7 +66,7 @@ struct DecSmem {
   static constexpr int kP = kQ + 2 * kQBytes;                // bf16 [2 halves of the tile][16][64], swizzled
   // what the CTAs of a cluster send one another when their unit ends: f32 [rank][16 maxima and sums], then numerators
   static constexpr int kInbox = kP + 4096;
-  template <int G> static constexpr int bytes() { return kInbox + (8 * 16 + G * D) * 4; }
+  template <int G> static constexpr int bytes() { return kInbox + (8 * 16 + G * D + 8) * 4; }   // (a slice is rounded up)
   // (the query operand's columns 8-15, which nobody reads, are whatever follows a sub-tile of kQ: always inside)
 };
 
@@ -109,7 +112,7 @@ struct DecWalk {
 template <int D, int G, bool kEarly>
 __global__ void __launch_bounds__(kDecThreads, 2)
 decode_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapV,
-              keepkv_params p,
+              keepkv_params p, int ranges,
               keepkv_cache c, const __nv_bfloat16 *__restrict__ q, __nv_bfloat16 *__restrict__ out,
               float *__restrict__ lse, int update_scores, int *counters, PartRec<D, G> *pool, int32_t *status_dev,
               const uint4 *__restrict__ k_new, const uint4 *__restrict__ v_new, int spin_limit, int withhold) {
@@ -146,7 +149,7 @@ decode_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ 
     mbar_fence_init();
   }
   if (tid == 32) { prefetch_tensormap(&mapK); prefetch_tensormap(&mapV); }
-  const int csize = (int)cluster_nctarank(), crank = (int)cluster_ctarank(), cshift = 31 - __clz(csize);   // (1, 2, 4 or 8)
+  const int csize = (int)cluster_nctarank(), crank = (int)cluster_ctarank();   // (1 to 8)
   if (csize > 1) cluster_arrive();   // waited for below: nobody writes to a CTA that has not started
   if (!kEarly) {
     pdl_wait();      // everything above ran while the previous kernel of the stream was finishing
@@ -190,19 +193,25 @@ decode_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ 
     gb_max = max(gb_max, s_tbmax[w]);
   }
   const int T = total_b * p.H_kv;   // (below 2^26: the rows of a cache are indexed by 32-bit TMA coordinates)
-  // one cluster per unit, if the launch has them and no sequence is much longer than the average
-  const bool split = grid == U << cshift && (long long)gb_max * p.B * 4 <= 5LL * total_b;
-  int chunk = max((T + grid - 1) / grid, kMinGroups);
+  int chunk = max((T + ranges - 1) / ranges, kMinGroups);
+  const bool even = gb_max * p.B == total_b;
+  // The cuts through units cost an equal range 3 to 6 us -- tickets, two segments in a row -- about what a CTA takes for
+  // kSlack groups.  So a cluster takes its whole unit, if the launch has one per unit, unless that leaves the CTAs of
+  // the longest unit more than kSlack groups, or a quarter, above an equal range.  (56 units of 121-485 entries, d = 64:
+  // 13.1 -> 8.0 us; 64 of 425-1702, d = 128: 17.4 -> 14.6 us; 64 of 2000-8000, 63 groups against 39: equal.)  Where the
+  // launch has more units than are resident at once, the equal ranges are the worse only for short units of unequal
+  // length (384 of 175-700: 27.5 -> 22.6 us; 512 of 442: 27.6 -> 28.8 us; 400 of 375-1500: equal).
+  const bool split = grid == U * csize && (U <= ranges ? gb_max <= (chunk + max(kSlack, chunk / 4)) * csize : !even && gb_max <= kSlack);
   // Equal ranges: when every unit has the same number of groups and a range holds more than one unit, the range is
-  // rounded up to whole units (if that costs at most an eighth more): no unit is then cut between two CTAs.
-  if (gb_max > 0 && gb_max * p.B == total_b && chunk > gb_max) {
+  // rounded up to whole units, if that costs at most an eighth, or a tile, more: no unit is then cut between two CTAs.
+  if (gb_max > 0 && even && chunk > gb_max) {
     const int up = (chunk + gb_max - 1) / gb_max * gb_max;
-    if (up * 8 <= chunk * 9) chunk = up;
+    if (up <= chunk + max(kDecTile / kGroup, chunk / 8)) chunk = up;
   }
   if (split) {
     if (tid == 0) {
-      const int u = cta >> cshift, b = u / p.H_kv, gb = groups_of(b);
-      const int lo = (crank * gb) >> cshift, hi = ((crank + 1) * gb) >> cshift;
+      const int u = cta / csize, b = u / p.H_kv, gb = groups_of(b);
+      const int lo = crank * gb / csize, hi = (crank + 1) * gb / csize;
       s_start[0] = b; s_start[1] = u % p.H_kv; s_start[2] = lo; s_start[3] = 0; s_start[4] = hi - lo;
     }
   } else {
@@ -591,6 +600,8 @@ decode_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ 
           nparts = (w.start + w.gb - 1) / chunk - c_first + 1;
         }
         const size_t head0 = (size_t)w.b * p.H_q + w.h * G;
+        // (what per_slice is rounded up by adds idx / 2^20 < 1 / slice to the quotient)
+        const int slice = (G * D + csize - 1) / csize, per_slice = ((1 << 20) + slice - 1) / slice;
         if (!dead && tid < D) {
           PartRec<D, G> *rec = pool + (size_t)cta * 2 + (c_first == cta ? 1 : 0);
 #pragma unroll
@@ -601,9 +612,8 @@ decode_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ 
               out[(head0 + g) * D + tid] = __float2bfloat16_rn(Ls > 0.f ? o[g] / Ls : 0.f);
               if (lse && tid == 0) lse[head0 + g] = Ls > 0.f ? (m[g] + lg2f(Ls)) * kLn2 : -CUDART_INF_F;
             } else if (split) {   // to the CTA of the cluster that folds this output
-              // (slices of G * D / csize outputs, powers of two)
-              const int sshift = 31 - __clz(G * D) - cshift, idx = g * D + tid, to = idx >> sshift;
-              st_shared_cluster_f32(mapa_shared(inbox + (128 + ((crank - to) << sshift) + idx) * 4, to), o[g]);
+              const int idx = g * D + tid, to = (uint32_t)(idx * per_slice) >> 20;   // idx / slice
+              st_shared_cluster_f32(mapa_shared(inbox + (128 + (crank - to) * slice + idx) * 4, to), o[g]);
               if (tid < csize) {
                 st_shared_cluster_f32(mapa_shared(inbox + (crank * 16 + g) * 4, tid), m[g]);
                 st_shared_cluster_f32(mapa_shared(inbox + (crank * 16 + 8 + g) * 4, tid), Ls);
@@ -684,10 +694,10 @@ decode_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ 
   if (split && csize > 1 && warp < 4 && total_b > 0) {
     // ---- every CTA of the cluster folds its slice of the unit's outputs, in rank order
     const float *in = reinterpret_cast<const float *>(smem + SL::kInbox);
-    const int slice = (G * D) >> cshift, u = cta >> cshift, b = u / p.H_kv, h = u % p.H_kv;
+    const int slice = (G * D + csize - 1) / csize, u = cta / csize, b = u / p.H_kv, h = u % p.H_kv;
     if (len_of(b) > 0) {
-      for (int j = tid; j < slice; j += 128) {
-        const int idx = crank * slice + j, g = idx / D;
+      for (int j = tid, idx; j < slice && (idx = crank * slice + j) < G * D; j += 128) {
+        const int g = idx / D;
         float M = -CUDART_INF_F, Ls = 0.f, acc = 0.f;
 #pragma unroll
         for (int r = 0; r < 8; ++r)
@@ -763,18 +773,47 @@ static bool cached_maps(CUtensorMap *out, void *base, uint64_t rows, int D) {
   maps[at][i] = *out;
   return true;
 }
+
+// Clusters of k CTAs of a kernel with two CTAs per SM that are resident at once: twice those of one CTA per SM, which is
+// what is asked for (more than half of an SM's shared memory each).  A device's answer is kept.
+template <typename K>
+static int resident_clusters(K kernel, int k) {
+  static std::atomic<int> known[64][9];
+  int dev = 0;
+  cudaGetDevice(&dev);
+  std::atomic<int> &at = known[dev & 63][k];
+  int n = at.load(std::memory_order_relaxed);
+  if (n == 0) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)k);
+    cfg.blockDim = dim3(kDecThreads);
+    cfg.dynamicSmemBytes = kOneCtaSmem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)k;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) { (void)cudaGetLastError(); n = 0; }
+    n = 2 * n + 1;   // (odd: never 0)
+    at.store(n, std::memory_order_relaxed);
+  }
+  return n - 1;
+}
+
 template <int D, int G, bool E>
 static void launch_t(const keepkv_params &p, const keepkv_cache &c, const void *q, void *out, float *lse,
                      int update_scores, char *ws, const WsLayout &L, int32_t *status_dev, const void *k_new,
                      const void *v_new, LaunchCtx &ctx) {
   using SL = DecSmem<D>;
   constexpr size_t smem_bytes = (size_t)SL::template bytes<G>() + 1024;
+  static_assert(smem_bytes <= kOneCtaSmem, "attribute below");
   static_assert(sizeof(PartRec<D, G>) == (16 + G * D) * 4, "partial record layout");
   static bool attr_done_dev[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
   if (!attr_done_dev[dev & 63]) {
-    cudaFuncSetAttribute(decode_kernel<D, G, E>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+    cudaFuncSetAttribute(decode_kernel<D, G, E>, cudaFuncAttributeMaxDynamicSharedMemorySize, kOneCtaSmem);
     attr_done_dev[dev & 63] = true;
   }
   CUtensorMap mapK, mapV;
@@ -786,27 +825,23 @@ static void launch_t(const keepkv_params &p, const keepkv_cache &c, const void *
   // Two CTAs per SM.  One per SM, with the next launch's CTAs resident beside this one's, measured 10-15 % slower: three
   // slots of 32 KB on an SM do not cover the latency of a loaded memory system, six do.
   const int U = p.B * p.H_kv, slots = 2 * sm_count() < kDecMaxCtas ? 2 * sm_count() : kDecMaxCtas;
-  // One cluster of 8, 4, 2 or 1 CTAs per unit, the most that are resident at once and still get a tile each (8 units of
-  // 1656 entries: 6.3 us with 8 CTAs, 7.8 us with 4, 9.6 us with 18 that meet in global memory).
-  int cs = U <= slots ? 1 : 0;
-  for (int k = 8; k > 1 && cs == 1; k >>= 1)
-    if (U * k <= slots && p.N_cap / k >= kDecTile) cs = k;
+  // One cluster of 8 to 1 CTAs per unit, the most that are resident at once and still get a tile each (8 units of 1656
+  // entries: 6.3 us with 8 CTAs, 7.8 us with 4, 9.6 us with 18 that meet in global memory).  A cluster lives inside one
+  // GPC: 30 clusters of 8 are resident, not 37.
+  int cs = U <= 2 * slots ? 1 : 0;
+  for (int k = 8; k > 1 && cs == 1; --k)
+    if (U * k <= slots && p.N_cap / k >= kDecTile && U <= resident_clusters(decode_kernel<D, G, E>, k)) cs = k;
   // Few long units: clusters would leave most of the chip idle, so the list of groups is cut into equal ranges (16 units
   // of 32768: 51 us against 54 us; the gap widens with fewer units).
   if (5 * U * cs < 2 * slots && p.N_cap > 1024 * cs) cs = 0;
-  if (cs > 1) {
-    launch_pdl_cluster(decode_kernel<D, G, E>, dim3((unsigned)(U * cs)), dim3(kDecThreads), smem_bytes, ctx.stream, cs,
-      mapK, mapV, p, c, reinterpret_cast<const __nv_bfloat16 *>(q), reinterpret_cast<__nv_bfloat16 *>(out), lse,
-      update_scores, reinterpret_cast<int *>(ws + L.counters), reinterpret_cast<PartRec<D, G> *>(ws + L.part_pool),
-      status_dev, reinterpret_cast<const uint4 *>(k_new), reinterpret_cast<const uint4 *>(v_new), g_dbg_spin, g_dbg_withhold);
-    KEEPKV_CHECK_LAUNCH(ctx);
-    return;
-  }
-  const int grid = cs ? U : slots;
-  launch_pdl(decode_kernel<D, G, E>, dim3((unsigned)grid), dim3(kDecThreads), smem_bytes, ctx.stream,
-      mapK, mapV, p, c, reinterpret_cast<const __nv_bfloat16 *>(q), reinterpret_cast<__nv_bfloat16 *>(out), lse,
-      update_scores, reinterpret_cast<int *>(ws + L.counters), reinterpret_cast<PartRec<D, G> *>(ws + L.part_pool),
-      status_dev, reinterpret_cast<const uint4 *>(k_new), reinterpret_cast<const uint4 *>(v_new), g_dbg_spin, g_dbg_withhold);
+  const int grid = cs ? U * cs : slots, ranges = grid < slots ? grid : slots;
+  auto launch = [&](auto &&...args) {
+    if (cs > 1) launch_pdl_cluster(decode_kernel<D, G, E>, dim3((unsigned)grid), dim3(kDecThreads), smem_bytes, ctx.stream, cs, args...);
+    else launch_pdl(decode_kernel<D, G, E>, dim3((unsigned)grid), dim3(kDecThreads), smem_bytes, ctx.stream, args...);
+  };
+  launch(mapK, mapV, p, ranges, c, reinterpret_cast<const __nv_bfloat16 *>(q), reinterpret_cast<__nv_bfloat16 *>(out), lse,
+         update_scores, reinterpret_cast<int *>(ws + L.counters), reinterpret_cast<PartRec<D, G> *>(ws + L.part_pool),
+         status_dev, reinterpret_cast<const uint4 *>(k_new), reinterpret_cast<const uint4 *>(v_new), g_dbg_spin, g_dbg_withhold);
   KEEPKV_CHECK_LAUNCH(ctx);
 }
 

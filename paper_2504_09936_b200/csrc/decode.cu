@@ -37,6 +37,7 @@
 // Every wait is bounded.  One that runs out marks the CTA (s_abort): its warps go on through their barriers without
 // waiting and without arithmetic, copies and products in flight get a bounded time to end, KEEPKV_DEV_TIMEOUT is raised.
 #include <atomic>
+#include <climits>
 #include <mutex>
 
 #include "common.cuh"
@@ -825,12 +826,20 @@ static void launch_t(const keepkv_params &p, const keepkv_cache &c, const void *
   // Two CTAs per SM.  One per SM, with the next launch's CTAs resident beside this one's, measured 10-15 % slower: three
   // slots of 32 KB on an SM do not cover the latency of a loaded memory system, six do.
   const int U = p.B * p.H_kv, slots = 2 * sm_count() < kDecMaxCtas ? 2 * sm_count() : kDecMaxCtas;
-  // One cluster of 8 to 1 CTAs per unit, the most that are resident at once and still get a tile each (8 units of 1656
-  // entries: 6.3 us with 8 CTAs, 7.8 us with 4, 9.6 us with 18 that meet in global memory).  A cluster lives inside one
-  // GPC: 30 clusters of 8 are resident, not 37.
-  int cs = U <= 2 * slots ? 1 : 0;
-  for (int k = 8; k > 1 && cs == 1; --k)
-    if (U * k <= slots && p.N_cap / k >= kDecTile && U <= resident_clusters(decode_kernel<D, G, E>, k)) cs = k;
+  // One cluster of k CTAs per unit, 1 <= k <= 8, resident at once (a cluster lives inside one GPC: 30 clusters of 8 are, not
+  // 37), with at least a tile per CTA.  In a loop of launches a tile of a CTA's share costs about 1 us; where the next
+  // launch's CTAs do not fit beside this one's they start behind it, 2.5 us; a k that is no power of two costs half a
+  // microsecond.  The k of the least sum, the smaller one of equals.  (Lengths are not known here: the capacity stands for
+  // them.  96 units of 250 entries: 5.4 us with k = 1, 8.1 with 2; 32 of 1700: 10.1 with 4, 11.7 with 6; 64 of 1702: 17.1
+  // with 2, 16.0 with 4; 8 of 1655: 7.0 with 8, 8.2 with 4, 9.6 with 18 CTAs that meet in global memory.)
+  int cs = 0, least = INT_MAX;
+  for (int k = 1; k <= 8; ++k) {
+    const int fit = k == 1 ? slots : resident_clusters(decode_kernel<D, G, E>, k);
+    if (k > 1 && (U * k > slots || U > fit || p.N_cap / k < kDecTile)) continue;
+    const int cost = 2 * ((p.N_cap + k * kDecTile - 1) / (k * kDecTile)) + (2 * U > fit ? 5 : 0) + ((k & (k - 1)) ? 1 : 0);
+    if (cost < least) { least = cost; cs = k; }
+  }
+  if (U > 2 * slots) cs = 0;
   // Few long units: clusters would leave most of the chip idle, so the list of groups is cut into equal ranges (16 units
   // of 32768: 51 us against 54 us; the gap widens with fewer units).
   if (5 * U * cs < 2 * slots && p.N_cap > 1024 * cs) cs = 0;

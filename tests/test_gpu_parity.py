@@ -81,7 +81,7 @@ def test_decode_one_cluster_per_unit(B, H_kv, G, d, lens):
 @pytest.mark.parametrize("lens", [
     [1, 31, 32, 33, 127, 128, 129, 160, 255, 257, 384, 515],    # one cluster of four CTAs per unit
     [509, 510, 511, 512, 513, 514],
-    [63, 400, 511], [610, 1, 639], [767, 130, 700], [895, 64],  # clusters of 3, 5, 6 and 7
+    [63, 300, 383], [610, 1, 639], [767, 130, 700], [895, 64],  # clusters of 3, 5, 6 and 7
     [2500] + [1, 33, 128, 31, 160, 257] * 10,                   # one much longer: equal ranges over the list of 32-entry groups
     [1, 33, 128, 31, 160, 257] * 26,                            # more units than are resident: unequal, a CTA per unit
     [90] * 160,                                                 # and equal, ranges of whole units

@@ -96,6 +96,13 @@ struct PartRec {
   float acc[G * D];
 };
 
+// How the launch is divided.
+struct DecGrid {
+  uint32_t per_csize;      // clusters of c > 1 CTAs: x / c = (x * per_csize) >> 32 for x < 2^26 (rounded up: adds < x * 8 / 2^32)
+  int slice;               // outputs of a unit that a CTA of the cluster folds
+  uint32_t per_slice;      // i / slice = (i * per_slice) >> 20 for i < 1024
+};
+
 // Position of a role in its CTA's range.
 struct DecWalk {
   int b, h;        // sequence, kv head
@@ -113,7 +120,7 @@ struct DecWalk {
 template <int D, int G, bool kEarly>
 __global__ void __launch_bounds__(kDecThreads, 2)
 decode_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapV,
-              keepkv_params p, int ranges,
+              keepkv_params p, DecGrid gr,
               keepkv_cache c, const __nv_bfloat16 *__restrict__ q, __nv_bfloat16 *__restrict__ out,
               float *__restrict__ lse, int update_scores, int *counters, PartRec<D, G> *pool, int32_t *status_dev,
               const uint4 *__restrict__ k_new, const uint4 *__restrict__ v_new, int spin_limit, int withhold) {
@@ -127,6 +134,7 @@ decode_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ 
   __shared__ float s_wsum[4][8];                      // per-warp sums of a segment
   __shared__ int s_scan[8], s_tbmax[8];
   __shared__ int s_start[5];        // b, h, group, unit's list position, groups of this CTA's range
+  __shared__ int s_step[2];         // sequences and heads from a unit of this CTA to its next
   __shared__ uint32_t s_tmem;
   __shared__ volatile int s_abort;
   __shared__ int s_last, s_finisher;
@@ -194,26 +202,38 @@ decode_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ 
     gb_max = max(gb_max, s_tbmax[w]);
   }
   const int T = total_b * p.H_kv;   // (below 2^26: the rows of a cache are indexed by 32-bit TMA coordinates)
-  int chunk = max((T + ranges - 1) / ranges, kMinGroups);
   const bool even = gb_max * p.B == total_b;
   // The cuts through units cost an equal range 3 to 6 us -- tickets, two segments in a row -- about what a CTA takes for
   // kSlack groups.  So a cluster takes its whole unit, if the launch has one per unit, unless that leaves the CTAs of
   // the longest unit more than kSlack groups, or a quarter, above an equal range.  (56 units of 121-485 entries, d = 64:
-  // 13.1 -> 8.0 us; 64 of 425-1702, d = 128: 17.4 -> 14.6 us; 64 of 2000-8000, 63 groups against 39: equal.)  Where the
-  // launch has more units than are resident at once, the equal ranges are the worse only for short units of unequal
-  // length (384 of 175-700: 27.5 -> 22.6 us; 512 of 442: 27.6 -> 28.8 us; 400 of 375-1500: equal).
-  const bool split = grid == U * csize && (U <= ranges ? gb_max <= (chunk + max(kSlack, chunk / 4)) * csize : !even && gb_max <= kSlack);
-  // Equal ranges: when every unit has the same number of groups and a range holds more than one unit, the range is
-  // rounded up to whole units, if that costs at most an eighth, or a tile, more: no unit is then cut between two CTAs.
-  if (gb_max > 0 && even && chunk > gb_max) {
-    const int up = (chunk + gb_max - 1) / gb_max * gb_max;
-    if (up <= chunk + max(kDecTile / kGroup, chunk / 8)) chunk = up;
+  // 13.1 -> 8.0 us; 64 of 425-1702, d = 128: 17.4 -> 14.6 us; 64 of 2000-8000, 63 groups against 39: equal.)  With up to
+  // two units per CTA the same holds for short units of unequal length: CTA c takes units c and c + grid (384 of
+  // 175-700: 27.5 -> 22.6 us; 400 of 375-1500: equal).
+  bool split = grid == U * csize && gb_max <= kSlack * csize;
+  int chunk = 0;
+  if (!split) {
+    chunk = max((T + grid - 1) / grid, kMinGroups);
+    split = U <= grid ? grid == U * csize && gb_max <= (chunk + max(kSlack, chunk / 4)) * csize
+                      : U <= 2 * grid && !even && gb_max <= kSlack;
+    // Equal ranges: when every unit has the same number of groups and a range holds more than one unit, the range is
+    // rounded up to whole units, if that costs at most an eighth, or a tile, more: no unit is then cut between two CTAs.
+    if (gb_max > 0 && even && chunk > gb_max) {
+      const int up = (chunk + gb_max - 1) / gb_max * gb_max;
+      if (up <= chunk + max(kDecTile / kGroup, chunk / 8)) chunk = up;
+    }
   }
+  if (tid == 32) { s_step[0] = split ? grid / p.H_kv : 0; s_step[1] = split ? grid % p.H_kv : 1; }
   if (split) {
     if (tid == 0) {
-      const int u = cta / csize, b = u / p.H_kv, gb = groups_of(b);
-      const int lo = crank * gb / csize, hi = (crank + 1) * gb / csize;
-      s_start[0] = b; s_start[1] = u % p.H_kv; s_start[2] = lo; s_start[3] = 0; s_start[4] = hi - lo;
+      const int u = (int)cluster_id(), b = u / p.H_kv, gb = groups_of(b);
+      int lo = 0, hi = gb;
+      if (csize > 1) {
+        lo = (int)__umulhi((uint32_t)(crank * gb), gr.per_csize);
+        hi = crank + 1 == csize ? gb : (int)__umulhi((uint32_t)((crank + 1) * gb), gr.per_csize);
+      }
+      const int gb2 = u + grid < U ? groups_of((u + grid) / p.H_kv) : 0;
+      s_start[0] = b; s_start[1] = u % p.H_kv; s_start[2] = lo; s_start[3] = 0; s_start[4] = hi - lo + gb2;
+      if (gb == 0 && gb2 > 0) { s_start[0] = (u + grid) / p.H_kv; s_start[1] = (u + grid) % p.H_kv; }
     }
   } else {
     const int g0 = (int)min((long long)T, (long long)cta * chunk), g1 = min(T, g0 + chunk);
@@ -246,15 +266,14 @@ decode_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ 
       w.g = 0;
       w.first = true;
       w.start += w.gb;
-      if (++w.h == p.H_kv) {
-        w.h = 0;
-        do {
-          ++w.b;
-          w.len = len_of(w.b);
-          w.gb = (w.len + kGroup - 1) / kGroup;
-        } while (w.gb == 0);   // (sequences without entries have no groups)
-        w.fresh = fresh_of(w.b);
-      }
+      do {   // (sequences without entries have no groups)
+        w.b += s_step[0];
+        w.h += s_step[1];
+        if (w.h >= p.H_kv) { w.h -= p.H_kv; ++w.b; }
+        w.len = len_of(w.b);
+        w.gb = (w.len + kGroup - 1) / kGroup;
+      } while (w.gb == 0);
+      w.fresh = fresh_of(w.b);
     }
   };
   // row inside the current tile of the entry this call appends, -1 if the tile does not hold it
@@ -601,8 +620,6 @@ decode_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ 
           nparts = (w.start + w.gb - 1) / chunk - c_first + 1;
         }
         const size_t head0 = (size_t)w.b * p.H_q + w.h * G;
-        // (what per_slice is rounded up by adds idx / 2^20 < 1 / slice to the quotient)
-        const int slice = (G * D + csize - 1) / csize, per_slice = ((1 << 20) + slice - 1) / slice;
         if (!dead && tid < D) {
           PartRec<D, G> *rec = pool + (size_t)cta * 2 + (c_first == cta ? 1 : 0);
 #pragma unroll
@@ -613,8 +630,8 @@ decode_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ 
               out[(head0 + g) * D + tid] = __float2bfloat16_rn(Ls > 0.f ? o[g] / Ls : 0.f);
               if (lse && tid == 0) lse[head0 + g] = Ls > 0.f ? (m[g] + lg2f(Ls)) * kLn2 : -CUDART_INF_F;
             } else if (split) {   // to the CTA of the cluster that folds this output
-              const int idx = g * D + tid, to = (uint32_t)(idx * per_slice) >> 20;   // idx / slice
-              st_shared_cluster_f32(mapa_shared(inbox + (128 + (crank - to) * slice + idx) * 4, to), o[g]);
+              const int idx = g * D + tid, to = (int)((uint32_t)idx * gr.per_slice >> 20);   // idx / slice
+              st_shared_cluster_f32(mapa_shared(inbox + (128 + (crank - to) * gr.slice + idx) * 4, to), o[g]);
               if (tid < csize) {
                 st_shared_cluster_f32(mapa_shared(inbox + (crank * 16 + g) * 4, tid), m[g]);
                 st_shared_cluster_f32(mapa_shared(inbox + (crank * 16 + 8 + g) * 4, tid), Ls);
@@ -695,7 +712,7 @@ decode_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ 
   if (split && csize > 1 && warp < 4 && total_b > 0) {
     // ---- every CTA of the cluster folds its slice of the unit's outputs, in rank order
     const float *in = reinterpret_cast<const float *>(smem + SL::kInbox);
-    const int slice = (G * D + csize - 1) / csize, u = cta / csize, b = u / p.H_kv, h = u % p.H_kv;
+    const int slice = gr.slice, u = (int)cluster_id(), b = u / p.H_kv, h = u % p.H_kv;
     if (len_of(b) > 0) {
       for (int j = tid, idx; j < slice && (idx = crank * slice + j) < G * D; j += 128) {
         const int g = idx / D;
@@ -778,10 +795,8 @@ static bool cached_maps(CUtensorMap *out, void *base, uint64_t rows, int D) {
 // Clusters of k CTAs of a kernel with two CTAs per SM that are resident at once: twice those of one CTA per SM, which is
 // what is asked for (more than half of an SM's shared memory each).  A device's answer is kept.
 template <typename K>
-static int resident_clusters(K kernel, int k) {
+static int resident_clusters(K kernel, int dev, int k) {
   static std::atomic<int> known[64][9];
-  int dev = 0;
-  cudaGetDevice(&dev);
   std::atomic<int> &at = known[dev & 63][k];
   int n = at.load(std::memory_order_relaxed);
   if (n == 0) {
@@ -833,22 +848,25 @@ static void launch_t(const keepkv_params &p, const keepkv_cache &c, const void *
   // them.  96 units of 250 entries: 5.4 us with k = 1, 8.1 with 2; 32 of 1700: 10.1 with 4, 11.7 with 6; 64 of 1702: 17.1
   // with 2, 16.0 with 4; 8 of 1655: 7.0 with 8, 8.2 with 4, 9.6 with 18 CTAs that meet in global memory.)
   int cs = 0, least = INT_MAX;
-  for (int k = 1; k <= 8; ++k) {
-    const int fit = k == 1 ? slots : resident_clusters(decode_kernel<D, G, E>, k);
+  for (int k = 1; k <= 8 && U <= slots; ++k) {
+    const int fit = k == 1 ? slots : resident_clusters(decode_kernel<D, G, E>, dev, k);
     if (k > 1 && (U * k > slots || U > fit || p.N_cap / k < kDecTile)) continue;
     const int cost = 2 * ((p.N_cap + k * kDecTile - 1) / (k * kDecTile)) + (2 * U > fit ? 5 : 0) + ((k & (k - 1)) ? 1 : 0);
     if (cost < least) { least = cost; cs = k; }
   }
-  if (U > 2 * slots) cs = 0;
   // Few long units: clusters would leave most of the chip idle, so the list of groups is cut into equal ranges (16 units
   // of 32768: 51 us against 54 us; the gap widens with fewer units).
   if (5 * U * cs < 2 * slots && p.N_cap > 1024 * cs) cs = 0;
-  const int grid = cs ? U * cs : slots, ranges = grid < slots ? grid : slots;
+  const int grid = cs ? U * cs : slots, csize = cs ? cs : 1;
+  DecGrid gr;
+  gr.per_csize = csize > 1 ? (uint32_t)((0x100000000ull + csize - 1) / csize) : 0;
+  gr.slice = (G * D + csize - 1) / csize;
+  gr.per_slice = (uint32_t)(((1 << 20) + gr.slice - 1) / gr.slice);
   auto launch = [&](auto &&...args) {
     if (cs > 1) launch_pdl_cluster(decode_kernel<D, G, E>, dim3((unsigned)grid), dim3(kDecThreads), smem_bytes, ctx.stream, cs, args...);
     else launch_pdl(decode_kernel<D, G, E>, dim3((unsigned)grid), dim3(kDecThreads), smem_bytes, ctx.stream, args...);
   };
-  launch(mapK, mapV, p, ranges, c, reinterpret_cast<const __nv_bfloat16 *>(q), reinterpret_cast<__nv_bfloat16 *>(out), lse,
+  launch(mapK, mapV, p, gr, c, reinterpret_cast<const __nv_bfloat16 *>(q), reinterpret_cast<__nv_bfloat16 *>(out), lse,
          update_scores, reinterpret_cast<int *>(ws + L.counters), reinterpret_cast<PartRec<D, G> *>(ws + L.part_pool),
          status_dev, reinterpret_cast<const uint4 *>(k_new), reinterpret_cast<const uint4 *>(v_new), g_dbg_spin, g_dbg_withhold);
   KEEPKV_CHECK_LAUNCH(ctx);

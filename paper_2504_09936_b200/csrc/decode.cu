@@ -135,6 +135,7 @@ decode_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ 
   __shared__ int s_scan[8], s_tbmax[8];
   __shared__ int s_start[5];        // b, h, group, unit's list position, groups of this CTA's range
   __shared__ int s_step[2];         // sequences and heads from a unit of this CTA to its next
+  __shared__ int s_slice;           // gr.slice
   __shared__ uint32_t s_tmem;
   __shared__ volatile int s_abort;
   __shared__ int s_last, s_finisher;
@@ -159,6 +160,7 @@ decode_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ 
   }
   if (tid == 32) { prefetch_tensormap(&mapK); prefetch_tensormap(&mapV); }
   const int csize = (int)cluster_nctarank(), crank = (int)cluster_ctarank();   // (1 to 8)
+  const int cluster = (int)cluster_id();
   if (csize > 1) cluster_arrive();   // waited for below: nobody writes to a CTA that has not started
   if (!kEarly) {
     pdl_wait();      // everything above ran while the previous kernel of the stream was finishing
@@ -222,10 +224,10 @@ decode_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ 
       if (up <= chunk + max(kDecTile / kGroup, chunk / 8)) chunk = up;
     }
   }
-  if (tid == 32) { s_step[0] = split ? grid / p.H_kv : 0; s_step[1] = split ? grid % p.H_kv : 1; }
+  if (tid == 32) { s_step[0] = split ? grid / p.H_kv : 0; s_step[1] = split ? grid % p.H_kv : 1; s_slice = gr.slice; }
   if (split) {
     if (tid == 0) {
-      const int u = (int)cluster_id(), b = u / p.H_kv, gb = groups_of(b);
+      const int u = cluster, b = u / p.H_kv, gb = groups_of(b);
       int lo = 0, hi = gb;
       if (csize > 1) {
         lo = (int)__umulhi((uint32_t)(crank * gb), gr.per_csize);
@@ -631,7 +633,7 @@ decode_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ 
               if (lse && tid == 0) lse[head0 + g] = Ls > 0.f ? (m[g] + lg2f(Ls)) * kLn2 : -CUDART_INF_F;
             } else if (split) {   // to the CTA of the cluster that folds this output
               const int idx = g * D + tid, to = (int)((uint32_t)idx * gr.per_slice >> 20);   // idx / slice
-              st_shared_cluster_f32(mapa_shared(inbox + (128 + (crank - to) * gr.slice + idx) * 4, to), o[g]);
+              st_shared_cluster_f32(mapa_shared(inbox + (128 + (crank - to) * s_slice + idx) * 4, to), o[g]);
               if (tid < csize) {
                 st_shared_cluster_f32(mapa_shared(inbox + (crank * 16 + g) * 4, tid), m[g]);
                 st_shared_cluster_f32(mapa_shared(inbox + (crank * 16 + 8 + g) * 4, tid), Ls);
@@ -712,9 +714,11 @@ decode_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ 
   if (split && csize > 1 && warp < 4 && total_b > 0) {
     // ---- every CTA of the cluster folds its slice of the unit's outputs, in rank order
     const float *in = reinterpret_cast<const float *>(smem + SL::kInbox);
-    const int slice = gr.slice, u = (int)cluster_id(), b = u / p.H_kv, h = u % p.H_kv;
+    const int slice = s_slice, b = s_start[0], h = s_start[1];
     if (len_of(b) > 0) {
-      for (int j = tid, idx; j < slice && (idx = crank * slice + j) < G * D; j += 128) {
+      const int mine_n = min(slice, G * D - crank * slice);
+      for (int j = tid; j < mine_n; j += 128) {
+        const int idx = crank * slice + j;
         const int g = idx / D;
         float M = -CUDART_INF_F, Ls = 0.f, acc = 0.f;
 #pragma unroll

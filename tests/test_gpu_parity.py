@@ -719,6 +719,14 @@ def test_prefill_scores_windowed_initialisation(G, d, W, alpha):
         check_close(after.lscore[u, :n], ref, f"prefill scores u={u}", ulps=None, max_abs=1e-3, mean_rel=1e-4)
 
 
+@pytest.mark.parametrize("G,d", [(1, 128), (2, 64), (4, 128), (8, 64), (8, 128)])
+@pytest.mark.parametrize("W", [8, 9, 16, 17, 32])
+def test_prefill_scores_window_columns(G, d, W):
+    """Windows at the edges of the 8, 16 and 32 columns a head takes: one to eight accumulators of the tensor product, one
+    or two per tile.  Checks and bounds of the test above."""
+    test_prefill_scores_windowed_initialisation(G, d, W, 0.9)
+
+
 def _copy_params(p, **kw):
     args = dict(B=p.B, H_q=p.H_q, H_kv=p.H_kv, d=p.d, N_cap=p.N_cap, period=p.period, n_sink=p.n_sink,
                 n_recent=p.n_recent, sm_scale=p.sm_scale, ema_alpha=p.ema_alpha, merge_threshold=p.merge_threshold,

@@ -62,9 +62,18 @@ void launch_append(const keepkv_params &p, const keepkv_cache &c, const void *k_
                    int32_t *status_dev, LaunchCtx &ctx);
 void launch_fresh_state(const keepkv_params &p, const keepkv_cache &c, LaunchCtx &ctx);
 // k_new / v_new: the step's token to append inside the same launch (keepkv_decode_step), or null
+// What a launch moves between page-locked host memory and the device, in 16-byte units: a layer's queries, keys and values
+// in, a layer's results out.
+struct HostMoves {
+  const uint4 *q_src, *k_src, *v_src, *out_src;
+  uint4 *q_dst, *k_dst, *v_dst, *out_dst;
+  int n_q, n_kv, n_out;   // n_kv: of the keys, and again of the values
+  __host__ __device__ int n_in() const { return n_q + 2 * n_kv; }
+};
 void launch_decode(const keepkv_params &p, const keepkv_cache &c, const void *q, void *out, float *lse,
                    int update_scores, char *ws, const WsLayout &L, int32_t *status_dev, LaunchCtx &ctx,
-                   const void *k_new = nullptr, const void *v_new = nullptr);
+                   const void *k_new = nullptr, const void *v_new = nullptr, const HostMoves &moves = HostMoves{});
+void launch_host_moves(const HostMoves &moves, LaunchCtx &ctx);
 void launch_compress(const keepkv_params &p, const keepkv_cache &src, const keepkv_cache &dst,
                      const int32_t *budget_dev, int32_t budget_scalar, const int32_t *n_recent_dev, int32_t *ret_idx,
                      int32_t *target, keepkv_stats *stats, char *ws, const WsLayout &L, int32_t *status_dev,

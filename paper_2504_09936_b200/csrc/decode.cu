@@ -96,6 +96,29 @@ struct PartRec {
   float acc[G * D];
 };
 
+// The i-th 16 bytes of a layer's inputs.  (Reads bypass L1: the host writes between launches.)
+__device__ __forceinline__ const uint4 *host_in_src(const HostMoves &m, int i) {
+  return i < m.n_q ? m.q_src + i : i < m.n_q + m.n_kv ? m.k_src + (i - m.n_q) : m.v_src + (i - m.n_q - m.n_kv);
+}
+__device__ __forceinline__ uint4 *host_in_dst(const HostMoves &m, int i) {
+  return i < m.n_q ? m.q_dst + i : i < m.n_q + m.n_kv ? m.k_dst + (i - m.n_q) : m.v_dst + (i - m.n_q - m.n_kv);
+}
+__device__ __forceinline__ uint4 load_host(const uint4 *p) { return __ldcv(p); }
+
+__global__ void __launch_bounds__(256) host_moves_kernel(const HostMoves m) {
+  pdl_wait();
+  pdl_trigger();
+  const int i0 = blockIdx.x * 256 + threadIdx.x, step = gridDim.x * 256;
+  for (int i = i0; i < m.n_in(); i += step) *host_in_dst(m, i) = load_host(host_in_src(m, i));
+  for (int i = i0; i < m.n_out; i += step) m.out_dst[i] = __ldcg(m.out_src + i);
+}
+
+void launch_host_moves(const HostMoves &m, LaunchCtx &ctx) {
+  const int n = m.n_in() + m.n_out, blocks = (n + 255) / 256;
+  launch_pdl(host_moves_kernel, dim3((unsigned)(blocks < sm_count() ? blocks : sm_count())), dim3(256), 0, ctx.stream, m);
+  KEEPKV_CHECK_LAUNCH(ctx);
+}
+
 // How the launch is divided.
 struct DecGrid {
   uint32_t per_csize;      // clusters of c > 1 CTAs: x / c = (x * per_csize) >> 32 for x < 2^26 (rounded up: adds < x * 8 / 2^32)
@@ -123,7 +146,8 @@ decode_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ 
               keepkv_params p, DecGrid gr,
               keepkv_cache c, const __nv_bfloat16 *__restrict__ q, __nv_bfloat16 *__restrict__ out,
               float *__restrict__ lse, int update_scores, int *counters, PartRec<D, G> *pool, int32_t *status_dev,
-              const uint4 *__restrict__ k_new, const uint4 *__restrict__ v_new, int spin_limit, int withhold) {
+              const uint4 *__restrict__ k_new, const uint4 *__restrict__ v_new, int spin_limit, int withhold,
+              const HostMoves moves) {
   using SL = DecSmem<D>;
   constexpr int S = SL::kSlots;
   constexpr int NO = D == 128 ? 16 : 32;   // columns of the second product
@@ -391,6 +415,18 @@ decode_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ 
       }
       __syncwarp();
     }
+    // Moves of a loop over layers whose inputs and results live on the host: the next layer's inputs come in, the previous
+    // one's results go out.  This warp has time: its first product waits for a tile, its logits and its weights.  The
+    // first load of a lane is stored when the tiles are done, a trip over PCIe later.
+    const int mv0 = cta * 32 + lane, mv_step = grid * 32, n_in = vals ? moves.n_in() : 0;
+    uint4 mv = make_uint4(0, 0, 0, 0);
+    if (vals) {
+      if (mv0 < n_in) mv = load_host(host_in_src(moves, mv0));
+      for (int i = mv0; i < moves.n_out; i += mv_step) moves.out_dst[i] = __ldcg(moves.out_src + i);
+#pragma unroll 4
+      for (int i = mv0 + mv_step; i < n_in; i += mv_step) *host_in_dst(moves, i) = load_host(host_in_src(moves, i));
+      __syncwarp();
+    }
     auto swz = [](int row, int chunk) { return (chunk >> 3) * SL::kSubBytes + row * 128 + (((chunk & 7) ^ (row & 7)) << 4); };
     bool ok = true;
     for (int t = 0, seg = -1; w.left > 0; ++t) {
@@ -463,6 +499,7 @@ decode_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ 
       __syncwarp();
       advance(w, n);
     }
+    if (mv0 < n_in) *host_in_dst(moves, mv0) = mv;
     if (!ok) {   // products in flight retire (bounded) before tensor memory is given back
       s_abort = 1;
       if (elect_one()) umma_commit(bar_drain + 8 * (warp & 1));
@@ -824,7 +861,7 @@ static int resident_clusters(K kernel, int dev, int k) {
 template <int D, int G, bool E>
 static void launch_t(const keepkv_params &p, const keepkv_cache &c, const void *q, void *out, float *lse,
                      int update_scores, char *ws, const WsLayout &L, int32_t *status_dev, const void *k_new,
-                     const void *v_new, LaunchCtx &ctx) {
+                     const void *v_new, const HostMoves &moves, LaunchCtx &ctx) {
   using SL = DecSmem<D>;
   constexpr size_t smem_bytes = (size_t)SL::template bytes<G>() + 1024;
   static_assert(smem_bytes <= kOneCtaSmem, "attribute below");
@@ -872,19 +909,19 @@ static void launch_t(const keepkv_params &p, const keepkv_cache &c, const void *
   };
   launch(mapK, mapV, p, gr, c, reinterpret_cast<const __nv_bfloat16 *>(q), reinterpret_cast<__nv_bfloat16 *>(out), lse,
          update_scores, reinterpret_cast<int *>(ws + L.counters), reinterpret_cast<PartRec<D, G> *>(ws + L.part_pool),
-         status_dev, reinterpret_cast<const uint4 *>(k_new), reinterpret_cast<const uint4 *>(v_new), g_dbg_spin, g_dbg_withhold);
+         status_dev, reinterpret_cast<const uint4 *>(k_new), reinterpret_cast<const uint4 *>(v_new), g_dbg_spin, g_dbg_withhold, moves);
   KEEPKV_CHECK_LAUNCH(ctx);
 }
 
 void launch_decode(const keepkv_params &p, const keepkv_cache &c, const void *q, void *out, float *lse,
                    int update_scores, char *ws, const WsLayout &L, int32_t *status_dev, LaunchCtx &ctx, const void *k_new,
-                   const void *v_new) {
+                   const void *v_new, const HostMoves &moves) {
   const int G = p.H_q / p.H_kv;
   const bool early = (p.flags & KEEPKV_FLAG_CACHE_IDLE) != 0;
 #define KEEPKV_DISPATCH(DD, GG) \
   if (p.d == DD && G == GG) \
-    return early ? launch_t<DD, GG, true>(p, c, q, out, lse, update_scores, ws, L, status_dev, k_new, v_new, ctx) \
-                 : launch_t<DD, GG, false>(p, c, q, out, lse, update_scores, ws, L, status_dev, k_new, v_new, ctx);
+    return early ? launch_t<DD, GG, true>(p, c, q, out, lse, update_scores, ws, L, status_dev, k_new, v_new, moves, ctx) \
+                 : launch_t<DD, GG, false>(p, c, q, out, lse, update_scores, ws, L, status_dev, k_new, v_new, moves, ctx);
   KEEPKV_DISPATCH(128, 1) KEEPKV_DISPATCH(128, 2) KEEPKV_DISPATCH(128, 4) KEEPKV_DISPATCH(128, 8)
   KEEPKV_DISPATCH(64, 1) KEEPKV_DISPATCH(64, 2) KEEPKV_DISPATCH(64, 4) KEEPKV_DISPATCH(64, 8)
 #undef KEEPKV_DISPATCH

@@ -569,6 +569,36 @@ def test_decode_step_host_layers_matches_per_layer_calls(packed):
     assert int(st.item()) == 0
 
 
+@pytest.mark.parametrize("B,H_kv,G,d,layers", [
+    (33, 8, 8, 128, 3),   # five 16-byte pieces of a layer's inputs per lane of the warps that move them
+    (1, 1, 1, 64, 2),     # fewer pieces than lanes
+    (5, 2, 2, 64, 1),     # one layer: no launch moves another layer's data
+])
+def test_decode_step_host_layers_pinned_and_pageable_agree(B, H_kv, G, d, layers):
+    """Page-locked arrays are moved by the layers' own launches, others by copies: same results, same caches, same staging
+    buffers, bit for bit, in two steps."""
+    p = kb.make_params(B=B, H_q=H_kv * G, H_kv=H_kv, d=d, N_cap=128)
+    lens = [1 + (37 * b) % 100 for b in range(B)]
+    results = []
+    for pin in (True, False):
+        caches = [random_cache(p, lens, seed=50 + l) for l in range(layers)]
+        rng = np.random.default_rng(9)
+        mk = lambda *s: torch.from_numpy(rng.standard_normal(s).astype(np.float32)).bfloat16()
+        ws, st = kb.new_workspace(p), kb.new_status()
+        for _ in range(2):
+            h = [mk(layers, B, p.H_q, d), mk(layers, B, H_kv, d), mk(layers, B, H_kv, d), torch.zeros(layers, B, p.H_q, d, dtype=torch.bfloat16)]
+            if pin:
+                h = [t.pin_memory() for t in h]
+            dev = [torch.zeros_like(t, device="cuda") for t in h]
+            kb.keepkv_decode_step_host_layers(p, caches, *h, *dev, True, ws, st)
+            torch.cuda.synchronize()
+            assert int(st.item()) == 0
+            assert torch.equal(dev[3].cpu().view(torch.int16), h[3].view(torch.int16))
+        results.append([t.cpu() for t in h + dev] + [getattr(c, f).cpu() for c in caches for f in ("K", "V", "votes", "lscore", "seq_len")])
+    for x, y in zip(*results):
+        assert torch.equal(x.contiguous().view(torch.uint8), y.contiguous().view(torch.uint8))
+
+
 @pytest.mark.parametrize("B,H_kv,G,d,n_cap,base_len,graph", [
     (8, 8, 4, 128, 2048, 1700, True),     # 64 units: one cluster of four per unit, the launches back to back in a graph
     (6, 4, 4, 128, 256, 120, False),      # 24 units: clusters of eight, lengths that cross a tile edge

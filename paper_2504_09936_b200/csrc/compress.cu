@@ -612,11 +612,48 @@ static void launch_compress_t(const keepkv_params &p, const keepkv_cache &src, c
 //   compact     -> kept rows to dst
 //   group       -> keys sorted into groups, few groups merged at once
 //   merge       -> Eq. A.3 for units with many groups
+
+// Calls f(i, |k_i|^2) in one lane for every row i < len of a unit's keys (rows: the first one) that want(i) holds for, with
+// 0 for the others.  grid (x, U), 256 threads; sixteen lanes per row, eight rows of a warp in flight: with two, 288 CTAs took
+// 33 us for 32 units of 6007 rows, a trip to memory per sweep.
+constexpr int kNormRows = 64;   // rows of a CTA and sweep
+template <int D, typename Want, typename F>
+__device__ __forceinline__ void each_row_norm(const uint4 *rows, int len, Want want, F f) {
+  constexpr int CH = D / 8;
+  const int lane = threadIdx.x & 31, ch = lane & 15, sub = lane >> 4, warp = threadIdx.x >> 5;
+  for (int r0 = blockIdx.x * kNormRows; r0 < len; r0 += gridDim.x * kNormRows) {
+    uint4 kv[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int i = r0 + warp * 8 + r * 2 + sub;
+      kv[r] = make_uint4(0, 0, 0, 0);
+      if (i < len && ch < CH && want(i)) kv[r] = rows[(size_t)i * CH + ch];
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int i = r0 + warp * 8 + r * 2 + sub;
+      float ss = 0.f;
+      const uint32_t w[4] = {kv[r].x, kv[r].y, kv[r].z, kv[r].w};
+#pragma unroll
+      for (int q = 0; q < 4; ++q) { const float a = bf16_lo(w[q]), b = bf16_hi(w[q]); ss = fmaf(a, a, ss); ss = fmaf(b, b, ss); }
+      ss += __shfl_xor_sync(0xffffffffu, ss, 1);
+      ss += __shfl_xor_sync(0xffffffffu, ss, 2);
+      ss += __shfl_xor_sync(0xffffffffu, ss, 4);
+      ss += __shfl_xor_sync(0xffffffffu, ss, 8);
+      if (i < len && ch == 0) f(i, ss);
+    }
+  }
+}
+// CTAs per unit: what is resident (eight per SM), as far as there are rows.
+static int norm_grid(const keepkv_params &p) {
+  const int most = (p.N_cap + kNormRows - 1) / kNormRows, n = 8 * sm_count() / (p.B * p.H_kv);
+  return n < 1 ? 1 : n < most ? n : most;
+}
+
 template <int D>
 __global__ void __launch_bounds__(256)
 mf_prepare_kernel(keepkv_params p, keepkv_cache src, int32_t *ev_idx, UnitInfo *unit_info, float *__restrict__ inv_norm,
                   uint4 *__restrict__ norm_ext) {
-  constexpr int CH = D / 8;
   pdl_wait();
   pdl_trigger();
   const int u = blockIdx.y, b = u / p.H_kv;
@@ -626,22 +663,11 @@ mf_prepare_kernel(keepkv_params p, keepkv_cache src, int32_t *ev_idx, UnitInfo *
     UnitInfo ui{len, len, len, 0, 0, 0, 0, 0};
     unit_info[u] = ui;
   }
-  const uint4 *sK = reinterpret_cast<const uint4 *>(src.K);
-  const int lane = threadIdx.x & 31, ch = lane & 15, sub = lane >> 4, warp = threadIdx.x >> 5;
-  for (int r0 = blockIdx.x * 16; r0 < len; r0 += gridDim.x * 16) {   // sixteen lanes per row, two rows per warp
-    const int i = r0 + warp * 2 + sub;
-    uint4 kv = make_uint4(0, 0, 0, 0);
-    if (i < len && ch < CH) kv = sK[(base + i) * CH + ch];
-    float ss = 0.f;
-    const uint32_t w[4] = {kv.x, kv.y, kv.z, kv.w};
-#pragma unroll
-    for (int q = 0; q < 4; ++q) { const float a = bf16_lo(w[q]), bb = bf16_hi(w[q]); ss = fmaf(a, a, ss); ss = fmaf(bb, bb, ss); }
-    ss += __shfl_xor_sync(0xffffffffu, ss, 1);
-    ss += __shfl_xor_sync(0xffffffffu, ss, 2);
-    ss += __shfl_xor_sync(0xffffffffu, ss, 4);
-    ss += __shfl_xor_sync(0xffffffffu, ss, 8);
-    if (i < len && ch == 0) { inv_norm[base + i] = rsqrtf(ss); norm_ext[base + i] = ext_col(sqrtf(ss)); ev_idx[base + i] = i; }
-  }
+  each_row_norm<D>(reinterpret_cast<const uint4 *>(src.K) + base * (D / 8), len, [](int) { return true; }, [&](int i, float ss) {
+    inv_norm[base + i] = rsqrtf(ss);
+    norm_ext[base + i] = ext_col(sqrtf(ss));
+    ev_idx[base + i] = i;
+  });
 }
 
 // One CTA per unit.  partner[e] (in `target`): the entry e would merge into, or -1.  Writes the kept list (ret_idx),
@@ -783,9 +809,7 @@ static void launch_compress_merge_first_t(const keepkv_params &p, const keepkv_c
     attr_done_dev[dev & 63] = true;
   }
   // ---- pass 1: similar entries merged with each other, cache -> scratch (every head keeps its own length for now)
-  int gx = 2 * sm_count() / U;
-  gx = gx < 1 ? 1 : (gx > 32 ? 32 : gx);
-  launch_pdl(mf_prepare_kernel<D>, dim3(gx, U), dim3(256), 0, ctx.stream, p, cache, ev_idx, ui, inv_norm, norm_ext);
+  launch_pdl(mf_prepare_kernel<D>, dim3(norm_grid(p), U), dim3(256), 0, ctx.stream, p, cache, ev_idx, ui, inv_norm, norm_ext);
   KEEPKV_CHECK_LAUNCH(ctx);
   // rows and columns are the same keys: the "retained" operand of the search is the prompt itself
   launch_nominate(p, cache, cache, ev_idx, ui, inv_norm, norm_ext, sched, nom_v, nom_si, L.nom_chunks, status_dev, ctx, 1);
@@ -849,33 +873,18 @@ template <int D>
 __global__ void __launch_bounds__(256)
 ip_prepare_kernel(keepkv_params p, keepkv_cache c, const int32_t *__restrict__ target, int32_t *ident, UnitInfo *unit_info,
                   float *__restrict__ inv_norm, uint4 *__restrict__ norm_ext) {
-  constexpr int CH = D / 8;
   pdl_wait();
   pdl_trigger();
   const int u = blockIdx.y;
   const int len = unit_info[u].len;
   const size_t base = (size_t)u * p.N_cap;
-  const uint4 *sK = reinterpret_cast<const uint4 *>(c.K);
-  const int lane = threadIdx.x & 31, ch = lane & 15, sub = lane >> 4, warp = threadIdx.x >> 5;
-  for (int r0 = blockIdx.x * 16; r0 < len; r0 += gridDim.x * 16) {   // sixteen lanes per row, two rows per warp
-    const int i = r0 + warp * 2 + sub;
-    const bool kept = i < len && target[base + i] == -2;
-    uint4 kv = make_uint4(0, 0, 0, 0);
-    if (kept && ch < CH) kv = sK[(base + i) * CH + ch];
-    float ss = 0.f;
-    const uint32_t w[4] = {kv.x, kv.y, kv.z, kv.w};
-#pragma unroll
-    for (int q = 0; q < 4; ++q) { const float a = bf16_lo(w[q]), bb = bf16_hi(w[q]); ss = fmaf(a, a, ss); ss = fmaf(bb, bb, ss); }
-    ss += __shfl_xor_sync(0xffffffffu, ss, 1);
-    ss += __shfl_xor_sync(0xffffffffu, ss, 2);
-    ss += __shfl_xor_sync(0xffffffffu, ss, 4);
-    ss += __shfl_xor_sync(0xffffffffu, ss, 8);
-    if (i < len && ch == 0) {
-      norm_ext[base + i] = ext_col(kept ? sqrtf(ss) : kExtNever);
-      inv_norm[base + i] = kept ? rsqrtf(ss) : __int_as_float(0x7fffffff);   // a row that is not retained is no column
-      ident[base + i] = i;   // the slot of a target is its row
-    }
-  }
+  auto kept = [&](int i) { return target[base + i] == -2; };
+  each_row_norm<D>(reinterpret_cast<const uint4 *>(c.K) + base * (D / 8), len, kept, [&](int i, float ss) {
+    const bool k = kept(i);
+    norm_ext[base + i] = ext_col(k ? sqrtf(ss) : kExtNever);
+    inv_norm[base + i] = k ? rsqrtf(ss) : __int_as_float(0x7fffffff);   // a row that is not retained is no column
+    ident[base + i] = i;   // the slot of a target is its row
+  });
 }
 
 // The search's column count is the unit's length (all rows lie in the operand); the rest of the record stays.
@@ -964,9 +973,7 @@ static void launch_compress_inplace_t(const keepkv_params &p, const keepkv_cache
              budget_dev, budget_scalar, n_recent_dev, kept, target, ev_idx, ui, stats, (const float *)nullptr,
              (const int32_t *)nullptr, pos, (const int32_t *)pos_len, (const int32_t *)n_seen, status_dev);
   KEEPKV_CHECK_LAUNCH(ctx);
-  int gx = 2 * sm_count() / U;
-  gx = gx < 1 ? 1 : (gx > 32 ? 32 : gx);
-  launch_pdl(ip_prepare_kernel<D>, dim3(gx, U), dim3(256), 0, ctx.stream, p, c, (const int32_t *)target, ident, ui, inv_norm, norm_ext);
+  launch_pdl(ip_prepare_kernel<D>, dim3(norm_grid(p), U), dim3(256), 0, ctx.stream, p, c, (const int32_t *)target, ident, ui, inv_norm, norm_ext);
   KEEPKV_CHECK_LAUNCH(ctx);
   const bool merges = !(isinf(p.merge_threshold) && p.merge_threshold > 0.f);
   if (merges) {

@@ -1,6 +1,6 @@
-"""ctypes binding over libkeepkv.so: same names as the C ABI (``include/keepkv.h``), argument
-marshalling only.  torch supplies device memory and streams; every step of the path runs in the
-library's CUDA kernels.  There is no fallback: if the compiled library is missing, loading raises.
+"""Binding over libkeepkv.so: same names as the C ABI (``include/keepkv.h``), argument marshalling only -- by ctypes, the
+calls made for every token by an extension module.  torch supplies device memory and streams; every step of the path runs
+in the library's CUDA kernels.  There is no fallback: if the compiled library is missing, loading raises.
 """
 from __future__ import annotations
 
@@ -43,6 +43,7 @@ STATS_FIELDS = ("n_retained", "n_evicted", "n_merged", "n_below_T", "n_guard_gro
                 "reserved")
 
 _lib = None
+_native = None   # the extension module with the calls made for every token (csrc/native.c)
 _raw_stream, _current_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
 
 
@@ -155,22 +156,33 @@ def new_status(device="cuda") -> torch.Tensor:
     return torch.zeros(1, dtype=torch.int32, device=device)
 
 
+def _calls():
+    """The extension module (loaded with the library)."""
+    global _native
+    lib()
+    from . import _native as module
+    _native = module
+    return module
+
+
 def keepkv_append(p, cache: Cache, k_new, v_new, status, stream=None):
-    _check(lib().keepkv_append(C.byref(p), cache.ref(), k_new.data_ptr(), v_new.data_ptr(), status.data_ptr(),
-                               _stream(stream)), "keepkv_append")
+    rc = (_native or _calls()).append(p, cache.c(), k_new, v_new, status, _stream(stream))
+    if rc:
+        _check(rc, "keepkv_append")
 
 
 def keepkv_decode_attention(p, cache: Cache, q, out, lse, update_scores: bool, ws, status, stream=None):
-    _check(lib().keepkv_decode_attention(C.byref(p), cache.ref(), q.data_ptr(), out.data_ptr(), _ptr(lse),
-                                         int(update_scores), ws.data_ptr(), ws.numel(), status.data_ptr(),
-                                         _stream(stream)), "keepkv_decode_attention")
+    rc = (_native or _calls()).decode_attention(p, cache.c(), q, out, lse, update_scores, ws, status, _stream(stream))
+    if rc:
+        _check(rc, "keepkv_decode_attention")
 
 
 def keepkv_decode_step(p, cache: Cache, q, k_new, v_new, out, lse, update_scores: bool, ws, status, stream=None):
     """keepkv_append followed by keepkv_decode_attention in one launch."""
-    _check(lib().keepkv_decode_step(C.byref(p), cache.ref(), q.data_ptr(), k_new.data_ptr(), v_new.data_ptr(),
-                                    out.data_ptr(), _ptr(lse), int(update_scores), ws.data_ptr(), ws.numel(),
-                                    status.data_ptr(), _stream(stream)), "keepkv_decode_step")
+    rc = (_native or _calls()).decode_step(p, cache.c(), q, k_new, v_new, out, lse, update_scores, ws, status,
+                                           _stream(stream))
+    if rc:
+        _check(rc, "keepkv_decode_step")
 
 
 def keepkv_decode_attention_static(p, cache: Cache, q, out, lse, update_scores: bool, status, stream=None):
@@ -260,12 +272,11 @@ def keepkv_decode_step_host(p, cache: Cache, q_host, k_new_host, v_new_host, out
 def keepkv_decode_step_host_layers(p, caches, q_host, k_new_host, v_new_host, out_host, q_dev, k_new_dev, v_new_dev,
                                    out_dev, update_scores: bool, ws, status, stream=None):
     """caches: list of Cache, one per layer; host / staging tensors carry the layers as their first axis."""
-    arr = (keepkv_cache * len(caches))(*[c.c() for c in caches])
-    _check(lib().keepkv_decode_step_host_layers(C.byref(p), arr, len(caches), q_host.data_ptr(), k_new_host.data_ptr(),
-                                                v_new_host.data_ptr(), out_host.data_ptr(), q_dev.data_ptr(),
-                                                k_new_dev.data_ptr(), v_new_dev.data_ptr(), out_dev.data_ptr(),
-                                                int(update_scores), ws.data_ptr(), ws.numel(), status.data_ptr(),
-                                                _stream(stream)), "keepkv_decode_step_host_layers")
+    rc = (_native or _calls()).decode_step_host_layers(
+        p, [c.c() for c in caches], q_host, k_new_host, v_new_host, out_host, q_dev, k_new_dev, v_new_dev, out_dev,
+        update_scores, ws, status, _stream(stream))
+    if rc:
+        _check(rc, "keepkv_decode_step_host_layers")
 
 
 def keepkv_debug_decode(spin_limit: int = 0, withhold_tile: int = -1):

@@ -1,14 +1,16 @@
-"""Compile libkeepkv.so (sm_100a only) in-tree with nvcc."""
+"""Compile libkeepkv.so (sm_100a only) in-tree with nvcc, and the extension module that calls it from Python."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_HERE)
 CSRC = os.path.join(_HERE, "csrc")
 LIB = os.path.join(_HERE, "libkeepkv.so")
+NATIVE = os.path.join(_HERE, "_native.so")
 SOURCES = ["api.cu", "append.cu", "decode.cu", "decode_static.cu", "compress.cu", "compress_steady.cu", "nominate.cu",
            "prefill.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC",
@@ -16,9 +18,9 @@ NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", 
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(NATIVE):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(NATIVE))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(_ROOT, "include", "keepkv.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 
@@ -46,6 +48,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if failed:
         raise RuntimeError("nvcc failed")
     subprocess.run([nvcc, "-shared", "-o", LIB, *objs, "-lcudart"], check=True)
+    subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I", os.path.join(_ROOT, "include"),
+                    "-I", sysconfig.get_paths()["include"], os.path.join(CSRC, "native.c"), "-o", NATIVE,
+                    "-L", _HERE, "-l:libkeepkv.so", "-Wl,-rpath,$ORIGIN"], check=True)
     return LIB
 
 

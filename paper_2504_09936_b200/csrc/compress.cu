@@ -51,6 +51,7 @@ select_kernel(keepkv_params p, keepkv_cache src, int32_t *dst_seq_len, const int
   const int nthr = min((int)blockDim.x, len > 4096 ? 1024 : (len > 1024 ? 512 : 128)), nw = nthr >> 5;
   if (tid >= nthr) return;
   const int lane = tid & 31, warp = tid >> 5;
+  uint32_t k_lo = 0xffffffffu, k_hi = 0u;   // the range of the candidates' keys
   if (pos) {
     // A cache that is not in token order (in-place compression): sinks and recent window are told by the token
     // position of a row, not by the row.  Rows from pos_len[b] on are the tokens appended since the last call, in
@@ -65,7 +66,10 @@ select_kernel(keepkv_params p, keepkv_cache src, int32_t *dst_seq_len, const int
       if (i >= first_fresh) { ps = n_seen[b] + (i - first_fresh); pos[base + i] = ps; }
       const bool fixed = all || ps < n_sink || ps >= n_total - n_recent;
       n_fixed += (!all && fixed) ? 1 : 0;
-      keys[i] = fixed ? 0u : kappa_key(src.votes[base + i], src.lscore[base + i]);
+      const uint32_t k = fixed ? 0u : kappa_key(src.votes[base + i], src.lscore[base + i]);
+      keys[i] = k;
+      k_lo = min(k_lo, k);
+      k_hi = max(k_hi, k);
     }
     int tot;
     block_excl_sum(n_fixed, warp_tot, tot, nw);
@@ -78,18 +82,17 @@ select_kernel(keepkv_params p, keepkv_cache src, int32_t *dst_seq_len, const int
 #pragma unroll 4
     for (int i = tid; i < len; i += nthr) {
       // the caller's scores where given, else kappa = ln p + lscore
-      keys[i] = select_key ? ordered_key(select_key[base + i]) : kappa_key(src.votes[base + i], src.lscore[base + i]);
+      const uint32_t k = select_key ? ordered_key(select_key[base + i]) : kappa_key(src.votes[base + i], src.lscore[base + i]);
+      keys[i] = k;
+      if (i >= lo && i < hi) { k_lo = min(k_lo, k); k_hi = max(k_hi, k); }
     }
   }
-  // the range of the candidates' keys (a thread reads back what it wrote)
-  uint32_t k_lo = 0xffffffffu, k_hi = 0u;
-  for (int i = tid; i < len; i += nthr)
-    if (i >= lo && i < hi) { k_lo = min(k_lo, keys[i]); k_hi = max(k_hi, keys[i]); }
   k_lo = __reduce_min_sync(0xffffffffu, k_lo);
   k_hi = __reduce_max_sync(0xffffffffu, k_hi);
   if (lane == 0) { warp_min[warp] = k_lo; warp_max[warp] = k_hi; }
   __syncthreads();
-  for (int w = 0; w < nw; ++w) { k_lo = min(k_lo, warp_min[w]); k_hi = max(k_hi, warp_max[w]); }
+  k_lo = __reduce_min_sync(0xffffffffu, lane < nw ? warp_min[lane] : 0xffffffffu);
+  k_hi = __reduce_max_sync(0xffffffffu, lane < nw ? warp_max[lane] : 0u);
 
   uint32_t kth = 0;    // the n_heavy-th largest key
   int n_tie = 0;       // how many entries equal to it are taken, lowest index first
@@ -116,16 +119,19 @@ select_kernel(keepkv_params p, keepkv_cache src, int32_t *dst_seq_len, const int
   }
   if (lane == 0) { warp_tot[warp] = n_k; warp_tie[warp] = n_t; }
   __syncthreads();
-  int slot = 0, tie_rank = 0, base_keep = 0;
-  {
-    int ties = 0;
-    for (int w = 0; w < nw; ++w) {
-      if (w == warp) { slot = base_keep; tie_rank = ties; }
-      base_keep += warp_tot[w];
-      if (rank_ties) base_keep += max(0, min(n_tie - ties, warp_tie[w]));
-      ties += warp_tie[w];
-    }
+  // a warp's counts per lane: ties before it, then what the warps before it keep
+  const int ties_w = lane < nw ? warp_tie[lane] : 0;
+  int ties_before = ties_w;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, ties_before, o);
+    if (lane >= o) ties_before += y;
   }
+  ties_before -= ties_w;
+  const int kept_w = (lane < nw ? warp_tot[lane] : 0) + (rank_ties ? max(0, min(n_tie - ties_before, ties_w)) : 0);
+  const int base_keep = __reduce_add_sync(0xffffffffu, kept_w);
+  int slot = __reduce_add_sync(0xffffffffu, lane < warp ? kept_w : 0);
+  int tie_rank = __shfl_sync(0xffffffffu, ties_before, warp);
   for (int i0 = e0; i0 < e1; i0 += 32) {
     const int i = i0 + lane;
     bool keep, tie;

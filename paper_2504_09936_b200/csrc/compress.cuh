@@ -12,6 +12,13 @@ constexpr float kRankEps = 1e-4f;   // tensor-core cosines closer than this are 
 // ------------------------------------------------------------------ block scans
 // The barrier of the threads that take part (the block, unless the kernel has warps with other work).
 struct BlockSync { __device__ __forceinline__ void operator()() const { __syncthreads(); } };
+// The sums of warp_tot over the warps before this one and over all nw <= 32, a warp's value per lane.  (A loop over 32 warps is
+// half a microsecond of shared-memory latency.)
+__device__ __forceinline__ int warps_before(const int *warp_tot, int &total, int nw) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, v = lane < nw ? warp_tot[lane] : 0;
+  total = __reduce_add_sync(0xffffffffu, v);
+  return __reduce_add_sync(0xffffffffu, lane < warp ? v : 0);
+}
 // Exclusive prefix count of `flag` over the first nw warps of the block in thread order (the other
 // warps have left the kernel); total returned through `total`.
 template <typename Sync = BlockSync>
@@ -22,14 +29,7 @@ __device__ __forceinline__ int block_excl_count(bool flag, int *warp_tot, int &t
   sync();  // warp_tot may still be read from the previous call
   if (lane == 0) warp_tot[warp] = __popc(bal);
   sync();
-  int off = 0, tot = 0;
-  for (int w = 0; w < nw; ++w) {
-    const int t = warp_tot[w];
-    if (w < warp) off += t;
-    tot += t;
-  }
-  total = tot;
-  return off + in_warp;
+  return warps_before(warp_tot, total, nw) + in_warp;
 }
 __device__ __forceinline__ int block_excl_count(bool flag, int *warp_tot, int &total) {
   return block_excl_count(flag, warp_tot, total, (int)(blockDim.x >> 5));
@@ -48,14 +48,7 @@ __device__ __forceinline__ int block_excl_sum(int v, int *warp_tot, int &total, 
   sync();
   if (lane == 31) warp_tot[warp] = x;
   sync();
-  int off = 0, tot = 0;
-  for (int w = 0; w < nw; ++w) {
-    const int t = warp_tot[w];
-    if (w < warp) off += t;
-    tot += t;
-  }
-  total = tot;
-  return off + x - v;
+  return warps_before(warp_tot, total, nw) + x - v;
 }
 
 // ------------------------------------------------------------------ selection key
@@ -87,6 +80,7 @@ __device__ __forceinline__ void range_select(const uint32_t *keys, int lo, int h
     const int shift = max(0, 21 - __clz(k_hi - k_lo));   // (bits of the span less the 11 of a bin number)
     for (int i = tid; i < kSelBins; i += nthr) hist[i] = 0;
     sync();
+#pragma unroll 4
     for (int i = lo + tid; i < hi; i += nthr) {
       const uint32_t k = keys[i];
       if (k >= k_lo && k <= k_hi) atomicAdd(&hist[(k - k_lo) >> shift], 1);

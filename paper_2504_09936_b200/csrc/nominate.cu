@@ -114,7 +114,6 @@ nominate_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, const
                 const float *__restrict__ inv_norm, const uint4 *__restrict__ norm_ext, int32_t *sched,
                 float4 *__restrict__ nom_v, int32_t *__restrict__ nom_si, int C_max, int32_t *status_dev, int self_mask) {
   using SL = NomSmem<D>;
-  constexpr uint32_t IDESC = umma_idesc_bf16(kNomM, kNomN);
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   // a_ready[2], a_empty[2], b_full[4], b_empty[4], t_full[2], t_empty[2], drain, x_full[4][2]
   __shared__ __align__(8) uint64_t bars[4 + 2 * kNomStages + 4 + 1 + 8];
@@ -241,6 +240,8 @@ nominate_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, const
       if (it.n_ev < 0) break;
       for (int t = it.t0; ok && t < it.t1; ++t, ++acc) {
         const int a = acc & 1;
+        // a unit's last tile is multiplied as far as it has columns, in sixteens
+        const uint32_t idesc = umma_idesc_bf16(kNomM, min(kNomN, (it.n_ret - t * kNomN + 15) & ~15));
         ok = __all_sync(0xffffffffu, !s_abort && mbar_wait(bar_t_empty + 8 * a, ((acc >> 1) & 1) ^ 1));
 #pragma unroll
         for (int sub = 0; sub < SL::kSub; ++sub, ++ring) {
@@ -254,12 +255,12 @@ nominate_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, const
             const uint32_t dt = tmem + a * kNomN;
 #pragma unroll
             for (int k = 0; k < 4; ++k)   // (descriptor addresses count 16-byte units)
-              umma_bf16(dt, ad + k * 2, bd + k * 2, IDESC, sub + k > 0 ? 1u : 0u);
+              umma_bf16(dt, ad + k * 2, bd + k * 2, idesc, sub + k > 0 ? 1u : 0u);
             if (sub == SL::kSub - 1) {
               const uint32_t zero = sbase + SL::kZero;
               if (kCut)
                 umma_bf16(dt, umma_desc_plain(sbase + SL::kAX + buf * (kNomM * 16), zero),
-                          umma_desc_plain(sbase + SL::kBX + acc % SL::kTiles * (kNomN * 16), zero), IDESC, 1u);
+                          umma_desc_plain(sbase + SL::kBX + acc % SL::kTiles * (kNomN * 16), zero), idesc, 1u);
               umma_commit(bar_t_full + 8 * a);
             }
             umma_commit(bar_b_empty + 8 * s);   // the stage may be refilled once these have read it

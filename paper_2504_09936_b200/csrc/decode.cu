@@ -232,20 +232,21 @@ decode_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ 
   // The cuts through units cost an equal range 3 to 6 us -- tickets, two segments in a row -- about what a CTA takes for
   // kSlack groups.  So a cluster takes its whole unit, if the launch has one per unit, unless that leaves the CTAs of
   // the longest unit more than kSlack groups, or a quarter, above an equal range.  (56 units of 121-485 entries, d = 64:
-  // 13.1 -> 8.0 us; 64 of 425-1702, d = 128: 17.4 -> 14.6 us; 64 of 2000-8000, 63 groups against 39: equal.)  With up to
-  // two units per CTA the same holds for short units of unequal length: CTA c takes units c and c + grid (384 of
-  // 175-700: 27.5 -> 22.6 us; 400 of 375-1500: equal).
+  // 13.1 -> 8.0 us; 64 of 425-1702, d = 128: 17.4 -> 14.6 us; 64 of 2000-8000, 63 groups against 39: equal.)  With more
+  // units than CTAs the same holds for short units of unequal length: CTA c takes units c, c + grid, ..., up to two of
+  // them, or up to eight very short ones (384 of 175-700: 27.5 -> 22.6 us; 400 of 375-1500: equal; 960 of 50-200, d = 64:
+  // 24.6 -> 17.2; 1920 of 25-100: 45.7 -> 27.5).
   bool split = grid == U * csize && gb_max <= kSlack * csize;
   int chunk = 0;
   if (!split) {
     chunk = max((T + grid - 1) / grid, kMinGroups);
     split = U <= grid ? grid == U * csize && gb_max <= (chunk + max(kSlack, chunk / 4)) * csize
-                      : U <= 2 * grid && !even && gb_max <= kSlack;
+                      : !even && (U <= 2 * grid ? gb_max <= kSlack : U <= 8 * grid && gb_max <= kSlack / 4);
     // Equal ranges: when every unit has the same number of groups and a range holds more than one unit, the range is
-    // rounded up to whole units, if that costs at most an eighth, or a tile, more: no unit is then cut between two CTAs.
+    // rounded up to whole units, if that costs at most an eighth, or two tiles, more: no unit is then cut between two CTAs.
     if (gb_max > 0 && even && chunk > gb_max) {
       const int up = (chunk + gb_max - 1) / gb_max * gb_max;
-      if (up <= chunk + max(kDecTile / kGroup, chunk / 8)) chunk = up;
+      if (up <= chunk + max(2 * kDecTile / kGroup, chunk / 8)) chunk = up;
     }
   }
   if (tid == 32) { s_step[0] = split ? grid / p.H_kv : 0; s_step[1] = split ? grid % p.H_kv : 1; s_slice = gr.slice; }
@@ -257,9 +258,12 @@ decode_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ 
         lo = (int)__umulhi((uint32_t)(crank * gb), gr.per_csize);
         hi = crank + 1 == csize ? gb : (int)__umulhi((uint32_t)((crank + 1) * gb), gr.per_csize);
       }
-      const int gb2 = u + grid < U ? groups_of((u + grid) / p.H_kv) : 0;
-      s_start[0] = b; s_start[1] = u % p.H_kv; s_start[2] = lo; s_start[3] = 0; s_start[4] = hi - lo + gb2;
-      if (gb == 0 && gb2 > 0) { s_start[0] = (u + grid) / p.H_kv; s_start[1] = (u + grid) % p.H_kv; }
+      int first = u, n = hi - lo;
+      for (int v = u + grid; v < U; v += grid) {   // further units of this CTA
+        if (n == 0) first = v;                     // (the first one that is not empty)
+        n += groups_of(v / p.H_kv);
+      }
+      s_start[0] = first / p.H_kv; s_start[1] = first % p.H_kv; s_start[2] = lo; s_start[3] = 0; s_start[4] = n;
     }
   } else {
     const int g0 = (int)min((long long)T, (long long)cta * chunk), g1 = min(T, g0 + chunk);

@@ -85,6 +85,7 @@ def test_decode_one_cluster_per_unit(B, H_kv, G, d, lens):
     [2500] + [1, 33, 128, 31, 160, 257] * 10,                   # one much longer: equal ranges over the list of 32-entry groups
     [1, 33, 128, 31, 160, 257] * 26,                            # more units than are resident: unequal, a CTA per unit
     [90] * 160,                                                 # and equal, ranges of whole units
+    [5, 90, 33, 120] * 85,                                      # three short units per CTA, every 296th
     [2900],                                                     # two long units: ranges of a unit that meet in memory
 ])
 def test_decode_group_and_tile_edges(G, d, lens):

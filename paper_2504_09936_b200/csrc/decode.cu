@@ -3,10 +3,10 @@
 //
 // Work.  Every unit's entries are cut into groups of 32; a CTA owns a contiguous range of groups and walks it in tiles
 // of up to 128 entries, a segment being the part of its range that lies in one unit.  Up to two units per SM, the grid is
-// one cluster of 8, 4, 2 or 1 CTAs per unit; if the units are about equally long -- every steady-state step -- the CTAs
-// of a cluster split their unit evenly and send their partial results to each other's shared memory: one cluster
-// barrier, then each folds its share of the outputs in rank order.  (Through global memory -- fence, ticket, the last to
-// arrive reads the others' partials -- the same meeting took 1.5 to 4 us behind the next launch's loads.)  Otherwise the
+// one cluster of 1 to 8 CTAs per unit, which split their unit evenly and send their partial results to each other's shared
+// memory: one cluster barrier, then each folds its share of the outputs in rank order.  (Through global memory -- fence,
+// ticket, the last to arrive reads the others' partials -- the same meeting took 1.5 to 4 us behind the next launch's
+// loads.)  More units than that are dealt out whole to two CTAs per SM where they are short or alike.  Otherwise the
 // list of all groups is cut into equal ranges, and a unit that lies in several of them is finished through global memory
 // by the last of their CTAs to arrive (one ticket per unit), in a fixed order, so results are bit-reproducible.
 //

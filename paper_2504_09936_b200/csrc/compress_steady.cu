@@ -14,16 +14,20 @@
 //      warps drain the accumulator of the previous tile with tcgen05.ld while the next product runs: a thread
 //      owns one evicted row and half of the columns and keeps the row's two best cosines with their slots, of those
 //      above the merge threshold (an entry whose best cosine does not exceed it is dropped whatever its best column was);
-//   3. leave their two best per row in the workspace; the last CTA of the unit to arrive folds them, settles
+//   3. are a cluster: every evicted row has one of them that gets its candidates from all through shared memory, folds them and settles
 //      arg-max and threshold (Algorithm 1, arg-max and threshold step) with the interface's exact fp32 chain wherever the tensor-core ranking is
-//      closer than kRankEps, sorts the entries to merge into groups and merges them (Eq. A.3; Algorithm 1, merge step).
+//      closer than kRankEps, and tells all of them; each sorts the entries to merge into the same groups and its warps merge their
+//      share of them (Eq. A.3; Algorithm 1, merge step).
 // Decisions, and therefore all outputs, are the same bits as the general pipeline's (compress.cu).
-// Bound: the chain selection (6 us) -> evicted keys and first tile (5 us) -> tiles (12 us) -> the last CTA's tail (10 us); the
+// Bound: the chain selection (6 us) -> evicted keys and first tile (5 us) -> tiles (12 us) -> decisions and merges (5 us); the
 // bytes of 64 units of 1766 entries, 112 MB, take 17 us at the copy rate.  Every warp copying, searching and selecting in
 // turn took 69 us a layer; values through the registers of two copying warps 85 us (they ended at 60-70 us, the search at
-// 24); values by bulk copies through shared memory 45 us.
+// 24); values by bulk copies through shared memory 45 us; with the candidates in global memory and all decisions and merges the
+// last CTA's, 29 groups on eight warps.  Shared out over the cluster: 40 us.
 // Every wait on the tensor core and on a bulk copy is bounded; one that runs out raises KEEPKV_DEV_TIMEOUT and the CTA goes
 // on without further products (its unit's result is then unspecified), frees its tensor memory and returns.
+#include <atomic>
+
 #include "compress.cuh"
 #include "ptx.cuh"
 
@@ -38,6 +42,8 @@ constexpr int kStRet = 16384;    // retained entries per unit
 constexpr int kStN = 64;         // retained slots per tile (columns of the product)
 constexpr int kStTmemCols = 128; // two accumulators of kStN columns
 constexpr int kStRows = 32;      // rows of a block of values
+constexpr int kStOneCtaSmem = 120 * 1024;   // more than half of an SM's shared memory
+constexpr int kStMaxCtas = 8;    // CTAs per unit: a cluster
 
 // Barriers of parts of the CTA.  (Not the aligned form: a warp may come to them from a branch of its lanes.)
 struct StSync { __device__ __forceinline__ void operator()() const { asm volatile("barrier.sync 1, 256;" ::: "memory"); } };
@@ -59,7 +65,10 @@ struct StSmem {
   static constexpr int kXchg = kEinv + kStEv * 4;                // u32 [kStEv][4] column-half exchange
   static constexpr int kHeavy = kXchg + kStEv * 16;              // i32 [kStCand] source index of kept candidates
   static constexpr int kEv = kHeavy + kStCand * 4;               // i32 [kStEv]   source index of evicted entries
-  static constexpr int kBytes = kEv + kStEv * 4;
+  // what the CTAs of a unit tell one another: a row's candidates go to the CTA that settles it, its target to all
+  static constexpr int kInbox = kEv + kStEv * 4;                 // uint4 [R][kStEv / R, rounded up]
+  static constexpr int kDec = kInbox + (kStEv + kStMaxCtas) * 16; // i32 [kStEv]   slot to merge into, or -1
+  static constexpr int kBytes = kDec + kStEv * 4;
   static constexpr int kKeys = kA;                               // u32 [kStCand] selection keys, gone before A is staged
   static constexpr int kHist = kRing + 2 * kStageBytes;          // i32 [kSelBins] in the stage that is filled last
   // scratch of the last CTA, laid over the operand tiles once the similarity search is over
@@ -73,13 +82,14 @@ struct StSmem {
   static_assert(kSelBins * 4 <= kStageBytes, "selection bins must fit a stage");
 };
 
-template <int D>
+// kCluster: a unit's CTAs are a cluster, which settles the candidates and the merges together.  Otherwise they leave them in
+// global memory (nom), and the unit's last CTA to arrive does all of it.
+template <int D, bool kCluster>
 __global__ void __launch_bounds__(kStAll, 2)
 steady_compress_kernel(const __grid_constant__ CUtensorMap mapD, keepkv_params p, keepkv_cache src, keepkv_cache dst,
                        const int32_t *budget_dev, int budget_scalar,
-                       const int32_t *n_recent_dev, int32_t *ret_idx, int32_t *target, float4 *nom_v,
-                       int32_t *nom_si, int C_max, int *counters, keepkv_stats *stats, int32_t *status_dev,
-                       const float *__restrict__ select_key, int spin_limit, int withhold) {
+                       const int32_t *n_recent_dev, int32_t *ret_idx, int32_t *target, uint4 *nom, int C_max, int *counters,
+                       keepkv_stats *stats, int32_t *status_dev, const float *__restrict__ select_key, int spin_limit, int withhold) {
   using SL = StSmem<D>;
   constexpr int KSTEPS = D / 16;          // k-steps of the similarity product
   constexpr int CH = D / 8;               // 16-byte chunks of a row
@@ -451,21 +461,38 @@ steady_compress_kernel(const __grid_constant__ CUtensorMap mapD, keepkv_params p
     xchg[row * 4 + 2] = __float_as_uint(top.second); xchg[row * 4 + 3] = (uint32_t)top.si;
   }
   sync();
-  const bool valid = tid < n_ev;   // threads 0..127 are the first column half of rows 0..127
+  const int tr = kCluster ? r : 0, tR = kCluster ? R : 1;   // of the CTAs that go on
+  const int per = (kStEv + tR - 1) / tR;           // CTA tr settles rows tr, tr + tR, ..: thread i the i-th of them
+  const int j = tr + tid * tR;
+  const bool valid = tid < per && j < n_ev;
   Top2 mine;
   mine.init(0.f);
-  if (valid) {
+  if (tid < n_ev) {                // threads 0..127 are the first column half of rows 0..127
     mine = top;
     mine.insert_any(__uint_as_float(xchg[row * 4]), (int)xchg[row * 4 + 1]);
     mine.insert_any(__uint_as_float(xchg[row * 4 + 2]), (int)xchg[row * 4 + 3]);
     mine.best *= einv[row];
     mine.second *= einv[row];
   }
-  if (R > 1) {
-    if (valid) {
-      nom_v[(base + tid) * C_max + r] = make_float4(mine.best, mine.second, 0.f, __int_as_float(mine.bi));
-      nom_si[(base + tid) * C_max + r] = mine.si;
-    }
+  auto fold = [&](const uint4 v) {   // slices hold ascending slots: strict comparisons keep the lower slot on ties
+    mine.insert(__uint_as_float(v.x), (int)v.z);
+    mine.insert(__uint_as_float(v.y), (int)v.w);
+  };
+  if (kCluster) {
+    if (tid < n_ev)
+      st_shared_cluster_v4(mapa_shared(sbase + SL::kInbox + (r * per + tid / R) * 16, (uint32_t)(tid % R)), __float_as_uint(mine.best),
+                           __float_as_uint(mine.second), (uint32_t)mine.bi, (uint32_t)mine.si);
+    if (r == 0 && tid == 0) stats[u] = keepkv_stats{};   // (before any CTA of the unit adds to it)
+    __threadfence();
+    __syncwarp();
+    cluster_sync_all();            // every CTA's candidates are here, and its rows in place
+    mine.init(0.f);
+    if (valid)
+      for (int c = 0; c < R; ++c) fold(*reinterpret_cast<const uint4 *>(st_smem + SL::kInbox + (c * per + tid) * 16));
+  } else if (R > 1) {
+    if (valid)
+      nom[(base + tid) * C_max + r] =
+          make_uint4(__float_as_uint(mine.best), __float_as_uint(mine.second), (uint32_t)mine.bi, (uint32_t)mine.si);
     __threadfence();
     sync();
     if (tid == 0) {
@@ -475,14 +502,9 @@ steady_compress_kernel(const __grid_constant__ CUtensorMap mapD, keepkv_params p
     sync();
     if (!s_last) return;
     __threadfence();
-    if (valid) {
-      mine.init(0.f);
-      for (int c = 0; c < R; ++c) {   // chunks hold ascending slots: strict comparisons keep the lower slot on ties
-        const float4 v = __ldcg(&nom_v[(base + tid) * C_max + c]);
-        mine.insert(v.x, __float_as_int(v.w));
-        mine.insert(v.y, __ldcg(&nom_si[(base + tid) * C_max + c]));
-      }
-    }
+    mine.init(0.f);
+    if (valid)
+      for (int c = 0; c < R; ++c) fold(__ldcg(&nom[(base + tid) * C_max + c]));
   }
 
   // ---- Algorithm 1, arg-max and threshold step: arg-max and threshold; the interface's exact arithmetic where the ranking is too close to call
@@ -497,7 +519,7 @@ steady_compress_kernel(const __grid_constant__ CUtensorMap mapD, keepkv_params p
   int e = 0, slot = -1, kind = 0;
   bool merge = false;
   if (valid) {
-    e = ev[tid];
+    e = ev[j];
     if (mine.bi >= 0) {
       slot = mine.bi;
       if (!(mine.best - mine.second > kRankEps)) kind = mine.si >= 0 ? 1 : 2;
@@ -525,11 +547,24 @@ steady_compress_kernel(const __grid_constant__ CUtensorMap mapD, keepkv_params p
   sync();
   if (kind) { slot = res_slot[tid]; merge = res_merge[tid] != 0; }
 
-  // ---- groups: the entries to merge sorted by (slot, position)
+  // ---- the decisions, to every CTA of the unit
+  int *dec = reinterpret_cast<int *>(st_smem + SL::kDec);
+  if (valid) {
+    const int to = merge ? slot : -1;
+    target[base + e] = to;
+    if (!kCluster) dec[j] = to;
+    else
+      for (int c = 0; c < R; ++c) st_shared_cluster_u32(mapa_shared(sbase + SL::kDec + j * 4, (uint32_t)c), (uint32_t)to);
+  }
+  __syncwarp();
+  if (!kCluster) sync();
+  else cluster_sync_all();         // (behind it no CTA touches another's shared memory)
+
+  // ---- groups: the entries to merge sorted by (slot, position); every CTA makes the same list
+  const int to = tid < n_ev ? dec[tid] : -1;
   int M;
-  const int off = block_excl_count(merge, warp_tot, M, kStWarps, sync);
-  if (valid) target[base + e] = merge ? slot : -1;
-  if (merge) skey[off] = ((uint32_t)slot << 16) | (uint32_t)tid;
+  const int off = block_excl_count(to >= 0, warp_tot, M, kStWarps, sync);
+  if (to >= 0) skey[off] = ((uint32_t)to << 16) | (uint32_t)tid;
   sync();
   uint32_t mk = 0xFFFFFFFFu;
   int rank = 0;
@@ -546,22 +581,48 @@ steady_compress_kernel(const __grid_constant__ CUtensorMap mapD, keepkv_params p
   if (head) ghead[pos] = tid;
   if (tid == 0) {
     ghead[n_groups] = M;
-    keepkv_stats st;
-    st.n_retained = n_ret; st.n_evicted = n_ev; st.n_merged = 0; st.n_below_T = n_ev - M;
-    st.n_guard_groups = 0; st.n_groups = 0; st.max_group = 0; st.reserved = 0;
-    stats[u] = st;
-    if (h == 0) dst.seq_len[b] = n_ret;
+    if (tr == 0) {
+      if (!kCluster) stats[u] = keepkv_stats{};
+      stats[u].n_retained = n_ret;
+      stats[u].n_evicted = n_ev;
+      stats[u].n_below_T = n_ev - M;
+      if (h == 0) dst.seq_len[b] = n_ret;
+    }
   }
   sync();
-  // ---- Algorithm 1, merge step: one warp per group
+  // ---- Algorithm 1, merge step: one warp per group, of all the unit's CTAs
   MergeCount count;
-  for (int gi = warp; gi < n_groups; gi += kStWarps) {
+  for (int gi = tr * kStWarps + warp; gi < n_groups; gi += tR * kStWarps) {
     const int beg = ghead[gi], n = ghead[gi + 1] - beg;
     const int c = (int)(skey[beg] >> 16);
     merge_group<D>(p, src, dst, c, src, base + ret(c), [&](int t) { return ev[skey[beg + t] & 0xFFFFu]; }, n, target + base, base,
                    count);
   }
   count.flush(stats + u);
+}
+
+// Clusters of k CTAs that are resident at once: twice those of one CTA per SM (see decode.cu).  A device's answer is kept.
+template <typename K>
+static int steady_clusters(K kernel, int dev, int k) {
+  static std::atomic<int> known[64][kStMaxCtas + 1];
+  std::atomic<int> &at = known[dev & 63][k];
+  int n = at.load(std::memory_order_relaxed);
+  if (n == 0) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)k);
+    cfg.blockDim = dim3(kStAll);
+    cfg.dynamicSmemBytes = kStOneCtaSmem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)k;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) { (void)cudaGetLastError(); n = 0; }
+    n = 2 * n + 1;   // (odd: never 0)
+    at.store(n, std::memory_order_relaxed);
+  }
+  return n - 1;
 }
 
 template <int D>
@@ -572,11 +633,13 @@ static void launch_steady_t(const keepkv_params &p, const keepkv_cache &src, con
   using SL = StSmem<D>;
   const int U = p.B * p.H_kv;
   constexpr size_t smem_bytes = (size_t)SL::kBytes + 1024;   // slack to align the swizzled tiles
+  static_assert(smem_bytes <= kStOneCtaSmem && 2 * (smem_bytes + 2048) <= 228 * 1024, "two CTAs per SM");
   static bool attr_done_dev[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
   if (!attr_done_dev[dev & 63]) {
-    cudaFuncSetAttribute(steady_compress_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+    cudaFuncSetAttribute(steady_compress_kernel<D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kStOneCtaSmem);
+    cudaFuncSetAttribute(steady_compress_kernel<D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
     attr_done_dev[dev & 63] = true;
   }
   CUtensorMap mapD;
@@ -584,13 +647,23 @@ static void launch_steady_t(const keepkv_params &p, const keepkv_cache &src, con
     if (ctx.err == cudaSuccess) ctx.err = cudaErrorInvalidValue;
     return;
   }
-  // CTAs per unit: what two resident CTAs per SM can hold at once, at most one per column chunk of the workspace
+  // CTAs per unit: what two resident CTAs per SM can hold at once.  They are a cluster where all units' clusters are resident
+  // (one lives inside a GPC: 66 of four, 90 of three), also with fewer CTAs, unless more than a quarter of them would be given up:
+  // a launch for 72 units takes 43 us as clusters of three, 45 as four CTAs; one for 96 takes 60 as clusters of two, 53 as three.
   int R = 2 * sm_count() / U;
   R = R < 1 ? 1 : (R > L.nom_chunks ? L.nom_chunks : R);
-  launch_pdl(steady_compress_kernel<D>, dim3(R, U), dim3(kStAll), smem_bytes, ctx.stream, mapD, p, src, dst,
-             budget_dev, budget_scalar, n_recent_dev, ret_idx, target,
-             reinterpret_cast<float4 *>(ws + L.nom_v), reinterpret_cast<int32_t *>(ws + L.nom_si), L.nom_chunks,
-             reinterpret_cast<int *>(ws + L.counters), stats, status_dev, select_key, debug_spin_limit(), debug_withhold());
+  int k = R;
+  while (k > 1 && steady_clusters(steady_compress_kernel<D, true>, dev, k) < U) --k;
+  uint4 *nom = reinterpret_cast<uint4 *>(ws + L.nom_v);
+  int *counters = reinterpret_cast<int *>(ws + L.counters);
+  if (k > 1 && 4 * k >= 3 * R)
+    launch_pdl_cluster(steady_compress_kernel<D, true>, dim3(k, U), dim3(kStAll), smem_bytes, ctx.stream, (unsigned)k, mapD, p, src, dst,
+                       budget_dev, budget_scalar, n_recent_dev, ret_idx, target, nom, L.nom_chunks, counters, stats, status_dev,
+                       select_key, debug_spin_limit(), debug_withhold());
+  else
+    launch_pdl(steady_compress_kernel<D, false>, dim3(R, U), dim3(kStAll), smem_bytes, ctx.stream, mapD, p, src, dst, budget_dev,
+               budget_scalar, n_recent_dev, ret_idx, target, nom, L.nom_chunks, counters, stats, status_dev, select_key,
+               debug_spin_limit(), debug_withhold());
   KEEPKV_CHECK_LAUNCH(ctx);
 }
 

@@ -904,6 +904,22 @@ def test_compress_steady_flag_equals_pipeline(B, H_kv, G, d, lens, budget, n_rec
         check_compress_unit(p, u, budget, n_recent, hs, hd, ret, tgt, stats, what="single kernel")
 
 
+@pytest.mark.parametrize("units", [5, 31, 37, 45, 53, 67, 91, 148, 149])
+def test_compress_steady_clusters_of_every_size(units):
+    """A unit's CTAs are a cluster of one to eight, by the number of units; each settles its share of the evicted entries and
+    of the groups.  Same bits as the general kernels, with one evicted entry, some, and as many as there may be."""
+    lens = [200 + (1, 67, 128)[i % 3] for i in range(units)]
+    p = kb.make_params(B=units, H_q=1, H_kv=1, d=64, N_cap=384, n_sink=4, n_recent=90, merge_threshold=0.1)
+    src = random_cache(p, lens, seed=units, vote_max=3, scored_frac=1.0)
+    got, want = _run_compress(_copy_params(p, flags=kb.FLAG_COMPRESS_STEADY), src, 200), _run_compress(p, src, 200)
+    for name in ("K", "V", "votes", "lscore"):
+        x, y = (getattr(run[0], name)[:, :, :200].contiguous().view(torch.uint8) for run in (got, want))
+        assert torch.equal(x, y), name
+    assert np.array_equal(got[3], want[3]) and np.array_equal(got[1][:, :200], want[1][:, :200])
+    for b, n in enumerate(lens):
+        assert np.array_equal(got[2][b, :n], want[2][b, :n]), b
+
+
 @pytest.mark.parametrize("d", [64, 128])
 @pytest.mark.parametrize("withhold", [0, 1, 2])
 def test_compress_steady_bounded_wait_runs_out_and_the_next_call_is_normal(d, withhold):

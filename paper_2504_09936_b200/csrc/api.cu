@@ -37,8 +37,7 @@ WsLayout ws_layout(const keepkv_params &p) {
   // (the search reads whole 256-entry tiles of these two)
   L.inv_norm = take(U * N * 4);
   L.norm_ext = take(U * N * 16 + 4096);
-  L.nom_v = take(U * N * C * 16);
-  L.nom_si = take(U * N * C * 4);
+  L.nom = take(U * N * C * 16);
   L.grp_key = take(U * Np2 * 4);
   L.grp_head = take(U * N * 4);
   L.stats = take(U * sizeof(keepkv_stats));

@@ -30,8 +30,7 @@ struct WsLayout {
   size_t ev_idx;      // i32 [U,N]          source indices of evicted entries, ascending
   size_t inv_norm;    // f32 [U,N]          1/|k| of each retained key (tree-summed; only ranks candidates)
   size_t norm_ext;    // bf16 [U,N,8]       |k| of the same in three terms, as more channels of the search's columns
-  size_t nom_v;       // float4 [U,N,C]     per evicted row and column chunk: best, second cosine, unused, best slot
-  size_t nom_si;      // i32 [U,N,C]        slot of the second-best cosine
+  size_t nom;         // uint4 [C,U,N]      per column chunk and evicted row: best, second cosine (f32), their slots
   size_t grp_key;     // u32 [U,Npow2]      (slot << 16 | source index) of merged entries, sorted
   size_t grp_head;    // i32 [U,N]          position in grp_key where each group starts
   size_t stats;       // keepkv_stats [U]   used when the caller passes no stats array
@@ -80,8 +79,7 @@ void launch_compress(const keepkv_params &p, const keepkv_cache &src, const keep
                      LaunchCtx &ctx, const float *select_key = nullptr);
 // tcgen05 similarity search: for every evicted key the two largest cosines over the retained keys
 void launch_nominate(const keepkv_params &p, const keepkv_cache &src, const keepkv_cache &dst, const int32_t *ev_idx,
-                     const UnitInfo *unit_info, const float *inv_norm, const uint4 *norm_ext, int32_t *sched, float4 *nom_v, int32_t *nom_si,
-                     int nom_chunks, int32_t *status_dev, LaunchCtx &ctx, int self_mask = 0);
+                     const UnitInfo *unit_info, const float *inv_norm, const uint4 *norm_ext, int32_t *sched, uint4 *nom, int nom_chunks, int32_t *status_dev, LaunchCtx &ctx, int self_mask = 0);
 // Algorithm 1 in place on a cache with a position array (compress.cu)
 void launch_compress_inplace(const keepkv_params &p, const keepkv_cache &c, int32_t *pos, int32_t *pos_len, int32_t *n_seen,
                              const int32_t *budget_dev, int32_t budget_scalar, const int32_t *n_recent_dev,

@@ -242,8 +242,11 @@ compact_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, const int32_
 // (Three distinct cosines within the accumulation error of each other, the one case this cannot
 // settle, would need a coincidence of order 1e-8 per row; exact duplicates are handled, because equal
 // keys give equal values and the lower slot stays in front.)
-// Rows that need the exact chain are queued and shared out over the warps of the CTA (coalesced row
-// loads into shared memory, the sequential chains on three lanes).  A unit of at most kResolveThreads evicted
+// Rows that need the exact chain are taken one after the other by the warp that finds them (coalesced row
+// loads into shared memory, the sequential chains on three lanes).  Bound: the latency of a row's list; so the warps of the
+// resident CTAs (two per SM) walk the rows on their own, the next lists on their way, and no barrier is met: 64 units of 6554
+// rows 19 -> 13 us, 128 of up to 14746 41 -> 26 us against a CTA per 512 rows with a common queue and place in the list (and
+// lists whose chunks lay side by side, so that a row's sector was mostly unused).  A unit of at most kResolveThreads evicted
 // entries (every steady-state compression) is one CTA's: it sorts the entries to merge by (slot, position), which makes
 // every group contiguous and ascending, and merges them if the groups are few.  The entries to merge of larger units go to
 // a list that group_kernel sorts.
@@ -329,44 +332,47 @@ __device__ __forceinline__ void group_and_merge(const keepkv_params &p, const ke
 template <int D>
 __global__ void __launch_bounds__(kResolveThreads)
 resolve_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, const int32_t *__restrict__ ev_idx,
-               UnitInfo *unit_info, const float4 *__restrict__ nom_v, const int32_t *__restrict__ nom_si,
-               const int32_t *__restrict__ sched, int C_max, int32_t *target, uint32_t *grp_key, int key_stride, int32_t *grp_head, keepkv_stats *stats, int decide_only) {
+               UnitInfo *unit_info, const uint4 *__restrict__ nom, const int32_t *__restrict__ sched, int32_t *target,
+               uint32_t *grp_key, int key_stride, int32_t *grp_head, keepkv_stats *stats, int decide_only) {
   __shared__ uint32_t key_smem[kResolveThreads];
   __shared__ float ke_s[kResolveWarps][D];
   __shared__ float kc_s[kResolveWarps][2][D];
   __shared__ int warp_tot[32];
-  __shared__ int s_nq[2], s_base;
-  __shared__ int q_tid[kResolveThreads], q_e[kResolveThreads], q_kind[kResolveThreads], q_a[kResolveThreads],
-      q_b[kResolveThreads];
-  __shared__ int res_slot[kResolveThreads], res_merge[kResolveThreads];
-  const int u = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  __shared__ int s_keys;
+  const int u = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, step = gridDim.x * kResolveThreads;
   pdl_wait();
   pdl_trigger();
   const UnitInfo ui = unit_info[u];
-  const size_t base = (size_t)u * p.N_cap;
+  const int C = sched[0];
+  const size_t base = (size_t)u * p.N_cap, n_rows = (size_t)p.B * p.H_kv * p.N_cap;
   const __nv_bfloat16 *sK = reinterpret_cast<const __nv_bfloat16 *>(src.K) + base * D;
   const __nv_bfloat16 *dK = reinterpret_cast<const __nv_bfloat16 *>(dst.K) + base * D;
   uint32_t *gk = grp_key + (size_t)u * key_stride;
-  const int C = sched[0];
   const float T = p.merge_threshold;
   if ((int)blockIdx.x * kResolveThreads >= ui.n_ev) return;
-  const bool single = ui.n_ev <= kResolveThreads && !decide_only;
-  if (tid == 0) { s_nq[0] = s_nq[1] = 0; s_base = 0; }
+  const bool single = ui.n_ev <= kResolveThreads && !decide_only;   // this CTA holds all rows of the unit
+  if (tid == 0) s_keys = 0;
   __syncthreads();
 
-  int pass = 0;
-  for (int j0 = blockIdx.x * kResolveThreads; j0 < ui.n_ev; j0 += gridDim.x * kResolveThreads, ++pass) {
-    const int j = j0 + tid;
+  // The warps go their own ways; a row's list is on its way while the one before it is decided.
+  int j0 = blockIdx.x * kResolveThreads + warp * 32, e_next = 0;
+  uint4 v_next = make_uint4(0u, 0u, 0u, 0u);
+  auto fetch = [&](int j) {
+    if (j < ui.n_ev) { e_next = ev_idx[base + j]; v_next = nom[base + j]; }
+  };
+  fetch(j0 + lane);
+  for (; j0 < ui.n_ev; j0 += step) {
+    const int j = j0 + lane, e = e_next;
+    uint4 v = v_next;
+    fetch(j + step);
     const bool valid = j < ui.n_ev;
-    int e = 0, slot = -1, kind = 0, bi = -1, si = -1;
+    int slot = -1, kind = 0, bi = -1, si = -1;
     bool merge = false;
     if (valid) {
-      e = ev_idx[base + j];
       float best = -CUDART_INF_F, second = -CUDART_INF_F;
-      for (int c = 0; c < C; ++c) {   // chunks hold ascending slots: strict comparisons keep the lower slot on ties
-        const float4 v = nom_v[(base + j) * C_max + c];
-        const int vi[2] = {__float_as_int(v.w), nom_si[(base + j) * C_max + c]};
-        const float vv[2] = {v.x, v.y};
+      for (int c = 0;;) {   // chunks hold ascending slots: strict comparisons keep the lower slot on ties
+        const int vi[2] = {(int)v.z, (int)v.w};
+        const float vv[2] = {__uint_as_float(v.x), __uint_as_float(v.y)};
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
           const bool p1 = vv[t] > best, p2 = vv[t] > second;
@@ -375,6 +381,8 @@ resolve_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, const int32_
           bi = p1 ? vi[t] : bi;
           best = fmaxf(best, vv[t]);
         }
+        if (++c >= C) break;
+        v = nom[c * n_rows + base + j];
       }
       if (bi >= 0) {
         slot = bi;
@@ -383,52 +391,32 @@ resolve_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, const int32_
         else merge = best > T;
       }
     }
-    // ---- rows that need the interface's exact arithmetic, shared out over the warps
-    const int par = pass & 1;
-    if (kind) {
-      const int q = atomicAdd(&s_nq[par], 1);
-      q_tid[q] = tid; q_e[q] = e; q_kind[q] = kind; q_a[q] = bi; q_b[q] = si;
-    }
-    __syncthreads();
-    const int nq = s_nq[par];
-    if (tid == 0) s_nq[par ^ 1] = 0;   // the next pass counts in the other word
-    for (int q = warp; q < nq; q += kResolveWarps) {
-      const int ee = q_e[q], kd = q_kind[q], ca = q_a[q], cb = kd == 1 ? q_b[q] : q_a[q];
+    // ---- rows that need the interface's exact arithmetic, one after the other
+    for (unsigned need = __ballot_sync(0xffffffffu, kind != 0); need; need &= need - 1) {
+      const int l = __ffs(need) - 1, ee = __shfl_sync(0xffffffffu, e, l), ca = __shfl_sync(0xffffffffu, bi, l);
+      const int cb = __shfl_sync(0xffffffffu, kind == 1 ? si : bi, l);
       float u0, u1;
       exact_cosines<D>(sK + (size_t)ee * D, dK + (size_t)ca * D, dK + (size_t)cb * D, ke_s[warp], &kc_s[warp][0][0], u0, u1);
       int win = ca;
       float wu = u0;
-      if (kd == 1 && (u1 > u0 || (u1 == u0 && cb < ca))) { win = cb; wu = u1; }
-      if (lane == 0) { res_slot[q_tid[q]] = win; res_merge[q_tid[q]] = win >= 0 && wu > T; }
+      if (u1 > u0 || (u1 == u0 && cb < ca)) { win = cb; wu = u1; }
+      if (lane == l) { slot = win; merge = wu > T; }
     }
-    __syncthreads();
-    if (kind) { slot = res_slot[tid]; merge = res_merge[tid] != 0; }
-    if (decide_only) {   // the caller pairs the entries itself (merge-first policy): the partner above T, or -1
-      if (valid) target[base + e] = merge ? slot : -1;
-      continue;
-    }
-    // ---- record the decision; entries to merge go to the unit's key list (any order: it is sorted below)
-    int tot;
-    const int off = block_excl_count(merge, warp_tot, tot);
-    if (single) {   // this CTA holds all rows of the unit: its keys never leave shared memory
-      if (valid) {
-        target[base + e] = merge ? slot : -1;
-        if (merge) key_smem[off] = ((uint32_t)slot << 16) | (uint32_t)e;
-      }
-      if (tid == 0) s_base = tot;
-      __syncthreads();
-      continue;
-    }
-    if (tid == 0) s_base = tot ? atomicAdd(&unit_info[u].n_keys, tot) : 0;
-    __syncthreads();
-    if (valid) {
-      target[base + e] = merge ? slot : -1;
-      if (merge) gk[s_base + off] = ((uint32_t)slot << 16) | (uint32_t)e;
+    if (valid) target[base + e] = merge ? slot : -1;
+    if (decide_only) continue;   // the caller pairs the entries itself (merge-first policy): the partner above T, or -1
+    // ---- entries to merge go to the unit's key list (any order: it is sorted below)
+    const unsigned m = __ballot_sync(0xffffffffu, merge);
+    if (m) {
+      int at = 0;
+      if (lane == 0) at = atomicAdd(single ? &s_keys : &unit_info[u].n_keys, __popc(m));
+      at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
+      if (merge) (single ? key_smem : gk)[at] = ((uint32_t)slot << 16) | (uint32_t)e;
     }
   }
   if (!single) return;
+  __syncthreads();
   if (tid == 0) unit_info[u].ticket = 1;   // this unit's entries are sorted
-  group_and_merge<D, kResolveThreads>(p, src, dst, u, base, ui.n_ev, s_base, true, key_smem, kResolveThreads, gk, target, grp_head, unit_info, stats, warp_tot);
+  group_and_merge<D, kResolveThreads>(p, src, dst, u, base, ui.n_ev, s_keys, true, key_smem, kResolveThreads, gk, target, grp_head, unit_info, stats, warp_tot);
 }
 
 // One CTA per unit: the unit's key list (in global memory, any order) sorted into groups by counting -- a histogram of the
@@ -508,7 +496,10 @@ group_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, int32_t *targe
 }
 
 // What the two kernels are launched with.
-static int resolve_grid(const keepkv_params &p) { return (p.N_cap + kResolveThreads - 1) / kResolveThreads; }   // a pass each
+static int resolve_grid(const keepkv_params &p) {   // what is resident (two per SM), as far as there are rows
+  const int most = (p.N_cap + kResolveThreads - 1) / kResolveThreads, n = 2 * sm_count() / (p.B * p.H_kv);
+  return n < 1 ? 1 : n < most ? n : most;
+}
 static int merge_grid(const keepkv_params &p) {
   const int n = 4096 / (p.B * p.H_kv);
   return n < 1 ? 1 : (n > 128 ? 128 : n);
@@ -565,8 +556,7 @@ static void launch_compress_t(const keepkv_params &p, const keepkv_cache &src, c
   int32_t *ev_idx = reinterpret_cast<int32_t *>(ws + L.ev_idx);
   float *inv_norm = reinterpret_cast<float *>(ws + L.inv_norm);
   uint4 *norm_ext = reinterpret_cast<uint4 *>(ws + L.norm_ext);
-  float4 *nom_v = reinterpret_cast<float4 *>(ws + L.nom_v);
-  int32_t *nom_si = reinterpret_cast<int32_t *>(ws + L.nom_si);
+  uint4 *nom = reinterpret_cast<uint4 *>(ws + L.nom);
   uint32_t *grp_key = reinterpret_cast<uint32_t *>(ws + L.grp_key);
   int32_t *grp_head = reinterpret_cast<int32_t *>(ws + L.grp_head);
   const int ret_bound = budget_dev ? p.N_cap : (budget_scalar < p.N_cap ? budget_scalar : p.N_cap);
@@ -598,9 +588,9 @@ static void launch_compress_t(const keepkv_params &p, const keepkv_cache &src, c
              merges ? norm_ext : nullptr);
   KEEPKV_CHECK_LAUNCH(ctx);
   if (!merges) return;
-  launch_nominate(p, src, dst, ev_idx, ui, inv_norm, norm_ext, sched, nom_v, nom_si, L.nom_chunks, status_dev, ctx);
+  launch_nominate(p, src, dst, ev_idx, ui, inv_norm, norm_ext, sched, nom, L.nom_chunks, status_dev, ctx);
   launch_pdl(resolve_kernel<D>, dim3(resolve_grid(p), U), dim3(kResolveThreads), 0, ctx.stream,
-      p, src, dst, ev_idx, ui, nom_v, nom_si, sched, L.nom_chunks, target, grp_key, L.key_stride, grp_head,
+      p, src, dst, ev_idx, ui, nom, sched, target, grp_key, L.key_stride, grp_head,
       stats, 0);
   KEEPKV_CHECK_LAUNCH(ctx);
   if (!all_small(p, budget_dev, budget_scalar)) {
@@ -808,8 +798,7 @@ static void launch_compress_merge_first_t(const keepkv_params &p, const keepkv_c
   int32_t *ev_idx = reinterpret_cast<int32_t *>(ws + L.ev_idx);
   float *inv_norm = reinterpret_cast<float *>(ws + L.inv_norm);
   uint4 *norm_ext = reinterpret_cast<uint4 *>(ws + L.norm_ext);
-  float4 *nom_v = reinterpret_cast<float4 *>(ws + L.nom_v);
-  int32_t *nom_si = reinterpret_cast<int32_t *>(ws + L.nom_si);
+  uint4 *nom = reinterpret_cast<uint4 *>(ws + L.nom);
   uint32_t *grp_key = reinterpret_cast<uint32_t *>(ws + L.grp_key);
   int32_t *grp_head = reinterpret_cast<int32_t *>(ws + L.grp_head);
   keepkv_stats *st1 = reinterpret_cast<keepkv_stats *>(ws + L.stats2);
@@ -828,9 +817,9 @@ static void launch_compress_merge_first_t(const keepkv_params &p, const keepkv_c
   launch_pdl(mf_prepare_kernel<D>, dim3(norm_grid(p), U), dim3(256), 0, ctx.stream, p, cache, ev_idx, ui, inv_norm, norm_ext);
   KEEPKV_CHECK_LAUNCH(ctx);
   // rows and columns are the same keys: the "retained" operand of the search is the prompt itself
-  launch_nominate(p, cache, cache, ev_idx, ui, inv_norm, norm_ext, sched, nom_v, nom_si, L.nom_chunks, status_dev, ctx, 1);
+  launch_nominate(p, cache, cache, ev_idx, ui, inv_norm, norm_ext, sched, nom, L.nom_chunks, status_dev, ctx, 1);
   launch_pdl(resolve_kernel<D>, dim3(resolve_grid(p), U), dim3(kResolveThreads), 0, ctx.stream,
-      p, cache, cache, ev_idx, ui, nom_v, nom_si, sched, L.nom_chunks, target, grp_key, L.key_stride, grp_head,
+      p, cache, cache, ev_idx, ui, nom, sched, target, grp_key, L.key_stride, grp_head,
       st1, 1);
   KEEPKV_CHECK_LAUNCH(ctx);
   launch_pdl(mf_mark_kernel, dim3(U), dim3(1024), 0, ctx.stream, p, unit_len, ret1, target, ev_idx, grp_head, grp_key,
@@ -973,8 +962,7 @@ static void launch_compress_inplace_t(const keepkv_params &p, const keepkv_cache
   int32_t *ev_idx = reinterpret_cast<int32_t *>(ws + L.ev_idx);
   float *inv_norm = reinterpret_cast<float *>(ws + L.inv_norm);
   uint4 *norm_ext = reinterpret_cast<uint4 *>(ws + L.norm_ext);
-  float4 *nom_v = reinterpret_cast<float4 *>(ws + L.nom_v);
-  int32_t *nom_si = reinterpret_cast<int32_t *>(ws + L.nom_si);
+  uint4 *nom = reinterpret_cast<uint4 *>(ws + L.nom);
   uint32_t *grp_key = reinterpret_cast<uint32_t *>(ws + L.grp_key);
   int32_t *grp_head = reinterpret_cast<int32_t *>(ws + L.grp_head);
   static bool attr_done_dev[64] = {};
@@ -995,9 +983,9 @@ static void launch_compress_inplace_t(const keepkv_params &p, const keepkv_cache
   if (merges) {
     launch_pdl(ip_columns_kernel, dim3((U + 127) / 128), dim3(128), 0, ctx.stream, ui, U);
     KEEPKV_CHECK_LAUNCH(ctx);
-    launch_nominate(p, c, c, ev_idx, ui, inv_norm, norm_ext, sched, nom_v, nom_si, L.nom_chunks, status_dev, ctx);
+    launch_nominate(p, c, c, ev_idx, ui, inv_norm, norm_ext, sched, nom, L.nom_chunks, status_dev, ctx);
     launch_pdl(resolve_kernel<D>, dim3(resolve_grid(p), U), dim3(kResolveThreads), 0, ctx.stream,
-        p, c, c, ev_idx, ui, nom_v, nom_si, sched, L.nom_chunks, target, grp_key, L.key_stride, grp_head,
+        p, c, c, ev_idx, ui, nom, sched, target, grp_key, L.key_stride, grp_head,
         stats, 0);
     KEEPKV_CHECK_LAUNCH(ctx);
     if (!all_small(p, budget_dev, budget_scalar)) {

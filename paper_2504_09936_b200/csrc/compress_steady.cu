@@ -654,7 +654,7 @@ static void launch_steady_t(const keepkv_params &p, const keepkv_cache &src, con
   R = R < 1 ? 1 : (R > L.nom_chunks ? L.nom_chunks : R);
   int k = R;
   while (k > 1 && steady_clusters(steady_compress_kernel<D, true>, dev, k) < U) --k;
-  uint4 *nom = reinterpret_cast<uint4 *>(ws + L.nom_v);
+  uint4 *nom = reinterpret_cast<uint4 *>(ws + L.nom);
   int *counters = reinterpret_cast<int *>(ws + L.counters);
   if (k > 1 && 4 * k >= 3 * R)
     launch_pdl_cluster(steady_compress_kernel<D, true>, dim3(k, U), dim3(kStAll), smem_bytes, ctx.stream, (unsigned)k, mapD, p, src, dst,

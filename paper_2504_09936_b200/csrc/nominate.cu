@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(kNomThreads, 1)
 nominate_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, const __nv_bfloat16 *__restrict__ srcK,
                 const int32_t *__restrict__ ev_idx, const UnitInfo *__restrict__ unit_info,
                 const float *__restrict__ inv_norm, const uint4 *__restrict__ norm_ext, int32_t *sched,
-                float4 *__restrict__ nom_v, int32_t *__restrict__ nom_si, int C_max, int32_t *status_dev, int self_mask) {
+                uint4 *__restrict__ nom, int C_max, int32_t *status_dev, int self_mask) {
   using SL = NomSmem<D>;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   // a_ready[2], a_empty[2], b_full[4], b_empty[4], t_full[2], t_empty[2], drain, x_full[4][2]
@@ -133,6 +133,7 @@ nominate_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, const
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int U = p.B * p.H_kv;
+  const size_t n_rows = (size_t)U * p.N_cap;
 
   if (tid == 0) {
     for (int i = 0; i < 2; ++i) {
@@ -289,9 +290,7 @@ nominate_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, const
       const size_t ubase = (size_t)it.u * p.N_cap;
       if (it.n_ev >= 0 && it.t0 == it.t1) {   // a chunk without tiles (fewer tiles than chunks): an empty result
         for (int i = it.m0 + r0 + lane; i < min(it.m0 + r0 + RW, it.n_ev); i += 32) {
-          const size_t o = (ubase + i) * C_max + it.chunk;
-          nom_v[o] = make_float4(-CUDART_INF_F, -CUDART_INF_F, 0.f, __int_as_float(-1));
-          nom_si[o] = -1;
+          nom[it.chunk * n_rows + ubase + i] = make_uint4(0xff800000u, 0xff800000u, 0xffffffffu, 0xffffffffu);   // (-inf, none)
         }
         continue;
       }
@@ -459,9 +458,8 @@ nominate_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, const
           top.insert_any(__uint_as_float(x[3 * w + 1]), (int)(sl >> 16) - 1);
         }
         if (row_ok) {
-          const size_t o = (ubase + it.m0 + row) * C_max + it.chunk;
-          nom_v[o] = make_float4(top.best * rinv, top.second * rinv, 0.f, __int_as_float(top.bi));
-          nom_si[o] = top.si;
+          nom[it.chunk * n_rows + ubase + it.m0 + row] =
+              make_uint4(__float_as_uint(top.best * rinv), __float_as_uint(top.second * rinv), (uint32_t)top.bi, (uint32_t)top.si);
         }
       }
       x_phase ^= 1 << buf;
@@ -491,7 +489,7 @@ nominate_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, const
 template <int D, bool kCut>
 static void launch_nominate_t(const keepkv_params &p, const keepkv_cache &src, const keepkv_cache &dst,
                               const int32_t *ev_idx, const UnitInfo *unit_info, const float *inv_norm,
-                              const uint4 *norm_ext, int32_t *sched, float4 *nom_v, int32_t *nom_si, int nom_chunks, int32_t *status_dev, LaunchCtx &ctx,
+                              const uint4 *norm_ext, int32_t *sched, uint4 *nom, int nom_chunks, int32_t *status_dev, LaunchCtx &ctx,
                               int self_mask) {
   using SL = NomSmem<D>;
   constexpr size_t smem_bytes = (size_t)SL::kBytes + 1024;
@@ -508,18 +506,18 @@ static void launch_nominate_t(const keepkv_params &p, const keepkv_cache &src, c
     return;
   }
   launch_pdl(nominate_kernel<D, kCut>, dim3(sm_count()), dim3(kNomThreads), smem_bytes, ctx.stream,
-      mapB, p, reinterpret_cast<const __nv_bfloat16 *>(src.K), ev_idx, unit_info, inv_norm, norm_ext, sched, nom_v, nom_si,
+      mapB, p, reinterpret_cast<const __nv_bfloat16 *>(src.K), ev_idx, unit_info, inv_norm, norm_ext, sched, nom,
       nom_chunks, status_dev, self_mask);
   KEEPKV_CHECK_LAUNCH(ctx);
 }
 
 void launch_nominate(const keepkv_params &p, const keepkv_cache &src, const keepkv_cache &dst, const int32_t *ev_idx,
-                     const UnitInfo *unit_info, const float *inv_norm, const uint4 *norm_ext, int32_t *sched, float4 *nom_v, int32_t *nom_si,
+                     const UnitInfo *unit_info, const float *inv_norm, const uint4 *norm_ext, int32_t *sched, uint4 *nom,
                      int nom_chunks, int32_t *status_dev, LaunchCtx &ctx, int self_mask) {
   const bool cut = p.merge_threshold >= kNomStatic;
   auto launch = p.d == 128 ? (cut ? launch_nominate_t<128, true> : launch_nominate_t<128, false>)
                            : (cut ? launch_nominate_t<64, true> : launch_nominate_t<64, false>);
-  launch(p, src, dst, ev_idx, unit_info, inv_norm, norm_ext, sched, nom_v, nom_si, nom_chunks, status_dev, ctx, self_mask);
+  launch(p, src, dst, ev_idx, unit_info, inv_norm, norm_ext, sched, nom, nom_chunks, status_dev, ctx, self_mask);
 }
 
 }  // namespace keepkv

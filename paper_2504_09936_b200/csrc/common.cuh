@@ -79,7 +79,14 @@ void launch_compress(const keepkv_params &p, const keepkv_cache &src, const keep
                      LaunchCtx &ctx, const float *select_key = nullptr);
 // tcgen05 similarity search: for every evicted key the two largest cosines over the retained keys
 void launch_nominate(const keepkv_params &p, const keepkv_cache &src, const keepkv_cache &dst, const int32_t *ev_idx,
-                     const UnitInfo *unit_info, const float *inv_norm, const uint4 *norm_ext, int32_t *sched, uint4 *nom, int nom_chunks, int32_t *status_dev, LaunchCtx &ctx, int self_mask = 0);
+                     const UnitInfo *unit_info, const float *inv_norm, const uint4 *norm_ext, int32_t *sched, uint4 *nom, int nom_chunks, int32_t *status_dev, LaunchCtx &ctx, int columns, int self_mask = 0,
+                     unsigned long long *tri_best = nullptr);
+// The form for large prompts (nominate_pair.cu).  tri_best: rows and columns are the same entries, the lists are two words as a row
+// and two as a column for each of them, zero at first.
+bool nominate_pairs(const keepkv_params &p, int columns);
+void launch_nominate_pairs(const keepkv_params &p, const keepkv_cache &src, const keepkv_cache &dst, const int32_t *ev_idx,
+                           const UnitInfo *unit_info, const float *inv_norm, const uint4 *norm_ext, int32_t *sched, uint4 *nom,
+                           int nom_chunks, int32_t *status_dev, LaunchCtx &ctx, unsigned long long *tri_best);
 // Algorithm 1 in place on a cache with a position array (compress.cu)
 void launch_compress_inplace(const keepkv_params &p, const keepkv_cache &c, int32_t *pos, int32_t *pos_len, int32_t *n_seen,
                              const int32_t *budget_dev, int32_t budget_scalar, const int32_t *n_recent_dev,

@@ -329,11 +329,13 @@ __device__ __forceinline__ void group_and_merge(const keepkv_params &p, const ke
 }
 
 
-template <int D>
+// kTri: the search's lists are those of a triangle.
+template <int D, bool kTri>
 __global__ void __launch_bounds__(kResolveThreads)
 resolve_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, const int32_t *__restrict__ ev_idx,
                UnitInfo *unit_info, const uint4 *__restrict__ nom, const int32_t *__restrict__ sched, int32_t *target,
-               uint32_t *grp_key, int key_stride, int32_t *grp_head, keepkv_stats *stats, int decide_only) {
+               uint32_t *grp_key, int key_stride, int32_t *grp_head, keepkv_stats *stats, int decide_only,
+               const ulonglong2 *__restrict__ tri_best) {
   __shared__ uint32_t key_smem[kResolveThreads];
   __shared__ float ke_s[kResolveWarps][D];
   __shared__ float kc_s[kResolveWarps][2][D];
@@ -343,7 +345,7 @@ resolve_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, const int32_
   pdl_wait();
   pdl_trigger();
   const UnitInfo ui = unit_info[u];
-  const int C = sched[0];
+  const int C = kTri ? 0 : sched[0];
   const size_t base = (size_t)u * p.N_cap, n_rows = (size_t)p.B * p.H_kv * p.N_cap;
   const __nv_bfloat16 *sK = reinterpret_cast<const __nv_bfloat16 *>(src.K) + base * D;
   const __nv_bfloat16 *dK = reinterpret_cast<const __nv_bfloat16 *>(dst.K) + base * D;
@@ -357,20 +359,37 @@ resolve_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, const int32_
   // The warps go their own ways; a row's list is on its way while the one before it is decided.
   int j0 = blockIdx.x * kResolveThreads + warp * 32, e_next = 0;
   uint4 v_next = make_uint4(0u, 0u, 0u, 0u);
+  ulonglong2 l0_next = make_ulonglong2(0, 0), l1_next = l0_next;
   auto fetch = [&](int j) {
-    if (j < ui.n_ev) { e_next = ev_idx[base + j]; v_next = nom[base + j]; }
+    if (j >= ui.n_ev) return;
+    if (kTri) { e_next = j; l0_next = tri_best[(base + j) * 2]; l1_next = tri_best[(base + j) * 2 + 1]; }
+    else { e_next = ev_idx[base + j]; v_next = nom[base + j]; }
   };
   fetch(j0 + lane);
   for (; j0 < ui.n_ev; j0 += step) {
     const int j = j0 + lane, e = e_next;
     uint4 v = v_next;
+    const ulonglong2 l0 = l0_next, l1 = l1_next;
     fetch(j + step);
     const bool valid = j < ui.n_ev;
-    int slot = -1, kind = 0, bi = -1, si = -1;
+    int slot = -1, kind = 0, bi = -1, si = -1, ci = -1, di = -1;
     bool merge = false;
     if (valid) {
       float best = -CUDART_INF_F, second = -CUDART_INF_F;
-      for (int c = 0;;) {   // chunks hold ascending slots: strict comparisons keep the lower slot on ties
+      if constexpr (kTri) {
+        // Two lists of two, as the entry was a row and as it was a column.  In either, equal keys have equal cosines and the lower
+        // slot is in front; between them they can differ by rounding, so everything that is close to the best is looked at.
+        const unsigned long long first = l0.x > l1.x ? l0.x : l1.x, other = l0.x > l1.x ? l1.x : l0.x;
+        auto val = [](unsigned long long y) { return y ? __uint_as_float((uint32_t)(y >> 32)) : -CUDART_INF_F; };
+        auto idx = [](unsigned long long y) { return y ? (int)(0xffffffffu - (uint32_t)y) : -1; };
+        best = val(first);
+        bi = idx(first);
+        second = fmaxf(val(other), fmaxf(val(l0.y), val(l1.y)));
+        auto close = [&](unsigned long long y) { return y && !(best - val(y) > kRankEps) ? idx(y) : -1; };
+        si = close(other);
+        ci = close(l0.y);
+        di = close(l1.y);
+      } else for (int c = 0;;) {   // chunks hold ascending slots: strict comparisons keep the lower slot on ties
         const int vi[2] = {(int)v.z, (int)v.w};
         const float vv[2] = {__uint_as_float(v.x), __uint_as_float(v.y)};
 #pragma unroll
@@ -386,7 +405,7 @@ resolve_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, const int32_
       }
       if (bi >= 0) {
         slot = bi;
-        if (!(best - second > kRankEps)) kind = si >= 0 ? 1 : 2;
+        if (!(best - second > kRankEps)) kind = kTri || si >= 0 ? 1 : 2;
         else if (!(fabsf(best - T) > kRankEps)) kind = 2;
         else merge = best > T;
       }
@@ -394,12 +413,20 @@ resolve_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, const int32_
     // ---- rows that need the interface's exact arithmetic, one after the other
     for (unsigned need = __ballot_sync(0xffffffffu, kind != 0); need; need &= need - 1) {
       const int l = __ffs(need) - 1, ee = __shfl_sync(0xffffffffu, e, l), ca = __shfl_sync(0xffffffffu, bi, l);
-      const int cb = __shfl_sync(0xffffffffu, kind == 1 ? si : bi, l);
+      const int cb = __shfl_sync(0xffffffffu, kind == 1 && si >= 0 ? si : bi, l);
       float u0, u1;
       exact_cosines<D>(sK + (size_t)ee * D, dK + (size_t)ca * D, dK + (size_t)cb * D, ke_s[warp], &kc_s[warp][0][0], u0, u1);
       int win = ca;
       float wu = u0;
       if (u1 > u0 || (u1 == u0 && cb < ca)) { win = cb; wu = u1; }
+      if (kTri && __shfl_sync(0xffffffffu, max(ci, di), l) >= 0) {
+        int cc = __shfl_sync(0xffffffffu, ci, l), cd = __shfl_sync(0xffffffffu, di, l);
+        if (cc < 0) cc = cd;
+        if (cd < 0) cd = cc;
+        exact_cosines<D>(sK + (size_t)ee * D, dK + (size_t)cc * D, dK + (size_t)cd * D, ke_s[warp], &kc_s[warp][0][0], u0, u1);
+        if (u0 > wu || (u0 == wu && cc < win)) { win = cc; wu = u0; }
+        if (u1 > wu || (u1 == wu && cd < win)) { win = cd; wu = u1; }
+      }
       if (lane == l) { slot = win; merge = wu > T; }
     }
     if (valid) target[base + e] = merge ? slot : -1;
@@ -588,10 +615,11 @@ static void launch_compress_t(const keepkv_params &p, const keepkv_cache &src, c
              merges ? norm_ext : nullptr);
   KEEPKV_CHECK_LAUNCH(ctx);
   if (!merges) return;
-  launch_nominate(p, src, dst, ev_idx, ui, inv_norm, norm_ext, sched, nom, L.nom_chunks, status_dev, ctx);
-  launch_pdl(resolve_kernel<D>, dim3(resolve_grid(p), U), dim3(kResolveThreads), 0, ctx.stream,
+  launch_nominate(p, src, dst, ev_idx, ui, inv_norm, norm_ext, sched, nom, L.nom_chunks, status_dev, ctx,
+                  budget_dev ? p.N_cap / 10 : ret_bound);
+  launch_pdl(resolve_kernel<D, false>, dim3(resolve_grid(p), U), dim3(kResolveThreads), 0, ctx.stream,
       p, src, dst, ev_idx, ui, nom, sched, target, grp_key, L.key_stride, grp_head,
-      stats, 0);
+      stats, 0, (const ulonglong2 *)nullptr);
   KEEPKV_CHECK_LAUNCH(ctx);
   if (!all_small(p, budget_dev, budget_scalar)) {
     launch_pdl(group_kernel<D>, dim3(U), dim3(kGroupThreads), (size_t)group_words(p, L) * 4, ctx.stream, p, src, dst,
@@ -659,7 +687,7 @@ static int norm_grid(const keepkv_params &p) {
 template <int D>
 __global__ void __launch_bounds__(256)
 mf_prepare_kernel(keepkv_params p, keepkv_cache src, int32_t *ev_idx, UnitInfo *unit_info, float *__restrict__ inv_norm,
-                  uint4 *__restrict__ norm_ext) {
+                  uint4 *__restrict__ norm_ext, uint4 *__restrict__ tri_best) {
   pdl_wait();
   pdl_trigger();
   const int u = blockIdx.y, b = u / p.H_kv;
@@ -673,6 +701,7 @@ mf_prepare_kernel(keepkv_params p, keepkv_cache src, int32_t *ev_idx, UnitInfo *
     inv_norm[base + i] = rsqrtf(ss);
     norm_ext[base + i] = ext_col(sqrtf(ss));
     ev_idx[base + i] = i;
+    if (tri_best) tri_best[(base + i) * 2] = tri_best[(base + i) * 2 + 1] = make_uint4(0, 0, 0, 0);
   });
 }
 
@@ -813,14 +842,18 @@ static void launch_compress_merge_first_t(const keepkv_params &p, const keepkv_c
     cudaFuncSetAttribute(group_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGroupSmem);
     attr_done_dev[dev & 63] = true;
   }
+  // The search's lists, 32 bytes a row, lie where the scratch cache's keys come later.
+  unsigned long long *tri_best = nominate_pairs(p, p.N_cap) ? reinterpret_cast<unsigned long long *>(scratch.K) : nullptr;
   // ---- pass 1: similar entries merged with each other, cache -> scratch (every head keeps its own length for now)
-  launch_pdl(mf_prepare_kernel<D>, dim3(norm_grid(p), U), dim3(256), 0, ctx.stream, p, cache, ev_idx, ui, inv_norm, norm_ext);
+  launch_pdl(mf_prepare_kernel<D>, dim3(norm_grid(p), U), dim3(256), 0, ctx.stream, p, cache, ev_idx, ui, inv_norm, norm_ext,
+             reinterpret_cast<uint4 *>(tri_best));
   KEEPKV_CHECK_LAUNCH(ctx);
   // rows and columns are the same keys: the "retained" operand of the search is the prompt itself
-  launch_nominate(p, cache, cache, ev_idx, ui, inv_norm, norm_ext, sched, nom, L.nom_chunks, status_dev, ctx, 1);
-  launch_pdl(resolve_kernel<D>, dim3(resolve_grid(p), U), dim3(kResolveThreads), 0, ctx.stream,
-      p, cache, cache, ev_idx, ui, nom, sched, target, grp_key, L.key_stride, grp_head,
-      st1, 1);
+  launch_nominate(p, cache, cache, ev_idx, ui, inv_norm, norm_ext, sched, nom, L.nom_chunks, status_dev, ctx, p.N_cap, 1,
+                  tri_best);
+  launch_pdl(tri_best ? resolve_kernel<D, true> : resolve_kernel<D, false>, dim3(resolve_grid(p), U), dim3(kResolveThreads), 0,
+      ctx.stream, p, cache, cache, ev_idx, ui, nom, sched, target, grp_key, L.key_stride, grp_head,
+      st1, 1, (const ulonglong2 *)tri_best);
   KEEPKV_CHECK_LAUNCH(ctx);
   launch_pdl(mf_mark_kernel, dim3(U), dim3(1024), 0, ctx.stream, p, unit_len, ret1, target, ev_idx, grp_head, grp_key,
              L.key_stride, ui, st1);
@@ -983,10 +1016,10 @@ static void launch_compress_inplace_t(const keepkv_params &p, const keepkv_cache
   if (merges) {
     launch_pdl(ip_columns_kernel, dim3((U + 127) / 128), dim3(128), 0, ctx.stream, ui, U);
     KEEPKV_CHECK_LAUNCH(ctx);
-    launch_nominate(p, c, c, ev_idx, ui, inv_norm, norm_ext, sched, nom, L.nom_chunks, status_dev, ctx);
-    launch_pdl(resolve_kernel<D>, dim3(resolve_grid(p), U), dim3(kResolveThreads), 0, ctx.stream,
+    launch_nominate(p, c, c, ev_idx, ui, inv_norm, norm_ext, sched, nom, L.nom_chunks, status_dev, ctx, 0);
+    launch_pdl(resolve_kernel<D, false>, dim3(resolve_grid(p), U), dim3(kResolveThreads), 0, ctx.stream,
         p, c, c, ev_idx, ui, nom, sched, target, grp_key, L.key_stride, grp_head,
-        stats, 0);
+        stats, 0, (const ulonglong2 *)nullptr);
     KEEPKV_CHECK_LAUNCH(ctx);
     if (!all_small(p, budget_dev, budget_scalar)) {
       launch_pdl(group_kernel<D>, dim3(U), dim3(kGroupThreads), (size_t)group_words(p, L) * 4, ctx.stream, p, c, c,

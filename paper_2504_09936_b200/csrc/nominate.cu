@@ -39,6 +39,8 @@ constexpr int kNomDrainWarps = 16;
 constexpr int kNomGatherWarps = 2; // (20 warps in all: 96 registers a thread)
 constexpr int kNomThreads = 32 * (2 + kNomGatherWarps + kNomDrainWarps);
 constexpr float kNomStatic = 0.5f; // thresholds from here on are subtracted by the product
+constexpr int kNomPairCap = 4096;  // capacity and retained keys from which on pairs of CTAs search
+constexpr int kNomPairColumns = 800;
 
 template <int D>
 struct NomSmem {
@@ -511,9 +513,23 @@ static void launch_nominate_t(const keepkv_params &p, const keepkv_cache &src, c
   KEEPKV_CHECK_LAUNCH(ctx);
 }
 
+// Large prompts go to pairs of CTAs (nominate_pair.cu).  The buffer's capacity stands for their length, which the host does not know;
+// columns: how many retained keys it expects a unit to have, 0 where most rows have none or few are evicted (in place).  The whole
+// call, this form against pairs, us, 8 and 64 units: 4096 -> 410 entries 46.2 / 47.4 and 101 / 110, 4096 -> 1229 52.1 / 52.6 and
+// 131 / 129, 6000 -> 600 52.5 / 53.8 and 141 / 146, 6000 -> 1800 61.5 / 60.4 and 213 / 191, 8100 -> 810 66.0 / 64.7 and 206 / 195,
+// 12000 -> 3600 124 / 115 and 602 / 531; all pairs of 2500 100 / 102 and 316 / 290, of 4096 130 / 123 and 548 / 474.  (64 channels:
+// 16 units of 20000 -> 4000 553 / 694.)
+bool nominate_pairs(const keepkv_params &p, int columns) {
+  return p.d == 128 && p.merge_threshold >= kNomStatic && p.N_cap >= kNomPairCap && columns >= kNomPairColumns;
+}
+
 void launch_nominate(const keepkv_params &p, const keepkv_cache &src, const keepkv_cache &dst, const int32_t *ev_idx,
                      const UnitInfo *unit_info, const float *inv_norm, const uint4 *norm_ext, int32_t *sched, uint4 *nom,
-                     int nom_chunks, int32_t *status_dev, LaunchCtx &ctx, int self_mask) {
+                     int nom_chunks, int32_t *status_dev, LaunchCtx &ctx, int columns, int self_mask, unsigned long long *tri_best) {
+  if (tri_best || nominate_pairs(p, columns)) {
+    launch_nominate_pairs(p, src, dst, ev_idx, unit_info, inv_norm, norm_ext, sched, nom, nom_chunks, status_dev, ctx, tri_best);
+    return;
+  }
   const bool cut = p.merge_threshold >= kNomStatic;
   auto launch = p.d == 128 ? (cut ? launch_nominate_t<128, true> : launch_nominate_t<128, false>)
                            : (cut ? launch_nominate_t<64, true> : launch_nominate_t<64, false>);

@@ -1147,6 +1147,66 @@ def test_prefill_compression_merge_first_policy(d, G, T, guard):
     assert hd.seq_len[1] == 0 and hd.seq_len[2] == 1
 
 
+@pytest.mark.parametrize("d,n,T", [(128, 255, 0.8), (64, 257, 0.8), (128, 257, 0.8), (128, 513, 0.5), (128, 1300, 0.8), (128, 2100, 0.9)])
+def test_merge_first_equal_keys_far_apart(d, n, T):
+    """The merge-first search takes one product for two cosines and keeps what an entry hears from later and from earlier
+    entries apart: copies of a key in every 256-entry tile (equal cosines on both sides: the lowest index is the partner),
+    noisy copies around them, every length that ends a tile or just passes it, in a buffer that the search by pairs of CTAs takes
+    (not at 64 channels).  Kept rows and votes exact, rows rounded."""
+    B = 3
+    n_cap = 4096
+    lens = [n, n - 1, max(1, n - 256)]
+    p = kb.make_params(B=B, H_q=1, H_kv=1, d=d, N_cap=n_cap, period=0, n_sink=0, n_recent=0, merge_threshold=T,
+                       gamma_min=-math.inf, gamma_max=math.inf)
+    rng = np.random.default_rng(n + d)
+    K = rng.standard_normal((B, n_cap, d)).astype(np.float32)
+    for b in range(B):
+        base = 3.0 * rng.standard_normal((20, d)).astype(np.float32)
+        at = rng.permutation(lens[b])[:lens[b] // 2]
+        K[b, at] = base[rng.integers(0, 20, len(at))] + rng.choice([0.0, 0.0, 0.7], (len(at), 1)) * rng.standard_normal((len(at), d))
+    cache = random_cache(p, lens, seed=5, vote_max=3, scored_frac=1.0)
+    cache.K.copy_(f32_to_dev_bf16(K).view(B, 1, n_cap, d))
+    cache.lscore.mul_(0.25).add_(1.5)
+    scratch = kb.Cache.empty(p)
+    ret = torch.full((B, n_cap), -7, dtype=torch.int32, device="cuda")
+    ws, st = kb.new_workspace(p), kb.new_status()
+    hs = HostCache(cache)
+    kb.keepkv_compress_merge_first(p, cache, scratch, n_cap, ws, st, retained_idx=ret)
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0
+    hd = HostCache(cache)
+    for b in range(B):
+        ref = O.merge_similar(oracle_params(p), *hs.unit(b))
+        m = len(ref["ret_idx"])
+        assert ref["stats"]["n_merged"] >= lens[b] // 8
+        assert int(hd.seq_len[b]) == m
+        assert np.array_equal(ret[b, :m].cpu().numpy(), ref["ret_idx"])
+        dK, dV, dvotes, _ = hd.unit(b)
+        assert np.array_equal(dvotes, ref["votes"])
+        check_close(dK, ref["K"], f"K b={b}")
+        check_close(dV, ref["V"], f"V b={b}")
+
+
+@pytest.mark.parametrize("budget,T,n_cap", [(801, 0.5, 4096), (832, 0.8, 4096), (897, 0.6, 4160), (960, 0.7, 8192)])
+def test_compress_search_by_pairs_of_ctas(budget, T, n_cap):
+    """The search for large prompts: rows in tiles of 256 and columns in tiles of 128, one more and one less than both, a unit
+    that evicts nothing, a second half of a pair without rows, equal keys in different tiles."""
+    B, d, n_recent = 8, 128, 500
+    lens = [budget + e for e in (1, 127, 129, 255, 257, 513, 800)] + [budget - 5]
+    p = kb.make_params(B=B, H_q=4, H_kv=1, d=d, N_cap=n_cap, n_sink=4, n_recent=n_recent, merge_threshold=T)
+    rng = np.random.default_rng(budget)
+    centers = 3.0 * rng.standard_normal((60, d))
+    K = centers[rng.integers(0, 60, (B, n_cap))] + rng.choice([0.0, 0.6, 3.0], (B, n_cap, 1)) * rng.standard_normal((B, n_cap, d))
+    src = random_cache(p, lens, seed=budget, vote_max=3, scored_frac=1.0)
+    src.K.copy_(f32_to_dev_bf16(K.astype(np.float32)).view(B, 1, n_cap, d))
+    src.lscore.mul_(0.25).add_(1.5)
+    dst, ret, tgt, stats = _run_compress(p, src, budget if n_cap < 8192 else torch.full((B,), budget, dtype=torch.int32, device="cuda"))
+    assert stats[:, kb.STATS_FIELDS.index("n_merged")].sum() > 200
+    hs, hd = HostCache(src), HostCache(dst)
+    for u in range(B):
+        check_compress_unit(p, u, budget, n_recent, hs, hd, ret, tgt, stats, what="pairs")
+
+
 def _check_inplace_unit(p, u, budget, n_recent, before: HostCache, pos_before, after: HostCache, pos_after, moved, tgt, stats,
                         what, max_tolerated=0):
     """One unit of keepkv_compress_inplace against the oracle fed the same rows and positions: targets, moves and

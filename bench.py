@@ -503,7 +503,7 @@ def run_ours(args, w, rank, world):
             "achieved": inc_gbs, "peak": hbm, "unit": "GB/s", "frac": inc_gbs / hbm, "peak_source": src, "traffic": None,
             "bytes_per_call": inc_bytes, "us_per_call": t_inc_compress * 1e6},
         "roofline_compress_full": {
-            "bound": "tensor", "kernel": "nominate_kernel (similarity search of the first compression)",
+            "bound": "tensor", "kernel": "nominate_pair_kernel or nominate_kernel (similarity search of the first compression)",
             "achieved": gemm_flops / t_full_compress / 1e12, "peak": tens, "unit": "TFLOP/s",
             "frac": gemm_flops / t_full_compress / 1e12 / tens, "peak_source": src + " (sustained bf16)", "traffic": None,
             "flops_per_call": gemm_flops, "us_per_call": t_full_compress * 1e6},

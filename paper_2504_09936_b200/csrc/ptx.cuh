@@ -278,8 +278,9 @@ __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// The two halves of that barrier.
+// The two halves of that barrier; the relaxed arrival orders no memory.
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 // Address of this CTA's shared-memory location `addr` in the CTA of rank `rank` of the cluster, and a store to it.
 __device__ __forceinline__ uint32_t mapa_shared(uint32_t addr, uint32_t rank) {

@@ -54,3 +54,16 @@ def test_products_and_their_commits_are_issued_by_the_elected_thread(name):
                 assert any("elect_one()" in g for g in guards + [body[last:m.start()]]), (kernel, body[last:m.end()])
                 continue
             last = m.end()
+
+
+@pytest.mark.parametrize("name", SOURCES)
+def test_other_ctas_shared_memory_is_written_behind_a_cluster_barrier(name):
+    """A CTA may write to its neighbours' shared memory, or arrive at their barriers, when all of the cluster have started: the
+    whole barrier, or its waiting half, stands in front, and every thread of the CTA has arrived before its ways part."""
+    for kernel, body in kernels(name):
+        remote = re.search(r"\b(?:st_shared_cluster_\w+|mbar_arrive_cluster)\(", body)
+        if remote:
+            front = body[:remote.start()]
+            assert "cluster_wait()" in front or "cluster_sync_all()" in front, kernel
+            arrival = re.search(r"cluster_arrive\w*\(\)|cluster_sync_all\(\)", front).start()
+            assert "return;" not in front[:arrival], kernel

@@ -314,11 +314,12 @@ int keepkv_decode_attention_static(const keepkv_params *p, const keepkv_cache *c
                                    float *lse_or_null, int update_scores, int32_t *status_dev, void *stream);
 
 /* Test hook, not for production use: process-wide settings of the decode launches (keepkv_decode_attention,
- * keepkv_decode_step, their host and static variants) and of the KEEPKV_FLAG_COMPRESS_STEADY compressions that follow.
+ * keepkv_decode_step, their host and static variants) and of the compressions that follow.
  * spin_limit > 0 replaces the number of polls after which a
  * bounded wait inside the kernel gives up (0 restores the default).  withhold_tile >= 0 makes every CTA announce
- * the tile (compression: the block of value rows) at that position of its sequence without ever issuing its copies, so
- * that the wait for it runs out: the call then returns normally, KEEPKV_DEV_TIMEOUT is raised in *status_dev and the outputs of
+ * the tile (KEEPKV_FLAG_COMPRESS_STEADY: the block of value rows; other compressions: the tile of retained keys of the
+ * similarity search, of a search by pairs of CTAs the half tile, those of the two CTAs in turn) at that position of its
+ * sequence without ever issuing its copies, so that the wait for it runs out: the call then returns normally, KEEPKV_DEV_TIMEOUT is raised in *status_dev and the outputs of
  * that call are unspecified; -1 restores normal operation.  This is how the kernels' timeout path is exercised
  * without faulting or hanging a GPU. */
 int keepkv_debug_decode(int spin_limit, int withhold_tile);

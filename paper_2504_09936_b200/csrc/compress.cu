@@ -391,7 +391,9 @@ resolve_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, const int32_
         di = close(l1.y);
       } else for (int c = 0;;) {   // chunks hold ascending slots: strict comparisons keep the lower slot on ties
         const int vi[2] = {(int)v.z, (int)v.w};
-        const float vv[2] = {__uint_as_float(v.x), __uint_as_float(v.y)};
+        // (A search that gave up has left rows as they were: what names no slot is no candidate.)
+        const float vv[2] = {v.z < (uint32_t)ui.n_ret ? __uint_as_float(v.x) : -CUDART_INF_F,
+                             v.w < (uint32_t)ui.n_ret ? __uint_as_float(v.y) : -CUDART_INF_F};
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
           const bool p1 = vv[t] > best, p2 = vv[t] > second;

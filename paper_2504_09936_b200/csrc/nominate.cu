@@ -115,7 +115,8 @@ __global__ void __launch_bounds__(kNomThreads, 1)
 nominate_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, const __nv_bfloat16 *__restrict__ srcK,
                 const int32_t *__restrict__ ev_idx, const UnitInfo *__restrict__ unit_info,
                 const float *__restrict__ inv_norm, const uint4 *__restrict__ norm_ext, int32_t *sched,
-                uint4 *__restrict__ nom, int C_max, int32_t *status_dev, int self_mask) {
+                uint4 *__restrict__ nom, int C_max, int32_t *status_dev, int self_mask,
+                int spin_limit, int withhold) {
   using SL = NomSmem<D>;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   // a_ready[2], a_empty[2], b_full[4], b_empty[4], t_full[2], t_empty[2], drain, x_full[4][2]
@@ -208,7 +209,7 @@ nominate_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, const
     int ring = 0, n_tiles = 0;
     bool ok = true;
     for (int n_done = 0; ok; ++n_done) {   // (watches the rows' barrier only: an item's last product waits for its columns)
-      if (!__all_sync(0xffffffffu, !s_abort && mbar_wait(bar_a_ready + 8 * (n_done & 1), (n_done >> 1) & 1))) { s_abort = 1; break; }
+      if (!__all_sync(0xffffffffu, !s_abort && mbar_wait_n(bar_a_ready + 8 * (n_done & 1), (n_done >> 1) & 1, spin_limit))) { s_abort = 1; break; }
       const NomItem it = s_item[n_done & 1];
       if (it.n_ev < 0) break;
       for (int t = it.t0; ok && t < it.t1; ++t, ++n_tiles) {
@@ -216,9 +217,9 @@ nominate_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, const
 #pragma unroll
         for (int sub = 0; sub < SL::kSub; ++sub, ++ring) {
           const int s = ring % kNomStages;
-          ok = __all_sync(0xffffffffu, !s_abort && mbar_wait(bar_b_empty + 8 * s, ((ring / kNomStages) & 1) ^ 1));
+          ok = __all_sync(0xffffffffu, !s_abort && mbar_wait_n(bar_b_empty + 8 * s, ((ring / kNomStages) & 1) ^ 1, spin_limit));
           if (!ok) { s_abort = 1; break; }
-          if (elect_one()) {
+          if (n_tiles != withhold && elect_one()) {   // (test hook: this tile is never asked for)
             const uint32_t full = bar_b_full + 8 * s;
             const bool last = sub == SL::kSub - 1;
             mbar_expect_tx(full, SL::kBBytes + (last ? kNomN * 20 : 0));
@@ -238,7 +239,7 @@ nominate_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, const
     bool ok = true;
     for (int n_done = 0; ok; ++n_done) {
       const int buf = n_done & 1;
-      ok = __all_sync(0xffffffffu, !s_abort && mbar_wait(bar_a_ready + 8 * buf, (n_done >> 1) & 1));
+      ok = __all_sync(0xffffffffu, !s_abort && mbar_wait_n(bar_a_ready + 8 * buf, (n_done >> 1) & 1, spin_limit));
       if (!ok) break;
       const NomItem it = s_item[buf];
       if (it.n_ev < 0) break;
@@ -246,11 +247,11 @@ nominate_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, const
         const int a = acc & 1;
         // a unit's last tile is multiplied as far as it has columns, in sixteens
         const uint32_t idesc = umma_idesc_bf16(kNomM, min(kNomN, (it.n_ret - t * kNomN + 15) & ~15));
-        ok = __all_sync(0xffffffffu, !s_abort && mbar_wait(bar_t_empty + 8 * a, ((acc >> 1) & 1) ^ 1));
+        ok = __all_sync(0xffffffffu, !s_abort && mbar_wait_n(bar_t_empty + 8 * a, ((acc >> 1) & 1) ^ 1, spin_limit));
 #pragma unroll
         for (int sub = 0; sub < SL::kSub; ++sub, ++ring) {
           const int s = ring % kNomStages;
-          ok = ok && __all_sync(0xffffffffu, !s_abort && mbar_wait(bar_b_full + 8 * s, (ring / kNomStages) & 1));
+          ok = ok && __all_sync(0xffffffffu, !s_abort && mbar_wait_n(bar_b_full + 8 * s, (ring / kNomStages) & 1, spin_limit));
           if (!ok) break;
           tc_fence_after();
           if (elect_one()) {
@@ -277,7 +278,7 @@ nominate_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, const
     }
     if (!ok) s_abort = 1;
     if (elect_one()) umma_commit(bar_drain);
-    mbar_wait(bar_drain, 0);   // every product issued above has retired (bounded)
+    mbar_wait_n(bar_drain, 0, spin_limit);   // every product issued above has retired (bounded)
   } else if (warp < 2 + kNomGatherWarps) {
     // ------------------------------------------------------------ rows of the next item, kNomM / kNomGatherWarps a warp
     // Asynchronous copies straight into the swizzled tile, all in flight together; then a row per lane for the norms.
@@ -300,7 +301,7 @@ nominate_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, const
       int mine[RW / 32];
 #pragma unroll
       for (int k = 0; k < RW / 32; ++k) mine[k] = it.n_ev >= 0 && m0 + 32 * k + lane < it.n_ev ? ev_idx[ubase + m0 + 32 * k + lane] : -1;
-      if (n_done >= 2 && !__all_sync(0xffffffffu, !s_abort && mbar_wait(bar_a_empty + 8 * buf, ((n_done >> 1) - 1) & 1))) {
+      if (n_done >= 2 && !__all_sync(0xffffffffu, !s_abort && mbar_wait_n(bar_a_empty + 8 * buf, ((n_done >> 1) - 1) & 1, spin_limit))) {
         s_abort = 1;
         break;
       }
@@ -358,7 +359,7 @@ nominate_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, const
     int acc = 0, x_phase = 0;   // x_phase: a bit per set of A tiles
     for (int n_done = 0;; ++n_done) {
       const int buf = n_done & 1;
-      if (!__all_sync(0xffffffffu, !s_abort && mbar_wait(bar_a_ready + 8 * buf, (n_done >> 1) & 1))) { s_abort = 1; break; }
+      if (!__all_sync(0xffffffffu, !s_abort && mbar_wait_n(bar_a_ready + 8 * buf, (n_done >> 1) & 1, spin_limit))) { s_abort = 1; break; }
       const NomItem it = s_item[buf];
       if (it.n_ev < 0) break;
       const size_t ubase = (size_t)it.u * p.N_cap;
@@ -374,7 +375,7 @@ nominate_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, const
       bool ok = true;
       for (int t = it.t0; t < it.t1; ++t, ++acc) {
         const int a = acc & 1;
-        ok = __all_sync(0xffffffffu, !s_abort && mbar_wait(bar_t_full + 8 * a, (acc >> 1) & 1));
+        ok = __all_sync(0xffffffffu, !s_abort && mbar_wait_n(bar_t_full + 8 * a, (acc >> 1) & 1, spin_limit));
         if (!ok) break;
         tc_fence_after();
         const int c0 = t * kNomN + cq * 64, n_valid = it.n_ret - c0;   // this warp's columns that exist, if positive
@@ -452,7 +453,7 @@ nominate_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, const
         __syncwarp();
         if (lane == 0) mbar_arrive(xbar + 8 * buf);
       } else {
-        if (!__all_sync(0xffffffffu, !s_abort && mbar_wait(xbar + 8 * buf, (x_phase >> buf) & 1))) { s_abort = 1; break; }
+        if (!__all_sync(0xffffffffu, !s_abort && mbar_wait_n(xbar + 8 * buf, (x_phase >> buf) & 1, spin_limit))) { s_abort = 1; break; }
 #pragma unroll
         for (int w = 0; w < 3; ++w) {
           const uint32_t sl = x[3 * w + 2];
@@ -477,7 +478,7 @@ nominate_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, const
     if (tid == 0) {
       atomicOr(status_dev, KEEPKV_DEV_TIMEOUT);
       // copies still in flight get a bounded chance to land before the shared memory goes away
-      for (int i = 0; i < kNomStages; ++i) { mbar_wait(bar_b_full + 8 * i, 0); mbar_wait(bar_b_full + 8 * i, 1); }
+      for (int i = 0; i < kNomStages; ++i) { mbar_wait_n(bar_b_full + 8 * i, 0, spin_limit); mbar_wait_n(bar_b_full + 8 * i, 1, spin_limit); }
     }
     __syncthreads();
   }
@@ -509,7 +510,7 @@ static void launch_nominate_t(const keepkv_params &p, const keepkv_cache &src, c
   }
   launch_pdl(nominate_kernel<D, kCut>, dim3(sm_count()), dim3(kNomThreads), smem_bytes, ctx.stream,
       mapB, p, reinterpret_cast<const __nv_bfloat16 *>(src.K), ev_idx, unit_info, inv_norm, norm_ext, sched, nom,
-      nom_chunks, status_dev, self_mask);
+      nom_chunks, status_dev, self_mask, debug_spin_limit(), debug_withhold());
   KEEPKV_CHECK_LAUNCH(ctx);
 }
 

@@ -142,7 +142,7 @@ nominate_pair_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, 
                 const int32_t *__restrict__ ev_idx, const UnitInfo *__restrict__ unit_info,
                 const float *__restrict__ inv_norm, const uint4 *__restrict__ norm_ext, int32_t *sched,
                 uint4 *__restrict__ nom, int C_max, int32_t *status_dev,
-                unsigned long long *__restrict__ tri_best) {
+                unsigned long long *__restrict__ tri_best, int spin_limit, int withhold) {
   using SL = PairSmem<D>;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   constexpr int kStages = SL::kTiles;
@@ -246,7 +246,7 @@ nominate_pair_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, 
       int n_tiles = 0;
       bool ok = true;
       for (int n_done = 0; ok; ++n_done) {   // (watches the rows' barrier only: an item's last product waits for its columns)
-        ok = mbar_wait_or(bar_a_ready + 8 * (n_done & 1), (n_done >> 1) & 1, &s_abort);
+        ok = mbar_wait_or(bar_a_ready + 8 * (n_done & 1), (n_done >> 1) & 1, spin_limit, &s_abort);
         if (!ok) break;
         const PairItem it = s_item[n_done & 1];
         if (it.n_ev < 0) break;
@@ -255,8 +255,9 @@ nominate_pair_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, 
           const int first = it.u * p.N_cap + t * kPairN, row = first + (int)rank * (pair_cols(it, t) / 2);
           const int s = n_tiles % kStages;
           const uint32_t full = bar_b_full + 8 * s;
-          ok = mbar_wait_or(bar_b_empty + 8 * s, ((n_tiles / kStages) & 1) ^ 1, &s_abort);
+          ok = mbar_wait_or(bar_b_empty + 8 * s, ((n_tiles / kStages) & 1) ^ 1, spin_limit, &s_abort);
           if (!ok) break;
+          if (2 * n_tiles + (int)rank == withhold) continue;   // (test hook: this half of a tile is never asked for)
           mbar_expect_tx(full, SL::kBBytes + kPairHalf * 16 + kPairN * 4);
           tma_load_3d(sbase + SL::kB + s * SL::kBBytes, &mapB, 0, row, 0, full);
           bulk_load_1d(sbase + SL::kBX + s * (kPairHalf * 16), norm_ext + row, kPairHalf * 16, full);
@@ -274,7 +275,7 @@ nominate_pair_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, 
       const uint32_t zero = sbase + SL::kZero;
       for (int n_done = 0; ok; ++n_done) {
         const int buf = n_done & 1;
-        ok = mbar_wait_or(bar_rows + 8 * buf, (n_done >> 1) & 1, &s_abort);
+        ok = mbar_wait_or(bar_rows + 8 * buf, (n_done >> 1) & 1, spin_limit, &s_abort);
         if (!ok) break;
         const PairItem it = s_item[buf];
         if (it.n_ev < 0) break;
@@ -283,8 +284,8 @@ nominate_pair_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, 
           const int a = acc % kPairAcc, s = acc % kStages;
           const uint32_t idesc = umma_idesc_bf16(kPairRows, pair_cols(it, t)), dt = tmem + a * kPairN;
           const uint64_t bd = umma_desc_sw128(sbase + SL::kB + s * SL::kBBytes);
-          ok = mbar_wait_or(bar_b_full + 8 * s, (acc / kStages) & 1, &s_abort) &&
-               mbar_wait_or(bar_t_empty + 8 * a, ((acc / kPairAcc) & 1) ^ 1, &s_abort);
+          ok = mbar_wait_or(bar_b_full + 8 * s, (acc / kStages) & 1, spin_limit, &s_abort) &&
+               mbar_wait_or(bar_t_empty + 8 * a, ((acc / kPairAcc) & 1) ^ 1, spin_limit, &s_abort);
           if (!ok) break;
           tc_fence_after();
 #pragma unroll
@@ -301,7 +302,7 @@ nominate_pair_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, 
       }
       if (!ok) s_abort = 1;
       umma_commit(CtaPair{}, bar_drain);
-      mbar_wait(bar_drain, 0);   // every product issued above has retired (bounded)
+      mbar_wait_n(bar_drain, 0, spin_limit);   // every product issued above has retired (bounded)
     }
     __syncwarp();
   } else if (warp == 1) {
@@ -311,19 +312,19 @@ nominate_pair_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, 
       int n_tiles = 0;
       bool ok = true;
       for (int n_done = 0; ok; ++n_done) {
-        ok = mbar_wait_or(bar_a_ready + 8 * (n_done & 1), (n_done >> 1) & 1, &s_abort);
+        ok = mbar_wait_or(bar_a_ready + 8 * (n_done & 1), (n_done >> 1) & 1, spin_limit, &s_abort);
         if (!ok) break;
         const PairItem it = s_item[n_done & 1];
         if (it.n_ev < 0) break;
         for (int i = it.t1 - it.t0; i > 0; --i, ++n_tiles) {
           const int s = n_tiles % kStages;
-          ok = mbar_wait_or(bar_b_full + 8 * s, (n_tiles / kStages) & 1, &s_abort);
+          ok = mbar_wait_or(bar_b_full + 8 * s, (n_tiles / kStages) & 1, spin_limit, &s_abort);
           if (!ok) break;
           mbar_arrive_cluster(peer + 8 * s);
         }
       }
       if (!ok) s_abort = 1;
-      mbar_wait(bar_drain, 0);
+      mbar_wait_n(bar_drain, 0, spin_limit);
     }
     __syncwarp();
   } else if (warp < 2 + kPairGatherWarps) {
@@ -352,7 +353,7 @@ nominate_pair_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, 
       int mine[RW / 32];
 #pragma unroll
       for (int k = 0; k < RW / 32; ++k) mine[k] = it.n_ev >= 0 && m0 + 32 * k + lane < it.n_ev ? ev_idx[ubase + m0 + 32 * k + lane] : -1;
-      if (n_done >= 2 && !__all_sync(0xffffffffu, !s_abort && mbar_wait(bar_a_empty + 8 * buf, ((n_done >> 1) - 1) & 1))) {
+      if (n_done >= 2 && !__all_sync(0xffffffffu, !s_abort && mbar_wait_n(bar_a_empty + 8 * buf, ((n_done >> 1) - 1) & 1, spin_limit))) {
         s_abort = 1;
         break;
       }
@@ -415,7 +416,7 @@ nominate_pair_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, 
     int told_slot = 0, told_to = 0, n_told = 0;
     for (int n_done = 0;; ++n_done) {
       const int buf = n_done & 1;
-      if (!__all_sync(0xffffffffu, !s_abort && mbar_wait(bar_a_ready + 8 * buf, (n_done >> 1) & 1))) { s_abort = 1; break; }
+      if (!__all_sync(0xffffffffu, !s_abort && mbar_wait_n(bar_a_ready + 8 * buf, (n_done >> 1) & 1, spin_limit))) { s_abort = 1; break; }
       const PairItem it = s_item[buf];
       if (it.n_ev < 0) break;
       const size_t ubase = (size_t)it.u * p.N_cap;
@@ -432,7 +433,7 @@ nominate_pair_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, 
       for (int t = it.t0; t < it.t1; ++t, ++acc) {
         if (acc % kPairAcc != grp) continue;
         const bool beyond = t / (kPairRows / kPairN) > it.m0 / kPairRows;   // (of a square on the diagonal both halves are multiplied)
-        ok = __all_sync(0xffffffffu, mbar_wait_or(bar_t_full + 8 * grp, (acc / kPairAcc) & 1, &s_abort));
+        ok = __all_sync(0xffffffffu, mbar_wait_or(bar_t_full + 8 * grp, (acc / kPairAcc) & 1, spin_limit, &s_abort));
         if (!ok) break;
         tc_fence_after();
         const int c0 = t * kPairN, n_valid = min(kPairN, it.n_ret - c0);   // columns that exist
@@ -530,7 +531,7 @@ nominate_pair_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, 
         __syncwarp();
         if (lane == 0) mbar_arrive(xbar + 8 * buf);
       } else {
-        if (!__all_sync(0xffffffffu, !s_abort && mbar_wait(xbar + 8 * buf, (x_phase >> buf) & 1))) { s_abort = 1; break; }
+        if (!__all_sync(0xffffffffu, !s_abort && mbar_wait_n(xbar + 8 * buf, (x_phase >> buf) & 1, spin_limit))) { s_abort = 1; break; }
         if (lane == 0) s_done[buf][quarter] = 0;
 #pragma unroll
         for (int w = 0; w < 3; ++w) {
@@ -557,7 +558,7 @@ nominate_pair_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, 
     if (tid == 0) {
       atomicOr(status_dev, KEEPKV_DEV_TIMEOUT);
       // copies still in flight get a bounded chance to land before the shared memory goes away
-      for (int i = 0; i < kStages; ++i) { mbar_wait(bar_b_full + 8 * i, 0); mbar_wait(bar_b_full + 8 * i, 1); }
+      for (int i = 0; i < kStages; ++i) { mbar_wait_n(bar_b_full + 8 * i, 0, spin_limit); mbar_wait_n(bar_b_full + 8 * i, 1, spin_limit); }
     }
     __syncthreads();
   }
@@ -590,7 +591,7 @@ static void launch_pairs_t(const keepkv_params &p, const keepkv_cache &src, cons
   }
   launch_pdl_cluster(nominate_pair_kernel<D, kTri>, dim3(sm_count() & ~1), dim3(kPairThreads), smem_bytes, ctx.stream, 2u, mapB, p,
                      reinterpret_cast<const __nv_bfloat16 *>(src.K), ev_idx, unit_info, inv_norm, norm_ext, sched, nom, nom_chunks,
-                     status_dev, tri_best);
+                     status_dev, tri_best, debug_spin_limit(), debug_withhold());
   KEEPKV_CHECK_LAUNCH(ctx);
 }
 

@@ -53,9 +53,9 @@ __device__ __forceinline__ bool mbar_wait_n(uint32_t bar, uint32_t parity, int l
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) { return mbar_wait_n(bar, parity, kSpinLimit); }
 
 // The same for a loop in which every step counts: no vote, and the abort flag is only looked at while there is nothing to do.
-__device__ __forceinline__ bool mbar_wait_or(uint32_t bar, uint32_t parity, const volatile int *abort) {
+__device__ __forceinline__ bool mbar_wait_or(uint32_t bar, uint32_t parity, int limit, const volatile int *abort) {
   if (mbar_try_wait(bar, parity)) return true;
-  for (int it = 0; it < kSpinLimit && !*abort; ++it)
+  for (int it = 0; it < limit && !*abort; ++it)
     if (mbar_try_wait(bar, parity)) return true;
   return false;
 }

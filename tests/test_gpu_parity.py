@@ -1207,6 +1207,42 @@ def test_compress_search_by_pairs_of_ctas(budget, T, n_cap):
         check_compress_unit(p, u, budget, n_recent, hs, hd, ret, tgt, stats, what="pairs")
 
 
+@pytest.mark.parametrize("merge_first", [False, True])
+@pytest.mark.parametrize("d,n_cap,withhold", [(128, 4096, 0), (128, 4096, 1), (128, 4096, 5), (128, 1728, 0), (64, 1728, 1)])
+def test_similarity_search_bounded_wait_runs_out_and_the_next_call_is_normal(d, n_cap, withhold, merge_first):
+    """Retained keys that never come, of one CTA of a pair (a tile of every CTA, where CTAs search alone), in a workspace whose
+    lists name no entry: the call returns with KEEPKV_DEV_TIMEOUT, and the next one gives the bits it gives without all this."""
+    B, n, budget = 24, 1700, 820
+    p = kb.make_params(B=B, H_q=1, H_kv=1, d=d, N_cap=n_cap, n_sink=4, n_recent=400, merge_threshold=0.5)
+    src = random_cache(p, [n - 7 * i for i in range(B)], seed=d, vote_max=3, scored_frac=1.0)
+    ws, st = kb.new_workspace(p), kb.new_status()
+
+    def call():
+        cache, other = kb.Cache(*(t.clone() for t in (src.K, src.V, src.votes, src.lscore, src.seq_len))), kb.Cache.empty(p)
+        if merge_first:
+            kb.keepkv_compress_merge_first(p, cache, other, budget, ws, st)
+        else:
+            kb.keepkv_compress(p, cache, other, budget, ws, st)
+        torch.cuda.synchronize()
+        kept = cache if merge_first else other
+        return [t[:, :, :budget].contiguous().view(torch.uint8) for t in (kept.K, kept.V, kept.votes, kept.lscore)] + [kept.seq_len]
+
+    want = call()
+    assert int(st.item()) == 0
+    ws.fill_(0x5A)
+    kb._check(kb.lib().keepkv_workspace_init(kb.C.byref(p), ws.data_ptr(), ws.numel(), kb._stream()), "keepkv_workspace_init")
+    try:
+        kb.keepkv_debug_decode(spin_limit=4096, withhold_tile=withhold)
+        call()
+    finally:
+        kb.keepkv_debug_decode(0, -1)
+    assert int(st.item()) == kb.DEV_TIMEOUT
+    st.zero_()
+    for x, y in zip(call(), want):
+        assert torch.equal(x, y)
+    assert int(st.item()) == 0
+
+
 def _check_inplace_unit(p, u, budget, n_recent, before: HostCache, pos_before, after: HostCache, pos_after, moved, tgt, stats,
                         what, max_tolerated=0):
     """One unit of keepkv_compress_inplace against the oracle fed the same rows and positions: targets, moves and

@@ -16,6 +16,11 @@
 // per 256 columns: pairs with two accumulators 2189 (2853 with arrivals of the cluster's scope), copies and products
 // issued by one thread's loops 2041, four accumulators with groups 2064, the last group to be done folding an item 2018, one copy of
 // the code behind the screen 1876.
+// Where half a block's groups of four columns hold a candidate all its columns are looked at in line.  Keys along a common direction,
+// three quarters of the pairs above the threshold: 64 units of 8191 -> 1638 (the call) 1314 us with a loop over the groups, 1105 now,
+// 1161 in nominate.cu's form; merge-first, 32 units of 6007, 21.5 ms with an offer to a column for every pair, 1.03 ms with one for the
+// best of 32 rows, 1.05 ms in nominate.cu's form (0.92 / 0.97 / 1.42 ms for 64 centres).  With candidates rare the calls take as long
+// as before.
 // With 64 channels a tile's products are half as long as its drain, and this form is up to a quarter slower than nominate.cu's.
 // Every wait is bounded; a wait that runs out raises KEEPKV_DEV_TIMEOUT, every warp of the CTA leaves its loop, what is
 // in flight gets a bounded time to end, the pair meets, tensor memory is freed.
@@ -30,6 +35,8 @@ constexpr int kPairN = 128;         // retained columns per tile
 constexpr int kPairHalf = kPairN / 2; // ... of which a CTA holds these many
 constexpr int kPairAcc = 4;         // accumulators, each with a group of four drain warps
 constexpr int kPairDrainWarps = 4 * kPairAcc;
+constexpr int kPairMany = 4;        // of the eight groups of four columns of a block, see the drain
+constexpr int kPairTold = 32;       // entries of a drain warp's stash of offers; up to eight come at a time
 constexpr int kPairGatherWarps = 2; // (20 warps in all: 96 registers a thread)
 constexpr int kPairThreads = 32 * (2 + kPairGatherWarps + kPairDrainWarps);
 
@@ -52,15 +59,61 @@ struct PairSmem {
   static constexpr int kXchg = kRowInv + 2 * kPairM * 4;        // u32 [2][128][3][3]  results of the groups that are done first
   static constexpr int kCoarse = kXchg + 2 * kPairM * 36;       // i32 [kMaxUnits / 32]  row tiles before each 32 units
   static constexpr int kBytes = kCoarse + kMaxUnits / 32 * 4;
+  static constexpr int kTold = kXchg;   // a triangle's stashes of offers: nothing is exchanged there
+  static_assert(kTold % 16 == 0 && kPairDrainWarps * kPairTold * 16 <= 2 * kPairM * 36, "the stashes take the place of the exchange");
 };
 
 // Two words hold the two largest cosines offered so far, with their slots, in any order of the offers: equal values go to
-// the lower slot.  (All of them are above the threshold, so their bits are in order; an empty word is zero.)
+// the lower slot.  (Only positive ones count, so their bits are in order; an empty word is zero.  A look at the second word first is
+// a trip to L2 that few offers save: 447 -> 441 us for merge-first compressions without it.)
+__device__ __forceinline__ unsigned long long tri_word(float v, int slot) {
+  return (unsigned long long)__float_as_uint(v) << 32 | (0xffffffffu - (unsigned)slot);
+}
 __device__ __forceinline__ void tri_offer(unsigned long long *best, float v, int slot) {
-  const unsigned long long x = (unsigned long long)__float_as_uint(v) << 32 | (0xffffffffu - (unsigned)slot);
-  if (!(v > 0.f) || x <= __ldcg(best + 1)) return;
+  if (!(v > 0.f)) return;
+  const unsigned long long x = tri_word(v, slot);
   const unsigned long long old = atomicMax(best, x), less = old < x ? old : x;
   if (less) atomicMax(best + 1, less);
+}
+
+// Of the lanes m those with the two largest values (positive; of equal ones the lowest lanes).
+__device__ __forceinline__ unsigned two_largest(unsigned m, float v) {
+  const int lane = threadIdx.x & 31;
+  uint32_t left = m >> lane & 1u ? __float_as_uint(v) : 0u;
+  m = 0;
+#pragma unroll 1
+  for (int k = 0; k < 2; ++k) {
+    const uint32_t most = __reduce_max_sync(0xffffffffu, left);
+    const int l = __ffs(__ballot_sync(0xffffffffu, left == most)) - 1;
+    m |= 1u << l;
+    if (lane == l) left = 0u;
+  }
+  return m;
+}
+
+// A block of cosines, 32 rows (lanes) by 32 columns (r, positive floats): every lane gets the largest value of one column, its row --
+// of equal values the lowest -- and the second largest value.  Halves of the columns are exchanged between neighbouring ranges
+// of rows, step by step: 31 exchanges for the block.
+struct ColumnTop { uint32_t best, second; int row; };
+template <int kDist>
+__device__ __forceinline__ ColumnTop column_meet(const ColumnTop &lo, const ColumnTop &hi) {   // of the lower and the higher column
+  const bool up = threadIdx.x & kDist;
+  const ColumnTop own = up ? hi : lo, give = up ? lo : hi;
+  ColumnTop got;
+  got.best = __shfl_xor_sync(0xffffffffu, give.best, kDist);
+  got.second = kDist > 1 ? __shfl_xor_sync(0xffffffffu, give.second, kDist) : 0u;
+  got.row = kDist > 1 ? __shfl_xor_sync(0xffffffffu, give.row, kDist) : (int)((threadIdx.x & 31) ^ 1);
+  ColumnTop t;
+  t.row = got.best + (up ? 1u : 0u) > own.best ? got.row : own.row;   // (the upper lanes' partner has the lower rows)
+  t.best = max(own.best, got.best);
+  t.second = max(min(own.best, got.best), max(own.second, got.second));
+  return t;
+}
+// Column kFirst and the columns behind it, as many as lanes are met.
+template <int kDist, int kFirst, int kN>
+__device__ __forceinline__ ColumnTop column_top(const uint32_t (&r)[kN]) {
+  if constexpr (kDist == 0) return ColumnTop{r[kFirst], 0u, (int)(threadIdx.x & 31)};
+  else return column_meet<kDist>(column_top<kDist / 2, kFirst>(r), column_top<kDist / 2, kFirst + kDist>(r));
 }
 
 struct __align__(16) PairItem { int u, m0, chunk, t0, t1, n_ev, n_ret, pad; };
@@ -411,9 +464,25 @@ nominate_pair_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, 
     const float *rowinv = reinterpret_cast<const float *>(smem + SL::kRowInv);
     uint32_t *xchg = reinterpret_cast<uint32_t *>(smem + SL::kXchg);
     int acc = 0, x_phase = 0;   // x_phase: a bit per set of A tiles
-    // kTri: cosines that columns have yet to hear, one a lane: an offer is two trips to L2, which 32 of them make together
-    float told_v = 0.f;
-    int told_slot = 0, told_to = 0, n_told = 0;
+    // kTri: cosines that columns have yet to hear.  An offer is two trips to L2, which up to 32 of them make together.
+    const uint32_t told = sbase + SL::kTold + ew * (kPairTold * 16);   // uint4 [kPairTold]  value, row, column
+    int n_told = 0;
+    auto offer_told = [&] {
+      __syncwarp();
+      if (lane < n_told) {
+        const uint4 x = ld_shared_v4(told + lane * 16);
+        tri_offer(tri_best + (size_t)x.z * 4 + 2, __uint_as_float(x.x), (int)x.y);
+      }
+      __syncwarp();
+      n_told = 0;
+    };
+    // Lanes m have v for column `to`.  Of the warp's rows only two can be among the column's two best.
+    auto tell = [&](unsigned m, float v, int row, int to) {
+      if (__popc(m) > 2) m = two_largest(m, v);
+      if (m >> lane & 1u)
+        st_shared_v4(told + (n_told + __popc(m & ((1u << lane) - 1u))) * 16, make_uint4(__float_as_uint(v), (uint32_t)row, (uint32_t)to, 0u));
+      n_told += __popc(m);
+    };
     for (int n_done = 0;; ++n_done) {
       const int buf = n_done & 1;
       if (!__all_sync(0xffffffffu, !s_abort && mbar_wait_n(bar_a_ready + 8 * buf, (n_done >> 1) & 1, spin_limit))) { s_abort = 1; break; }
@@ -421,23 +490,23 @@ nominate_pair_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, 
       if (it.n_ev < 0) break;
       const size_t ubase = (size_t)it.u * p.N_cap;
       const bool row_ok = it.m0 + row < it.n_ev;
-      // Values are compared before the division by |k_e|: the closeness margin and the threshold scale with it.
+      // Values are compared before the division by |k_e|.
       const float rinv = rowinv[buf * kPairM + row];
       const bool live = it.m0 + quarter * 32 < it.n_ev;   // some of this warp's rows exist
       Top2 top, topb;   // two lists over alternate columns: two independent dependency chains
-      top.init(2.f * kRankEps / rinv);
-      topb.init(top.thr);
+      top.init(0.f);
+      topb.init(0.f);
       const float cut0 = (p.merge_threshold - 2.f * kRankEps) / rinv;
-      top.cut = row_ok && rinv < CUDART_INF_F ? cut0 : CUDART_INF_F;
       bool ok = true;
       for (int t = it.t0; t < it.t1; ++t, ++acc) {
         if (acc % kPairAcc != grp) continue;
         const bool beyond = t / (kPairRows / kPairN) > it.m0 / kPairRows;   // (of a square on the diagonal both halves are multiplied)
+        const int c0 = t * kPairN, n_valid = min(kPairN, it.n_ret - c0);   // columns that exist
         ok = __all_sync(0xffffffffu, mbar_wait_or(bar_t_full + 8 * grp, (acc / kPairAcc) & 1, spin_limit, &s_abort));
         if (!ok) break;
         tc_fence_after();
-        const int c0 = t * kPairN, n_valid = min(kPairN, it.n_ret - c0);   // columns that exist
         const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + grp * kPairN;
+        const uint32_t inv = sbase + SL::kInv + acc % SL::kInvTiles * (kPairN * 4);
         // rows and columns are the same entries: the column of the row's own key does not count
         const int diag = kTri ? it.m0 + row - c0 : -1;
         const int diag0 = it.m0 + quarter * 32 - c0;
@@ -453,7 +522,6 @@ nominate_pair_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, 
             for (int i = 0; i < 32; ++i)
               if (off + i >= n_valid || off + i == diag) r[i] = 0xff800000u;   // -inf
           }
-          const float4 *wv = reinterpret_cast<const float4 *>(smem + SL::kInv + acc % SL::kInvTiles * (kPairN * 4)) + off / 4;
           // groups of four columns; what lies above the row's cut is positive (NaNs never show)
           float gm[8];
 #pragma unroll
@@ -461,39 +529,99 @@ nominate_pair_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, 
             gm[i] = max3(fmaxf(__uint_as_float(r[4 * i]), __uint_as_float(r[4 * i + 1])), __uint_as_float(r[4 * i + 2]), __uint_as_float(r[4 * i + 3]));
           const float all = max3(max3(gm[0], gm[1], gm[2]), max3(gm[3], gm[4], gm[5]), fmaxf(gm[6], gm[7]));
           if (__any_sync(0xffffffffu, all > 0.f)) {
-            uint32_t some = 0;
+            uint32_t some = 0;   // groups of columns with a candidate
 #pragma unroll
             for (int i = 0; i < 8; ++i) some |= gm[i] > 0.f ? 1u << i : 0u;
             some = __reduce_or_sync(0xffffffffu, some);
-            // An eighth of the blocks, and mostly one group of theirs: read once more, so that there is one copy of this code
-            // (with eight copies of it, a tile took 1009 cycles, with one 938).
-#pragma unroll 1
-            for (; some; some &= some - 1) {
-              const int i = __ffs(some) - 1, c = c0 + off + 4 * i;
-              uint32_t q[4];
-              tmem_ld_32x4(taddr + off + 4 * i, q);
-              const float4 w = wv[i];
-              tmem_ld_wait();
-              float v[4] = {__uint_as_float(q[0]), __uint_as_float(q[1]), __uint_as_float(q[2]), __uint_as_float(q[3])};
-              const float n[4] = {w.x, w.y, w.z, w.w};
+            if (__popc(some) >= kPairMany) {
+              // Prompts of similar keys: the price of a block does not depend on how many pairs pass.  The rows' lists take all of
+              // them, the columns' what is best for each among the warp's rows.
 #pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                const bool counts = off + 4 * i + j < n_valid && off + 4 * i + j != diag;
-                v[j] = counts ? fmaf(v[j], fabsf(n[j]), cut0) : -CUDART_INF_F;
+              for (int i = 0; i < 8; ++i) {
+                const float4 w = ld_shared_f4(inv + (off + 4 * i) * 4);
+                const int c = c0 + off + 4 * i;
+                const float v[4] = {fmaf(__uint_as_float(r[4 * i]), fabsf(w.x), cut0), fmaf(__uint_as_float(r[4 * i + 1]), fabsf(w.y), cut0),
+                                    fmaf(__uint_as_float(r[4 * i + 2]), fabsf(w.z), cut0), fmaf(__uint_as_float(r[4 * i + 3]), fabsf(w.w), cut0)};
+                top.insert(v[0], c);
+                topb.insert(v[1], c + 1);
+                top.insert(v[2], c + 2);
+                topb.insert(v[3], c + 3);
               }
-              top.insert(v[0], c);
-              topb.insert(v[1], c + 1);
-              top.insert(v[2], c + 2);
-              topb.insert(v[3], c + 3);
-              if (kTri && beyond) {   // what the columns are to hear
+              if (kTri && beyond) {
+                unsigned long long *lists = tri_best + (ubase + c0 + off + lane) * 4 + 2;
+                const unsigned long long heard = off + lane < n_valid ? __ldcg(lists + 1) : ~0ull;
+                ColumnTop half[2];
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
-                  for (unsigned m = __ballot_sync(0xffffffffu, __uint_as_float(q[j]) > 0.f && v[j] > 0.f); m; m &= m - 1) {
-                    const int l = __ffs(m) - 1;
-                    const float pv = __shfl_sync(0xffffffffu, v[j] * rinv, l);
-                    if (lane == n_told) { told_v = pv; told_slot = it.m0 + quarter * 32 + l; told_to = (int)ubase + c + j; }
-                    if (++n_told == 32) { tri_offer(tri_best + (size_t)told_to * 4 + 2, told_v, told_slot); n_told = 0; }
+                for (int k = 0; k < 2; ++k) {   // (read once more: nothing spills)
+                  uint32_t q[16];
+                  tmem_ld_32x16(taddr + off + 16 * k, q);
+                  tmem_ld_wait();
+#pragma unroll
+                  for (int i = 0; i < 4; ++i) {
+                    const float4 w = ld_shared_f4(inv + (off + 16 * k + 4 * i) * 4);
+                    const float n[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)   // (a NaN is 0)
+                      q[4 * i + j] = __float_as_uint(fmaxf(fmaf(__uint_as_float(q[4 * i + j]), fabsf(n[j]), cut0) * rinv, 0.f));
                   }
+                  half[k] = column_top<8, 0>(q);
+                }
+                const ColumnTop mine = column_meet<16>(half[0], half[1]);
+
+                const float v = __uint_as_float(mine.best);
+                const int slot = it.m0 + quarter * 32 + mine.row;
+                const bool wants = v > p.merge_threshold - 2.f * kRankEps && tri_word(v, slot) > heard;
+                if (wants) tri_offer(lists, v, slot);
+                // (Seldom: rows of the warp that are as close to the column as its best but for the margin.  What is further
+                // below the warp's best is further below the column's, and the decision looks at nothing there.)
+                const float near = v - 2.f * kRankEps;
+#pragma unroll 1
+                for (unsigned ls = __ballot_sync(0xffffffffu, wants && __uint_as_float(mine.second) >= near); ls; ls &= ls - 1) {
+                  const int i = __ffs(ls) - 1;
+                  const int first = __shfl_sync(0xffffffffu, mine.row, i);
+                  const float lnear = __shfl_sync(0xffffffffu, near, i);
+                  uint32_t q;
+                  tmem_ld_32x1(taddr + off + i, q);
+                  const float n = ld_shared_f32(inv + (off + i) * 4);
+                  tmem_ld_wait();
+                  const float pv = fmaf(__uint_as_float(q), fabsf(n), cut0) * rinv;
+                  tell(__ballot_sync(0xffffffffu, pv >= lnear && lane != first), pv, it.m0 + row, (int)ubase + c0 + off + i);
+                  if (n_told > kPairTold - 8) offer_told();
+                }
+              }
+            } else {
+              // An eighth of the blocks, and mostly one group of theirs: read once more, so that there is one copy of this code
+              // (with eight copies of it, a tile took 1009 cycles, with one 938).
+#pragma unroll 1
+              for (; some; some &= some - 1) {
+                const int i = __ffs(some) - 1, c = c0 + off + 4 * i;
+                uint32_t q[4];
+                tmem_ld_32x4(taddr + off + 4 * i, q);
+                const float4 w = ld_shared_f4(inv + (off + 4 * i) * 4);
+                tmem_ld_wait();
+                float v[4] = {__uint_as_float(q[0]), __uint_as_float(q[1]), __uint_as_float(q[2]), __uint_as_float(q[3])};
+                const float n[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                  const bool counts = off + 4 * i + j < n_valid && off + 4 * i + j != diag;
+                  v[j] = counts ? fmaf(v[j], fabsf(n[j]), cut0) : -CUDART_INF_F;
+                }
+                top.insert(v[0], c);
+                topb.insert(v[1], c + 1);
+                top.insert(v[2], c + 2);
+                topb.insert(v[3], c + 3);
+                if (kTri && beyond) {   // what the columns are to hear
+                  uint32_t any4 = 0;
+#pragma unroll
+                  for (int j = 0; j < 4; ++j) any4 |= __uint_as_float(q[j]) > 0.f && v[j] > 0.f ? 1u << j : 0u;
+#pragma unroll 1
+                  for (unsigned js = __reduce_or_sync(0xffffffffu, any4); js; js &= js - 1) {
+                    const int j = __ffs(js) - 1;
+                    const float x = j & 2 ? (j & 1 ? v[3] : v[2]) : (j & 1 ? v[1] : v[0]);
+                    tell(__ballot_sync(0xffffffffu, any4 >> j & 1u), x * rinv, it.m0 + row, (int)ubase + c + j);
+                  }
+                  if (n_told > kPairTold - 8) offer_told();
+                }
               }
             }
           }
@@ -548,7 +676,7 @@ nominate_pair_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, 
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_a_empty + 8 * buf);
     }
-    if (kTri && lane < n_told) tri_offer(tri_best + (size_t)told_to * 4 + 2, told_v, told_slot);
+    if (kTri) offer_told();
   }
 
   // ---------------------------------------------------------------- teardown

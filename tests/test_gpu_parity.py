@@ -1207,6 +1207,61 @@ def test_compress_search_by_pairs_of_ctas(budget, T, n_cap):
         check_compress_unit(p, u, budget, n_recent, hs, hd, ret, tgt, stats, what="pairs")
 
 
+def _similar_keys(kind, U, n, d, seed):
+    """Keys [U, n, d] of which many pairs are similar: around common centres, along one direction (most cosines are above 0.8),
+    repeated, with every ninth row zero, or with every fortieth above 0.5 to all others, which are below it to one another."""
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    r = lambda *shape: torch.randn(*shape, device="cuda", generator=g)
+    if kind == "direction":
+        return 1.95 * r(U, 1, d) + r(U, n, d)
+    if kind == "hubs":
+        u, K = r(U, 1, d), r(U, n, d)
+        K += 0.8 * u
+        K[:, ::40] = u + 0.1 * K[:, ::40]
+        return K
+    centres = r(U, 50, d).gather(1, torch.randint(0, 50, (U, n, 1), device="cuda", generator=g).expand(-1, -1, d))
+    K = centres if kind == "repeated" else centres + 0.42 * r(U, n, d)
+    if kind == "zeros":
+        K[:, 4::9] = 0.0
+    return K
+
+
+@pytest.mark.parametrize("merge_first", [False, True])
+@pytest.mark.parametrize("kind", ["centres", "direction", "repeated", "zeros", "hubs"])
+def test_search_by_pairs_of_ctas_decides_as_the_other_search(kind, merge_first):
+    """The same prompts in a buffer of 4032 rows (one CTA searches) and of 4096 (pairs do): same bits.  Forty units, lengths of no
+    entry to 4000, so that rings, accumulators and lists of two levels are used many times over."""
+    B, H_kv, d, budget = 20, 2, 128, 900
+    lens = [4000, 0, 1, 2, 257, 901, 1000, 3999, 3841] + [3000 + 83 * i for i in range(B - 9)]
+    K = _similar_keys(kind, B * H_kv, 4032, d, seed=len(kind)).bfloat16().view(B, H_kv, 4032, d)
+    runs = []
+    for n_cap in (4032, 4096):
+        p = kb.make_params(B=B, H_q=H_kv, H_kv=H_kv, d=d, N_cap=n_cap, n_sink=4, n_recent=400, merge_threshold=0.5 if kind == "hubs" else 0.8)
+        g = torch.Generator(device="cuda").manual_seed(7)
+        cache, other = kb.Cache.empty(p), kb.Cache.empty(p)
+        cache.K[:, :, :4032] = K
+        cache.V[:, :, :4032] = torch.randn(B, H_kv, 4032, d, device="cuda", generator=g).bfloat16()
+        cache.lscore[:, :, :4032] = 0.25 * torch.randn(B, H_kv, 4032, device="cuda", generator=g) + 1.5
+        cache.seq_len.copy_(torch.tensor(lens, dtype=torch.int32))
+        ws, st = kb.new_workspace(p), kb.new_status()
+        ret = torch.full((B, H_kv, n_cap), -7, dtype=torch.int32, device="cuda")
+        stats = torch.zeros(B * H_kv, 8, dtype=torch.int32, device="cuda")
+        if merge_first:
+            kb.keepkv_compress_merge_first(p, cache, other, budget, ws, st, retained_idx=ret, stats=stats)
+        else:
+            kb.keepkv_compress(p, cache, other, budget, ws, st, retained_idx=ret, stats=stats)
+        torch.cuda.synchronize()
+        assert int(st.item()) == 0
+        kept = cache if merge_first else other
+        runs.append(([kept.K, kept.V, kept.votes, kept.lscore, ret], kept.seq_len, stats))
+    (x, len_x, stats_x), (y, len_y, stats_y) = runs
+    assert torch.equal(len_x, len_y) and torch.equal(stats_x, stats_y)
+    assert int(stats_x[:, kb.STATS_FIELDS.index("n_merged")].sum()) > 5000
+    for b, m in enumerate(len_x.tolist()):
+        for s, t in zip(x, y):
+            assert torch.equal(s[b, :, :m].contiguous().view(torch.uint8), t[b, :, :m].contiguous().view(torch.uint8)), b
+
+
 @pytest.mark.parametrize("merge_first", [False, True])
 @pytest.mark.parametrize("d,n_cap,withhold", [(128, 4096, 0), (128, 4096, 1), (128, 4096, 5), (128, 1728, 0), (64, 1728, 1)])
 def test_similarity_search_bounded_wait_runs_out_and_the_next_call_is_normal(d, n_cap, withhold, merge_first):

@@ -242,8 +242,11 @@ compact_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, const int32_
 // (Three distinct cosines within the accumulation error of each other, the one case this cannot
 // settle, would need a coincidence of order 1e-8 per row; exact duplicates are handled, because equal
 // keys give equal values and the lower slot stays in front.)
-// Rows that need the exact chain are taken one after the other by the warp that finds them (coalesced row
-// loads into shared memory, the sequential chains on three lanes).  Bound: the latency of a row's list; so the warps of the
+// Rows that need the exact chain are evaluated by the warp that finds them.  One or two: coalesced row loads into shared memory, the
+// sequential chains on three lanes.  More: ten at a time (six of a triangle), every candidate is a lane's, which walks its row and
+// the evicted one's in global memory (64 units, keys that repeat 27 times: 6554 rows a unit 1143 -> 840 us the call, 128 rows 127 -> 85;
+// 101 with a queue that the CTA's warps shared.  But a lone row takes twice as long, and in line the code cost the call 0.5 %).
+// Bound: the latency of a row's list; so the warps of the
 // resident CTAs (two per SM) walk the rows on their own, the next lists on their way, and no barrier is met: 64 units of 6554
 // rows 19 -> 13 us, 128 of up to 14746 41 -> 26 us against a CTA per 512 rows with a common queue and place in the list (and
 // lists whose chunks lay side by side, so that a row's sector was mostly unused).  A unit of at most kResolveThreads evicted
@@ -253,6 +256,7 @@ compact_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, const int32_
 constexpr int kMergeInline = 32;   // units with at most this many groups are merged where group_and_merge sorts them
 constexpr int kResolveThreads = 512;
 constexpr int kResolveWarps = kResolveThreads / 32;
+constexpr int kResolveFew = 2;
 constexpr int kGroupThreads = 1024;
 constexpr int kGroupSmem = 212992; // bytes of counters and keys group_kernel may hold
 constexpr int kGroupRank = 128;    // members of one group up to which a key finds its place among its neighbours
@@ -328,6 +332,45 @@ __device__ __forceinline__ void group_and_merge(const keepkv_params &p, const ke
   }
 }
 
+
+// The rows of lanes `need` in the interface's exact arithmetic, several at a time: a row is entry e, its candidates c0 and, of those that
+// are not negative, c1 to c3.  Returned: the best slot, with the sign bit where it is not above T.  (Not in line: most warps never come here.)
+template <int D, bool kTri>
+__device__ __noinline__ int exact_many(unsigned need, int e, int c0, int c1, int c2, int c3, const __nv_bfloat16 *sK, const __nv_bfloat16 *dK,
+                                       float T) {
+  constexpr int kCand = kTri ? 4 : 2, kLanes = kCand + 1, kRows = 32 / kLanes;   // a lane for each candidate and one for the row's norm
+  const int lane = threadIdx.x & 31, g = lane / kLanes, role = lane - g * kLanes;
+  int out = -1;
+  while (need) {
+    unsigned m = need;
+    for (int k = 0; k < g; ++k) m &= m - 1;
+    const int l = m ? __ffs(m) - 1 : 0;
+    const int ee = __shfl_sync(0xffffffffu, e, l);
+    int c = __shfl_sync(0xffffffffu, c0, l);
+    const int d1 = __shfl_sync(0xffffffffu, c1, l), d2 = __shfl_sync(0xffffffffu, c2, l), d3 = __shfl_sync(0xffffffffu, c3, l);
+    const int other = role == 2 ? d1 : role == 3 ? d2 : role == 4 ? d3 : -1;
+    if (other >= 0) c = other;
+    float u = 0.f, nn = 0.f;
+    if (m && g < kRows) exact_dot<D>(sK + (size_t)ee * D, role ? dK + (size_t)c * D : sK + (size_t)ee * D, u, nn);
+    const float ne = __shfl_sync(0xffffffffu, nn, min(g * kLanes, 31));
+    u = u / (sqrtf(ne) * sqrtf(nn));
+    const int at = __popc(need & ((1u << lane) - 1u));   // the row's place among those that are left
+    const bool mine = (need >> lane & 1u) && at < kRows;
+    int win = 0;
+    float wu = 0.f;
+#pragma unroll
+    for (int k = 0; k < kCand; ++k) {
+      const int from = mine ? at * kLanes + 1 + k : 0;
+      const float uk = __shfl_sync(0xffffffffu, u, from);
+      const int ck = __shfl_sync(0xffffffffu, c, from);
+      if (k == 0 || uk > wu || (uk == wu && ck < win)) { win = ck; wu = uk; }
+    }
+    if (mine) out = wu > T ? win : (int)0x80000000 | win;
+#pragma unroll
+    for (int k = 0; k < kRows; ++k) need &= need - 1;
+  }
+  return out;
+}
 
 // kTri: the search's lists are those of a triangle.
 template <int D, bool kTri>
@@ -412,8 +455,9 @@ resolve_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, const int32_
         else merge = best > T;
       }
     }
-    // ---- rows that need the interface's exact arithmetic, one after the other
-    for (unsigned need = __ballot_sync(0xffffffffu, kind != 0); need; need &= need - 1) {
+    // ---- rows that need the interface's exact arithmetic: one or two of them one after the other, more at a time
+    unsigned need = __ballot_sync(0xffffffffu, kind != 0);
+    for (; need && __popc(need) <= kResolveFew; need &= need - 1) {
       const int l = __ffs(need) - 1, ee = __shfl_sync(0xffffffffu, e, l), ca = __shfl_sync(0xffffffffu, bi, l);
       const int cb = __shfl_sync(0xffffffffu, kind == 1 && si >= 0 ? si : bi, l);
       float u0, u1;
@@ -430,6 +474,10 @@ resolve_kernel(keepkv_params p, keepkv_cache src, keepkv_cache dst, const int32_
         if (u1 > wu || (u1 == wu && cd < win)) { win = cd; wu = u1; }
       }
       if (lane == l) { slot = win; merge = wu > T; }
+    }
+    if (need) {
+      const int win = exact_many<D, kTri>(need, e, bi, kTri || kind == 1 ? si : -1, ci, di, sK, dK, T);
+      if (kind) { slot = win & 0xffff; merge = win >= 0; }
     }
     if (valid) target[base + e] = merge ? slot : -1;
     if (decide_only) continue;   // the caller pairs the entries itself (merge-first policy): the partner above T, or -1

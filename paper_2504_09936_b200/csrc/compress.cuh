@@ -224,6 +224,26 @@ __device__ __forceinline__ void exact_cosines(const __nv_bfloat16 *ke, const __n
   ub = __shfl_sync(0xffffffffu, uu, 1);
 }
 
+// The same sums by one thread: x . y and |y|^2.
+template <int D>
+__device__ __forceinline__ void exact_dot(const __nv_bfloat16 *x, const __nv_bfloat16 *y, float &dot, float &nn) {
+  const uint4 *xp = reinterpret_cast<const uint4 *>(x), *yp = reinterpret_cast<const uint4 *>(y);
+  dot = nn = 0.f;
+#pragma unroll 2
+  for (int k = 0; k < D / 8; ++k) {
+    const uint4 a = xp[k], b = yp[k];
+    const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, bw[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float b0 = bf16_lo(bw[q]), b1 = bf16_hi(bw[q]);
+      dot = fmaf(bf16_lo(aw[q]), b0, dot);
+      nn = fmaf(b0, b0, nn);
+      dot = fmaf(bf16_hi(aw[q]), b1, dot);
+      nn = fmaf(b1, b1, nn);
+    }
+  }
+}
+
 // ------------------------------------------------------------------ merge
 // One warp per group.  With a_i = ln p_i + lscore_i over the group K'_e (target first, then members
 // ascending):  omega = softmax(a),  v_r = sum omega_i v_i,  k_r = gamma * sum omega_i k_i,

@@ -1207,6 +1207,26 @@ def test_compress_search_by_pairs_of_ctas(budget, T, n_cap):
         check_compress_unit(p, u, budget, n_recent, hs, hd, ret, tgt, stats, what="pairs")
 
 
+@pytest.mark.parametrize("d,n,budget,copies", [(64, 700, 572, 3), (128, 700, 572, 40), (64, 1500, 600, 2), (128, 1500, 600, 25)])
+def test_compress_rows_that_need_the_exact_cosines(d, n, budget, copies):
+    """One row of a warp, a few, and all of them whose best cosines are equal or closer than the ranking's error: the lower slot
+    of equal ones, the larger of the others, in the interface's arithmetic."""
+    B, n_recent = 3, 300
+    p = kb.make_params(B=B, H_q=1, H_kv=1, d=d, N_cap=1536, n_sink=4, n_recent=n_recent, merge_threshold=0.6)
+    rng = np.random.default_rng(d + n)
+    centers = rng.standard_normal((B, -(-n // copies), d)).astype(np.float32)
+    K = np.repeat(centers, copies, axis=1)[:, rng.permutation(n)]
+    K[:, ::5] *= 1.0 + 2.0 ** -7                      # parallel keys: cosines that differ in the last places only
+    src = random_cache(p, [n, n - 1, n - 130], seed=d + copies, vote_max=3, scored_frac=1.0)
+    src.K[:, :, :n].copy_(f32_to_dev_bf16(K).view(B, 1, n, d))
+    src.lscore.mul_(0.25).add_(1.5)
+    dst, ret, tgt, stats = _run_compress(p, src, budget)
+    assert stats[0, kb.STATS_FIELDS.index("n_merged")] > 10
+    hs, hd = HostCache(src), HostCache(dst)
+    for u in range(B):
+        check_compress_unit(p, u, budget, n_recent, hs, hd, ret, tgt, stats, what="exact")
+
+
 def _similar_keys(kind, U, n, d, seed):
     """Keys [U, n, d] of which many pairs are similar: around common centres, along one direction (most cosines are above 0.8),
     repeated, with every ninth row zero, or with every fortieth above 0.5 to all others, which are below it to one another."""

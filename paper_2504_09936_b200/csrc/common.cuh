@@ -5,6 +5,7 @@
 #include <math_constants.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <utility>
 
 #include "keepkv.h"
@@ -142,6 +143,30 @@ inline void launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, 
   cfg.attrs = attr;
   cfg.numAttrs = 2;
   cudaLaunchKernelEx(&cfg, kernel, KArgs(std::forward<Args>(args))...);
+}
+// Clusters of k <= 8 CTAs of a kernel with two CTAs per SM that are resident at once: twice those of one CTA per SM, which is what
+// is asked for (one_cta_smem: more than half of an SM's shared memory).  A device's answer is kept, a failed query is not.
+template <auto kKernel>
+inline int resident_clusters(int dev, int k, int threads, size_t one_cta_smem) {
+  static std::atomic<int> known[64][9];
+  std::atomic<int> &at = known[dev & 63][k];
+  int n = at.load(std::memory_order_relaxed);
+  if (n == 0) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)k);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = one_cta_smem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)k;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&n, kKernel, &cfg) != cudaSuccess) { (void)cudaGetLastError(); return 0; }
+    n = 2 * n + 1;   // (odd: never 0)
+    at.store(n, std::memory_order_relaxed);
+  }
+  return n - 1;
 }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

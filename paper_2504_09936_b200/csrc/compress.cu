@@ -901,7 +901,9 @@ static void launch_compress_merge_first_t(const keepkv_params &p, const keepkv_c
   // rows and columns are the same keys: the "retained" operand of the search is the prompt itself
   launch_nominate(p, cache, cache, ev_idx, ui, inv_norm, norm_ext, sched, nom, L.nom_chunks, status_dev, ctx, p.N_cap, 1,
                   tri_best);
-  launch_pdl(tri_best ? resolve_kernel<D, true> : resolve_kernel<D, false>, dim3(resolve_grid(p), U), dim3(kResolveThreads), 0,
+  auto resolve = resolve_kernel<D, false>;
+  if constexpr (D == 128) { if (tri_best) resolve = resolve_kernel<D, true>; }   // (the search by pairs takes 128 channels)
+  launch_pdl(resolve, dim3(resolve_grid(p), U), dim3(kResolveThreads), 0,
       ctx.stream, p, cache, cache, ev_idx, ui, nom, sched, target, grp_key, L.key_stride, grp_head,
       st1, 1, (const ulonglong2 *)tri_best);
   KEEPKV_CHECK_LAUNCH(ctx);

@@ -26,8 +26,6 @@
 // last CTA's, 29 groups on eight warps.  Shared out over the cluster: 40 us.
 // Every wait on the tensor core and on a bulk copy is bounded; one that runs out raises KEEPKV_DEV_TIMEOUT and the CTA goes
 // on without further products (its unit's result is then unspecified), frees its tensor memory and returns.
-#include <atomic>
-
 #include "compress.cuh"
 #include "ptx.cuh"
 
@@ -43,7 +41,7 @@ constexpr int kStN = 64;         // retained slots per tile (columns of the prod
 constexpr int kStTmemCols = 128; // two accumulators of kStN columns
 constexpr int kStRows = 32;      // rows of a block of values
 constexpr int kStOneCtaSmem = 120 * 1024;   // more than half of an SM's shared memory
-constexpr int kStMaxCtas = 8;    // CTAs per unit: a cluster
+constexpr int kStMaxCtas = kNomChunksMax;   // CTAs per unit: a cluster
 
 // Barriers of parts of the CTA.  (Not the aligned form: a warp may come to them from a branch of its lanes.)
 struct StSync { __device__ __forceinline__ void operator()() const { asm volatile("barrier.sync 1, 256;" ::: "memory"); } };
@@ -606,30 +604,6 @@ steady_compress_kernel(const __grid_constant__ CUtensorMap mapD, keepkv_params p
   count.flush(stats + u);
 }
 
-// Clusters of k CTAs that are resident at once: twice those of one CTA per SM (see decode.cu).  A device's answer is kept.
-template <typename K>
-static int steady_clusters(K kernel, int dev, int k) {
-  static std::atomic<int> known[64][kStMaxCtas + 1];
-  std::atomic<int> &at = known[dev & 63][k];
-  int n = at.load(std::memory_order_relaxed);
-  if (n == 0) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)k);
-    cfg.blockDim = dim3(kStAll);
-    cfg.dynamicSmemBytes = kStOneCtaSmem;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)k;
-    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) { (void)cudaGetLastError(); n = 0; }
-    n = 2 * n + 1;   // (odd: never 0)
-    at.store(n, std::memory_order_relaxed);
-  }
-  return n - 1;
-}
-
 template <int D>
 static void launch_steady_t(const keepkv_params &p, const keepkv_cache &src, const keepkv_cache &dst,
                             const int32_t *budget_dev, int32_t budget_scalar, const int32_t *n_recent_dev,
@@ -658,7 +632,7 @@ static void launch_steady_t(const keepkv_params &p, const keepkv_cache &src, con
   int R = 2 * sm_count() / U;
   R = R < 1 ? 1 : (R > L.nom_chunks ? L.nom_chunks : R);
   int k = R;
-  while (k > 1 && steady_clusters(steady_compress_kernel<D, true>, dev, k) < U) --k;
+  while (k > 1 && resident_clusters<steady_compress_kernel<D, true>>(dev, k, kStAll, kStOneCtaSmem) < U) --k;
   uint4 *nom = reinterpret_cast<uint4 *>(ws + L.nom);
   int *counters = reinterpret_cast<int *>(ws + L.counters);
   if (k > 1 && 4 * k >= 3 * R)

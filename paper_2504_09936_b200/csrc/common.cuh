@@ -31,7 +31,8 @@ struct WsLayout {
   size_t ev_idx;      // i32 [U,N]          source indices of evicted entries, ascending
   size_t inv_norm;    // f32 [U,N]          1/|k| of each retained key (tree-summed; only ranks candidates)
   size_t norm_ext;    // bf16 [U,N,8]       |k| of the same in three terms, as more channels of the search's columns
-  size_t nom;         // uint4 [C,U,N]      per column chunk and evicted row: best, second cosine (f32), their slots
+  size_t nom;         // uint4 [C,U,N]      per column chunk and evicted row: best, second cosine (f32), their slots ([U,N,C] in the
+                      //                    single-kernel compression)
   size_t grp_key;     // u32 [U,Npow2]      (slot << 16 | source index) of merged entries, sorted
   size_t grp_head;    // i32 [U,N]          position in grp_key where each group starts
   size_t stats;       // keepkv_stats [U]   used when the caller passes no stats array

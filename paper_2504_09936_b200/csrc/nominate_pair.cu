@@ -29,6 +29,7 @@
 
 namespace keepkv {
 
+constexpr int kPairD = 128;         // channels
 constexpr int kPairM = 128;         // evicted rows per CTA (tensor-memory lanes)
 constexpr int kPairRows = 2 * kPairM; // ... and per item, which is a pair of CTAs'
 constexpr int kPairN = 128;         // retained columns per tile
@@ -40,8 +41,8 @@ constexpr int kPairTold = 32;       // entries of a drain warp's stash of offers
 constexpr int kPairGatherWarps = 2; // (20 warps in all: 96 registers a thread)
 constexpr int kPairThreads = 32 * (2 + kPairGatherWarps + kPairDrainWarps);
 
-template <int D>
 struct PairSmem {
+  static constexpr int D = kPairD;
   static constexpr int kSub = D / 64;                     // 64-channel (128-byte) K atoms per row
   static constexpr int kABytes = kSub * kPairM * 128;
   static constexpr int kBBytes = kSub * kPairHalf * 128;   // a CTA's half of a column tile
@@ -189,14 +190,15 @@ __device__ __forceinline__ int pair_cols(const PairItem &it, int t) { return min
 // only.  A pair of CTAs walks an equal range of all triangles' tiles.  What is above the threshold is offered to the row's list as
 // before, and beyond the square on the diagonal to the column's as well; both are in global memory, two words each (tri_offer).
 // Half the products, and the power they take: merge-first compression of 32 units of 6007 entries 493 -> 436 us.
-template <int D, bool kTri>
+template <bool kTri>
 __global__ void __launch_bounds__(kPairThreads, 1)
 nominate_pair_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, const __nv_bfloat16 *__restrict__ srcK,
                 const int32_t *__restrict__ ev_idx, const UnitInfo *__restrict__ unit_info,
                 const float *__restrict__ inv_norm, const uint4 *__restrict__ norm_ext, int32_t *sched,
                 uint4 *__restrict__ nom, int C_max, int32_t *status_dev,
                 unsigned long long *__restrict__ tri_best, int spin_limit, int withhold) {
-  using SL = PairSmem<D>;
+  using SL = PairSmem;
+  constexpr int D = kPairD;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   constexpr int kStages = SL::kTiles;
   // a_ready[2], a_empty[2], t_full, drain, x_full[4][2], b_full, b_empty; of the pair's first CTA: t_empty, both CTAs' rows[2]
@@ -251,7 +253,7 @@ nominate_pair_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, 
     tmem_relinquish(CtaPair{});
   }
   int total_m = 0, t_max = 0;
-  {   // exclusive prefix of 128-row tiles over the units, kept for every 32nd: one unit per thread and pass
+  {   // exclusive prefix of the units' row tiles (or tiles of triangles), kept for every 32nd: one unit per thread and pass
     for (int u0 = 0; u0 < U; u0 += kPairThreads) {
       const int u = u0 + tid;
       int t = 0, cols = 0;
@@ -283,7 +285,7 @@ nominate_pair_kernel(const __grid_constant__ CUtensorMap mapB, keepkv_params p, 
 
   const uint32_t tmem = s_tmem;
   // Column chunks per row tile: what makes the longest CTA shortest, an item costing about a tile and a half beside its
-  // tiles (first columns, publishing).  Without chunks 192 items on 148 CTAs take as long as 296.
+  // tiles (first columns, publishing).  Without chunks 96 items on 74 pairs take as long as 148.
   int C = 1;
   if (!kTri) {
     int cost = 0x7fffffff;
@@ -705,22 +707,21 @@ template <bool kTri>
 static void launch_pairs_t(const keepkv_params &p, const keepkv_cache &src, const keepkv_cache &dst, const int32_t *ev_idx,
                            const UnitInfo *unit_info, const float *inv_norm, const uint4 *norm_ext, int32_t *sched, uint4 *nom,
                            int nom_chunks, int32_t *status_dev, LaunchCtx &ctx, unsigned long long *tri_best) {
-  constexpr int D = 128;
-  using SL = PairSmem<D>;
+  using SL = PairSmem;
   constexpr size_t smem_bytes = (size_t)SL::kBytes + 1024;
   static bool attr_done_dev[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
   if (!attr_done_dev[dev & 63]) {
-    cudaFuncSetAttribute(nominate_pair_kernel<D, kTri>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+    cudaFuncSetAttribute(nominate_pair_kernel<kTri>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
     attr_done_dev[dev & 63] = true;
   }
   CUtensorMap mapB;
-  if (!make_bf16_tiles_map(&mapB, dst.K, (uint64_t)p.B * p.H_kv * p.N_cap, D, kPairHalf)) {
+  if (!make_bf16_tiles_map(&mapB, dst.K, (uint64_t)p.B * p.H_kv * p.N_cap, kPairD, kPairHalf)) {
     if (ctx.err == cudaSuccess) ctx.err = cudaErrorInvalidValue;
     return;
   }
-  launch_pdl_cluster(nominate_pair_kernel<D, kTri>, dim3(sm_count() & ~1), dim3(kPairThreads), smem_bytes, ctx.stream, 2u, mapB, p,
+  launch_pdl_cluster(nominate_pair_kernel<kTri>, dim3(sm_count() & ~1), dim3(kPairThreads), smem_bytes, ctx.stream, 2u, mapB, p,
                      reinterpret_cast<const __nv_bfloat16 *>(src.K), ev_idx, unit_info, inv_norm, norm_ext, sched, nom, nom_chunks,
                      status_dev, tri_best, debug_spin_limit(), debug_withhold());
   KEEPKV_CHECK_LAUNCH(ctx);

@@ -1227,6 +1227,20 @@ def test_compress_rows_that_need_the_exact_cosines(d, n, budget, copies):
         check_compress_unit(p, u, budget, n_recent, hs, hd, ret, tgt, stats, what="exact")
 
 
+def test_search_by_pairs_of_ctas_walks_many_columns():
+    """Two units of 8000 entries, 6200 kept: a pair's columns run through the rings several times within an item."""
+    B, n, budget, n_recent = 2, 8000, 6200, 5000
+    p = kb.make_params(B=B, H_q=1, H_kv=1, d=128, N_cap=8064, n_sink=4, n_recent=n_recent, merge_threshold=0.7)
+    src = random_cache(p, [n, n - 129], seed=11, vote_max=3, scored_frac=1.0)
+    src.K.copy_(_similar_keys("centres", B, 8064, 128, seed=3).bfloat16().view(B, 1, 8064, 128))
+    src.lscore.mul_(0.25).add_(1.5)
+    dst, ret, tgt, stats = _run_compress(p, src, budget)
+    assert stats[:, kb.STATS_FIELDS.index("n_merged")].min() > 500
+    hs, hd = HostCache(src), HostCache(dst)
+    for u in range(B):
+        check_compress_unit(p, u, budget, n_recent, hs, hd, ret, tgt, stats, what="columns")
+
+
 def _similar_keys(kind, U, n, d, seed):
     """Keys [U, n, d] of which many pairs are similar: around common centres, along one direction (most cosines are above 0.8),
     repeated, with every ninth row zero, or with every fortieth above 0.5 to all others, which are below it to one another."""

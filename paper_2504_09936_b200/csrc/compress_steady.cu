@@ -114,12 +114,10 @@ steady_compress_kernel(const __grid_constant__ CUtensorMap mapD, keepkv_params p
 
   const int u = blockIdx.y, r = blockIdx.x, R = gridDim.x, b = u / p.H_kv, h = u % p.H_kv;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // Nobody writes to a CTA that has not started.  (What is written is set up by nobody before, so the arrival orders no memory: as
-  // a release the launch took 0.8-1.5 us longer, 40 us.)
+  // Nobody writes to a CTA that has not started: waited for in front of the first such write, and of every return.  (What is written
+  // is set up by nobody before, so the arrival orders no memory: as a release the launch took 0.8 us longer, 40 us.)
   if (kCluster) cluster_arrive_relaxed();
   if (tid == 0) prefetch_tensormap(&mapD);
-  __syncwarp();
-  if (kCluster) cluster_wait();
   pdl_wait();
   pdl_trigger();
   // ---- the sets of Algorithm 1, selection step, exactly as the general selection defines them
@@ -141,6 +139,8 @@ steady_compress_kernel(const __grid_constant__ CUtensorMap mapD, keepkv_params p
   const int m_cand = hi - lo, n_ret = min(len, budget), n_ev = len - n_ret;
   if (m_cand > kStCand || n_ev > kStEv || n_ret > kStRet) {
     if (r == 0 && tid == 0) atomicOr(status_dev, KEEPKV_DEV_NOT_STEADY);   // the promise does not hold here
+    __syncwarp();
+    if (kCluster) cluster_wait();
     return;
   }
   const size_t base = (size_t)u * p.N_cap;
@@ -225,6 +225,8 @@ steady_compress_kernel(const __grid_constant__ CUtensorMap mapD, keepkv_params p
     }
     __threadfence();
     st_arrive_all(3);   // these rows are in place
+    __syncwarp();
+    if (kCluster) cluster_wait();
     return;
   }
 
@@ -482,6 +484,8 @@ steady_compress_kernel(const __grid_constant__ CUtensorMap mapD, keepkv_params p
     mine.insert(__uint_as_float(v.y), (int)v.w);
   };
   if (kCluster) {
+    __syncwarp();
+    cluster_wait();                // every CTA of the unit has started
     if (tid < n_ev)
       st_shared_cluster_v4(mapa_shared(sbase + SL::kInbox + (r * per + tid / R) * 16, (uint32_t)(tid % R)), __float_as_uint(mine.best),
                            __float_as_uint(mine.second), (uint32_t)mine.bi, (uint32_t)mine.si);

@@ -665,6 +665,8 @@ static void launch_compress_t(const keepkv_params &p, const keepkv_cache &src, c
              merges ? norm_ext : nullptr);
   KEEPKV_CHECK_LAUNCH(ctx);
   if (!merges) return;
+  // (Budgets on the device are taken for a tenth of the capacity.  Where they are more, the form for smaller prompts is kept: 64 units
+  // 6000 -> 1800 in 6016 rows 181 us, 157 with the budget on the host; where less, pairs search few columns: 16000 -> 100 227, 225.)
   launch_nominate(p, src, dst, ev_idx, ui, inv_norm, norm_ext, sched, nom, L.nom_chunks, status_dev, ctx,
                   budget_dev ? p.N_cap / 10 : ret_bound);
   launch_pdl(resolve_kernel<D, false>, dim3(resolve_grid(p), U), dim3(kResolveThreads), 0, ctx.stream,

@@ -516,10 +516,11 @@ static void launch_nominate_t(const keepkv_params &p, const keepkv_cache &src, c
 
 // Large prompts go to pairs of CTAs (nominate_pair.cu).  The buffer's capacity stands for their length, which the host does not know;
 // columns: how many retained keys it expects a unit to have, 0 where most rows have none or few are evicted (in place).  The whole
-// call, this form against pairs, us, 8 and 64 units: 4096 -> 410 entries 46.2 / 47.4 and 101 / 110, 4096 -> 1229 52.1 / 52.6 and
-// 131 / 129, 6000 -> 600 52.5 / 53.8 and 141 / 146, 6000 -> 1800 61.5 / 60.4 and 213 / 191, 8100 -> 810 66.0 / 64.7 and 206 / 195,
-// 12000 -> 3600 124 / 115 and 602 / 531; all pairs of 2500 100 / 102 and 316 / 290, of 4096 130 / 123 and 548 / 474.  (64 channels:
-// 16 units of 20000 -> 4000 553 / 694.)
+// call, this form against pairs, us, 8 and 64 units: 4096 -> 819 entries 40.1 / 39.0 and 101 / 93, 4096 -> 1229 42.9 / 42.6 and
+// 109 / 103, 6000 -> 1800 50.3 / 48.0 and 181 / 155, 8192 -> 819 51.8 / 49.8 and 169 / 151, 8192 -> 1638 57.2 / 53.9 and 230 / 194,
+// 16384 -> 1638 (8 and 32 units) 94.6 / 85.1 and 250 / 209; merge-first of 4095 (8 units) and 6007 entries (32) 101 / 83 and 382 / 230.
+// What the capacity misjudges, a cache that evicts 128 entries out of a large buffer: 1766 -> 1638 30.4 / 31.9 and 54.2 / 54.2,
+// 1002 -> 874 29.1 / 30.6 and 40.6 / 41.4: half of a pair's rows do not exist.  (64 channels: 16 units of 20000 -> 4000 553 / 694.)
 bool nominate_pairs(const keepkv_params &p, int columns) {
   return p.d == 128 && p.merge_threshold >= kNomStatic && p.N_cap >= kNomPairCap && columns >= kNomPairColumns;
 }
